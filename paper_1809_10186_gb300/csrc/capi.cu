@@ -4,8 +4,8 @@
 // type, one device workspace sized for a chunk of nodes, and a device flag word. Every
 // compute call loops over node chunks and enqueues, per chunk,
 //   1. the translate products                  P_r = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)]
-//      (tensor cores for Q(f, f) of F16S/BF16S plans, tc_gain.cu; Fourier-space translates for every
-//      other call, k_vss.cu; the dense circulant kernel, k_gain_simt.cuh, for the allocation-free
+//      (tensor cores for the tensor-core plans, tc_gain.cu and tc_gain3.cu; Fourier-space translates for
+//      FP32/FP64 plans, k_shift.cu; the dense circulant kernel, k_gain_simt.cuh, for the allocation-free
 //      call of FP32/FP64 plans)
 //   2. the radial projection                   X_s = sum_r Vr[s][r] w_r rho_r P_r
 //   3. forward DFTs of X_s and the loss operand
@@ -32,6 +32,7 @@
 #include "../../include/dgfs.h"
 #include "launchers.h"
 #include "plan_host.h"
+#include "shift.h"
 #include "tc_gain.h"
 
 using namespace dgfs;
@@ -111,6 +112,8 @@ struct dgfs_plan_s {
     int64_t xchunk = 0;
     size_t off_Xt = 0;
     const void* d_mu = nullptr;   // [Nrho][npairs][3][N] complex multipliers (inside d_vss)
+    ShiftDev<float> shf;          // shared-shift program of the translate products (inside d_vss)
+    ShiftDev<double> shd;
     size_t off_V = 0, vss_bytes = 0;
     void* d_vss = nullptr;   // A [Nrho][npairs][N^3] (T) | GL [N^3] (T) | mu [Nrho][npairs][3][N] (complex T)
     int xfields = 0;
@@ -325,9 +328,54 @@ template <typename T> DevTables<T>& tables(dgfs_plan_s* p);
 template <> DevTables<float>& tables<float>(dgfs_plan_s* p) { return p->tf; }
 template <> DevTables<double>& tables<double>(dgfs_plan_s* p) { return p->td; }
 
+template <typename T> ShiftDev<T>& shift_dev(dgfs_plan_s* p);
+template <> ShiftDev<float>& shift_dev<float>(dgfs_plan_s* p) { return p->shf; }
+template <> ShiftDev<double>& shift_dev<double>(dgfs_plan_s* p) { return p->shd; }
+
+// Appends the shared-shift program to blob (16-byte aligned parts); the pointers of d hold offsets
+// until rebase_shift.
+template <typename T>
+void pack_shift(const ShiftProgram& sp, std::vector<unsigned char>& blob, ShiftDev<T>& d) {
+    auto put = [&](const void* src, size_t bytes) {
+        const size_t o = align_up(blob.size(), 16);
+        blob.resize(o + bytes);
+        if (bytes) std::memcpy(blob.data() + o, src, bytes);
+        return o;
+    };
+    std::vector<T> mu(sp.mu.begin(), sp.mu.end());
+    d.nrows = sp.nrows;
+    d.nx = sp.nx;
+    d.nquad = (int)sp.quad.size();
+    d.nbil = (int)sp.bil.size();
+    d.mu = reinterpret_cast<const Cplx<T>*>(put(mu.data(), mu.size() * sizeof(T)));
+    d.quad = reinterpret_cast<const ShiftEntry*>(put(sp.quad.data(), sp.quad.size() * sizeof(ShiftEntry)));
+    d.bil = reinterpret_cast<const ShiftEntry*>(put(sp.bil.data(), sp.bil.size() * sizeof(ShiftEntry)));
+    d.xrows = reinterpret_cast<const int*>(put(sp.xrows.data(), sp.xrows.size() * sizeof(int)));
+}
+
+template <typename T>
+void rebase_shift(ShiftDev<T>& d, const void* base) {
+    auto fix = [&](auto& ptr) {
+        using P = std::remove_reference_t<decltype(ptr)>;
+        ptr = reinterpret_cast<P>(static_cast<const unsigned char*>(base) + reinterpret_cast<uintptr_t>(ptr));
+    };
+    fix(d.mu); fix(d.quad); fix(d.bil); fix(d.xrows);
+}
+
 unsigned char* ws(dgfs_plan_s* p, size_t off) { return static_cast<unsigned char*>(p->d_ws) + off; }
 
-enum class Op { Collide, Collide2, Jvp, Dgamma, Vjp };
+// Step: Q(f, f) of an SSP-RK stage (dgfs_ssprk)
+enum class Op { Collide, Collide2, Jvp, Dgamma, Vjp, Step };
+
+constexpr bool quadratic(Op op) { return op == Op::Collide || op == Op::Dgamma || op == Op::Step; }
+
+// FP32 calls whose results are carried on in FP64 (the moments of a stepped state, the gradient of gamma
+// summed over a node) keep the rounding of the transform-per-pair products bit for bit: a run's
+// diagnostics stay comparable to 1e-9, which no other order of FP32 operations would give.
+template <typename T>
+constexpr bool keeps_rounding(Op op) {
+    return std::is_same<T, float>::value && (op == Op::Dgamma || op == Op::Step);
+}
 
 // The VSS kernel (alpha != 1): gain^ = scale sum_r sum_p A_rp DFT(products of the translates by
 // +-s_rp), one transform per radial and sphere point (k_vss.cu), in batches of vchunk nodes;
@@ -345,7 +393,7 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     // equal transform batches of at most vchunk nodes (no small ragged tail batch)
     const int64_t nbatch = (nodes + p->vchunk - 1) / std::max<int64_t>(1, p->vchunk);
     const int64_t C = nbatch > 0 ? (nodes + nbatch - 1) / nbatch : p->vchunk;
-    const bool two = op != Op::Collide;
+    const bool two = !quadratic(op);
     const int sets = two ? 2 : 1, yf = op == Op::Jvp ? 3 : 2;
     const T scale = op == Op::Jvp ? T(2) : T(1);
     const T* a = f;
@@ -368,8 +416,8 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
         if (!e) e = launch_vss_loss_init<T>(Fh, two ? Gh : Fh, GL, N, nn, Y, yf, s);
         if (e) return cuda_fail(e, "VSS operand transforms");
         for (int r = 0; r < Nr && !e; ++r) {
-            e = launch_vss_inverse_planes<T>(Fh, two ? Gh : nullptr, mu + (size_t)r * np * 3 * N, dftw, N, np, sets, nn,
-                                             Z, s);
+            e = launch_vss_inverse_planes<T>(Fh, two ? Gh : nullptr, mu + (size_t)r * np * 3 * N, dftw, N, np, sets, 1,
+                                             nn, Z, s);
             if (!e) e = launch_vss_lines<T>(Z, dftw, N, np, sets, nn, W, s);
             if (!e) e = launch_vss_forward_planes<T>(dftw, N, nw, nn, W, s);
             if (!e) e = launch_vss_accumulate<T>(W, A + (size_t)r * np * n3, N, np, nn, scale, Y, yf, s);
@@ -387,36 +435,76 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     return DGFS_OK;
 }
 
-// P[node][r] = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)] with the translates taken in Fourier
-// space (k_vss.cu: one complex inverse transform gives T_s f + i T_-s g), in batches of xchunk nodes;
-// the same P as the dense circulant passes of launch_gain_products at a fifth of the arithmetic.
+// P[node][r] = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)] with the translates taken in Fourier space,
+// the x and (x, y) translates that several sphere points share taken once (k_shift.cu). The spectra
+// of a batch of (node, radial point) items live in the xchunk region: every radial point of as many nodes
+// as fit, or (a plan with a small max_batch) as many radial points of one node as fit.
 template <typename T>
-cudaError_t fft_gain_products(dgfs_plan_s* p, const T* f, const T* g, const int64_t* offs, int64_t nodes, T* P,
-                              cudaStream_t s) {
+cudaError_t shift_gain_products(dgfs_plan_s* p, const T* f, const T* g, const int64_t* offs, int64_t nodes, T* P,
+                                cudaStream_t s) {
     const DevTables<T>& t = tables<T>(p);
-    const int N = t.N, np = t.npairs, Nr = t.Nrho, sets = g ? 2 : 1;
-    const int64_t n3 = (int64_t)N * N * N, C = p->xchunk;
-    Cplx<T>* Fh = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Xt));
-    Cplx<T>* Gh = Fh + C * n3;
-    Cplx<T>* Z = Gh + C * n3;
-    const Cplx<T>* mu = static_cast<const Cplx<T>*>(p->d_mu);
-    const Cplx<T>* dftw = reinterpret_cast<const Cplx<T>*>(t.dftw);
+    const ShiftDev<T>& d = shift_dev<T>(p);
+    const int N = t.N, Nr = t.Nrho, ops = g ? 2 : 1;
+    const int64_t n3 = (int64_t)N * N * N, field = n3 / 2;   // complex elements of a half-spectrum field
+    const int64_t cap = p->xchunk * (2 + 2 * (int64_t)t.npairs) * n3 / (field * ops);   // fields per operand
+    // one (node, r) always fits: 1 + 2 nx <= 1 + 2 npairs fields per operand, cap >= 2 + 2 npairs
+    int64_t C = std::min<int64_t>(cap / (1 + (int64_t)Nr * 2 * d.nx), 65535);
+    int R = Nr;
+    if (C < 1) {
+        C = 1;
+        R = (int)std::max<int64_t>(1, (cap - 1) / (2 * d.nx));
+    }
+    const int64_t nbatch = (nodes + C - 1) / C;
+    C = (nodes + nbatch - 1) / nbatch;   // equal batches
+    Cplx<T>* Gf = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Xt));
+    Cplx<T>* Gg = g ? Gf + C * field : nullptr;
+    Cplx<T>* Hf = Gf + ops * C * field;
+    Cplx<T>* Hg = g ? Hf + C * R * 2 * d.nx * field : nullptr;
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
         const int64_t nn = std::min<int64_t>(C, nodes - n0);
-        cudaError_t e = offs ? launch_vss_load_t<T>(f, offs + n0, N, nn, Fh, s)
-                             : launch_vss_load_t<T>(f + n0 * n3, nullptr, N, nn, Fh, s);
-        if (!e) e = launch_dft3<T>(t, Fh, nn, true, s);
-        if (!e && g) e = offs ? launch_vss_load_t<T>(g, offs + n0, N, nn, Gh, s)
-                              : launch_vss_load_t<T>(g + n0 * n3, nullptr, N, nn, Gh, s);
-        if (!e && g) e = launch_dft3<T>(t, Gh, nn, true, s);
-        for (int r = 0; r < Nr && !e; ++r) {
-            e = launch_vss_inverse_planes<T>(Fh, g ? Gh : nullptr, mu + (size_t)r * np * 3 * N, dftw, N, np, sets, nn,
-                                             Z, s);
-            if (!e) e = launch_vss_lines_sum<T>(Z, dftw, t.wsig, N, np, sets, nn, (int64_t)Nr * n3,
-                                                P + n0 * Nr * n3 + (int64_t)r * n3, s);
+        const int64_t fo = offs ? 0 : n0 * n3;
+        cudaError_t e = launch_shift_forward<T>(f + fo, offs ? offs + n0 : nullptr, N, nn, Gf, s);
+        if (!e && g) e = launch_shift_forward<T>(g + fo, offs ? offs + n0 : nullptr, N, nn, Gg, s);
+        for (int r0 = 0; r0 < Nr && !e; r0 += R) {
+            const int nr = std::min(R, Nr - r0);
+            e = launch_shift_x<T>(d, Gf, N, r0, nr, nn, Hf, s);
+            if (!e && g) e = launch_shift_x<T>(d, Gg, N, r0, nr, nn, Hg, s);
+            if (!e) e = launch_shift_products<T>(d, Gf, Hf, Gg, Hg, t.wsig, N, r0, nr, nn, (int64_t)Nr * n3,
+                                                 P + n0 * Nr * n3, s);
+            if (p->prof) p->prof_launches += (d.nx ? ops : 0) + 1;
         }
         if (e) return e;
-        if (p->prof) p->prof_launches += (g ? 8 : 4) + 2 * (int64_t)Nr;
+        if (p->prof) p->prof_launches += ops;
+    }
+    return cudaSuccess;
+}
+
+// P[node][r] of Q(f, f) with a transform of its own for every sphere pair (k_vss.cu; keeps_rounding above), in
+// batches of (node, radial point) items whose spectra fit the xchunk region: every radial point of as many
+// nodes as fit (one launch of each kernel for a small batch), or a part of the radial points.
+cudaError_t pair_gain_products(dgfs_plan_s* p, const float* f, int64_t nodes, float* P, cudaStream_t s) {
+    const DevTables<float>& t = p->tf;
+    const int N = t.N, np = t.npairs, Nr = t.Nrho;
+    const int64_t n3 = (int64_t)N * N * N, cap = p->xchunk * (2 + 2 * (int64_t)np);   // complex fields
+    Cplx<float>* Fh = reinterpret_cast<Cplx<float>*>(ws(p, p->off_Xt));
+    const Cplx<float>* mu = static_cast<const Cplx<float>*>(p->d_mu);
+    const Cplx<float>* dftw = reinterpret_cast<const Cplx<float>*>(t.dftw);
+    const int64_t C = std::min<int64_t>(nodes, p->xchunk);
+    const int R = (int)std::max<int64_t>(1, std::min<int64_t>({Nr, (cap - C) / (C * np), 65535 / C}));
+    Cplx<float>* Z = Fh + C * n3;
+    for (int64_t n0 = 0; n0 < nodes; n0 += C) {
+        const int64_t nn = std::min<int64_t>(C, nodes - n0);
+        cudaError_t e = launch_vss_load_t<float>(f + n0 * n3, nullptr, N, nn, Fh, s);
+        if (!e) e = launch_dft3<float>(t, Fh, nn, true, s);
+        for (int r = 0; r < Nr && !e; r += R) {
+            const int nr = std::min(R, Nr - r);
+            e = launch_vss_inverse_planes<float>(Fh, nullptr, mu + (size_t)r * np * 3 * N, dftw, N, np, 1, nr, nn, Z, s);
+            if (!e) e = launch_vss_lines_sum<float>(Z, dftw, t.wsig, N, np, nr, nn, (int64_t)Nr * n3,
+                                                    P + n0 * Nr * n3 + (int64_t)r * n3, s);
+            if (p->prof) p->prof_launches += 2;
+        }
+        if (e) return e;
+        if (p->prof) p->prof_launches += 4;
     }
     return cudaSuccess;
 }
@@ -442,7 +530,7 @@ cudaError_t fft_vjp_products(dgfs_plan_s* p, const T* f, const T* U, int64_t nod
         if (!e) e = cudaMemsetAsync(Gh, 0, (size_t)nn * n3 * sizeof(Cplx<T>), s);
         for (int r = 0; r < Nr && !e; ++r) {
             const Cplx<T>* mu_r = mu + (size_t)r * np * 3 * N;
-            e = launch_vss_inverse_planes<T>(Fh, nullptr, mu_r, dftw, N, np, 1, nn, Z, s);
+            e = launch_vss_inverse_planes<T>(Fh, nullptr, mu_r, dftw, N, np, 1, 1, nn, Z, s);
             if (!e) e = launch_vjp_lines<T>(Z, U + n0 * Nr * n3 + (int64_t)r * n3, (int64_t)Nr * n3, dftw, N, np, nn, W, s);
             if (!e) e = launch_vss_forward_planes<T>(dftw, N, np, nn, W, s);
             if (!e) e = launch_vjp_accumulate<T>(W, mu_r, t.wsig, N, np, nn, Gh, s);
@@ -495,7 +583,7 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
         return DGFS_OK;
     }
     // gain products: Q(f,f) and dQ/dgamma use (f, f); Q(f,g) uses (f, g); JVP uses (f, v)
-    const T* gg = (op == Op::Collide || op == Op::Dgamma) ? nullptr : g;
+    const T* gg = quadratic(op) ? nullptr : g;
     NvtxRange translate_range("dgfs translate products");
     if (p->prof) {
         p->prof_launches += (spectral_supported(tables<T>(p)) ? 5 : 11 + (op == Op::Jvp ? 1 : 0)) +
@@ -523,7 +611,10 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
                                             reinterpret_cast<float*>(P), p->d_flags, s, 0, coef + nodes, 1);
         if (p->prof) p->prof_launches += 2;
     } else if (p->fftx) {
-        e = fft_gain_products<T>(p, f, gg, offs, nodes, P, s);
+        if constexpr (std::is_same<T, float>::value)
+            e = keeps_rounding<T>(op) ? pair_gain_products(p, f, nodes, P, s) : shift_gain_products<T>(p, f, gg, offs, nodes, P, s);
+        else
+            e = shift_gain_products<T>(p, f, gg, offs, nodes, P, s);
     } else {
         e = launch_gain_products(t, f, gg, offs, nodes, P, s);
     }
@@ -537,7 +628,7 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     // real fields packed two per complex slot: the rank projected fields, then the loss
     // operand(s): Q(f,g) -> field rank = g;  JVP -> field rank = v, field rank + 1 = f
     if (spectral_supported(t)) {   // the fused three-launch Fourier stage
-        const T* la = (op == Op::Collide || op == Op::Dgamma) ? f : g;
+        const T* la = quadratic(op) ? f : g;
         e = launch_spectral<T>(t, P, np, nodes, la, op == Op::Jvp ? f : nullptr, offs,
                                op == Op::Jvp ? T(2) : T(1), X, Y, f, op == Op::Jvp ? g : nullptr, out,
                                p->d_flags, s);
@@ -547,7 +638,7 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     const int nfields = rank + (op == Op::Jvp ? 2 : 1), xs = (nfields + 1) / 2;
     e = launch_project<T>(t, P, np, nodes, X, xs, s);
     if (e) return cuda_fail(e, "radial projection");
-    const T* loss0 = (op == Op::Collide || op == Op::Dgamma) ? f : g;
+    const T* loss0 = quadratic(op) ? f : g;
     e = launch_load_field<T>(t.N, loss0, nullptr, offs, nodes, X, xs, rank / 2, rank % 2, s);
     if (!e && op == Op::Jvp) e = launch_load_field<T>(t.N, f, nullptr, offs, nodes, X, xs, (rank + 1) / 2, (rank + 1) % 2, s);
     if (e) return cuda_fail(e, "loss operand");
@@ -709,6 +800,10 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
             if (es == 8) reinterpret_cast<double*>(mblob.data())[i] = p->hp.mu[i];
             else reinterpret_cast<float*>(mblob.data())[i] = (float)p->hp.mu[i];
         }
+        ShiftProgram sp;
+        build_shift_program(p->hp, sp);
+        if (es == 8) pack_shift(sp, mblob, p->shd);
+        else pack_shift(sp, mblob, p->shf);
         cudaError_t ev = cudaMalloc(&p->d_vss, mblob.size());
         if (ev != cudaSuccess) return fail(DGFS_ERR_OOM, std::string("translate multipliers: ") + cudaGetErrorString(ev));
         ev = cudaMemcpy(p->d_vss, mblob.data(), mblob.size(), cudaMemcpyHostToDevice);
@@ -718,6 +813,8 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
         }
         p->vss_bytes = mblob.size();
         p->d_mu = p->d_vss;
+        if (es == 8) rebase_shift(p->shd, p->d_vss);
+        else rebase_shift(p->shf, p->d_vss);
     }
     cudaError_t e = cudaMalloc(&p->d_tables, p->table_bytes + tc_bytes);
     if (e != cudaSuccess) {
@@ -1088,18 +1185,18 @@ dgfs_status ssprk_run(dgfs_plan_s* p, int order, T* f, int64_t B, double dt, dou
         const int64_t nn = std::min<int64_t>(p->chunk, B - n0), n = nn * n3;
         T* u = f + n0 * n3;
         for (int it = 0; it < nsteps; ++it) {
-            dgfs_status st = run_chunk<T>(p, Op::Collide, u, nullptr, q, nullptr, np, nn, s);
+            dgfs_status st = run_chunk<T>(p, Op::Step, u, nullptr, q, nullptr, np, nn, s);
             if (st != DGFS_OK) return st;
             cudaError_t e = launch_rk_combine<T>(n, 1.0, u, 0.0, nullptr, h, q, stage, p->d_flags, s);
             if (e) return cuda_fail(e, "SSP-RK stage");
-            st = run_chunk<T>(p, Op::Collide, stage, nullptr, q, nullptr, np, nn, s);
+            st = run_chunk<T>(p, Op::Step, stage, nullptr, q, nullptr, np, nn, s);
             if (st != DGFS_OK) return st;
             if (order == 2) {
                 e = launch_rk_combine<T>(n, 0.5, u, 0.5, stage, 0.5 * h, q, u, p->d_flags, s);
             } else {
                 e = launch_rk_combine<T>(n, 0.75, u, 0.25, stage, 0.25 * h, q, stage, p->d_flags, s);
                 if (!e) {
-                    st = run_chunk<T>(p, Op::Collide, stage, nullptr, q, nullptr, np, nn, s);
+                    st = run_chunk<T>(p, Op::Step, stage, nullptr, q, nullptr, np, nn, s);
                     if (st != DGFS_OK) return st;
                     e = launch_rk_combine<T>(n, 1.0 / 3.0, u, 2.0 / 3.0, stage, 2.0 / 3.0 * h, q, u, p->d_flags, s);
                 }

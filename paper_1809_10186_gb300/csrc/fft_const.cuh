@@ -1,0 +1,163 @@
+// FFT lines in registers with compile-time twiddles, for the lengths of the velocity grid
+// (8, 16, 32 and 12, 24 = 3 * 2^m). Decimation in time: element k of a line goes into slot
+// line_slot<N>(k) (fourier_dev.cuh), the result is in natural order, unnormalised.
+//
+// A butterfly with a twiddle w other than 1 and -+i takes six fused multiply-adds,
+//   s = u + w v (two chains of two),  d = 2 u - s,
+// instead of two products, two FMAs and four additions; d carries the rounding of s, which is of
+// the size of its own. The twiddles are immediate operands, so a line loads nothing but its data:
+// 388 instructions for N = 32.
+#pragma once
+
+#include "fourier_dev.cuh"
+
+namespace dgfs {
+namespace cfft {
+
+using fdev::bitrev;
+using fdev::line_slot;
+
+// cos(2 pi m / 32), m = 0 .. 8, and cos(2 pi m / 24), m = 0 .. 6; other angles by symmetry
+__host__ __device__ constexpr double quarter32(int m) {
+    return m == 0 ? 1.0
+         : m == 1 ? 0.980785280403230449126182236134239037
+         : m == 2 ? 0.923879532511286756128183189396788287
+         : m == 3 ? 0.831469612302545237078788377617905757
+         : m == 4 ? 0.707106781186547524400844362104849039
+         : m == 5 ? 0.555570233019602224742830813948532874
+         : m == 6 ? 0.382683432365089771728459984030398867
+         : m == 7 ? 0.195090322016128267848284868477022241
+         : 0.0;
+}
+__host__ __device__ constexpr double quarter24(int m) {
+    return m == 0 ? 1.0
+         : m == 1 ? 0.965925826289068286749743199728897368
+         : m == 2 ? 0.866025403784438646763723170752936183
+         : m == 3 ? 0.707106781186547524400844362104849039
+         : m == 4 ? 0.5
+         : m == 5 ? 0.258819045102520762348898837624048328
+         : 0.0;
+}
+// cos(2 pi m / D) for D dividing 32 or 24
+template <int D>
+__host__ __device__ constexpr double cos_of(int m) {
+    constexpr int B = 32 % D == 0 ? 32 : 24, Q = B / 4;
+    m = ((m * (B / D)) % B + B) % B;
+    const int h = m <= 2 * Q ? m : B - m;                      // cos is even
+    const int q = h <= Q ? h : 2 * Q - h;
+    const double c = B == 32 ? quarter32(q) : quarter24(q);
+    return h <= Q ? c : -c;
+}
+template <int D>
+__host__ __device__ constexpr double sin_of(int m) {
+    constexpr int B = 32 % D == 0 ? 32 : 24;
+    return cos_of<B>(m * (B / D) - B / 4);
+}
+
+// u + v, u - v and 2 u - s of complex values. In FP32 both parts go through one packed instruction
+// (f32x2, each half rounded as the scalar operation): the lines are bound by instruction issue.
+template <typename T>
+__device__ __forceinline__ Cplx<T> add(Cplx<T> u, Cplx<T> v) { return Cplx<T>{u.x + v.x, u.y + v.y}; }
+template <typename T>
+__device__ __forceinline__ Cplx<T> sub(Cplx<T> u, Cplx<T> v) { return Cplx<T>{u.x - v.x, u.y - v.y}; }
+template <typename T>
+__device__ __forceinline__ Cplx<T> twice_minus(Cplx<T> u, Cplx<T> s) {
+    return Cplx<T>{fma(T(2), u.x, -s.x), fma(T(2), u.y, -s.y)};
+}
+__device__ __forceinline__ unsigned long long pack(Cplx<float> a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ Cplx<float> unpack(unsigned long long r) {
+    Cplx<float> a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+template <>
+__device__ __forceinline__ Cplx<float> add<float>(Cplx<float> u, Cplx<float> v) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack(u)), "l"(pack(v)));
+    return unpack(r);
+}
+template <>
+__device__ __forceinline__ Cplx<float> sub<float>(Cplx<float> u, Cplx<float> v) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack(u)), "l"(pack(v)));
+    return unpack(r);
+}
+template <>
+__device__ __forceinline__ Cplx<float> twice_minus<float>(Cplx<float> u, Cplx<float> s) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack(u)), "l"(pack(Cplx<float>{2.f, 2.f})),
+        "l"(pack(Cplx<float>{-s.x, -s.y})));
+    return unpack(r);
+}
+
+// radix-2 stages of a length-S transform in a[OFF .. OFF + S), spans LEN, 2 LEN, ..., S
+template <typename T, int NA, int OFF, int S, int LEN, bool FWD>
+__device__ __forceinline__ void stages(Cplx<T> (&a)[NA]) {
+    constexpr int half = LEN / 2;
+#pragma unroll
+    for (int i = 0; i < S; i += LEN)
+#pragma unroll
+        for (int j = 0; j < half; ++j) {
+            const Cplx<T> u = a[OFF + i + j], v = a[OFF + i + j + half];
+            Cplx<T> s, d;
+            if (j == 0) {
+                s = add(u, v);
+                d = sub(u, v);
+            } else if (4 * j == LEN) {                         // twiddle -i (forward), +i (inverse)
+                const T sg = FWD ? T(1) : T(-1);
+                s = Cplx<T>{u.x + sg * v.y, u.y - sg * v.x};
+                d = Cplx<T>{u.x - sg * v.y, u.y + sg * v.x};
+            } else {
+                const T wr = (T)cos_of<LEN>(j), wi = FWD ? (T)(-sin_of<LEN>(j)) : (T)sin_of<LEN>(j);
+                s = Cplx<T>{fma(-wi, v.y, fma(wr, v.x, u.x)), fma(wi, v.x, fma(wr, v.y, u.y))};
+                d = twice_minus(u, s);
+            }
+            a[OFF + i + j] = s;
+            a[OFF + i + j + half] = d;
+        }
+    if constexpr (LEN < S) stages<T, NA, OFF, S, 2 * LEN, FWD>(a);
+}
+
+template <typename T, int N, bool FWD>
+__device__ __forceinline__ void line(Cplx<T> (&a)[N]) {
+    if constexpr ((N & (N - 1)) == 0) {
+        stages<T, N, 0, N, 2, FWD>(a);
+    } else {
+        constexpr int S = N / 3;
+        static_assert(N == 12 || N == 24, "lengths 8, 12, 16, 24 and 32");
+        stages<T, N, 0, S, 2, FWD>(a);
+        stages<T, N, S, S, 2, FWD>(a);
+        stages<T, N, 2 * S, S, 2, FWD>(a);
+        // X[q + m S], m = 0, 1, 2, from y0 and the twiddled y1, y2 (one radix-3 butterfly)
+        const T c3 = FWD ? (T)(-quarter24(2)) : (T)quarter24(2);   // -+ sin(2 pi / 3)
+#pragma unroll
+        for (int q = 0; q < S; ++q) {
+            const Cplx<T> y0 = a[q], y1 = a[S + q], y2 = a[2 * S + q];
+            Cplx<T> t1 = y1, t2 = y2;
+            if (q > 0) {
+                const T r1 = (T)cos_of<N>(q), i1 = FWD ? (T)(-sin_of<N>(q)) : (T)sin_of<N>(q);
+                const T r2 = (T)cos_of<N>(2 * q), i2 = FWD ? (T)(-sin_of<N>(2 * q)) : (T)sin_of<N>(2 * q);
+                t1 = Cplx<T>{fma(-i1, y1.y, r1 * y1.x), fma(i1, y1.x, r1 * y1.y)};
+                t2 = Cplx<T>{fma(-i2, y2.y, r2 * y2.x), fma(i2, y2.x, r2 * y2.y)};
+            }
+            const Cplx<T> p{t1.x + t2.x, t1.y + t2.y}, d{t1.x - t2.x, t1.y - t2.y};
+            const Cplx<T> m{fma(T(-0.5), p.x, y0.x), fma(T(-0.5), p.y, y0.y)};
+            a[q] = Cplx<T>{y0.x + p.x, y0.y + p.y};
+            a[S + q] = Cplx<T>{fma(-c3, d.y, m.x), fma(c3, d.x, m.y)};
+            a[2 * S + q] = Cplx<T>{fma(c3, d.y, m.x), fma(-c3, d.x, m.y)};
+        }
+    }
+}
+
+// 1 - (mean diagonal of inverse times forward line / N) with the twiddles rounded to FP32, the rest exact:
+// the relative loss of a round trip. |w| of the rounded twiddles of these lengths is below 1 on average.
+__host__ __device__ constexpr double line_loss(int N) {
+    return N == 8 ? 0.86e-8 : N == 12 ? 2.09e-8 : N == 16 ? 2.71e-8 : N == 24 ? 3.32e-8 : 4.55e-8;
+}
+
+}  // namespace cfft
+}  // namespace dgfs

@@ -1,0 +1,452 @@
+// Translate products of the CUDA-core plans (FP32, FP64; arXiv:1809.10186, Appendix eq. lowrank1):
+//   P_r = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)],   s = c_r sigma_p / 2,
+// with the translates taken in Fourier space, one axis after the other, and every translate that
+// several sphere points share taken once. T_s is separable, T_s = X(s_x) Y(s_y) Z(s_z), and the points
+// of a symmetric rule have few distinct components: the 38 points of M = 38 have 8 nonzero signed s_x
+// and 25 distinct (s_x, s_y). Per radial point, in lines of one axis (complex, N points; the spectra of
+// real fields are kept for kz >= 0 only), a separate transform per pair took 57 N^2 lines; this takes
+// 4 N^2 (x) + 12.5 N^2 (y) + 19 N^2 (z; T_s f + i T_-s g share one line).
+//
+//   k_shift_forward   (y, z) spectra of every x plane of f                                  -> G
+//   k_shift_x         x spectra, then per r and signed s_x: phase, inverse x transform      -> H
+//   k_shift_products  per (node, r, XC planes x): per (s_x, s_y): phase, inverse y transform into
+//                     shared memory; per pair: phase, inverse z transform of one line per thread,
+//                     product summed in registers; P_r written once
+//
+// Measured (GB300, FP32, N = 32, M = 38, 256 nodes, whole Q): 8.4 ms, 22.2 ms with a transform of its own
+// per pair (two launches per radial point, 9.5 MB of spectra through DRAM per radial point and node
+// against 2.2 MB here); N = 16, M = 6, FP64, one node: 0.20 ms, 0.97 ms before. k_shift_products takes 73 %
+// of the FP32 step: 70 % of the issue slots and 56 % of the FMA pipe (ncu, 40 nodes); k_shift_x 15 %, at
+// 81 % of the DRAM throughput.
+//
+// Half spectra: kz = 0 .. N/2 - 1, with the spectra of kz = 0 and kz = N/2 (both of real (x, y)
+// fields, which x and y translates keep real) in the real and imaginary part of slot kz = 0.
+#include <algorithm>
+#include <map>
+
+#include "fft_const.cuh"
+#include "shift.h"
+
+namespace dgfs {
+
+void build_shift_program(const HostPlan& h, ShiftProgram& p) {
+    const int N = h.N, np = h.npairs, MP = shift_mu_pitch(N);
+    p = ShiftProgram();
+    std::map<double, int> rows, xs;
+    std::vector<std::pair<int, int>> at;   // a (pair, axis) that carries each row
+    for (int q = 0; q < np; ++q)
+        for (int a = 0; a < 3; ++a) {
+            const double v = std::fabs(h.sig[3 * q + a]);
+            if (v == 0.0) continue;
+            if (rows.emplace(v, (int)rows.size()).second) at.push_back({q, a});
+            if (a == 0 && xs.emplace(v, (int)xs.size()).second) p.xrows.push_back(rows[v]);
+        }
+    p.nrows = (int)rows.size();
+    p.nx = (int)xs.size();
+    p.mu.assign((size_t)h.Nrho * p.nrows * MP * 2, 0.0);
+    for (int r = 0; r < h.Nrho; ++r)
+        for (int d = 0; d < p.nrows; ++d) {
+            const double* m = &h.mu[(((size_t)r * np + at[d].first) * 3 + at[d].second) * N * 2];
+            const double sg = h.sig[3 * at[d].first + at[d].second] < 0 ? -1.0 : 1.0;
+            double* o = &p.mu[((size_t)r * p.nrows + d) * MP * 2];
+            for (int k = 0; k <= N / 2; ++k) {
+                o[2 * k] = m[2 * k];
+                o[2 * k + 1] = k == N / 2 ? 0.0 : sg * m[2 * k + 1];
+            }
+        }
+    struct Key { double x, y, z; int q; };
+    auto program = [&](bool both) {
+        std::vector<Key> keys;
+        for (int q = 0; q < np; ++q)
+            for (int sg = 1; sg >= (both ? -1 : 1); sg -= 2)
+                keys.push_back({sg * h.sig[3 * q], sg * h.sig[3 * q + 1], sg * h.sig[3 * q + 2], q});
+        std::stable_sort(keys.begin(), keys.end(),
+                         [](const Key& a, const Key& b) { return a.x != b.x ? a.x < b.x : a.y < b.y; });
+        std::vector<ShiftEntry> out;
+        for (size_t i = 0; i < keys.size(); ++i) {
+            const Key& k = keys[i];
+            auto row = [&](double v) { return v == 0.0 ? -1 : rows[std::fabs(v)]; };
+            const int fx = k.x == 0.0 ? -1 : 2 * xs[std::fabs(k.x)], neg = k.x < 0;
+            out.push_back({fx < 0 ? -1 : fx + neg, fx < 0 ? -1 : fx + 1 - neg, row(k.y), k.y < 0, row(k.z), k.z < 0, k.q,
+                           i == 0 || k.x != keys[i - 1].x || k.y != keys[i - 1].y});
+        }
+        return out;
+    };
+    p.quad = program(false);
+    p.bil = program(true);
+}
+
+namespace {
+
+using fdev::line_slot;
+
+template <typename T> struct Pair2;
+template <> struct Pair2<float> { using type = float2; };
+template <> struct Pair2<double> { using type = double2; };
+template <typename T>
+__device__ __forceinline__ Cplx<T> ld(const Cplx<T>* p) {
+    const typename Pair2<T>::type v = *reinterpret_cast<const typename Pair2<T>::type*>(p);
+    return Cplx<T>{v.x, v.y};
+}
+template <typename T>
+__device__ __forceinline__ Cplx<T> ldg(const Cplx<T>* p) {
+    const typename Pair2<T>::type v = __ldg(reinterpret_cast<const typename Pair2<T>::type*>(p));
+    return Cplx<T>{v.x, v.y};
+}
+template <typename T>
+__device__ __forceinline__ void st(Cplx<T>* p, Cplx<T> c) {
+    typename Pair2<T>::type v;
+    v.x = c.x;
+    v.y = c.y;
+    *reinterpret_cast<typename Pair2<T>::type*>(p) = v;
+}
+
+// two consecutive complex values from an even index (one 16-byte access in FP32)
+template <bool GLOBAL>
+__device__ __forceinline__ void ld_two(const Cplx<float>* p, Cplx<float>& a, Cplx<float>& b) {
+    const float4 v = GLOBAL ? __ldg(reinterpret_cast<const float4*>(p)) : *reinterpret_cast<const float4*>(p);
+    a = Cplx<float>{v.x, v.y};
+    b = Cplx<float>{v.z, v.w};
+}
+template <bool GLOBAL>
+__device__ __forceinline__ void ld_two(const Cplx<double>* p, Cplx<double>& a, Cplx<double>& b) {
+    a = GLOBAL ? ldg(p) : ld(p);
+    b = GLOBAL ? ldg(p + 1) : ld(p + 1);
+}
+
+template <typename T>
+__device__ __forceinline__ Cplx<T> cmul(Cplx<T> a, T br, T bi) {
+    return Cplx<T>{fma(-a.y, bi, a.x * br), fma(a.x, bi, a.y * br)};
+}
+
+// ---- forward (y, z) spectra ------------------------------------------------------------------
+
+template <int N>
+struct ForwardGeo {
+    // planes per CTA, N/2 lines each: about one warp, so that one node already spreads over many SMs
+    static constexpr int PX = N == 32 ? 2 : N == 12 ? 6 : N == 8 ? 8 : 4;
+    static constexpr int NT = PX * N / 2;
+    static constexpr int PITCH = N / 2 + 1;
+};
+
+// grid (N / PX, nodes). Lines along z of rows y and y + N/2 as real and imaginary part, separated into
+// half spectra; then lines along y of every slot kz.
+template <typename T, int N>
+__global__ void __launch_bounds__(ForwardGeo<N>::NT)
+k_shift_forward(const T* __restrict__ f, const int64_t* __restrict__ offs, Cplx<T>* __restrict__ G) {
+    using Geo = ForwardGeo<N>;
+    constexpr int NH = N / 2, PX = Geo::PX, NT = Geo::NT, PITCH = Geo::PITCH;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    T* rows = reinterpret_cast<T*>(sm_raw);                // [PX][N][N + 1], then S overwrites it
+    Cplx<T>* S = reinterpret_cast<Cplx<T>*>(sm_raw);       // [PX][N][PITCH]
+    const int tid = threadIdx.x, x0 = blockIdx.x * PX, pl = tid / NH, j = tid % NH;
+    const int64_t node = blockIdx.y, n3 = (int64_t)N * N * N;
+    const T* fn = f + (offs ? offs[node] : node * n3) + (int64_t)x0 * N * N;
+    for (int e = tid; e < PX * N * N; e += NT) rows[(e / N) * (N + 1) + e % N] = fn[e];
+    __syncthreads();
+    Cplx<T> v[N];
+#pragma unroll
+    for (int z = 0; z < N; ++z)
+        v[line_slot<N>(z)] = Cplx<T>{rows[(pl * N + j) * (N + 1) + z], rows[(pl * N + j + NH) * (N + 1) + z]};
+    __syncthreads();
+    cfft::line<T, N, true>(v);
+    Cplx<T>* a = S + (pl * N + j) * PITCH;
+    Cplx<T>* b = a + NH * PITCH;
+    st(a, Cplx<T>{v[0].x, v[NH].x});
+    st(b, Cplx<T>{v[0].y, v[NH].y});
+#pragma unroll
+    for (int k = 1; k < NH; ++k) {
+        const Cplx<T> p = v[k], m = v[N - k];
+        st(a + k, Cplx<T>{T(0.5) * (p.x + m.x), T(0.5) * (p.y - m.y)});
+        st(b + k, Cplx<T>{T(0.5) * (p.y + m.y), T(0.5) * (m.x - p.x)});
+    }
+    __syncthreads();
+#pragma unroll
+    for (int y = 0; y < N; ++y) v[line_slot<N>(y)] = ld(S + (pl * N + y) * PITCH + j);   // slot kz = j
+    cfft::line<T, N, true>(v);
+    const T sc = T(1) / (T(N) * T(N));
+    Cplx<T>* g = G + node * (n3 / 2) + (int64_t)(x0 + pl) * N * NH + j;
+#pragma unroll
+    for (int k = 0; k < N; ++k) st(g + k * NH, Cplx<T>{sc * v[k].x, sc * v[k].y});
+}
+
+// ---- x translates ----------------------------------------------------------------------------
+
+// One thread per column (ky, kz): the x spectrum of its line once, then for r = r0 + blockIdx.z RG .. and
+// every signed x shift the phase and the inverse transform. grid (ceil(N^2 / 2 / NT), nodes, ceil(nr / RG)).
+// Bound by its stores of H (1 MB per radial point and node at N = 32, M = 38).
+template <typename T, int N, int NT>
+__global__ void __launch_bounds__(NT)
+k_shift_x(const Cplx<T>* __restrict__ G, const Cplx<T>* __restrict__ mu, const int* __restrict__ xrows, int nrows, int nx,
+          int r0, int nr, int RG, Cplx<T>* __restrict__ H) {
+    constexpr int NH = N / 2, COLS = N * NH, MP = shift_mu_pitch(N);
+    constexpr int64_t FS = (int64_t)N * COLS;                // one half-spectrum field
+    const int c = blockIdx.x * NT + threadIdx.x;
+    if (c >= COLS) return;
+    const int64_t node = blockIdx.y;
+    Cplx<T> F[N];
+    const Cplx<T>* g = G + node * FS + c;
+#pragma unroll
+    for (int x = 0; x < N; ++x) F[line_slot<N>(x)] = ldg(g + (int64_t)x * COLS);
+    cfft::line<T, N, true>(F);
+    const T sc = T(1) / T(N);
+#pragma unroll
+    for (int k = 0; k < N; ++k) F[k] = Cplx<T>{sc * F[k].x, sc * F[k].y};
+    const int rl1 = min(nr, (int)(blockIdx.z + 1) * RG);
+    for (int rl = blockIdx.z * RG; rl < rl1; ++rl) {
+        Cplx<T>* h = H + (node * nr + rl) * (2 * nx) * FS + c;
+        for (int fi = 0; fi < 2 * nx; ++fi, h += FS) {
+            const Cplx<T>* m = mu + ((int64_t)(r0 + rl) * nrows + __ldg(xrows + (fi >> 1))) * MP;
+            const T sg = fi & 1 ? T(-1) : T(1);
+            Cplx<T> v[N];
+            v[0] = F[0];
+#pragma unroll
+            for (int k = 1; k < NH; ++k) {
+                const Cplx<T> w = ldg(m + k);
+                v[line_slot<N>(k)] = cmul(F[k], w.x, sg * w.y);
+                v[line_slot<N>(N - k)] = cmul(F[N - k], w.x, -sg * w.y);
+            }
+            const T wn = ldg(m + NH).x;
+            v[line_slot<N>(NH)] = Cplx<T>{F[NH].x * wn, F[NH].y * wn};
+            cfft::line<T, N, false>(v);
+#pragma unroll
+            for (int x = 0; x < N; ++x) st(h + (int64_t)x * COLS, v[x]);
+        }
+    }
+}
+
+// ---- y and z translates, products ------------------------------------------------------------
+
+// Row pitch (complex elements) of the y-translated fields in shared memory: a thread's kz row starts
+// 16-byte aligned and eight consecutive rows fall into different 16-byte bank groups.
+template <typename T, int N>
+__host__ __device__ constexpr int row_pitch() {
+    if (sizeof(T) == 8) return N / 2 + 1;
+    return N == 32 ? 18 : N == 24 ? 14 : N == 16 ? 10 : 6;
+}
+
+template <typename T, int N, int XC>
+struct ProductGeo {
+    static constexpr int NT = XC * N;                        // z lines; y lines: 2 XC N / 2
+    static constexpr int PITCH = row_pitch<T, N>();
+    static constexpr size_t smem = (size_t)2 * XC * N * PITCH * sizeof(Cplx<T>);
+    // resident CTAs the registers are budgeted for (a line and its sums are 96 values at N = 32: with four
+    // CTAs of 128 threads it spilled 100 bytes and measured 1 % slower than with three)
+    static constexpr int MINB = sizeof(T) == 8 ? 1 : N == 32 ? 384 / NT : N == 24 ? 480 / NT : 768 / NT;
+};
+
+// grid (N / XC, nr, nodes); H [node][r][2 nx fields][x][ky][kz], G [node][x][ky][kz]
+template <typename T, int N, int XC>
+__global__ void __launch_bounds__(ProductGeo<T, N, XC>::NT, ProductGeo<T, N, XC>::MINB)
+k_shift_products(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, const Cplx<T>* __restrict__ Gg,
+                 const Cplx<T>* __restrict__ Hg, const Cplx<T>* __restrict__ mu, const ShiftEntry* __restrict__ prog,
+                 int nprog, T wscale, const T* __restrict__ wsig, int nrows, int nx, int r0, int64_t node_stride,
+                 T* __restrict__ P) {
+    using Geo = ProductGeo<T, N, XC>;
+    constexpr int NH = N / 2, PITCH = Geo::PITCH, NT = Geo::NT, MP = shift_mu_pitch(N);
+    constexpr int64_t FS = (int64_t)N * N * NH, n3 = (int64_t)N * N * N;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    Cplx<T>* Y = reinterpret_cast<Cplx<T>*>(sm_raw);         // [sign][XC][y][PITCH]
+    const int tid = threadIdx.x, x0 = blockIdx.x * XC, rl = blockIdx.y, nr = gridDim.y;
+    const int64_t node = blockIdx.z;
+    // this thread's y line: operand (0: +s of f, 1: -s of g), plane, kz
+    const int op = tid / (XC * NH), ypl = (tid / NH) % XC, ykz = tid % NH;
+    const int64_t ybase = (int64_t)(x0 + ypl) * N * NH + ykz;
+    const Cplx<T>* Gy = (op ? Gg : Gf) + node * FS + ybase;
+    const Cplx<T>* Hy = (op ? Hg : Hf) + (node * nr + rl) * (2 * nx) * FS + ybase;
+    Cplx<T>* ydst = Y + ((op * XC + ypl) * N) * PITCH + ykz;
+    // this thread's z line: plane tid / N, y = tid % N
+    const Cplx<T>* zp = Y + tid * PITCH;
+    const Cplx<T>* zm = Y + (NT + tid) * PITCH;
+    const Cplx<T>* mu_r = mu + (int64_t)(r0 + rl) * nrows * MP;
+    T acc[N];
+#pragma unroll
+    for (int z = 0; z < N; ++z) acc[z] = T(0);
+    Cplx<T> v[N];
+    for (int i = 0; i < nprog; ++i) {
+        const ShiftEntry e = prog[i];
+        if (e.newy) {
+            const int fi = op ? e.fm : e.fp;
+            const Cplx<T>* src = fi < 0 ? Gy : Hy + fi * FS;
+#pragma unroll
+            for (int k = 0; k < N; ++k) v[line_slot<N>(k)] = ldg(src + k * NH);
+            if (e.yrow >= 0) {
+                const Cplx<T>* m = mu_r + e.yrow * MP;
+                const T sg = (e.yneg ^ op) ? T(-1) : T(1);
+#pragma unroll
+                for (int k2 = 0; k2 < NH; k2 += 2) {
+                    Cplx<T> w2[2];
+                    ld_two<true>(m + k2, w2[0], w2[1]);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int k = k2 + h;
+                        if (k == 0) continue;
+                        const T wi = sg * w2[h].y;
+                        v[line_slot<N>(k)] = cmul(v[line_slot<N>(k)], w2[h].x, wi);
+                        v[line_slot<N>(N - k)] = cmul(v[line_slot<N>(N - k)], w2[h].x, -wi);
+                    }
+                }
+                const T wn = ldg(m + NH).x;
+                v[line_slot<N>(NH)].x *= wn;
+                v[line_slot<N>(NH)].y *= wn;
+            }
+            cfft::line<T, N, false>(v);
+            __syncthreads();   // the previous (s_x, s_y) has been read
+#pragma unroll
+            for (int y = 0; y < N; ++y) st(ydst + y * PITCH, v[y]);
+            __syncthreads();
+        }
+        // z line of T_s f + i T_-s g from the half spectra a (+s) and b (-s, the conjugate phase)
+        const T wgt = wscale * __ldg(wsig + e.pair);
+        const bool zs = e.zrow >= 0;
+        const Cplx<T>* m = mu_r + (zs ? e.zrow : 0) * MP;
+        const T sg = e.zneg ? T(-1) : T(1);
+#pragma unroll
+        for (int k2 = 0; k2 < NH; k2 += 2) {
+            Cplx<T> a2[2], b2[2], w2[2];
+            ld_two<false>(zp + k2, a2[0], a2[1]);
+            ld_two<false>(zm + k2, b2[0], b2[1]);
+            if (zs) ld_two<true>(m + k2, w2[0], w2[1]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = k2 + h;
+                Cplx<T> a = a2[h], b = b2[h];
+                if (k == 0) {   // kz = 0 and kz = N/2, both real
+                    const T wn = zs ? ldg(m + NH).x : T(1);
+                    v[0] = Cplx<T>{a.x, b.x};
+                    v[line_slot<N>(NH)] = Cplx<T>{wn * a.y, wn * b.y};
+                } else {
+                    if (zs) {
+                        const T wi = sg * w2[h].y;
+                        a = cmul(a, w2[h].x, wi);
+                        b = cmul(b, w2[h].x, -wi);
+                    }
+                    v[line_slot<N>(k)] = Cplx<T>{a.x - b.y, a.y + b.x};
+                    v[line_slot<N>(N - k)] = Cplx<T>{a.x + b.y, b.x - a.y};
+                }
+            }
+        }
+        cfft::line<T, N, false>(v);
+#pragma unroll
+        for (int z = 0; z < N; ++z) acc[z] = fma(wgt * v[z].x, v[z].y, acc[z]);
+    }
+    if constexpr (sizeof(T) == 4) {
+        // Two systematic factors of the FP32 constants scale every P_r alike, a bias that the loss does not
+        // share: 1/N^2 and 1/N are rounded for N = 12, 24, and the rounded twiddles return a line that goes
+        // forward and back (three axes, two operands) shorter by line_loss. One FMA takes both out again;
+        // without it the FP32 error of Q at N = 24 grew from 1.6e-6 to 2.8e-6 (two-Maxwellian batch).
+        constexpr double sc = (double)(T(1) / (T(N) * T(N))) * (double)(T(1) / T(N)) * (double)n3;
+        constexpr T corr = (T)(1.0 / (sc * sc) - 1.0 + 6.0 * cfft::line_loss(N));
+#pragma unroll
+        for (int z = 0; z < N; ++z) acc[z] = fma(acc[z], corr, acc[z]);
+    }
+    // P_r of the planes x0 .. x0 + XC - 1 through shared memory (coalesced)
+    T* tile = reinterpret_cast<T*>(sm_raw);                  // [NT][N + 1]
+    __syncthreads();
+#pragma unroll
+    for (int z = 0; z < N; ++z) tile[tid * (N + 1) + z] = acc[z];
+    __syncthreads();
+    T* out = P + node * node_stride + (int64_t)(r0 + rl) * n3 + (int64_t)x0 * N * N;
+    for (int e = tid; e < NT * N; e += NT) out[e] = tile[(e / N) * (N + 1) + e % N];
+}
+
+template <typename T, int N>
+cudaError_t forward_n(const T* f, const int64_t* offs, int64_t nodes, Cplx<T>* G, cudaStream_t s) {
+    using Geo = ForwardGeo<N>;
+    constexpr size_t sm = (size_t)Geo::PX * N * Geo::PITCH * sizeof(Cplx<T>);
+    k_shift_forward<T, N><<<dim3(N / Geo::PX, (unsigned)nodes), Geo::NT, sm, s>>>(f, offs, G);
+    return cudaGetLastError();
+}
+
+template <typename T, int N>
+cudaError_t shift_x_n(const ShiftDev<T>& d, const Cplx<T>* G, int r0, int nr, int64_t nodes, Cplx<T>* H, cudaStream_t s) {
+    if (d.nx == 0 || nr == 0) return cudaSuccess;
+    constexpr int COLS = N * N / 2, NT = COLS < 128 ? COLS : COLS % 128 ? 96 : 128;
+    static_assert(COLS % NT == 0, "whole column blocks");
+    // radial points per CTA (the x spectrum is formed once for them) while the launch fills the GPU
+    // several times; a small batch takes one each, in one-warp CTAs, to reach more SMs
+    const int64_t blocks = (int64_t)(COLS / NT) * nodes * nr;
+    if (blocks >= 8192) {
+        k_shift_x<T, N, NT><<<dim3(COLS / NT, (unsigned)nodes, (unsigned)((nr + 3) / 4)), NT, 0, s>>>(
+            G, d.mu, d.xrows, d.nrows, d.nx, r0, nr, 4, H);
+    } else {
+        k_shift_x<T, N, 32><<<dim3((COLS + 31) / 32, (unsigned)nodes, (unsigned)nr), 32, 0, s>>>(
+            G, d.mu, d.xrows, d.nrows, d.nx, r0, nr, 1, H);
+    }
+    return cudaGetLastError();
+}
+
+template <typename T, int N, int XC>
+cudaError_t products_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
+                       const T* wsig, int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
+    using Geo = ProductGeo<T, N, XC>;
+    auto kern = k_shift_products<T, N, XC>;
+    if (Geo::smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo::smem);
+        if (e != cudaSuccess) return e;
+    }
+    const bool bil = Gg != nullptr;
+    kern<<<dim3(N / XC, (unsigned)nr, (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
+        Gf, Hf, bil ? Gg : Gf, bil ? Hg : Hf, d.mu, bil ? d.bil : d.quad, bil ? d.nbil : d.nquad, bil ? T(1) : T(2), wsig,
+        d.nrows, d.nx, r0, node_stride, P);
+    return cudaGetLastError();
+}
+
+template <typename T, int N>
+cudaError_t products_n(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
+                       const T* wsig, int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
+    constexpr int XC = N == 32 || N == 24 ? 4 : N == 12 ? 12 : 8;
+    // two planes per CTA while whole CTAs of XC planes would not fill the 152 SMs about four deep
+    if ((int64_t)(N / XC) * nr * nodes < 608)
+        return products_x<T, N, 2>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
+    return products_x<T, N, XC>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
+}
+
+}  // namespace
+
+#define DGFS_BY_N(CALL)                       \
+    if (nodes <= 0) return cudaSuccess;       \
+    if (nodes > 65535) return cudaErrorInvalidValue; \
+    if (N == 8) return CALL(8);               \
+    if (N == 12) return CALL(12);             \
+    if (N == 16) return CALL(16);             \
+    if (N == 24) return CALL(24);             \
+    if (N == 32) return CALL(32);             \
+    return cudaErrorInvalidValue
+
+template <typename T>
+cudaError_t launch_shift_forward(const T* f, const int64_t* offs, int N, int64_t nodes, Cplx<T>* G, cudaStream_t s) {
+#define CALL(n) forward_n<T, n>(f, offs, nodes, G, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+
+template <typename T>
+cudaError_t launch_shift_x(const ShiftDev<T>& d, const Cplx<T>* G, int N, int r0, int nr, int64_t nodes, Cplx<T>* H,
+                           cudaStream_t s) {
+#define CALL(n) shift_x_n<T, n>(d, G, r0, nr, nodes, H, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+
+template <typename T>
+cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg,
+                                  const Cplx<T>* Hg, const T* wsig, int N, int r0, int nr, int64_t nodes,
+                                  int64_t node_stride, T* P, cudaStream_t s) {
+#define CALL(n) products_n<T, n>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+
+#define DGFS_SHIFT_INST(T)                                                                                            \
+    template cudaError_t launch_shift_forward<T>(const T*, const int64_t*, int, int64_t, Cplx<T>*, cudaStream_t);     \
+    template cudaError_t launch_shift_x<T>(const ShiftDev<T>&, const Cplx<T>*, int, int, int, int64_t, Cplx<T>*,      \
+                                           cudaStream_t);                                                             \
+    template cudaError_t launch_shift_products<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*, \
+                                                  const Cplx<T>*, const T*, int, int, int, int64_t, int64_t, T*,      \
+                                                  cudaStream_t);
+DGFS_SHIFT_INST(float)
+DGFS_SHIFT_INST(double)
+#undef DGFS_SHIFT_INST
+
+}  // namespace dgfs

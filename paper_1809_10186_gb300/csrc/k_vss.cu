@@ -20,8 +20,7 @@
 //   k_vss_planes<FWD>   forward transforms along x and y of the packed spectra, in place
 //   k_vss_accumulate    Y[n][0](k) += scale sum_p A_rp(k) P^_p(k) (the mirror -k is taken per
 //                       axis, so any axis order works)
-// The VHS path uses the same plane kernel and k_vss_lines_sum, which sums the products over the
-// sphere in registers. Lines are transformed in registers: radix 2 for N = 8, 16, 32, one radix-3
+// The VHS translate products (no transform per point) are in k_shift.cu. Lines are transformed in registers: radix 2 for N = 8, 16, 32, one radix-3
 // stage over three radix-2 transforms for N = 12, 24 (fourier_dev.cuh).
 #include <cstdint>
 
@@ -103,13 +102,13 @@ struct PlaneGeo {
 
 // INV: field f = set * npairs + p of node n; planes kz0 .. kz0 + KZ - 1 of the translate spectra
 // (set 0: mu f^ + i conj(mu) g^, set 1: the same with conj(mu) for mu), then inverse transforms
-// along x and y; output Z[n][f] plane-major. !INV: forward transforms (scale 1/N each) along x and y
+// along x and y; output Z[n][r][f] plane-major for nr radial points (item n nr + r in blockIdx.z). !INV: forward transforms (scale 1/N each) along x and y
 // of X[n][f] in place. grid (N / KZ, fields, nodes). The x lines are read straight from global
 // memory (consecutive threads take consecutive ky: coalesced), the y lines go through shared memory.
 template <typename T, int N, bool INV>
 __global__ void __launch_bounds__(PlaneGeo<T, N>::NT)
     k_vss_planes(const Cplx<T>* __restrict__ Fh, const Cplx<T>* __restrict__ Gh, const Cplx<T>* __restrict__ mu_r,
-                 const Cplx<T>* __restrict__ dftw, int npairs, Cplx<T>* __restrict__ X) {
+                 const Cplx<T>* __restrict__ dftw, int npairs, int nr, Cplx<T>* __restrict__ X) {
     using G = PlaneGeo<T, N>;
     constexpr int KZ = G::KZ, NT = G::NT, P = G::P;
     constexpr int64_t n2 = (int64_t)N * N, n3 = n2 * N;
@@ -118,15 +117,17 @@ __global__ void __launch_bounds__(PlaneGeo<T, N>::NT)
     __shared__ Cplx<T> tw[N];
     __shared__ Cplx<T> m[3 * N];
     const int tid = threadIdx.x, kz0 = blockIdx.x * KZ, f = blockIdx.y, nf = gridDim.y;
-    const int64_t n = blockIdx.z;
+    const unsigned node = INV && nr > 1 ? blockIdx.z / (unsigned)nr : blockIdx.z;
+    const int rl = (int)(blockIdx.z - node * (unsigned)nr);   // radial point of the item (INV)
+    const int64_t n = node, item = blockIdx.z;
     const int pl = tid / N, ln = tid % N;
     if (tid < N) tw[tid] = dftw[N + tid];
-    Cplx<T>* Xf = X + (n * nf + f) * n3 + (int64_t)kz0 * n2;
+    Cplx<T>* Xf = X + (item * nf + f) * n3 + (int64_t)kz0 * n2;
     Cplx<T> v[N];
     if constexpr (INV) {
         const int p = f % npairs;
         const T sgn = f < npairs ? T(1) : T(-1);   // set 1 takes conj(mu) where set 0 takes mu
-        for (int i = tid; i < 3 * N; i += NT) m[i] = mu_r[(int64_t)p * 3 * N + i];
+        for (int i = tid; i < 3 * N; i += NT) m[i] = mu_r[((int64_t)rl * npairs + p) * 3 * N + i];
         __syncthreads();
         const Cplx<T>* Fp = Fh + n * n3 + (int64_t)(kz0 + pl) * n2 + ln;
         const Cplx<T>* Gp = (Gh ? Gh : Fh) + n * n3 + (int64_t)(kz0 + pl) * n2 + ln;
@@ -208,14 +209,16 @@ __global__ void __launch_bounds__(128) k_vss_lines(const Cplx<T>* __restrict__ Z
     for (int k = 0; k < N; ++k) w[k * n2] = Cplx<T>{v[k].x * sc, v[k].y * sc};
 }
 
-// VHS radial products in Fourier space (the isotropic kernel needs no per-point transform): for
+// VHS radial products with a transform per pair (dgfs_ssprk and dgfs_collide_dgamma of FP32 plans, which
+// keep this arithmetic bit for bit; every other call takes the shared translates of k_shift.cu): for
 // z-line (x, y) of node n, the inverse z transforms of every sphere point's translate lines give
-//   P_r(x, y, z) = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)]     (2 w_p (T_s f)(T_-s f) for g = f)
+//   P_r(x, y, z) = sum_p 2 w_p (T_s f)(T_-s f)
 // summed in registers; P_r is written in the standard layout [x][y][z] through shared memory.
-// grid (N^2 / 128, nodes); Z plane-major [n][set][p][kz][x][y]; P_r = P + n stride + r N^3.
+// grid (N^2 / 128, nodes, nr); Z plane-major [n][r][p][kz][x][y]; P_r = P + n stride + r N^3. All radial
+// points of a batch in one launch: one launch per r left 74 CTAs at N = 16 and 37 nodes.
 template <typename T, int N>
 __global__ void __launch_bounds__(128) k_vss_lines_sum(const Cplx<T>* __restrict__ Z, const Cplx<T>* __restrict__ dftw,
-                                                       const T* __restrict__ wsig, int npairs, int sets,
+                                                       const T* __restrict__ wsig, int npairs,
                                                        int64_t node_stride, T* __restrict__ P) {
     constexpr int64_t n2 = (int64_t)N * N, n3 = n2 * N;
     constexpr int LINES = 128;
@@ -224,29 +227,27 @@ __global__ void __launch_bounds__(128) k_vss_lines_sum(const Cplx<T>* __restrict
     if (threadIdx.x < N) tw[threadIdx.x] = dftw[N + threadIdx.x];
     __syncthreads();
     const int64_t l0 = (int64_t)blockIdx.x * LINES, l = l0 + threadIdx.x;
-    const int64_t n = blockIdx.y;
+    const int64_t n = blockIdx.y, item = n * gridDim.z + blockIdx.z;
     T acc[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) acc[k] = T(0);
     Cplx<T> v[N];
     if (l < n2) {
         for (int p = 0; p < npairs; ++p) {
-            const T w = wsig[p] * (sets == 1 ? T(2) : T(1));
-            for (int s = 0; s < sets; ++s) {
-                const Cplx<T>* z = Z + ((n * sets + s) * npairs + p) * n3 + l;
+            const T w = wsig[p] * T(2);
+            const Cplx<T>* z = Z + (item * npairs + p) * n3 + l;
 #pragma unroll
-                for (int k = 0; k < N; ++k) v[line_slot<N>(k)] = z[k * n2];
-                line_fft<T, N>(v, tw, false);
+            for (int k = 0; k < N; ++k) v[line_slot<N>(k)] = z[k * n2];
+            line_fft<T, N>(v, tw, false);
 #pragma unroll
-                for (int k = 0; k < N; ++k) acc[k] = fma(w * v[k].x, v[k].y, acc[k]);
-            }
+            for (int k = 0; k < N; ++k) acc[k] = fma(w * v[k].x, v[k].y, acc[k]);
         }
 #pragma unroll
         for (int k = 0; k < N; ++k) tile[threadIdx.x * (N + 1) + k] = acc[k];
     }
     __syncthreads();
     const int nl = (int)((n2 - l0) < LINES ? (n2 - l0) : LINES);
-    T* out = P + n * node_stride + l0 * N;
+    T* out = P + n * node_stride + blockIdx.z * n3 + l0 * N;
     for (int e = threadIdx.x; e < nl * N; e += LINES) out[e] = tile[(e / N) * (N + 1) + e % N];
 }
 
@@ -376,14 +377,14 @@ inline unsigned nblk(int64_t n) { return (unsigned)((n + 255) / 256); }
 
 template <typename T, int N, bool INV>
 cudaError_t planes_launch(const Cplx<T>* Fh, const Cplx<T>* Gh, const Cplx<T>* mu_r, const Cplx<T>* dftw, int npairs,
-                          int fields, int64_t nodes, Cplx<T>* X, cudaStream_t s) {
+                          int fields, int nr, int64_t nodes, Cplx<T>* X, cudaStream_t s) {
     using G = PlaneGeo<T, N>;
     auto kern = k_vss_planes<T, N, INV>;
     if (G::smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem);
         if (e != cudaSuccess) return e;
     }
-    kern<<<dim3(N / G::KZ, (unsigned)fields, (unsigned)nodes), G::NT, G::smem, s>>>(Fh, Gh, mu_r, dftw, npairs, X);
+    kern<<<dim3(N / G::KZ, (unsigned)fields, (unsigned)(nodes * nr)), G::NT, G::smem, s>>>(Fh, Gh, mu_r, dftw, npairs, nr, X);
     return cudaGetLastError();
 }
 
@@ -404,15 +405,15 @@ cudaError_t launch_vss_load_t(const T* f, const int64_t* offs, int N, int64_t no
 
 template <typename T>
 cudaError_t launch_vss_inverse_planes(const Cplx<T>* Fh, const Cplx<T>* Gh, const Cplx<T>* mu_r, const Cplx<T>* dftw,
-                                      int N, int npairs, int sets, int64_t nodes, Cplx<T>* Z, cudaStream_t s) {
+                                      int N, int npairs, int sets, int nr, int64_t nodes, Cplx<T>* Z, cudaStream_t s) {
     if (nodes <= 0) return cudaSuccess;
-    if (nodes > 65535) return cudaErrorInvalidValue;
+    if (nodes * nr > 65535) return cudaErrorInvalidValue;
     const int fields = sets * npairs;
-    if (N == 8) return planes_launch<T, 8, true>(Fh, Gh, mu_r, dftw, npairs, fields, nodes, Z, s);
-    if (N == 12) return planes_launch<T, 12, true>(Fh, Gh, mu_r, dftw, npairs, fields, nodes, Z, s);
-    if (N == 16) return planes_launch<T, 16, true>(Fh, Gh, mu_r, dftw, npairs, fields, nodes, Z, s);
-    if (N == 24) return planes_launch<T, 24, true>(Fh, Gh, mu_r, dftw, npairs, fields, nodes, Z, s);
-    if (N == 32) return planes_launch<T, 32, true>(Fh, Gh, mu_r, dftw, npairs, fields, nodes, Z, s);
+    if (N == 8) return planes_launch<T, 8, true>(Fh, Gh, mu_r, dftw, npairs, fields, nr, nodes, Z, s);
+    if (N == 12) return planes_launch<T, 12, true>(Fh, Gh, mu_r, dftw, npairs, fields, nr, nodes, Z, s);
+    if (N == 16) return planes_launch<T, 16, true>(Fh, Gh, mu_r, dftw, npairs, fields, nr, nodes, Z, s);
+    if (N == 24) return planes_launch<T, 24, true>(Fh, Gh, mu_r, dftw, npairs, fields, nr, nodes, Z, s);
+    if (N == 32) return planes_launch<T, 32, true>(Fh, Gh, mu_r, dftw, npairs, fields, nr, nodes, Z, s);
     return cudaErrorInvalidValue;
 }
 
@@ -436,25 +437,25 @@ cudaError_t launch_vss_forward_planes(const Cplx<T>* dftw, int N, int fields, in
                                       cudaStream_t s) {
     if (nodes <= 0) return cudaSuccess;
     if (nodes > 65535) return cudaErrorInvalidValue;
-    if (N == 8) return planes_launch<T, 8, false>(nullptr, nullptr, nullptr, dftw, 0, fields, nodes, W, s);
-    if (N == 12) return planes_launch<T, 12, false>(nullptr, nullptr, nullptr, dftw, 0, fields, nodes, W, s);
-    if (N == 16) return planes_launch<T, 16, false>(nullptr, nullptr, nullptr, dftw, 0, fields, nodes, W, s);
-    if (N == 24) return planes_launch<T, 24, false>(nullptr, nullptr, nullptr, dftw, 0, fields, nodes, W, s);
-    if (N == 32) return planes_launch<T, 32, false>(nullptr, nullptr, nullptr, dftw, 0, fields, nodes, W, s);
+    if (N == 8) return planes_launch<T, 8, false>(nullptr, nullptr, nullptr, dftw, 0, fields, 1, nodes, W, s);
+    if (N == 12) return planes_launch<T, 12, false>(nullptr, nullptr, nullptr, dftw, 0, fields, 1, nodes, W, s);
+    if (N == 16) return planes_launch<T, 16, false>(nullptr, nullptr, nullptr, dftw, 0, fields, 1, nodes, W, s);
+    if (N == 24) return planes_launch<T, 24, false>(nullptr, nullptr, nullptr, dftw, 0, fields, 1, nodes, W, s);
+    if (N == 32) return planes_launch<T, 32, false>(nullptr, nullptr, nullptr, dftw, 0, fields, 1, nodes, W, s);
     return cudaErrorInvalidValue;
 }
 
 template <typename T>
-cudaError_t launch_vss_lines_sum(const Cplx<T>* Z, const Cplx<T>* dftw, const T* wsig, int N, int npairs, int sets,
+cudaError_t launch_vss_lines_sum(const Cplx<T>* Z, const Cplx<T>* dftw, const T* wsig, int N, int npairs, int nr,
                                  int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
     if (nodes <= 0) return cudaSuccess;
     if (nodes > 65535) return cudaErrorInvalidValue;
-    const dim3 grid((unsigned)((N * N + 127) / 128), (unsigned)nodes);
-    if (N == 8) k_vss_lines_sum<T, 8><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, sets, node_stride, P);
-    else if (N == 12) k_vss_lines_sum<T, 12><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, sets, node_stride, P);
-    else if (N == 16) k_vss_lines_sum<T, 16><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, sets, node_stride, P);
-    else if (N == 24) k_vss_lines_sum<T, 24><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, sets, node_stride, P);
-    else if (N == 32) k_vss_lines_sum<T, 32><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, sets, node_stride, P);
+    const dim3 grid((unsigned)((N * N + 127) / 128), (unsigned)nodes, (unsigned)nr);
+    if (N == 8) k_vss_lines_sum<T, 8><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, node_stride, P);
+    else if (N == 12) k_vss_lines_sum<T, 12><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, node_stride, P);
+    else if (N == 16) k_vss_lines_sum<T, 16><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, node_stride, P);
+    else if (N == 24) k_vss_lines_sum<T, 24><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, node_stride, P);
+    else if (N == 32) k_vss_lines_sum<T, 32><<<grid, 128, 0, s>>>(Z, dftw, wsig, npairs, node_stride, P);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
@@ -536,7 +537,7 @@ cudaError_t launch_vss_loss_init(const Cplx<T>* Ah, const Cplx<T>* Bh, const T* 
                                                  Cplx<T>*, int, cudaStream_t);                                    \
     template cudaError_t launch_vss_load_t<T>(const T*, const int64_t*, int, int64_t, Cplx<T>*, cudaStream_t);                    \
     template cudaError_t launch_vss_inverse_planes<T>(const Cplx<T>*, const Cplx<T>*, const Cplx<T>*,            \
-                                                      const Cplx<T>*, int, int, int, int64_t, Cplx<T>*,           \
+                                                      const Cplx<T>*, int, int, int, int, int64_t, Cplx<T>*,      \
                                                       cudaStream_t);                                              \
     template cudaError_t launch_vss_lines<T>(const Cplx<T>*, const Cplx<T>*, int, int, int, int64_t, Cplx<T>*,   \
                                              cudaStream_t);                                                       \
@@ -547,11 +548,11 @@ cudaError_t launch_vss_loss_init(const Cplx<T>* Ah, const Cplx<T>* Bh, const T* 
                                              Cplx<T>*, cudaStream_t);                                             \
     template cudaError_t launch_vjp_accumulate<T>(const Cplx<T>*, const Cplx<T>*, const T*, int, int, int64_t,     \
                                                   Cplx<T>*, cudaStream_t);                                        \
-    template cudaError_t launch_vjp_real_t<T>(const Cplx<T>*, int, int64_t, T*, cudaStream_t);                    \
-    template cudaError_t launch_vss_lines_sum<T>(const Cplx<T>*, const Cplx<T>*, const T*, int, int, int, int64_t, \
-                                                 int64_t, T*, cudaStream_t);
+    template cudaError_t launch_vjp_real_t<T>(const Cplx<T>*, int, int64_t, T*, cudaStream_t);
 DGFS_VSS_INST(float)
 DGFS_VSS_INST(double)
 #undef DGFS_VSS_INST
+template cudaError_t launch_vss_lines_sum<float>(const Cplx<float>*, const Cplx<float>*, const float*, int, int, int,
+                                                 int64_t, int64_t, float*, cudaStream_t);
 
 }  // namespace dgfs

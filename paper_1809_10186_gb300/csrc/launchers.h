@@ -120,7 +120,7 @@ cudaError_t launch_vss_load_t(const T* f, const int64_t* offs, int N, int64_t no
 // Z[n][set][p] = inverse x, y transforms of the translate spectra
 template <typename T>
 cudaError_t launch_vss_inverse_planes(const Cplx<T>* Fh, const Cplx<T>* Gh, const Cplx<T>* mu_r, const Cplx<T>* dftw,
-                                      int N, int npairs, int sets, int64_t nodes, Cplx<T>* Z, cudaStream_t s);
+                                      int N, int npairs, int sets, int nr, int64_t nodes, Cplx<T>* Z, cudaStream_t s);
 // W[n][j] = forward z transform of P_2j + i P_2j+1 after the inverse z transform of the Z lines
 template <typename T>
 cudaError_t launch_vss_lines(const Cplx<T>* Z, const Cplx<T>* dftw, int N, int npairs, int sets, int64_t nodes,
@@ -129,9 +129,10 @@ cudaError_t launch_vss_lines(const Cplx<T>* Z, const Cplx<T>* dftw, int N, int n
 template <typename T>
 cudaError_t launch_vss_forward_planes(const Cplx<T>* dftw, int N, int fields, int64_t nodes, Cplx<T>* W,
                                       cudaStream_t s);
-// VHS: P[n][r] (standard layout, node stride node_stride) = sum_p w_p (products of the translate lines of Z)
+// VHS with a transform per pair: P[n][r] (standard layout, node stride node_stride), nr radial points, from
+// the translate lines Z[n][r][pair]
 template <typename T>
-cudaError_t launch_vss_lines_sum(const Cplx<T>* Z, const Cplx<T>* dftw, const T* wsig, int N, int npairs, int sets,
+cudaError_t launch_vss_lines_sum(const Cplx<T>* Z, const Cplx<T>* dftw, const T* wsig, int N, int npairs, int nr,
                                  int64_t nodes, int64_t node_stride, T* P, cudaStream_t s);
 // adjoint gain in Fourier space (see k_vss.cu): W[n][p] = DFT_z(U_r b + i U_r a) of the translate lines,
 // G^[n] += sum_p 2 w_p [conj(mu_s) P1^ + mu_s P2^], and the real part of the transformed-back G^ in the

@@ -1,0 +1,66 @@
+// Shared-shift translate products of the CUDA-core plans (k_shift.cu): the host side of the
+// program that the product kernel walks, and the launchers.
+#pragma once
+
+#include <cstdint>
+#include <vector>
+
+#include <cuda_runtime.h>
+
+#include "launchers.h"
+#include "plan_host.h"
+
+namespace dgfs {
+
+// One product term w (T_s f)(T_-s g). Its x translates are two fields of the x pass (-1: shift 0), its
+// y and z multipliers rows of the shift table (-1: shift 0) with a sign.
+struct ShiftEntry {
+    int fp, fm;      // x-pass fields of +s_x (of f) and -s_x (of g)
+    int yrow, yneg;  // |s_y|, 1 when s_y < 0
+    int zrow, zneg;  // |s_z|, 1 when s_z < 0
+    int pair;        // sphere pair (weight)
+    int newy;        // 1: another (s_x, s_y) than the entry before it
+};
+
+// Entries sorted by (s_x, s_y), so that equal x and (x, y) translates are neighbours: M = 38 has 19 pairs
+// but 8 nonzero signed x shifts and 13 (x, y) shifts up to sign; a rule without coinciding components
+// gets an entry of its own for each.
+struct ShiftProgram {
+    int nrows = 0;                       // distinct nonzero |component| over all pairs and axes
+    int nx = 0;                          // distinct nonzero |s_x|; fields 2i (+) and 2i + 1 (-)
+    std::vector<int> xrows;              // [nx] row of the shift table
+    std::vector<ShiftEntry> quad, bil;   // g = f: one entry per pair (weight 2 w_p); f, g: both signs (w_p)
+    std::vector<double> mu;              // [Nrho][nrows][MP][2] e^{i pi k s / L}, k = 0 .. N/2 (Nyquist cos)
+};
+
+// Row pitch of the shift table: N/2 + 1 modes, padded to an even count (16-byte FP32 rows).
+constexpr int shift_mu_pitch(int N) { return N / 2 + 2; }
+
+void build_shift_program(const HostPlan& h, ShiftProgram& p);
+
+// Device side of the program, in the compute type.
+template <typename T>
+struct ShiftDev {
+    int nrows = 0, nx = 0, nquad = 0, nbil = 0;
+    const int* xrows = nullptr;
+    const ShiftEntry *quad = nullptr, *bil = nullptr;
+    const Cplx<T>* mu = nullptr;
+};
+
+// G[node][x][ky][kz], kz = 0 .. N/2 - 1: the (y, z) spectra (times 1/N^2) of every x plane of the real
+// field f; the real spectra of kz = 0 and kz = N/2 share the complex slot kz = 0. offs: element offset of
+// every node (nullptr: node N^3).
+template <typename T>
+cudaError_t launch_shift_forward(const T* f, const int64_t* offs, int N, int64_t nodes, Cplx<T>* G, cudaStream_t s);
+// H[node][r - r0][field][x][ky][kz] for r in [r0, r0 + nr): the x translates of G by every signed x shift
+template <typename T>
+cudaError_t launch_shift_x(const ShiftDev<T>& d, const Cplx<T>* G, int N, int r0, int nr, int64_t nodes, Cplx<T>* H,
+                           cudaStream_t s);
+// P[node][r] = sum of the program's terms over the fields Hf/Gf (operand f) and Hg/Gg (operand g; Hg ==
+// nullptr: g = f); P + node node_stride + r N^3.
+template <typename T>
+cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg,
+                                  const Cplx<T>* Hg, const T* wsig, int N, int r0, int nr, int64_t nodes,
+                                  int64_t node_stride, T* P, cudaStream_t s);
+
+}  // namespace dgfs
