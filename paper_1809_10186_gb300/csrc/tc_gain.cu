@@ -133,7 +133,8 @@ struct Items {
     int64_t n_items;   // nodes * rblocks
     int rblocks;       // radial blocks per node (N_rho / rpc)
     int rpc;           // radial points per item
-    int nseq;          // (radial point, pair) steps per item: rpc * npairs
+    int nseq;          // (radial point, group) steps per item: rpc * groups
+    TcGroups groups;   // pairs that share passes 1 and 2 with the pair before them
 };
 
 struct Bars {
@@ -146,6 +147,7 @@ struct Bars {
     uint64_t a2_full[2], a2_free[2];   // pass-2 operand ring: epilogue -> MMA, MMA completion -> epilogue
     uint64_t a3_full, a3_free;         // pass-3 operands (both signs)
     uint64_t filt[2], fdone[2];        // filter buffers: copy landed; all MMAs of the step using it done
+    uint64_t filt_b[2], p1_done;       // y filters of a group's second pair landed; its pass-1 MMAs complete
     uint64_t item_full[kRing], item_free[kRing];   // work-item ring: published; read by every consumer warp
     uint64_t f_ready, f_free;          // f of the current item in TMEM; pass-1 MMAs of an item complete
     uint64_t scan[2];                  // max |f| partial maxima of an item written (item % 2)
@@ -205,7 +207,7 @@ template <int N, bool BF>
 __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uint32_t sb, uint32_t tmem,
                                             const unsigned char* filt, int npairs, const Items& it, long long first,
                                             volatile long long* s_item, int* queue, volatile int* abort,
-                                            int& copies0, int& copies1, int& waited0, int& waited1) {
+                                            int& copies0, int& copies1, int& waited0, int& waited1, int& second0, int& second1) {
     using G = Geo<N>;
     uint32_t used = 0, ph_free = 0, ph_fdone = 0;   // bit masks (bit i = slot or buffer i)
     constexpr uint32_t id1 = tc::idesc_f16(BF, false, false, 2 * N, 128);
@@ -213,6 +215,7 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
     const uint32_t sb16 = sb >> 4;
     long long cur = first;
     int64_t g = 0;
+    uint32_t ph_p1 = 0;
     for (int k = 0; cur >= 0; ++k) {
         // the next item is claimed now: its first filter block is copied during this item's last step
         long long nxt = -1;
@@ -220,8 +223,11 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
         const unsigned char* fcur = item_filters<N>(filt, cur, it, npairs);
         const unsigned char* fnxt = nxt >= 0 ? item_filters<N>(filt, nxt, it, npairs) : nullptr;
         DGFS_WAITW(&bars.f_ready, (uint32_t)(k & 1));   // f of this item is in TMEM
+        int pair = 0, off = 0;   // first pair of the step's group, its filter block within the item
         for (int s = 0; s < it.nseq; ++s, ++g) {
             const int fbuf = (int)(g & 1);
+            const int cnt = it.groups.count(pair);
+            const unsigned char* fstep = fcur + (size_t)off * G::F_BLOCK;
             DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((g >> 1) & 1));
             if (fbuf) ++waited1;
             else ++waited0;
@@ -249,7 +255,7 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
                 // the set-up copied steps 0 and 1, unless step 1 belongs to the next item (one-step items).
                 // With the epilogue's look-ahead the wait comes after tile 1: step g - 1 completes only
                 // after warpgroup 0 has turned tiles 0 and 1 of step g into pass-2 operands.
-                const unsigned char* src = s + 1 < it.nseq ? fcur + (size_t)(s + 1) * G::F_BLOCK : fnxt;
+                const unsigned char* src = s + 1 < it.nseq ? fstep + (size_t)cnt * G::F_BLOCK : fnxt;
                 if (t == (G::LOOKAHEAD ? 1 : 0) && (g >= 1 || it.nseq == 1) && src) {
                     const int nb = (int)((g + 1) & 1);
                     if (g >= 1) {   // buffer nb held step g - 1
@@ -265,7 +271,22 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
                     else ++copies0;
                 }
             }
+            if (cnt == 2) {   // the second pair's y filters take the place of the x filters, which are done with
+                tc::mma_commit_warp(&bars.p1_done);
+                DGFS_WAITW(&bars.p1_done, ph_p1);
+                ph_p1 ^= 1u;
+                if (tc::elect_one()) {
+                    tc::mbar_expect_tx(&bars.filt_b[fbuf], 2 * G::B23_BYTES);
+                    tc::bulk_g2s(smem + G::S_F + fbuf * G::F_BLOCK + G::OFF_B1, fstep + G::F_BLOCK + G::OFF_B3, 2 * G::B23_BYTES,
+                                 &bars.filt_b[fbuf]);
+                }
+                __syncwarp();
+                if (fbuf) ++second1;
+                else ++second0;
+            }
             tc::mma_commit_warp(&bars.fdone[fbuf]);
+            off += cnt;
+            pair = pair + cnt < npairs ? pair + cnt : 0;
         }
         tc::mma_commit_warp(&bars.f_free);   // f of this item may be replaced once these MMAs complete
         cur = nxt;
@@ -328,12 +349,12 @@ __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tm
 // also orders every pass-2 drain of the slot before these MMAs). Each sign's half of the slot has
 // its own completion (full3p / full3m) and release (free3p / free3m): the + MMAs of tile k + 1 wait
 // only for the + half of tile k to be read, so they run while the epilogue reads the - half and
-// forms the products (completions 0..2 of the step's four).
+// forms the products. A group's second pair reads the same operands with its own y filters.
 template <int N, bool BF, int b>
-__device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tmem, const Items& it,
+__device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tmem, int npairs, const Items& it,
                                             const volatile long long* s_item, volatile int* abort) {
     using G = Geo<N>;
-    uint32_t ph_a3full = 0;
+    uint32_t ph_a3full = 0, ph_b = 0, drained = 0;   // drained: drains of the slot handed over so far
     constexpr uint32_t id23 = tc::idesc_f16(BF, true, false, 2 * N, 128);
     constexpr uint64_t dF = tc::sdesc_base(G::FB_LBO, G::FB_SBO);
     constexpr uint64_t dA3 = tc::sdesc_base(G::A3_LBO, G::A3_SBO);
@@ -342,30 +363,41 @@ __device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tm
     for (int ki = 0;; ++ki) {
         long long item;
         if (!ring_take(bars, s_item, ki, item, abort) || item < 0) return;
+        int pair = 0;
         for (int s = 0; s < it.nseq; ++s, ++g) {
             const int fbuf = (int)(g & 1);
+            const int cnt = it.groups.count(pair);
+            pair = pair + cnt < npairs ? pair + cnt : 0;
             DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((g >> 1) & 1));
             const uint32_t f16 = sb16 + (G::S_F + fbuf * G::F_BLOCK) / 16;
             DGFS_WAITW(&bars.a3_full, ph_a3full);
             ph_a3full ^= 1;
             tc::tc_fence_after();
-            for (int k = 0; k < G::TW; ++k) {
-                const int u = 2 * k + b;
-                const uint32_t d = tmem + (b ? G::C_S3 : G::C_S2);
-                const uint32_t a16 = sb16 + G::S_A3 / 16 + u * (G::A3_TS / 16);
+            for (int i = 0; i < cnt; ++i) {   // pairs of the group: same operands, their own y filters
+                if (i == 1) {
+                    DGFS_WAITW(&bars.filt_b[fbuf], (ph_b >> fbuf) & 1u);
+                    ph_b ^= 1u << fbuf;
+                    tc::tc_fence_after();
+                }
+                const uint32_t fy16 = f16 + (i == 1 ? G::OFF_B1 : G::OFF_B3) / 16;
+                for (int k = 0; k < G::TW; ++k) {
+                    const int u = 2 * k + b;
+                    const uint32_t d = tmem + (b ? G::C_S3 : G::C_S2);
+                    const uint32_t a16 = sb16 + G::S_A3 / 16 + u * (G::A3_TS / 16);
 #pragma unroll
-                for (int gs = 0; gs < 2; ++gs) {   // sign +, then sign -
-                    if (k > 0) {
-                        DGFS_WAITW(gs ? &bars.free3m[b] : &bars.free3p[b], (uint32_t)((k - 1) & 1));   // four per step
-                        tc::tc_fence_after();
+                    for (int gs = 0; gs < 2; ++gs) {   // sign +, then sign -
+                        if (i > 0 || k > 0) {   // the previous tile of this step has been read
+                            DGFS_WAITW(gs ? &bars.free3m[b] : &bars.free3p[b], (drained - 1) & 1u);
+                            tc::tc_fence_after();
+                        }
+#pragma unroll
+                        for (int ks = 0; ks < G::KSTEPS; ++ks)
+                            tc::mma_ss_warp(d + gs * 2 * N,
+                                            tc::sdesc_at(dA3, a16 + (gs * G::A3_BYTES + ks * 2 * G::A3_LBO) / 16),
+                                            tc::sdesc_at(dF, fy16 + (gs * G::B23_BYTES + ks * 2 * G::FB_LBO) / 16), id23, ks);
+                        tc::mma_commit_warp(gs ? &bars.full3m[b] : &bars.full3p[b]);
                     }
-#pragma unroll
-                    for (int ks = 0; ks < G::KSTEPS; ++ks)
-                        tc::mma_ss_warp(d + gs * 2 * N,
-                                        tc::sdesc_at(dA3, a16 + (gs * G::A3_BYTES + ks * 2 * G::A3_LBO) / 16),
-                                        tc::sdesc_at(dF, f16 + (G::OFF_B3 + gs * G::B23_BYTES + ks * 2 * G::FB_LBO) / 16),
-                                        id23, ks);
-                    tc::mma_commit_warp(gs ? &bars.full3m[b] : &bars.full3p[b]);
+                    ++drained;
                 }
             }
             tc::mma_commit_warp(&bars.a3_free);
@@ -403,7 +435,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
     const uint32_t sb = tc::smem_u32(smem);
 
     // filter copies issued and waited per buffer 0 / 1 (used by the MMA warp and the drain)
-    int copies0 = 0, copies1 = 0, waited0 = 0, waited1 = 0;
+    int copies0 = 0, copies1 = 0, waited0 = 0, waited1 = 0, second0 = 0, second1 = 0;
     long long first = -1;
 
     // ---- set-up: barriers, the first item and its first filter copies, TMEM (MMA warp) -----------
@@ -423,6 +455,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                 tc::mbar_init(&bars.a2_free[i], 1);
                 tc::mbar_init(&bars.filt[i], 1);
                 tc::mbar_init(&bars.fdone[i], 4);   // one commit from each MMA warp
+                tc::mbar_init(&bars.filt_b[i], 1);
             }
             for (int i = 0; i < kRing; ++i) {
                 tc::mbar_init(&bars.item_full[i], 1);
@@ -430,6 +463,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
             }
             tc::mbar_init(&bars.f_ready, 256);      // the epilogue warpgroups
             tc::mbar_init(&bars.f_free, 1);
+            tc::mbar_init(&bars.p1_done, 1);
             tc::mbar_init(&bars.scan[0], G::EPI_WARPS);
             tc::mbar_init(&bars.scan[1], G::EPI_WARPS);
             tc::mbar_init(&bars.a3_full, 128);     // the pass-2 epilogue warpgroup
@@ -442,9 +476,10 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
         ring_claim(bars, s_item, queue, it, 0, first, abort);   // slot 0: no wait
         if (lane == 0 && first >= 0) {
             const unsigned char* f0 = item_filters<N>(filt, first, it, npairs);
-            for (int p = 0; p < 2 && p < it.nseq; ++p) {
+            for (int p = 0; p < 2 && p < it.nseq; ++p) {   // the first two groups
                 tc::mbar_expect_tx(&bars.filt[p], G::F_BLOCK);
-                tc::bulk_g2s(smem + G::S_F + p * G::F_BLOCK, f0 + (size_t)p * G::F_BLOCK, G::F_BLOCK, &bars.filt[p]);
+                tc::bulk_g2s(smem + G::S_F + p * G::F_BLOCK, f0, G::F_BLOCK, &bars.filt[p]);
+                f0 += (size_t)it.groups.count(0) * G::F_BLOCK;
             }
         }
         __syncwarp();
@@ -464,13 +499,13 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
       // ============================ MMA warps (converged) =====================================
       if (warp == G::ISSUER)
         mma_p1_loop<N, BF>(bars, smem, sb, tmem, filt, npairs, it, first, s_item, queue, abort, copies0, copies1,
-                           waited0, waited1);
+                           waited0, waited1, second0, second1);
       else if (warp == G::ISSUER + 1)
         mma_p2_loop<N, BF>(bars, sb, tmem, it, s_item, abort);
       else if (warp == G::ISSUER + 2)
-        mma_p3_loop<N, BF, 0>(bars, sb, tmem, it, s_item, abort);
+        mma_p3_loop<N, BF, 0>(bars, sb, tmem, npairs, it, s_item, abort);
       else
-        mma_p3_loop<N, BF, 1>(bars, sb, tmem, it, s_item, abort);
+        mma_p3_loop<N, BF, 1>(bars, sb, tmem, npairs, it, s_item, abort);
     } else {
         tc::setmaxnreg_inc<G::REG_EPI>();
         // ============================== epilogue warpgroups ===================================
@@ -587,13 +622,15 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
           tc::mbar_arrive(&bars.f_ready);
           int ahead = 0;   // pass-1 tiles of the current step that warpgroup 0 handled during the last back
           for (int rr = 0; rr < it.rpc; ++rr) {
-          for (int pp = 0; pp < npairs; ++pp, ++g) {
+          int cnt = 1;   // pairs of the step's group
+          for (int pp = 0; pp < npairs; pp += cnt, ++g) {
+            cnt = it.groups.count(pp);
             if (w == 0) {
                 // the step's remaining tiles, then, when the next step belongs to this item, its first
                 // LOOKAHEAD tiles (virtual tiles T, T + 1): their pass-1 MMAs and operand buffers do not
                 // depend on this step's pass 3, so warpgroup 0 fills the wait for the pass-3 operands
                 // with them (a third would wait for the next step's pass 2, i.e. for this step's back)
-                const int tend = G::T + ((pp + 1 < npairs || rr + 1 < it.rpc) ? G::LOOKAHEAD : 0);
+                const int tend = G::T + ((pp + cnt < npairs || rr + 1 < it.rpc) ? G::LOOKAHEAD : 0);
                 for (int t = ahead; t < tend; ++t) {   // pass-1 tile t (slot t % 2) -> pass-2 operands (buffer t % 2)
                     const int b = t & 1;
                     if (g > 0 || t >= 2) {   // pass 2 of tile t - 2 (of this or the previous step) has read buffer b
@@ -670,8 +707,10 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                 // failure test: the first CTA withholds the signal for its first step
                 if (!(fault == 1 && g == 0 && blockIdx.x == 0)) tc::mbar_arrive(&bars.a3_full);
             }
-            // pass-3 tiles u = 2k + w (slot w): products of the two translates
+            // pass-3 tiles u = 2k + w (slot w) of every pair of the group: products of the two translates
             const uint32_t tB = trow + (w ? G::C_S3 : G::C_S2);
+#pragma unroll 1
+            for (int i = 0; i < cnt; ++i) {
 #pragma unroll
             for (int k = 0; k < G::TW; ++k) {
                 // + half, released before the - half is awaited
@@ -706,7 +745,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                     if (c == N / 16 - 1) {
                         tc::tc_fence_before();
                         tc::mbar_arrive(&bars.free3m[w]);
-                        if (k == G::TW - 1) tc::mbar_arrive(&bars.free3x[w]);
+                        if (k == G::TW - 1 && i == cnt - 1) tc::mbar_arrive(&bars.free3x[w]);
                     }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
@@ -715,6 +754,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                         acc[k][8 * c + j] = tc::ffma2(xp[8 * c + j], xm, acc[k][8 * c + j]);
                     }
                 }
+            }
             }
           }
           // radial point r0 + rr done: P_r out, sums cleared
@@ -771,6 +811,9 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                         atomicOr(flags, 1);
                         break;
                     }
+            for (int i = 0; i < 2; ++i)   // the latest copy of a second pair's filters
+                if (const int n = i ? second1 : second0; n > 0 && !tc::mbar_wait(&bars.filt_b[i], (uint32_t)((n - 1) & 1)))
+                    atomicOr(flags, 1);
         }
         __syncwarp();
         tc::tc_fence_after();
@@ -793,7 +836,8 @@ cudaError_t launch_n(const TcTables& t, const float* f, const int64_t* offs, int
     Items it;
     it.rpc = tc_resolve_rpc(t, BF ? DGFS_PREC_BF16S : DGFS_PREC_F16S, nodes, sms);
     it.rblocks = t.Nrho / it.rpc;
-    it.nseq = it.rpc * t.npairs;
+    it.groups = t.groups;
+    it.nseq = it.rpc * t.ngroups;
     it.n_items = nodes * it.rblocks;
     if (it.n_items > (int64_t)0x7FFFFFFF - 4096 || it.nseq < 1) return cudaErrorInvalidValue;
     int* queue = flags + kQueueWord;
@@ -899,6 +943,20 @@ size_t build_tc_tables(const HostPlan& hp, int prec, std::vector<unsigned char>&
                         put(blk + b1 + 2 * b23 + g * b23, N + i, j, lo);
                     }
         }
+    // a pair whose x and z filters (the weight included) equal the pair's before it (the same (s_x, s_z) with
+    // the other s_y) shares its passes 1 and 2
+    t.ngroups = np;
+    for (int p = 1; p < np && p < 32 * TcGroups::kWords; ++p) {
+        bool same = t.groups.count(p - 1) == 1 && !t.groups.second(p - 1);
+        for (int r = 0; r < Nr && same; ++r) {
+            const unsigned char* a = blob.data() + ((size_t)r * np + p) * block;
+            same = std::memcmp(a, a - block, b1 + 2 * b23) == 0;
+        }
+        if (same) {
+            t.groups.w[p / 32] |= 1u << (p % 32);
+            --t.ngroups;
+        }
+    }
     t.N = N;
     t.nsrc = Nd;
     t.Nrho = Nr;

@@ -10,8 +10,19 @@
 
 namespace dgfs {
 
+// Sphere pairs grouped by their first two passes: bit p is set when pair p shares the x and z filters of
+// pair p - 1 (groups have one or two pairs: unit vectors with equal s_x, s_z differ in the sign of s_y).
+struct TcGroups {
+    static constexpr int kWords = 8;   // M <= 512
+    uint32_t w[kWords] = {};
+    __host__ __device__ bool second(int p) const { return p < 32 * kWords && (w[p / 32] >> (p % 32) & 1u); }
+    __host__ __device__ int count(int p) const { return second(p + 1) ? 2 : 1; }   // of the group that p begins
+};
+
 struct TcTables {
     int N = 0, Nrho = 0, npairs = 0;   // N: points per axis of the tiles
+    TcGroups groups;
+    int ngroups = 0;
     int nsrc = 0;                   // points per axis of f and P_r (N, or 24 on 32-point tiles)
     const void* mats = nullptr;     // per (r, pair, axis, sign) N x N operand tiles
     const float* wsig = nullptr;
