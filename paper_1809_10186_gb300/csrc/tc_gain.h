@@ -38,6 +38,9 @@ int tc_resolve_rpc(const TcTables& t, int prec, int64_t nodes, int sms);
 // N = 16, 32; N = 24 on the 32-point tiles (zero-padded filters and data), every tensor-core precision.
 bool tc_supported(int N, int prec);
 int tc_extra_launches(int prec);   // launches the tensor-core path adds per chunk (beyond one)
+// Groups adjacent pairs whose filter blocks (`block` bytes each, [Nrho][npairs]) agree in their first `front`
+// bytes, the x and z filters of every radial point (the weight included): the same (s_x, s_z), the other s_y.
+void tc_group_pairs(const std::vector<unsigned char>& blob, size_t block, size_t front, int Nrho, int npairs, TcTables& t);
 size_t build_tc_tables(const HostPlan& hp, int prec, std::vector<unsigned char>& blob, TcTables& t);
 void rebase_tc_tables(TcTables& t, void* base);
 // Word of the plan's device flag array that counts the work items claimed by the persistent

@@ -129,7 +129,8 @@ struct Bars3 {
     uint64_t free3x[2];                // last pass-3 drain of a slot in a pair
     uint64_t a3_full;                  // the 128 pass-2 epilogue threads (of both CTAs) that own rows here wrote them
     uint64_t a3_free;                  // both CTAs' pass-3 MMAs read this pair's operands
-    uint64_t filt[2], fdone[2];        // filter buffers: copy landed; all MMAs of the pair using it done
+    uint64_t filt[2], fdone[2];        // filter buffers: copy landed; all MMAs of the step using it done
+    uint64_t filt_b[2], p1_done;       // y filters of a group's second pair landed; its pass-1 MMAs complete
     uint64_t drain;
 };
 
@@ -145,10 +146,13 @@ struct Bars3 {
 // Pass 1 of the CTA's front tiles i (both signs) into the pass-1 slot; refills the filter buffers.
 template <int N, bool BF>
 __device__ __forceinline__ void mma3_p1_loop(Bars3& bars, unsigned char* smem, uint32_t sb, uint32_t tmem,
-                                             const unsigned char* fglob, int nseq, volatile int* abort,
-                                             int& copies0, int& copies1, int& waited0, int& waited1) {
+                                             const unsigned char* fglob, int npairs, const TcGroups& groups, int nseq,
+                                             volatile int* abort, int& copies0, int& copies1, int& waited0, int& waited1,
+                                             int& second0, int& second1) {
     using G = Geo3<N>;
-    uint32_t ph_free = 0;
+    uint32_t ph_free = 0, ph_p1 = 0;
+    int pair = 0;                            // first pair of the step's group
+    const unsigned char* fstep = fglob;      // its filter block
     int uses = 0;
     uint32_t ph_fdone = 0;
     constexpr uint32_t idw = tc::idesc_f16(BF, false, false, 4 * N, 128);   // [+hi; -hi; +lo; -lo]
@@ -157,6 +161,7 @@ __device__ __forceinline__ void mma3_p1_loop(Bars3& bars, unsigned char* smem, u
     const uint32_t sb16 = sb >> 4;
     for (int p = 0; p < nseq; ++p) {
         const int fbuf = p & 1;
+        const int cnt = groups.count(pair);
         DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((p >> 1) & 1));
         if (fbuf) ++waited1;
         else ++waited0;
@@ -184,7 +189,7 @@ __device__ __forceinline__ void mma3_p1_loop(Bars3& bars, unsigned char* smem, u
                 ph_fdone ^= 1u << nb;
                 if (tc::elect_one()) {
                     tc::mbar_expect_tx(&bars.filt[nb], G::F_BLOCK);
-                    tc::bulk_g2s(smem + G::S_F + nb * G::F_BLOCK, fglob + (size_t)(p + 1) * G::F_BLOCK, G::F_BLOCK,
+                    tc::bulk_g2s(smem + G::S_F + nb * G::F_BLOCK, fstep + (size_t)cnt * G::F_BLOCK, G::F_BLOCK,
                                  &bars.filt[nb]);
                 }
                 __syncwarp();
@@ -192,7 +197,22 @@ __device__ __forceinline__ void mma3_p1_loop(Bars3& bars, unsigned char* smem, u
                 else ++copies0;
             }
         }
+        if (cnt == 2) {   // the second pair's y filters take the place of the x filters, which are done with
+            tc::mma_commit_warp(&bars.p1_done);
+            DGFS_WAITW(&bars.p1_done, ph_p1);
+            ph_p1 ^= 1u;
+            if (tc::elect_one()) {
+                tc::mbar_expect_tx(&bars.filt_b[fbuf], 2 * G::SB_BYTES);
+                tc::bulk_g2s(smem + G::S_F + fbuf * G::F_BLOCK + G::OFF_B1, fstep + G::F_BLOCK + G::OFF_B3, 2 * G::SB_BYTES,
+                             &bars.filt_b[fbuf]);
+            }
+            __syncwarp();
+            if (fbuf) ++second1;
+            else ++second0;
+        }
         tc::mma_commit_warp(&bars.fdone[fbuf]);
+        fstep += (size_t)cnt * G::F_BLOCK;
+        pair = pair + cnt < npairs ? pair + cnt : 0;
     }
 }
 
@@ -257,51 +277,52 @@ __device__ __forceinline__ void mma3_p2_loop(Bars3& bars, uint32_t sb, uint32_t 
 // both CTAs' epilogues are complete (warpgroup b drains the slot); the release of the operands is
 // signalled to both CTAs (multicast commit).
 template <int N, bool BF, int b>
-__device__ __forceinline__ void mma3_p3_loop(Bars3& bars, uint32_t sb, uint32_t tmem, int nseq, volatile int* abort) {
+__device__ __forceinline__ void mma3_p3_loop(Bars3& bars, uint32_t sb, uint32_t tmem, int npairs, const TcGroups& groups, int nseq,
+                                             volatile int* abort) {
     using G = Geo3<N>;
-    uint32_t ph_a3full = 0, ph_f3p = 0, ph_f3m = 0;
+    uint32_t ph_a3full = 0, ph_b = 0, drained = 0;   // drained: tiles of the slot handed over so far
+    int pair = 0;
     constexpr uint32_t idw = tc::idesc_f16(BF, true, false, 2 * N, 128);
     constexpr uint32_t idn = tc::idesc_f16(BF, true, false, N, 128);
     constexpr uint64_t dF = tc::sdesc_base(G::FB_LBO, G::FB_SBO);
     constexpr uint64_t dA3 = tc::sdesc_base(G::A3_LBO, G::A3_SBO);
     const uint32_t sb16 = sb >> 4;
     for (int p = 0; p < nseq; ++p) {
-        const int fbuf = p & 1;
+        const int fbuf = p & 1, cnt = groups.count(pair);
+        pair = pair + cnt < npairs ? pair + cnt : 0;
         DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((p >> 1) & 1));
         const uint32_t f16 = sb16 + (G::S_F + fbuf * G::F_BLOCK) / 16;
         DGFS_WAITWC(&bars.a3_full, ph_a3full);
         ph_a3full ^= 1u;
         tc::fence_proxy_async();   // the peer's st.async rows, acquired with the barrier, to the tensor core
         tc::tc_fence_after();
-        int n = 0;
-        for (int k = b; k < G::TH; k += 2, ++n) {
-            const uint32_t d = tmem + (b ? G::C_S3 : G::C_S2);
-#pragma unroll
-            for (int sg = 0; sg < 2; ++sg) {   // sign +, then sign -; each half reused once it is read
-                if (n > 0) {
-                    if (sg) {
-                        DGFS_WAITW(&bars.free3m[b], ph_f3m);
-                        ph_f3m ^= 1u;
-                    } else {
-                        DGFS_WAITW(&bars.free3p[b], ph_f3p);
-                        ph_f3p ^= 1u;
-                    }
-                    tc::tc_fence_after();
-                }
-                const uint32_t a16 = sb16 + (G::S_A3 + sg * 2 * G::A3_BYTES + k * G::A3_TS) / 16;
-#pragma unroll
-                for (int ks = 0; ks < G::KSTEPS; ++ks) {
-                    const uint64_t bd = tc::sdesc_at(dF, f16 + (G::OFF_B3 + sg * G::SB_BYTES + ks * 2 * G::FB_LBO) / 16);
-                    tc::mma_ss_warp(d + sg * 2 * N, tc::sdesc_at(dA3, a16 + (ks * 2 * G::A3_LBO) / 16), bd, idw, ks);
-                    tc::mma_ss_warp(d + sg * 2 * N + N, tc::sdesc_at(dA3, a16 + (G::A3_BYTES + ks * 2 * G::A3_LBO) / 16),
-                                    bd, idn, 1);
-                }
-                tc::mma_commit_warp(sg ? &bars.full3m[b] : &bars.full3p[b]);
+        for (int i = 0; i < cnt; ++i) {   // pairs of the group: same operands, their own y filters
+            if (i == 1) {
+                DGFS_WAITW(&bars.filt_b[fbuf], (ph_b >> fbuf) & 1u);
+                ph_b ^= 1u << fbuf;
+                tc::tc_fence_after();
             }
-        }
-        if (n > 0) {   // the pair's last drains of the slot (not waited here)
-            ph_f3p ^= 1u;
-            ph_f3m ^= 1u;
+            const uint32_t fy16 = f16 + (i == 1 ? G::OFF_B1 : G::OFF_B3) / 16;
+            for (int k = b; k < G::TH; k += 2) {
+                const uint32_t d = tmem + (b ? G::C_S3 : G::C_S2);
+#pragma unroll
+                for (int sg = 0; sg < 2; ++sg) {   // sign +, then sign -; each half reused once it is read
+                    if (i > 0 || k > b) {   // the previous tile of this step
+                        DGFS_WAITW(sg ? &bars.free3m[b] : &bars.free3p[b], (drained - 1) & 1u);
+                        tc::tc_fence_after();
+                    }
+                    const uint32_t a16 = sb16 + (G::S_A3 + sg * 2 * G::A3_BYTES + k * G::A3_TS) / 16;
+#pragma unroll
+                    for (int ks = 0; ks < G::KSTEPS; ++ks) {
+                        const uint64_t bd = tc::sdesc_at(dF, fy16 + (sg * G::SB_BYTES + ks * 2 * G::FB_LBO) / 16);
+                        tc::mma_ss_warp(d + sg * 2 * N, tc::sdesc_at(dA3, a16 + (ks * 2 * G::A3_LBO) / 16), bd, idw, ks);
+                        tc::mma_ss_warp(d + sg * 2 * N + N, tc::sdesc_at(dA3, a16 + (G::A3_BYTES + ks * 2 * G::A3_LBO) / 16),
+                                        bd, idn, 1);
+                    }
+                    tc::mma_commit_warp(sg ? &bars.full3m[b] : &bars.full3p[b]);
+                }
+                ++drained;
+            }
         }
         tc::mma_commit_multicast_warp(&bars.a3_free, 0x3);
         tc::mma_commit_warp(&bars.fdone[fbuf]);
@@ -316,8 +337,8 @@ __device__ __forceinline__ void mma3_p3_loop(Bars3& bars, uint32_t sb, uint32_t 
 template <int N, bool BF, bool PAD>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Geo3<N>::THREADS, 1)
 k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const unsigned char* __restrict__ filt,
-           int npairs, int Nrho, int rpc, int nsrc, float* __restrict__ P, int* __restrict__ flags, int fault,
-           const float* __restrict__ coef, int accum) {
+           int npairs, int Nrho, int rpc, TcGroups groups, int ngroups, int nsrc, float* __restrict__ P,
+           int* __restrict__ flags, int fault, const float* __restrict__ coef, int accum) {
     using G = Geo3<N>;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) Bars3 bars;
@@ -329,7 +350,7 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool issuer = warp == G::ISSUER;
     const uint32_t crank = tc::cluster_rank();   // front y-tiles and back x'-tiles [crank TH, crank TH + TH)
-    const int r0 = (blockIdx.x >> 1) * rpc, nseq = npairs * rpc;
+    const int r0 = (blockIdx.x >> 1) * rpc, nseq = ngroups * rpc;   // (radial point, group) steps
     const int64_t node = blockIdx.y;
     constexpr int64_t n3 = (int64_t)N * N * N;
     const int64_t n3s = PAD ? (int64_t)nsrc * nsrc * nsrc : n3;
@@ -338,6 +359,7 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
     const unsigned char* fglob = filt + (size_t)r0 * npairs * G::F_BLOCK;
 
     int copies0 = nseq > 0 ? 1 : 0, copies1 = nseq > 1 ? 1 : 0, waited0 = 0, waited1 = 0;
+    int second0 = 0, second1 = 0;
 
     if (issuer) {
         if (lane == 0) {
@@ -357,17 +379,20 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
                 tc::mbar_init(&bars.free3x[i], 128);
                 tc::mbar_init(&bars.filt[i], 1);
                 tc::mbar_init(&bars.fdone[i], 4);
+                tc::mbar_init(&bars.filt_b[i], 1);
             }
             // the epilogue threads of this CTA whose pass-3 rows are here; the peer's rows arrive as
             // st.async bytes (expect_tx registered by one of these arrivals)
             tc::mbar_init(&bars.a3_full, 128);
             tc::mbar_init(&bars.a3_free, 4);     // the pass-3 MMA warps of both CTAs
+            tc::mbar_init(&bars.p1_done, 1);
             tc::mbar_init(&bars.drain, 4);
             tc::fence_mbar_init();
             s_abort = 0;
             for (int p = 0; p < 2 && p < nseq; ++p) {
                 tc::mbar_expect_tx(&bars.filt[p], G::F_BLOCK);
-                tc::bulk_g2s(smem + G::S_F + p * G::F_BLOCK, fglob + (size_t)p * G::F_BLOCK, G::F_BLOCK, &bars.filt[p]);
+                tc::bulk_g2s(smem + G::S_F + p * G::F_BLOCK, fglob + (size_t)(p ? groups.count(0) : 0) * G::F_BLOCK,
+                             G::F_BLOCK, &bars.filt[p]);   // the first two groups
             }
         }
         __syncwarp();
@@ -452,13 +477,14 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
     if (warp >= G::EPI_WARPS) {
         tc::setmaxnreg_dec<G::REG_MMA>();
         if (warp == G::ISSUER)
-            mma3_p1_loop<N, BF>(bars, smem, sb, tmem, fglob, nseq, abort, copies0, copies1, waited0, waited1);
+            mma3_p1_loop<N, BF>(bars, smem, sb, tmem, fglob, npairs, groups, nseq, abort, copies0, copies1, waited0, waited1,
+                                second0, second1);
         else if (warp == G::ISSUER + 1)
             mma3_p2_loop<N, BF>(bars, sb, tmem, nseq, abort);
         else if (warp == G::ISSUER + 2)
-            mma3_p3_loop<N, BF, 0>(bars, sb, tmem, nseq, abort);
+            mma3_p3_loop<N, BF, 0>(bars, sb, tmem, npairs, groups, nseq, abort);
         else
-            mma3_p3_loop<N, BF, 1>(bars, sb, tmem, nseq, abort);
+            mma3_p3_loop<N, BF, 1>(bars, sb, tmem, npairs, groups, nseq, abort);
     } else {
         tc::setmaxnreg_inc<G::REG_EPI>();
         // warpgroup w: the epilogues of sign w (w = 0: +s, 1: -s) and the back tiles k = w, w + 2, ...
@@ -493,9 +519,10 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
     do {                                                                \
         if (!tc::warp_wait_cluster((bar), (ph), abort)) goto epi_done;  \
     } while (0)
+        int p = 0;   // (radial point, group) step
         for (int rr = 0; rr < rpc; ++rr) {
-          for (int pp = 0; pp < npairs; ++pp) {
-            const int p = rr * npairs + pp;
+          for (int pp = 0, cnt; pp < npairs; pp += cnt, ++p) {
+            cnt = groups.count(pp);
             // front, software-pipelined over the front tiles: pass-1 epilogue of tile s, then the pass-2
             // epilogue of tile s - 1 (whose pass-2 MMAs ran meanwhile)
             for (int st = 0; st <= G::TH; ++st) {
@@ -588,6 +615,8 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
             }
             // back: pass-3 tiles k = w, w + 2, ... in slot 2 + w, products of the two translates
             const uint32_t tB = trow + (w ? G::C_S3 : G::C_S2);
+#pragma unroll 1
+            for (int ip = 0; ip < cnt; ++ip) {   // pairs of the group
 #pragma unroll
             for (int n = 0; n < NB; ++n) {
                 const int k = w + 2 * n;   // warp-uniform
@@ -626,7 +655,7 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
                     if (c == N / 16 - 1) {
                         tc::tc_fence_before();
                         tc::mbar_arrive(&bars.free3m[w]);
-                        if (k + 2 >= G::TH) tc::mbar_arrive(&bars.free3x[w]);
+                        if (k + 2 >= G::TH && ip == cnt - 1) tc::mbar_arrive(&bars.free3x[w]);
                     }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
@@ -635,6 +664,7 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
                         acc[n][8 * c + j] = tc::ffma2(xp[8 * c + j], xm, acc[n][8 * c + j]);
                     }
                 }
+            }
             }
           }
           // radial point r0 + rr done: P_r of this warpgroup's back tiles out, sums cleared
@@ -692,6 +722,9 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
                         atomicOr(flags, 1);
                         break;
                     }
+            for (int i = 0; i < 2; ++i)   // the latest copy of a second pair's filters
+                if (const int n = i ? second1 : second0; n > 0 && !tc::mbar_wait(&bars.filt_b[i], (uint32_t)((n - 1) & 1)))
+                    atomicOr(flags, 1);
         }
         __syncwarp();
         tc::tc_fence_after();
@@ -720,7 +753,7 @@ cudaError_t launch3_n(const TcTables& t, const float* f, const int64_t* offs, in
         const int64_t nn = nodes - n0 < 65535 ? nodes - n0 : 65535;
         kern<<<dim3(2 * (t.Nrho / rpc), (unsigned)nn), G::THREADS, G::S_TOTAL, s>>>(
             f + (offs ? 0 : n0 * n3), offs ? offs + n0 : nullptr, static_cast<const unsigned char*>(t.mats),
-            t.npairs, t.Nrho, rpc, nsrc, P + n0 * t.Nrho * n3, flags, n0 == 0 ? fault : 0, coef ? coef + n0 : nullptr,
+            t.npairs, t.Nrho, rpc, t.groups, t.ngroups, nsrc, P + n0 * t.Nrho * n3, flags, n0 == 0 ? fault : 0, coef ? coef + n0 : nullptr,
             accum);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -800,6 +833,7 @@ size_t build_tc3_tables(const HostPlan& hp, int prec, std::vector<unsigned char>
                         put(blk + (4 + sign) * sbytes, N + i, j, lo);
                     }
         }
+    tc_group_pairs(blob, block, 4 * sbytes, Nr, np, t);
     t.N = N;
     t.nsrc = Nd;
     t.Nrho = Nr;
