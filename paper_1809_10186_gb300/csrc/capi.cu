@@ -222,6 +222,9 @@ void fill_tables(dgfs_plan_s* p, std::vector<unsigned char>& blob, DevTables<T>&
     const size_t o_Uq = take((size_t)h.rank * nq2 * sizeof(T));
     const size_t o_Vr = take(h.Vr.size() * sizeof(T));
     const size_t o_Lr = take(h.Lr.size() * sizeof(T));
+    // the paper's loss weight depends on |k| only (the sphere rule's own weight does not)
+    const bool loss_radial = h.loss_mode == DGFS_LOSS_PAPER && !h.aniso;
+    const size_t o_Lq = take(loss_radial ? (size_t)h.Nrho * nq2 * sizeof(T) : 0);
     const size_t o_GL0 = take(n3 * sizeof(T));
     const size_t o_GLd = take(n3 * sizeof(T));
     const size_t o_W = take((size_t)N * N * 2 * sizeof(T));
@@ -251,6 +254,15 @@ void fill_tables(dgfs_plan_s* p, std::vector<unsigned char>& blob, DevTables<T>&
     }
     put(o_Vr, h.Vr);
     put(o_Lr, h.Lr);
+    if (loss_radial) {
+        T* d = reinterpret_cast<T*>(blob.data() + o_Lq);
+        auto sk = [N](int q) { return q < N / 2 ? q : q - N; };
+        for (size_t i = 0; i < n3; ++i) {
+            const int kx = sk((int)(i / ((size_t)N * N))), ky = sk((int)((i / N) % N)), kz = sk((int)(i % N));
+            for (int r = 0; r < h.Nrho; ++r)
+                d[(size_t)r * nq2 + kx * kx + ky * ky + kz * kz] = (T)h.Lr[(size_t)r * n3 + i];
+        }
+    }
     {
         // loss multiplier of the plan's kernel and its gamma-derivative, summed over r in FP64
         std::vector<double> g0(n3, 0.0), gd(n3, 0.0);
@@ -288,6 +300,7 @@ void fill_tables(dgfs_plan_s* p, std::vector<unsigned char>& blob, DevTables<T>&
     t.Uq = reinterpret_cast<const T*>(o_Uq);
     t.Vr = reinterpret_cast<const T*>(o_Vr);
     t.Lr = reinterpret_cast<const T*>(o_Lr);
+    t.Lq = loss_radial ? reinterpret_cast<const T*>(o_Lq) : nullptr;
     t.GL0 = reinterpret_cast<const T*>(o_GL0);
     t.GLd = reinterpret_cast<const T*>(o_GLd);
     t.dftw = reinterpret_cast<const T*>(o_W);
@@ -320,7 +333,7 @@ void rebase(DevTables<T>& t, void* base) {
         using P = std::remove_reference_t<decltype(ptr)>;
         ptr = reinterpret_cast<P>(static_cast<unsigned char*>(base) + reinterpret_cast<uintptr_t>(ptr));
     };
-    fix(t.filt); fix(t.wsig); fix(t.cr); fix(t.wr); fix(t.Uk); fix(t.Uq); fix(t.Vr); fix(t.Lr); fix(t.GL0); fix(t.GLd);
+    fix(t.filt); fix(t.wsig); fix(t.cr); fix(t.wr); fix(t.Uk); fix(t.Uq); fix(t.Vr); fix(t.Lr); if (t.Lq) fix(t.Lq); fix(t.GL0); fix(t.GLd);
     fix(t.dftw);
 }
 
@@ -584,9 +597,11 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     }
     // gain products: Q(f,f) and dQ/dgamma use (f, f); Q(f,g) uses (f, g); JVP uses (f, v)
     const T* gg = quadratic(op) ? nullptr : g;
+    // (N = 12, 24: the separate kernels where keeps_rounding holds on to their rounding)
+    const bool fused = spectral_supported(t) && !(keeps_rounding<T>(op) && t.N % 3 == 0);
     NvtxRange translate_range("dgfs translate products");
     if (p->prof) {
-        p->prof_launches += (spectral_supported(tables<T>(p)) ? 5 : 11 + (op == Op::Jvp ? 1 : 0)) +
+        p->prof_launches += (fused ? 5 : 11 + (op == Op::Jvp ? 1 : 0)) +
                             tc_extra_launches(p->prec);
         p->prof_gain += 1;
         p->prof_nodes += nodes;
@@ -627,7 +642,7 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     }
     // real fields packed two per complex slot: the rank projected fields, then the loss
     // operand(s): Q(f,g) -> field rank = g;  JVP -> field rank = v, field rank + 1 = f
-    if (spectral_supported(t)) {   // the fused three-launch Fourier stage
+    if (fused) {   // the fused Fourier stage
         const T* la = quadratic(op) ? f : g;
         e = launch_spectral<T>(t, P, np, nodes, la, op == Op::Jvp ? f : nullptr, offs,
                                op == Op::Jvp ? T(2) : T(1), X, Y, f, op == Op::Jvp ? g : nullptr, out,

@@ -94,6 +94,17 @@ __device__ __forceinline__ Cplx<float> twice_minus<float>(Cplx<float> u, Cplx<fl
     return unpack(r);
 }
 
+// a + c x with the constant c in two FP32 terms (the first a multiple of 1/128, the second's rounding below
+// 4e-10): N = 12, 24 take the constants sqrt(1/2) and sqrt(3)/2 of their short stages this way, because both
+// round 1.7e-8 down and shorten every line (a round trip at N = 24 loses 1.3e-8 instead of 3.3e-8).
+constexpr double kHalfRoot = quarter32(4), kRoot34 = quarter24(2);
+template <typename T>
+__device__ __forceinline__ T plus_scaled(T a, T x, double c) {
+    if (sizeof(T) == 8) return fma((T)c, x, a);
+    const double head = (double)(int)(c * 128.0) / 128.0;
+    return fma((T)(c - head), x, fma((T)head, x, a));
+}
+
 // radix-2 stages of a length-S transform in a[OFF .. OFF + S), spans LEN, 2 LEN, ..., S
 template <typename T, int NA, int OFF, int S, int LEN, bool FWD>
 __device__ __forceinline__ void stages(Cplx<T> (&a)[NA]) {
@@ -111,6 +122,11 @@ __device__ __forceinline__ void stages(Cplx<T> (&a)[NA]) {
                 const T sg = FWD ? T(1) : T(-1);
                 s = Cplx<T>{u.x + sg * v.y, u.y - sg * v.x};
                 d = Cplx<T>{u.x - sg * v.y, u.y + sg * v.x};
+            } else if (sizeof(T) == 4 && NA % 3 == 0 && LEN == 8) {   // (+-1 +- i) sqrt(1/2), exact to 1e-10
+                const T sr = cos_of<8>(j) > 0 ? T(1) : T(-1), si = FWD ? T(-1) : T(1);
+                const Cplx<T> t{sr * v.x - si * v.y, si * v.x + sr * v.y};
+                s = Cplx<T>{plus_scaled<T>(u.x, t.x, kHalfRoot), plus_scaled<T>(u.y, t.y, kHalfRoot)};
+                d = twice_minus(u, s);
             } else {
                 const T wr = (T)cos_of<LEN>(j), wi = FWD ? (T)(-sin_of<LEN>(j)) : (T)sin_of<LEN>(j);
                 s = Cplx<T>{fma(-wi, v.y, fma(wr, v.x, u.x)), fma(wi, v.x, fma(wr, v.y, u.y))};
@@ -133,7 +149,7 @@ __device__ __forceinline__ void line(Cplx<T> (&a)[N]) {
         stages<T, N, S, S, 2, FWD>(a);
         stages<T, N, 2 * S, S, 2, FWD>(a);
         // X[q + m S], m = 0, 1, 2, from y0 and the twiddled y1, y2 (one radix-3 butterfly)
-        const T c3 = FWD ? (T)(-quarter24(2)) : (T)quarter24(2);   // -+ sin(2 pi / 3)
+        constexpr double c3 = FWD ? -kRoot34 : kRoot34;   // -+ sin(2 pi / 3)
 #pragma unroll
         for (int q = 0; q < S; ++q) {
             const Cplx<T> y0 = a[q], y1 = a[S + q], y2 = a[2 * S + q];
@@ -147,8 +163,8 @@ __device__ __forceinline__ void line(Cplx<T> (&a)[N]) {
             const Cplx<T> p{t1.x + t2.x, t1.y + t2.y}, d{t1.x - t2.x, t1.y - t2.y};
             const Cplx<T> m{fma(T(-0.5), p.x, y0.x), fma(T(-0.5), p.y, y0.y)};
             a[q] = Cplx<T>{y0.x + p.x, y0.y + p.y};
-            a[S + q] = Cplx<T>{fma(-c3, d.y, m.x), fma(c3, d.x, m.y)};
-            a[2 * S + q] = Cplx<T>{fma(c3, d.y, m.x), fma(-c3, d.x, m.y)};
+            a[S + q] = Cplx<T>{plus_scaled<T>(m.x, d.y, -c3), plus_scaled<T>(m.y, d.x, c3)};
+            a[2 * S + q] = Cplx<T>{plus_scaled<T>(m.x, d.y, c3), plus_scaled<T>(m.y, d.x, -c3)};
         }
     }
 }
@@ -156,7 +172,7 @@ __device__ __forceinline__ void line(Cplx<T> (&a)[N]) {
 // 1 - (mean diagonal of inverse times forward line / N) with the twiddles rounded to FP32, the rest exact:
 // the relative loss of a round trip. |w| of the rounded twiddles of these lengths is below 1 on average.
 __host__ __device__ constexpr double line_loss(int N) {
-    return N == 8 ? 0.86e-8 : N == 12 ? 2.09e-8 : N == 16 ? 2.71e-8 : N == 24 ? 3.32e-8 : 4.55e-8;
+    return N == 8 ? 0.86e-8 : N == 12 ? 0.90e-8 : N == 16 ? 2.71e-8 : N == 24 ? 1.27e-8 : 4.55e-8;
 }
 
 }  // namespace cfft

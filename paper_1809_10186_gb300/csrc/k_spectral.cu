@@ -1,4 +1,4 @@
-// Fused Fourier stage for power-of-two grids (N = 8, 16, 32): the same arithmetic as the
+// Fused Fourier stage (N = 8, 12, 16, 24, 32): the same operations as the
 // projection, forward DFT, Fourier combine, inverse DFT and finalisation kernels of
 // k_fourier.cu (arXiv:1809.10186, Appendix, eqs. realGG, lowrank1, apndx_fs_Glm_Qk), in four
 // launches whose intermediates stay in shared memory or registers between the axis passes:
@@ -20,7 +20,7 @@
 // Twiddles are compile-time constants (cos 2 pi m / 32), so the FFT lines load nothing but data.
 #include <cstdint>
 
-#include "fourier_dev.cuh"
+#include "fft_const.cuh"
 #include "launchers.h"
 
 namespace dgfs {
@@ -34,12 +34,15 @@ struct SpecGeo {
     static constexpr int N2 = N * N;
     static constexpr int ROW = N + 1;                          // padded plane row (complex values)
     static constexpr int PLANE = N * ROW;
-    static constexpr int T1 = N == 8 ? 64 : 256;                // k_spec_xz: V points per thread
+    // k_spec_xz: V points per thread (2 at N = 12, 24: four would need 104 accumulators for the 26 fields
+    // of an uncompressed kernel, or a second pass over P)
+    static constexpr int T1 = N == 8 ? 64 : N == 12 ? 72 : N == 24 ? 288 : 256;
     static constexpr int V = N2 / T1;
     static constexpr int RB = N == 32 ? 5 : 8;                  // radial points of P in flight per thread
-    static constexpr int T2 = 256;                             // k_spec_y
-    static constexpr int YP = N * N <= 256 ? N : 256 / N;      // k_spec_xout: planes y per CTA
-    static_assert(V == 1 || V == 4, "points per thread");
+    static constexpr int T2 = N % 3 == 0 ? 192 : 256;          // k_spec_y: whole planes of lines
+    static constexpr int YP = N == 24 ? 8 : N * N <= 256 ? N : 256 / N;   // k_spec_xout: planes y per CTA
+    static_assert(V == 1 || V == 2 || V == 4, "points per thread");
+    static_assert(N2 % T1 == 0 && T2 % N == 0 && N % YP == 0, "whole lines and planes");
 };
 
 // ---- constant twiddles ------------------------------------------------------------------
@@ -88,11 +91,11 @@ __device__ __forceinline__ void fftc_stage(Cplx<T> (&a)[N]) {
     if constexpr (LEN < N) fftc_stage<T, N, 2 * LEN, FWD>(a);
 }
 
-// Unnormalised DFT of one line in registers (element k loaded into a[bitrev(k)]), natural order out.
+// Unnormalised DFT of one line in registers (element k loaded into a[line_slot(k)]), natural order out.
 template <typename T, int N, bool FWD>
 __device__ __forceinline__ void fftc(Cplx<T> (&a)[N]) {
-    static_assert(N <= 32 && (N & (N - 1)) == 0, "power-of-two lines up to 32");
-    fftc_stage<T, N, 2, FWD>(a);
+    if constexpr ((N & (N - 1)) == 0) fftc_stage<T, N, 2, FWD>(a);
+    else cfft::line<T, N, FWD>(a);   // N = 12, 24
 }
 
 // 8- or 16-byte accesses of one complex value (Cplx<T> itself is only T-aligned)
@@ -122,7 +125,7 @@ template <typename T, int N, bool FWD>
 __device__ __forceinline__ void fftc_smem_line(Cplx<T>* base, int stride) {
     Cplx<T> a[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) a[bitrev<N>(k)] = ldc(base + k * stride);
+    for (int k = 0; k < N; ++k) a[line_slot<N>(k)] = ldc(base + k * stride);
     fftc<T, N, FWD>(a);
 #pragma unroll
     for (int k = 0; k < N; ++k) stc(base + k * stride, a[k]);
@@ -158,16 +161,30 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 }
 
 // ---- kernel 0: projection coefficients ---------------------------------------------------
-// C[node][r][s] = Vr[s][r] (w_r rho_r(node)): one block per node (or one for the whole launch).
+// C[node][r][s] = Vr[s][r] (w_r rho_r(node)): one block per node (or one for the whole launch). With Lq
+// (per-node gamma or b, a loss weight of |k| alone), also the loss multiplier GLq[node][|k|^2]: the same FP64
+// sum over r as loss_multiplier, once for each of the 3 (N/2)^2 + 1 values of |k|^2 instead of at every mode
+// (the ragged cavity batch spent 1.2 of 14.3 ms on those sums at N = 32 alone).
 template <typename T>
 __global__ void k_spec_coef(const T* __restrict__ Vr, const double* __restrict__ cr, const double* __restrict__ wr,
-                            NodeParams np, int Nrho, int rank, T* __restrict__ C) {
+                            NodeParams np, int Nrho, int rank, T* __restrict__ C, const T* __restrict__ Lq, int nq2,
+                            T* __restrict__ GLq) {
     __shared__ T wrho[64];
+    __shared__ double rho[64];
     const int64_t node = blockIdx.x;
     const double gam = np.gamma ? np.gamma[node] : np.gamma0;
     const double bb = np.b ? np.b[node] : np.b0;
-    for (int r = threadIdx.x; r < Nrho; r += blockDim.x) wrho[r] = (T)wr[r] * radial_rho<T>(bb, gam, cr[r], np.dlog);
+    for (int r = threadIdx.x; r < Nrho; r += blockDim.x) {
+        wrho[r] = (T)wr[r] * radial_rho<T>(bb, gam, cr[r], np.dlog);
+        if (Lq) rho[r] = radial_rho<double>(bb, gam, cr[r], np.dlog);
+    }
     __syncthreads();
+    if (Lq)
+        for (int q = threadIdx.x; q < nq2; q += blockDim.x) {
+            double g = 0.0;
+            for (int r = 0; r < Nrho; ++r) g = fma(rho[r], (double)Lq[r * nq2 + q], g);
+            GLq[node * nq2 + q] = (T)g;
+        }
     T* Cn = C + node * Nrho * rank;
     for (int e = threadIdx.x; e < Nrho * rank; e += blockDim.x) {
         const int r = e / rank, s = e % rank;
@@ -179,13 +196,13 @@ __global__ void k_spec_coef(const T* __restrict__ Vr, const double* __restrict__
 // CTA (slot group g, plane y) of a node: slots [g slg, g slg + ns) of the packed fields (every slot
 // in one group when they fit, so that the plane of P, Nrho N^2 values, is read once).
 template <typename T, int N, int SL>
-__global__ void __launch_bounds__(SpecGeo<N>::T1, N == 32 ? 2 : 1)
+__global__ void __launch_bounds__(SpecGeo<N>::T1, N == 32 || (N == 24 && sizeof(T) == 4) ? 2 : 1)
 k_spec_xz(const T* __restrict__ P, const T* __restrict__ Cg, int64_t c_stride, int Nrho, int rank,
           const T* __restrict__ la, const T* __restrict__ lb, const int64_t* __restrict__ offs, int nloss,
           Cplx<T>* __restrict__ X, int xs, int groups, int slg) {
     using G = SpecGeo<N>;
     constexpr int FG = 2 * SL;                                  // fields of one slot group (at most)
-    constexpr bool PAIRS = sizeof(T) == 4 && G::V == 4;         // two points per FP32 FMA instruction
+    constexpr bool PAIRS = sizeof(T) == 4 && G::V >= 2;         // two points per FP32 FMA instruction
     extern __shared__ __align__(16) unsigned char sm_raw[];
     Cplx<T>* F = reinterpret_cast<Cplx<T>*>(sm_raw);           // [SL][PLANE]
     T* C = reinterpret_cast<T*>(F + SL * G::PLANE);             // [Nrho][FG] (pairs {c, c}: [Nrho][FG][2])
@@ -221,26 +238,34 @@ k_spec_xz(const T* __restrict__ P, const T* __restrict__ Cg, int64_t c_stride, i
 #pragma unroll
         for (int r = 0; r < G::RB; ++r) issue(r, r);
         if constexpr (PAIRS) {
-            float2 acc[2][FG];
+            constexpr int H = G::V / 2;   // point pairs
+            float2 acc[H][FG];
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+            for (int h = 0; h < H; ++h)
 #pragma unroll
                 for (int i = 0; i < FG; ++i) acc[h][i] = make_float2(0.f, 0.f);
             int slot = 0;
 #pragma unroll 1
             for (int r = 0; r < Nrho; ++r) {
                 cp_async_wait_group<G::RB - 1>();   // the copy of P_r has landed
-                const float4 p = *reinterpret_cast<const float4*>(mine + slot * (G::T1 * G::V));
-                const float2 p01 = make_float2(p.x, p.y), p23 = make_float2(p.z, p.w);
+                float2 p[H];
+                if constexpr (H == 2) {
+                    const float4 v = *reinterpret_cast<const float4*>(mine + slot * (G::T1 * G::V));
+                    p[0] = make_float2(v.x, v.y);
+                    p[1] = make_float2(v.z, v.w);
+                } else {
+                    p[0] = *reinterpret_cast<const float2*>(mine + slot * (G::T1 * G::V));
+                }
                 const float4* c4 = reinterpret_cast<const float4*>(C + 2 * r * FG);
 #pragma unroll
                 for (int i = 0; i < FG; i += 2) {
                     const float4 cc = c4[i / 2];    // {c_i, c_i, c_i+1, c_i+1}
                     const float2 ci = make_float2(cc.x, cc.y), cj = make_float2(cc.z, cc.w);
-                    acc[0][i] = fma2(ci, p01, acc[0][i]);
-                    acc[1][i] = fma2(ci, p23, acc[1][i]);
-                    acc[0][i + 1] = fma2(cj, p01, acc[0][i + 1]);
-                    acc[1][i + 1] = fma2(cj, p23, acc[1][i + 1]);
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        acc[h][i] = fma2(ci, p[h], acc[h][i]);
+                        acc[h][i + 1] = fma2(cj, p[h], acc[h][i + 1]);
+                    }
                 }
                 issue(r + G::RB, slot);   // after the FMAs that consumed the slot's values
                 slot = slot + 1 == G::RB ? 0 : slot + 1;
@@ -250,10 +275,11 @@ k_spec_xz(const T* __restrict__ P, const T* __restrict__ Cg, int64_t c_stride, i
             for (int i = 0; i < FG; i += 2)
                 if (i / 2 < ns) {
                     Cplx<T>* d = F + (i / 2) * G::PLANE + x * G::ROW + z0;
-                    stc(d + 0, Cplx<T>{acc[0][i].x, acc[0][i + 1].x});
-                    stc(d + 1, Cplx<T>{acc[0][i].y, acc[0][i + 1].y});
-                    stc(d + 2, Cplx<T>{acc[1][i].x, acc[1][i + 1].x});
-                    stc(d + 3, Cplx<T>{acc[1][i].y, acc[1][i + 1].y});
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        stc(d + 2 * h, Cplx<T>{acc[h][i].x, acc[h][i + 1].x});
+                        stc(d + 2 * h + 1, Cplx<T>{acc[h][i].y, acc[h][i + 1].y});
+                    }
                 }
         } else {
             T acc[G::V][FG];
@@ -331,22 +357,18 @@ k_spec_xz(const T* __restrict__ P, const T* __restrict__ Cg, int64_t c_stride, i
 // rank, so the gain sum runs without branches. The loss field(s) are picked up in a separate pass
 // of the group that holds them and parked, times their multiplier, in this CTA's planes of Y until
 // the inverse transforms.
-template <int N>
-constexpr int ilog2() { return N == 8 ? 3 : N == 16 ? 4 : 5; }
-
 // Row stride of k_spec_y's factor table: every field of a slot group, plus one pair of padding (an
 // even stride, so that a pair of factors loads as 8 bytes; 18 at N = 32 spreads a warp's rows over
 // the banks).
 template <int N>
-constexpr int spec_y_table_stride() { return 2 * (256 / N) + 2; }
+constexpr int spec_y_table_stride() { return 2 * (SpecGeo<N>::T2 / N) + 2; }
 
 template <typename T, int N, int NL>
 __global__ void __launch_bounds__(SpecGeo<N>::T2, 2)
 k_spec_y(const Cplx<T>* __restrict__ X, int xs, const T* __restrict__ Uq, int nq2, const T* __restrict__ Lr,
-         const T* __restrict__ GL0, const T* __restrict__ GLd, const double* __restrict__ cr, NodeParams np,
-         int Nrho, int rank, int lf0, int lf1, T gscale, T lscale, Cplx<T>* __restrict__ Y, int yf) {
+         const T* __restrict__ GL0, const T* __restrict__ GLd, const T* __restrict__ GLq, const double* __restrict__ cr,
+         NodeParams np, int Nrho, int rank, int lf0, int lf1, T gscale, T lscale, Cplx<T>* __restrict__ Y, int yf) {
     using G = SpecGeo<N>;
-    constexpr int LN = ilog2<N>();
     constexpr int GSX = G::T2 / N;                      // slots (planes) of the buffer: a group of one-plane CTAs
     constexpr int PT = (2 * G::N2 + G::T2 - 1) / G::T2; // combine points per thread (two planes)
     constexpr int MR = 2 * (N / 2) * (N / 2) + 1;       // |ky|^2 + |kz|^2 = 0 .. 2 (N/2)^2
@@ -358,18 +380,18 @@ k_spec_y(const Cplx<T>* __restrict__ X, int xs, const T* __restrict__ Uq, int nq
     double* rho = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(Us + MR * US) + 15) & ~uintptr_t(15));
     const int c = blockIdx.x, t = threadIdx.x;
     const int npl = (c == 0 || c == N / 2) ? 1 : 2, sh = npl - 1;
-    const int kx0 = c, kx1 = N - c, GS = G::T2 >> (LN + sh);
+    const int kx0 = c, kx1 = N - c, GS = (G::T2 / N) >> sh;
     const int kq = signed_q<N>(kx0), kx2 = kq * kq;
     const int64_t node = blockIdx.y, n3 = (int64_t)N * G::N2;
     const bool per_node = np.gamma || np.b;
-    if (per_node) {
+    if (per_node && !GLq) {
         const double gam = np.gamma ? np.gamma[node] : np.gamma0;
         const double bb = np.b ? np.b[node] : np.b0;
         for (int r = t; r < Nrho; r += G::T2) rho[r] = radial_rho<double>(bb, gam, cr[r], np.dlog);
     }
     const Cplx<T>* Xn = X + node * (int64_t)xs * n3;
     // this thread's y line
-    const int ljm = t >> (LN + sh), lpl = (t >> LN) & sh, lkz = t & (N - 1);
+    const int ljm = (t / N) >> sh, lpl = (t / N) & sh, lkz = t % N;
     const int64_t loff = (int64_t)(lpl ? kx1 : kx0) * G::N2 + lkz;   // X[m][kx][y][kz] at y = 0
     const int npts = npl * G::N2;
     // this thread's combine points e = t + i T2: plane e / N^2, (ky, kz); row |ky|^2 + |kz|^2 of the table
@@ -377,19 +399,19 @@ k_spec_y(const Cplx<T>* __restrict__ X, int xs, const T* __restrict__ Uq, int nq
     T gr[PT], gi[PT];
 #pragma unroll
     for (int i = 0; i < PT; ++i) {
-        const int e = t + i * G::T2, ky = (e >> LN) & (N - 1), kz = e & (N - 1);
+        const int e = t + i * G::T2, ky = (e / N) % N, kz = e % N;
         mrow[i] = signed_q<N>(ky) * signed_q<N>(ky) + signed_q<N>(kz) * signed_q<N>(kz);
         gr[i] = gi[i] = T(0);
     }
     Cplx<T>* Yn = Y + node * (int64_t)yf * n3;
     auto kidx = [&](int e) {   // spectrum index of point e
-        const int pl = e >> (2 * LN), ky = (e >> LN) & (N - 1), kz = e & (N - 1);
+        const int pl = e / G::N2, ky = (e / N) % N, kz = e % N;
         return ((int64_t)(pl ? kx1 : kx0) * N + ky) * N + kz;
     };
     // the two spectra a slot packs at point e (times 2): field 2m in fa, field 2m + 1 in fb
     auto unpack = [&](int e, int jm, Cplx<T>& fa, Cplx<T>& fb) {
-        const int pl = e >> (2 * LN), ky = (e >> LN) & (N - 1), kz = e & (N - 1);
-        const int pm = npl == 2 ? 1 - pl : pl, kym = (N - ky) & (N - 1), kzm = (N - kz) & (N - 1);
+        const int pl = e / G::N2, ky = (e / N) % N, kz = e % N;
+        const int pm = npl == 2 ? 1 - pl : pl, kym = ky ? N - ky : 0, kzm = kz ? N - kz : 0;
         const Cplx<T> z = ldc(buf + (jm * npl + pl) * G::PLANE + ky * G::ROW + kz);
         const Cplx<T> w = ldc(buf + (jm * npl + pm) * G::PLANE + kym * G::ROW + kzm);
         fa = Cplx<T>{z.x + w.x, z.y - w.y};
@@ -400,7 +422,7 @@ k_spec_y(const Cplx<T>* __restrict__ X, int xs, const T* __restrict__ Uq, int nq
         if (g0 + ljm < xs) {
             const Cplx<T>* src = Xn + (int64_t)(g0 + ljm) * n3 + loff;
 #pragma unroll
-            for (int k = 0; k < N; ++k) a[bitrev<N>(k)] = ldgc(src + k * N);
+            for (int k = 0; k < N; ++k) a[line_slot<N>(k)] = ldgc(src + k * N);
         }
     };
     // factors of the group's fields [f0, f0 + nf) at |k|^2 = |kx|^2 + row, into table columns
@@ -464,7 +486,8 @@ k_spec_y(const Cplx<T>* __restrict__ X, int xs, const T* __restrict__ Uq, int nq
                 unpack(e, jm, fa, fb);
                 const Cplx<T> v = h ? fb : fa;
                 const int64_t k = kidx(e);
-                const T GL = lscale * loss_multiplier<T>(GL0, GLd, Lr, rho, per_node, np.dlog, Nrho, n3, k);
+                const T GL = lscale * (GLq ? __ldg(GLq + node * nq2 + kx2 + mrow[i])
+                                           : loss_multiplier<T>(GL0, GLd, Lr, rho, per_node, np.dlog, Nrho, n3, k));
                 stc(Yn + (1 + jl) * n3 + k, Cplx<T>{GL * v.x, GL * v.y});
             }
         }
@@ -475,7 +498,7 @@ k_spec_y(const Cplx<T>* __restrict__ X, int xs, const T* __restrict__ Uq, int nq
     for (int i = 0; i < PT; ++i) {
         const int e = t + i * G::T2;
         if (e >= npts) continue;
-        const int pl = e >> (2 * LN), ky = (e >> LN) & (N - 1), kz = e & (N - 1);
+        const int pl = e / G::N2, ky = (e / N) % N, kz = e % N;
         const int64_t k = kidx(e);
         const int o = pl * G::PLANE + ky * G::ROW + kz;
         stc(buf + o, Cplx<T>{gscale * gr[i], gscale * gi[i]});
@@ -484,17 +507,17 @@ k_spec_y(const Cplx<T>* __restrict__ X, int xs, const T* __restrict__ Uq, int nq
     }
     __syncthreads();
     for (int id = t; id < yf * npl * N; id += G::T2) {   // inverse along y: line (field, plane, kz)
-        const int fp = id >> LN, kz = id & (N - 1);     // fp = field npl + plane
+        const int fp = id / N, kz = id % N;             // fp = field npl + plane
         fftc_smem_line<T, N, false>(buf + fp * G::PLANE + kz, G::ROW);
     }
     __syncthreads();
     for (int id = t; id < yf * npl * N; id += G::T2) {   // inverse along z: line (field, plane, y)
-        const int fp = id >> LN, yy = id & (N - 1);
+        const int fp = id / N, yy = id % N;
         fftc_smem_line<T, N, false>(buf + fp * G::PLANE + yy * G::ROW, 1);
     }
     __syncthreads();
     for (int e = t; e < yf * npl * G::N2; e += G::T2) {   // Y[field][kx][y][z]
-        const int fp = e >> (2 * LN), fo = fp >> sh, pl = fp & sh, yy = (e >> LN) & (N - 1), z = e & (N - 1);
+        const int fp = e / G::N2, fo = fp >> sh, pl = fp & sh, yy = (e / N) % N, z = e % N;
         stc(Yn + fo * n3 + ((int64_t)(pl ? kx1 : kx0) * N + yy) * N + z, ldc(buf + fp * G::PLANE + yy * G::ROW + z));
     }
 }
@@ -512,7 +535,7 @@ k_spec_xout(const Cplx<T>* __restrict__ Y, int yf, const T* __restrict__ a, cons
     Cplx<T> line[N];
     T q[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) line[bitrev<N>(k)] = ldgc(Yn + k * G::N2);
+    for (int k = 0; k < N; ++k) line[line_slot<N>(k)] = ldgc(Yn + k * G::N2);
     fftc<T, N, false>(line);
 #pragma unroll
     for (int k = 0; k < N; ++k) q[k] = line[k].x;
@@ -520,7 +543,7 @@ k_spec_xout(const Cplx<T>* __restrict__ Y, int yf, const T* __restrict__ a, cons
     for (int fo = 1; fo < yf; ++fo) {
         const T* mul = fo == 1 ? a : c;
 #pragma unroll
-        for (int k = 0; k < N; ++k) line[bitrev<N>(k)] = ldgc(Yn + fo * n3 + k * G::N2);
+        for (int k = 0; k < N; ++k) line[line_slot<N>(k)] = ldgc(Yn + fo * n3 + k * G::N2);
         fftc<T, N, false>(line);
 #pragma unroll
         for (int k = 0; k < N; ++k) q[k] -= mul[base + k * G::N2] * line[k].x;
@@ -539,7 +562,7 @@ cudaError_t launch_xz(const T* P, const T* C, int64_t c_stride, int Nrho, int ra
                       const int64_t* offs, int nloss, Cplx<T>* X, int xs, int groups, int slg, unsigned nn,
                       cudaStream_t s) {
     using G = SpecGeo<N>;
-    constexpr bool PAIRS = sizeof(T) == 4 && G::V == 4;
+    constexpr bool PAIRS = sizeof(T) == 4 && G::V >= 2;
     const size_t sm = sizeof(Cplx<T>) * (size_t)SL * G::PLANE + sizeof(T) * (size_t)Nrho * 2 * SL * (PAIRS ? 2 : 1) +
                       16 + sizeof(T) * (size_t)G::RB * G::T1 * G::V;
     cudaError_t e = cudaFuncSetAttribute(k_spec_xz<T, N, SL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -550,15 +573,15 @@ cudaError_t launch_xz(const T* P, const T* C, int64_t c_stride, int Nrho, int ra
 }
 
 // Largest slot group of one k_spec_xz CTA: the plane buffer stays within ~85 KB so that two CTAs
-// share an SM (N = 32) and the accumulators within the register budget.
+// share an SM (N = 24, 32) and the accumulators within the register budget.
 template <typename T, int N>
 constexpr int max_group_slots() {
-    return N == 32 ? 10 : 17;
+    return N == 32 ? 10 : N % 3 == 0 ? 13 : 17;   // 13: every field of an uncompressed N = 24 kernel
 }
 
 template <typename T, int N>
 cudaError_t spectral_n(const DevTables<T>& t, const T* P, NodeParams np, int64_t nodes, const T* la,
-                       const T* lb, const int64_t* offs, T gain_scale, const T* C, int64_t c_stride,
+                       const T* lb, const int64_t* offs, T gain_scale, const T* C, int64_t c_stride, const T* GLq,
                        Cplx<T>* X, Cplx<T>* Y, const T* fa, const T* fc, T* out, int* flags, cudaStream_t s) {
     using G = SpecGeo<N>;
     const int nloss = lb ? 2 : 1, nfields = t.rank + nloss, xs = (nfields + 1) / 2, yf = lb ? 3 : 2;
@@ -587,7 +610,7 @@ cudaError_t spectral_n(const DevTables<T>& t, const T* P, NodeParams np, int64_t
         auto kern = lb ? k_spec_y<T, N, 2> : k_spec_y<T, N, 1>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        kern<<<dim3(N / 2 + 1, nn), G::T2, sm, s>>>(X, xs, t.Uq, 3 * (N / 2) * (N / 2) + 1, t.Lr, t.GL0, t.GLd, t.cr, np,
+        kern<<<dim3(N / 2 + 1, nn), G::T2, sm, s>>>(X, xs, t.Uq, 3 * (N / 2) * (N / 2) + 1, t.Lr, t.GL0, t.GLd, GLq, t.cr, np,
                                                 t.Nrho, t.rank, t.rank, lb ? t.rank + 1 : -1, gain_scale * post, post,
                                                 Y, yf);
         e = cudaGetLastError();
@@ -602,8 +625,8 @@ cudaError_t spectral_n(const DevTables<T>& t, const T* P, NodeParams np, int64_t
 template <typename T>
 bool spectral_supported(const DevTables<T>& t) {
     if (t.rank < 1 || t.rank > 32 || t.Nrho > 64) return false;
-    if (t.N == 8 || t.N == 16) return true;
-    return t.N == 32 && sizeof(T) == 4;
+    if (t.N == 8 || t.N == 12 || t.N == 16) return true;
+    return (t.N == 24 || t.N == 32) && sizeof(T) == 4;
 }
 
 template <typename T>
@@ -619,12 +642,16 @@ cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, in
     const bool per_node = np.gamma || np.b;
     T* C = reinterpret_cast<T*>(X + nodes * xs * n3);
     const int64_t c_stride = per_node ? (int64_t)t.Nrho * t.rank : 0;
+    // the per-node loss table after the coefficients (one complex field per node is left past the slots)
+    const int nq2 = 3 * (t.N / 2) * (t.N / 2) + 1;
+    T* GLq = per_node && t.Lq ? C + nodes * c_stride : nullptr;
     for (int64_t n0 = 0; n0 < (per_node ? nodes : 1); n0 += 65535) {
         const int64_t nn = (per_node ? nodes : 1) - n0 < 65535 ? (per_node ? nodes : 1) - n0 : 65535;
         NodeParams np0 = np;
         if (np.gamma) np0.gamma = np.gamma + n0;
         if (np.b) np0.b = np.b + n0;
-        k_spec_coef<T><<<(unsigned)nn, 128, 0, s>>>(t.Vr, t.cr, t.wr, np0, t.Nrho, t.rank, C + n0 * c_stride);
+        k_spec_coef<T><<<(unsigned)nn, 128, 0, s>>>(t.Vr, t.cr, t.wr, np0, t.Nrho, t.rank, C + n0 * c_stride,
+                                                          GLq ? t.Lq : nullptr, nq2, GLq ? GLq + n0 * nq2 : nullptr);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -642,18 +669,18 @@ cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, in
         const T* fc0 = fc ? fc + fo : nullptr;
         T* out0 = out + fo;
         const T* C0 = C + n0 * c_stride;
+        const T* Q0 = GLq ? GLq + n0 * nq2 : nullptr;
         NodeParams np0 = np;
         if (np.gamma) np0.gamma = np.gamma + n0;
         if (np.b) np0.b = np.b + n0;
         cudaError_t e = cudaErrorNotSupported;
-        if (t.N == 8)
-            e = spectral_n<T, 8>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, X0, Y0, fa0, fc0, out0, flags, s);
-        else if (t.N == 16)
-            e = spectral_n<T, 16>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, X0, Y0, fa0, fc0, out0, flags,
-                                  s);
-        else if constexpr (sizeof(T) == 4)
-            e = spectral_n<T, 32>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, X0, Y0, fa0, fc0, out0, flags,
-                                  s);
+        switch (t.N) {
+            case 8: e = spectral_n<T, 8>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
+            case 12: e = spectral_n<T, 12>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
+            case 16: e = spectral_n<T, 16>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
+            case 24: if constexpr (sizeof(T) == 4) e = spectral_n<T, 24>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
+            case 32: if constexpr (sizeof(T) == 4) e = spectral_n<T, 32>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
+        }
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

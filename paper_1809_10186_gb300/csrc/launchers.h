@@ -19,6 +19,7 @@ struct DevTables {
     const T* Uq;        // [rank][3 (N/2)^2 + 1]: Uk[s](k) = Uq[s][|k|^2] (signed lattice index)
     const T* Vr;        // [rank][Nrho]
     const T* Lr;        // [Nrho][N^3]  DFT index order
+    const T* Lq;        // [Nrho][3 (N/2)^2 + 1]: Lr[r](k) = Lq[r][|k|^2]; nullptr when Lr depends on k itself
     const T* GL0;       // [N^3] sum_r rho_r(gamma, b) Lr[r]: loss multiplier of the plan's kernel
     const T* GLd;       // [N^3] sum_r ln(c_r) rho_r Lr[r]: its derivative with respect to gamma
     const T* dftw;      // [N][N] complex (re, im interleaved): e^{-2 pi i q j / N}

@@ -34,7 +34,9 @@
 // tile i, then the pass-2 epilogue of tile i - 1, whose MMAs ran meanwhile); in the back it forms
 // the products of the pass-3 tiles in slot 2 + w, accumulating P_r in registers (the slot's two sign
 // halves are completed and released separately, so the next tile's + MMAs overlap the read of the
-// - half). Every wait is bounded; on
+// - half). Adjacent pairs with the same x and z filters (tc_group_pairs) share the front: the second one's
+// y filters are copied over the x filters and pass 3 runs again on the same operands (M = 38: 15 fronts
+// for 19 pairs; 333 nodes at N = 32: 18.6 -> 16.6 ms, the same bits). Every wait is bounded; on
 // timeout the CTA raises flag bit 0, every role stops at its next wait, the MMAs and copies in
 // flight are drained, TMEM is freed and no P_r is written; both CTAs meet at a final cluster barrier.
 #include <cmath>
