@@ -5,14 +5,14 @@
 // compute call loops over node chunks and enqueues, per chunk,
 //   1. the translate products                  P_r = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)]
 //      (tensor cores for the tensor-core plans, tc_gain.cu and tc_gain3.cu; Fourier-space translates for
-//      FP32/FP64 plans, k_shift.cu; the dense circulant kernel, k_gain_simt.cuh, for the allocation-free
+//      FP32/FP64 plans, k_shift.cu and k_pair.cu; the dense circulant kernel, k_gain_simt.cuh, for the allocation-free
 //      call of FP32/FP64 plans)
 //   2. the radial projection                   X_s = sum_r Vr[s][r] w_r rho_r P_r
 //   3. forward DFTs of X_s and the loss operand
 //   4. the Fourier combine                     sum_s Uk[s] X^_s + i G_loss g^
 //   5. one inverse DFT and the finalisation    Q = Re - f Im
 // on the caller's stream; nothing is allocated after dgfs_plan_create. Plans of the VSS kernel
-// (alpha != 1) take the per-sphere-point path of k_vss.cu instead (vss_chunk below).
+// (alpha != 1) take the per-sphere-point path of k_shift_sum.cu instead (vss_chunk below).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -103,11 +103,10 @@ struct dgfs_plan_s {
     DevTables<double> td{};
     TcTables tc{};           // tensor-core translate tables (16-bit precisions only)
     // workspace carve (byte offsets into d_ws)
-    size_t off_P = 0, off_G = 0, off_X = 0, off_Y = 0, off_io = 0, off_node = 0;
+    size_t off_P = 0, off_X = 0, off_Y = 0, off_io = 0, off_node = 0;
     // VSS kernel: nodes per transform batch, its workspace region and the device tables
     int64_t vchunk = 0;
-    bool vss_planes = false;   // fused plane/line kernels, plane-major fields and tables
-    // VHS translate products in Fourier space (FP32/FP64, N = 8, 16, 32): nodes per transform batch
+    // VHS translates in Fourier space: sizes the region of their batches (nodes with 2 + 2 npairs complex fields)
     bool fftx = false;
     int64_t xchunk = 0;
     size_t off_Xt = 0;
@@ -115,7 +114,7 @@ struct dgfs_plan_s {
     ShiftDev<float> shf;          // shared-shift program of the translate products (inside d_vss)
     ShiftDev<double> shd;
     size_t off_V = 0, vss_bytes = 0;
-    void* d_vss = nullptr;   // A [Nrho][npairs][N^3] (T) | GL [N^3] (T) | mu [Nrho][npairs][3][N] (complex T)
+    void* d_vss = nullptr;   // VSS: half tables A, GL [N^3], shift program; VHS: mu [Nrho][npairs][3][N], shift program
     int xfields = 0;
     std::mutex host_mu;      // serialises host-side staging of per-node arrays
     int fault = 0;           // failure-test injection for the next tensor-core launch (dgfs_debug_inject)
@@ -168,11 +167,11 @@ void destroy_io(dgfs_plan_s* p) {
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-// Bytes of the VSS path per node of a transform batch: the operand spectra (2), the translate
-// spectra (2 sets x npairs), the packed products ((npairs + 1) / 2) and the output spectra (3).
+// Bytes of the VSS path per node of its workspace: half-spectrum fields (N^3/2 complex values) for one radial point
+// of a bilinear call (2 operands, 4 npairs x fields at most, 2 npairs products, a partial sum, 3 results).
 size_t vss_node_bytes(const HostPlan& h, int prec) {
     const size_t n3 = (size_t)h.N * h.N * h.N;
-    return 2 * elem_size(prec) * n3 * (2 + 2 * (size_t)h.npairs + (size_t)(h.npairs + 1) / 2 + 3);
+    return elem_size(prec) * n3 * (6 * (size_t)h.npairs + 8);
 }
 
 // Per-node workspace bytes (all operations share one layout). VSS plans use only the staging
@@ -186,14 +185,13 @@ void workspace_layout(dgfs_plan_s* p, int64_t C) {
     auto take = [&](size_t bytes) { const size_t o = off; off = align_up(off + bytes, 256); return o; };
     if (p->hp.aniso) {
         p->off_V = take((size_t)p->vchunk * vss_node_bytes(p->hp, p->prec));
-        p->off_P = p->off_G = p->off_X = p->off_Y = p->off_V;
+        p->off_P = p->off_X = p->off_Y = p->off_V;
         p->off_io = take(C * 2 * n3 * es);
         p->off_node = take(C * (sizeof(int64_t) + 2 * sizeof(double)));
         p->ws_bytes = off;
         return;
     }
-    p->off_P = take(C * Nr * n3 * es);                 // P_r (also K_r u for the VJP)
-    p->off_G = take(C * n3 * es);                      // VJP: the gain's radial sum
+    p->off_P = take(C * Nr * n3 * es);                 // P_r
     // X also holds, during the translate stage of a bilinear call of a tensor-core plan, the
     // polarisation operands (2 fields per node) and their per-node factors
     p->off_X = take(C * std::max<size_t>((size_t)p->xfields * n3 * 2 * es, 2 * n3 * es + 2 * sizeof(float)));
@@ -306,25 +304,33 @@ void fill_tables(dgfs_plan_s* p, std::vector<unsigned char>& blob, DevTables<T>&
     t.dftw = reinterpret_cast<const T*>(o_W);
 }
 
-// VSS tables in the compute type: A = w_r w_p F(k, c_r, sigma_p), the loss weight, the multipliers;
-// A and the loss weight plane-major ([kz][kx][ky]) for the fused kernels.
+// VSS tables in the compute type, the parts even in k (they act on real fields): A = w_r w_p F(k, c_r, sigma_p) as half
+// tables [r][p] of [kx][ky][kz < N/2] in the order of the folded plane kz = 0 (k_shift_sum.cu: rows ky < N/2 hold
+// (ky, 0), the others (ky - N/2, N/2)), then [2][kx] the values at ky = N/2 of its two packed columns; and the loss
+// weight [N^3], DFT index order.
 template <typename T>
-void fill_vss_tables(const HostPlan& h, bool planes, std::vector<unsigned char>& blob) {
-    const int N = h.N;
-    const size_t n3 = (size_t)N * N * N;
-    blob.assign((h.Fa.size() + h.GLa.size() + h.mu.size()) * sizeof(T), 0);
+void fill_vss_tables(const HostPlan& h, std::vector<unsigned char>& blob) {
+    const int N = h.N, NH = N / 2;
+    const size_t n3 = (size_t)N * N * N, half = n3 / 2 + 2 * (size_t)N, fields = h.Fa.size() / n3;
+    blob.assign((fields * half + n3) * sizeof(T), 0);
     T* d = reinterpret_cast<T*>(blob.data());
-    auto dst = [&](size_t i) {   // standard index (kx N + ky) N + kz -> stored index
-        if (!planes) return i;
-        const size_t kx = i / ((size_t)N * N), ky = (i / N) % N, kz = i % N;
-        return (kz * N + kx) * N + ky;
+    auto even = [&](const double* a, int kx, int ky, int kz) {
+        const size_t i = ((size_t)kx * N + ky) * N + kz;
+        const size_t m = ((size_t)((N - kx) % N) * N + (N - ky) % N) * N + (N - kz) % N;
+        return (T)(0.5 * (a[i] + a[m]));
     };
-    for (size_t f = 0; f < h.Fa.size() / n3; ++f)
-        for (size_t i = 0; i < n3; ++i) d[f * n3 + dst(i)] = (T)h.Fa[f * n3 + i];
-    d += h.Fa.size();
-    for (size_t i = 0; i < n3; ++i) d[dst(i)] = (T)h.GLa[i];
-    d += n3;
-    for (size_t i = 0; i < h.mu.size(); ++i) d[i] = (T)h.mu[i];
+    for (size_t f = 0; f < fields; ++f, d += half) {
+        const double* a = &h.Fa[f * n3];
+        for (int kx = 0; kx < N; ++kx) {
+            for (int ky = 0; ky < N; ++ky) {
+                d[((size_t)kx * N + ky) * NH] = even(a, kx, ky % NH, ky < NH ? 0 : NH);
+                for (int kz = 1; kz < NH; ++kz) d[((size_t)kx * N + ky) * NH + kz] = even(a, kx, ky, kz);
+            }
+            d[n3 / 2 + kx] = even(a, kx, NH, 0);
+            d[n3 / 2 + N + kx] = even(a, kx, NH, NH);
+        }
+    }
+    for (size_t i = 0; i < n3; ++i) d[i] = even(h.GLa.data(), (int)(i / ((size_t)N * N)), (int)((i / N) % N), (int)(i % N));
 }
 
 template <typename T>
@@ -364,6 +370,8 @@ void pack_shift(const ShiftProgram& sp, std::vector<unsigned char>& blob, ShiftD
     d.quad = reinterpret_cast<const ShiftEntry*>(put(sp.quad.data(), sp.quad.size() * sizeof(ShiftEntry)));
     d.bil = reinterpret_cast<const ShiftEntry*>(put(sp.bil.data(), sp.bil.size() * sizeof(ShiftEntry)));
     d.xrows = reinterpret_cast<const int*>(put(sp.xrows.data(), sp.xrows.size() * sizeof(int)));
+    std::vector<T> kq(sp.kq.begin(), sp.kq.end());
+    d.kq = reinterpret_cast<const T*>(put(kq.data(), kq.size() * sizeof(T)));
 }
 
 template <typename T>
@@ -372,7 +380,7 @@ void rebase_shift(ShiftDev<T>& d, const void* base) {
         using P = std::remove_reference_t<decltype(ptr)>;
         ptr = reinterpret_cast<P>(static_cast<const unsigned char*>(base) + reinterpret_cast<uintptr_t>(ptr));
     };
-    fix(d.mu); fix(d.quad); fix(d.bil); fix(d.xrows);
+    fix(d.mu); fix(d.quad); fix(d.bil); fix(d.xrows); fix(d.kq);
 }
 
 unsigned char* ws(dgfs_plan_s* p, size_t off) { return static_cast<unsigned char*>(p->d_ws) + off; }
@@ -390,9 +398,14 @@ constexpr bool keeps_rounding(Op op) {
     return std::is_same<T, float>::value && (op == Op::Dgamma || op == Op::Step);
 }
 
-// The VSS kernel (alpha != 1): gain^ = scale sum_r sum_p A_rp DFT(products of the translates by
-// +-s_rp), one transform per radial and sphere point (k_vss.cu), in batches of vchunk nodes;
-// loss and finalisation as for VHS: out = Re gain - a Re(GL * b) [- b Re(GL * a) for the JVP].
+// Parts of the radial sum of k_shift_sum (columns of `nodes` nodes alone are few CTAs), at most `most`.
+int sum_parts(int64_t nodes, int nr, int64_t most) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>({(300 + nodes - 1) / nodes, 8, nr, most}));
+}
+
+// The VSS kernel (alpha != 1): gain^ = scale sum_r sum_p A_rp DFT(products of the translates by +-s_rp), one
+// transform per radial and sphere point (k_shift_sum.cu), in batches of (node, radial point) items that fit
+// the workspace; out = gain - a (GL * b) [- b (GL * a) for the JVP].
 template <typename T>
 dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, const int64_t* offs, int64_t nodes,
                       cudaStream_t s) {
@@ -401,47 +414,52 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     NvtxRange range("dgfs VSS chunk");
     if (offs) return fail(DGFS_ERR_UNSUPPORTED, "the VSS kernel (alpha != 1) takes no node offsets");
     const DevTables<T>& t = tables<T>(p);
-    const int N = t.N, np = t.npairs, Nr = t.Nrho, nw = (np + 1) / 2;
-    const int64_t n3 = (int64_t)N * N * N;
-    // equal transform batches of at most vchunk nodes (no small ragged tail batch)
-    const int64_t nbatch = (nodes + p->vchunk - 1) / std::max<int64_t>(1, p->vchunk);
-    const int64_t C = nbatch > 0 ? (nodes + nbatch - 1) / nbatch : p->vchunk;
+    const ShiftDev<T>& d = shift_dev<T>(p);
+    const int N = t.N, np = t.npairs, Nr = t.Nrho;
+    const int64_t n3 = (int64_t)N * N * N, field = n3 / 2;
     const bool two = !quadratic(op);
-    const int sets = two ? 2 : 1, yf = op == Op::Jvp ? 3 : 2;
-    const T scale = op == Op::Jvp ? T(2) : T(1);
+    const int ops = two ? 2 : 1, nprog = two ? d.nbil : d.nquad, nf = op == Op::Jvp ? 3 : 2;
     const T* a = f;
     const T* b = two ? g : f;
-    Cplx<T>* Fh = reinterpret_cast<Cplx<T>*>(ws(p, p->off_V));
-    Cplx<T>* Gh = Fh + C * n3;
-    Cplx<T>* Z = Gh + C * n3;
-    Cplx<T>* W = Z + C * 2 * np * n3;
-    Cplx<T>* Y = W + C * nw * n3;
     const T* A = static_cast<const T*>(p->d_vss);
-    const T* GL = A + (size_t)Nr * np * n3;
-    const Cplx<T>* mu = reinterpret_cast<const Cplx<T>*>(GL + n3);
-    const Cplx<T>* dftw = reinterpret_cast<const Cplx<T>*>(t.dftw);
+    const T* GL = A + (size_t)Nr * np * (field + 2 * N);
+    const double scale = (two ? 1.0 : 2.0) * (op == Op::Jvp ? 2.0 : 1.0) / (double)n3 * shift_gain_scale(N, sizeof(T) == 8);
+    // fields per node (operands, partial sums, results) and per item (x translates, products)
+    const int64_t cap = p->vchunk * (6 * (int64_t)np + 8), item = (int64_t)ops * 2 * d.nx + nprog;
+    int64_t C = std::min<int64_t>({nodes, cap / (ops + 1 + nf + item), 65535});
+    const int64_t nbatch = (nodes + C - 1) / C;
+    C = (nodes + nbatch - 1) / nbatch;   // equal batches
+    int parts = sum_parts(C, Nr, (cap / C - ops - nf - item));
+    const int R = (int)std::max<int64_t>(1, std::min<int64_t>(Nr, (cap / C - ops - parts - nf) / item));
+    parts = std::min(parts, R);
+    Cplx<T>* Gf = reinterpret_cast<Cplx<T>*>(ws(p, p->off_V));
+    Cplx<T>* Gg = two ? Gf + C * field : nullptr;
+    Cplx<T>* F = Gf + ops * C * field;             // [nf][C] results
+    Cplx<T>* part = F + nf * C * field;            // [C][parts]
+    Cplx<T>* Hf = part + C * parts * field;        // [C][R][2 nx]
+    Cplx<T>* Hg = two ? Hf + C * R * 2 * d.nx * field : nullptr;
+    Cplx<T>* W = Hf + ops * C * R * 2 * d.nx * field;   // [C][R][nprog]
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
         const int64_t nn = std::min<int64_t>(C, nodes - n0);
-        cudaError_t e = launch_vss_load_t<T>(a + n0 * n3, nullptr, N, nn, Fh, s);
-        if (!e) e = launch_dft3<T>(t, Fh, nn, true, s);
-        if (!e && two) e = launch_vss_load_t<T>(b + n0 * n3, nullptr, N, nn, Gh, s);
-        if (!e && two) e = launch_dft3<T>(t, Gh, nn, true, s);
-        if (!e) e = launch_vss_loss_init<T>(Fh, two ? Gh : Fh, GL, N, nn, Y, yf, s);
-        if (e) return cuda_fail(e, "VSS operand transforms");
-        for (int r = 0; r < Nr && !e; ++r) {
-            e = launch_vss_inverse_planes<T>(Fh, two ? Gh : nullptr, mu + (size_t)r * np * 3 * N, dftw, N, np, sets, 1,
-                                             nn, Z, s);
-            if (!e) e = launch_vss_lines<T>(Z, dftw, N, np, sets, nn, W, s);
-            if (!e) e = launch_vss_forward_planes<T>(dftw, N, nw, nn, W, s);
-            if (!e) e = launch_vss_accumulate<T>(W, A + (size_t)r * np * n3, N, np, nn, scale, Y, yf, s);
+        cudaError_t e = launch_shift_forward<T>(a + n0 * n3, nullptr, nullptr, N, nn, Gf, s);
+        if (!e && two) e = launch_shift_forward<T>(b + n0 * n3, nullptr, nullptr, N, nn, Gg, s);
+        for (int r0 = 0; r0 < Nr && !e; r0 += R) {
+            const int nr = std::min(R, Nr - r0);
+            e = launch_shift_x<T>(d, Gf, N, r0, nr, nn, Hf, s);
+            if (!e && two) e = launch_shift_x<T>(d, Gg, N, r0, nr, nn, Hg, s);
+            if (!e) e = launch_shift_vss<T>(d, Gf, Hf, Gg, Hg, N, r0, nr, nn, W, s);
+            if (!e) e = launch_shift_sum<T>(d, W, nprog, A, two, np, N, r0, nr, parts, r0 > 0, nn, part, s);
+            if (p->prof) p->prof_launches += (d.nx ? ops : 0) + 3;
         }
         if (e) return cuda_fail(e, "VSS gain");
-        e = launch_dft3<T>(t, Y, nn * yf, false, s);
-        if (!e) e = launch_vss_finalize_t<T>(Y, yf, a + n0 * n3, op == Op::Jvp ? b + n0 * n3 : nullptr, N, nn,
-                                             out + n0 * n3, p->d_flags, s);
+        e = launch_shift_reduce<T>(part, parts, (T)scale, N, nn, F, s);
+        if (!e) e = launch_shift_filter<T>(two ? Gg : Gf, GL, 0, N, 0, 1, nn, F + C * field, s);
+        if (!e && op == Op::Jvp) e = launch_shift_filter<T>(Gf, GL, 0, N, 0, 1, nn, F + 2 * C * field, s);
+        if (!e) e = launch_shift_out<T>(F, nf, C * field, true, a + n0 * n3, op == Op::Jvp ? b + n0 * n3 : nullptr, N, nn,
+                                        out + n0 * n3, p->d_flags, s);
         if (e) return cuda_fail(e, "VSS loss and finalisation");
         if (p->prof) {
-            p->prof_launches += (two ? 8 : 4) + 1 + (int64_t)Nr * 4 + 4;
+            p->prof_launches += ops + 1 + nf;
             p->prof_nodes += nn;
         }
     }
@@ -476,8 +494,8 @@ cudaError_t shift_gain_products(dgfs_plan_s* p, const T* f, const T* g, const in
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
         const int64_t nn = std::min<int64_t>(C, nodes - n0);
         const int64_t fo = offs ? 0 : n0 * n3;
-        cudaError_t e = launch_shift_forward<T>(f + fo, offs ? offs + n0 : nullptr, N, nn, Gf, s);
-        if (!e && g) e = launch_shift_forward<T>(g + fo, offs ? offs + n0 : nullptr, N, nn, Gg, s);
+        cudaError_t e = launch_shift_forward<T>(f + fo, nullptr, offs ? offs + n0 : nullptr, N, nn, Gf, s);
+        if (!e && g) e = launch_shift_forward<T>(g + fo, nullptr, offs ? offs + n0 : nullptr, N, nn, Gg, s);
         for (int r0 = 0; r0 < Nr && !e; r0 += R) {
             const int nr = std::min(R, Nr - r0);
             e = launch_shift_x<T>(d, Gf, N, r0, nr, nn, Hf, s);
@@ -492,7 +510,7 @@ cudaError_t shift_gain_products(dgfs_plan_s* p, const T* f, const T* g, const in
     return cudaSuccess;
 }
 
-// P[node][r] of Q(f, f) with a transform of its own for every sphere pair (k_vss.cu; keeps_rounding above), in
+// P[node][r] of Q(f, f) with a transform of its own for every sphere pair (k_pair.cu; keeps_rounding above), in
 // batches of (node, radial point) items whose spectra fit the xchunk region: every radial point of as many
 // nodes as fit (one launch of each kernel for a small batch), or a part of the radial points.
 cudaError_t pair_gain_products(dgfs_plan_s* p, const float* f, int64_t nodes, float* P, cudaStream_t s) {
@@ -507,13 +525,13 @@ cudaError_t pair_gain_products(dgfs_plan_s* p, const float* f, int64_t nodes, fl
     Cplx<float>* Z = Fh + C * n3;
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
         const int64_t nn = std::min<int64_t>(C, nodes - n0);
-        cudaError_t e = launch_vss_load_t<float>(f + n0 * n3, nullptr, N, nn, Fh, s);
+        cudaError_t e = launch_pair_load(f + n0 * n3, N, nn, Fh, s);
         if (!e) e = launch_dft3<float>(t, Fh, nn, true, s);
         for (int r = 0; r < Nr && !e; r += R) {
             const int nr = std::min(R, Nr - r);
-            e = launch_vss_inverse_planes<float>(Fh, nullptr, mu + (size_t)r * np * 3 * N, dftw, N, np, 1, nr, nn, Z, s);
-            if (!e) e = launch_vss_lines_sum<float>(Z, dftw, t.wsig, N, np, nr, nn, (int64_t)Nr * n3,
-                                                    P + n0 * Nr * n3 + (int64_t)r * n3, s);
+            e = launch_pair_planes(Fh, mu + (size_t)r * np * 3 * N, dftw, N, np, nr, nn, Z, s);
+            if (!e) e = launch_pair_sum(Z, dftw, t.wsig, N, np, nr, nn, (int64_t)Nr * n3,
+                                        P + n0 * Nr * n3 + (int64_t)r * n3, s);
             if (p->prof) p->prof_launches += 2;
         }
         if (e) return e;
@@ -522,36 +540,48 @@ cudaError_t pair_gain_products(dgfs_plan_s* p, const float* f, int64_t nodes, fl
     return cudaSuccess;
 }
 
-// Adjoint gain sum_r G_r (G_r = sum_p 2 w_p [T_-s(U_r T_-s f) + T_s(U_r T_s f)], U[node][r] = K_r u)
-// with the translates and back-translates in Fourier space (k_vss.cu), in batches of xchunk nodes:
-// Gsum [nodes][N^3], standard layout.
+// The adjoint: out = sum_r G_r - u (K_L f) - K_L (u f), G_r = sum_p 2 w_p [T_-s(U_r T_-s f) + T_s(U_r T_s f)] with
+// U_r = K_r u, on the shared translates (k_shift_sum.cu). The operands' and results' spectra live in the Y
+// region, partial sums in X, the (node, radial point) items in the xchunk region.
 template <typename T>
-cudaError_t fft_vjp_products(dgfs_plan_s* p, const T* f, const T* U, int64_t nodes, T* Gsum, cudaStream_t s) {
+cudaError_t shift_vjp(dgfs_plan_s* p, const T* f, const T* u, T* out, int64_t nodes, cudaStream_t s) {
     const DevTables<T>& t = tables<T>(p);
-    const int N = t.N, np = t.npairs, Nr = t.Nrho;
-    const int64_t n3 = (int64_t)N * N * N, C = p->xchunk;
-    Cplx<T>* Fh = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Xt));
-    Cplx<T>* Gh = Fh + C * n3;
-    Cplx<T>* Z = Gh + C * n3;
-    Cplx<T>* W = Z + C * np * n3;
-    const Cplx<T>* mu = static_cast<const Cplx<T>*>(p->d_mu);
-    const Cplx<T>* dftw = reinterpret_cast<const Cplx<T>*>(t.dftw);
+    const ShiftDev<T>& d = shift_dev<T>(p);
+    const int N = t.N, Nr = t.Nrho, nq2 = 3 * (N / 2) * (N / 2) + 1;
+    const int64_t n3 = (int64_t)N * N * N, field = n3 / 2;
+    const int64_t cap = p->xchunk * (4 + 4 * (int64_t)t.npairs), item = 4 * (int64_t)d.nx + 3;
+    int64_t C = std::min<int64_t>({nodes, cap / item, 65535});
+    const int64_t nbatch = (nodes + C - 1) / C;
+    C = (nodes + nbatch - 1) / nbatch;   // equal batches
+    const int R = (int)std::min<int64_t>(Nr, cap / (C * item));
+    const int parts = sum_parts(C, R, 2 * (int64_t)p->xfields);
+    const double scale = shift_gain_scale(N, sizeof(T) == 8) / (double)n3;
+    Cplx<T>* G = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Y));   // spectra of f, u and u f
+    Cplx<T>* F = G + 3 * C * field;                             // gain, K_L f, K_L(u f)
+    Cplx<T>* part = reinterpret_cast<Cplx<T>*>(ws(p, p->off_X));
+    Cplx<T>* H = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Xt));
+    Cplx<T>* Ur = H + C * R * 2 * d.nx * field;
+    Cplx<T>* V = Ur + C * R * field;
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
         const int64_t nn = std::min<int64_t>(C, nodes - n0);
-        cudaError_t e = launch_vss_load_t<T>(f + n0 * n3, nullptr, N, nn, Fh, s);
-        if (!e) e = launch_dft3<T>(t, Fh, nn, true, s);
-        if (!e) e = cudaMemsetAsync(Gh, 0, (size_t)nn * n3 * sizeof(Cplx<T>), s);
-        for (int r = 0; r < Nr && !e; ++r) {
-            const Cplx<T>* mu_r = mu + (size_t)r * np * 3 * N;
-            e = launch_vss_inverse_planes<T>(Fh, nullptr, mu_r, dftw, N, np, 1, 1, nn, Z, s);
-            if (!e) e = launch_vjp_lines<T>(Z, U + n0 * Nr * n3 + (int64_t)r * n3, (int64_t)Nr * n3, dftw, N, np, nn, W, s);
-            if (!e) e = launch_vss_forward_planes<T>(dftw, N, np, nn, W, s);
-            if (!e) e = launch_vjp_accumulate<T>(W, mu_r, t.wsig, N, np, nn, Gh, s);
+        const T *fn = f + n0 * n3, *un = u + n0 * n3;
+        cudaError_t e = launch_shift_forward<T>(fn, nullptr, nullptr, N, nn, G, s);
+        if (!e) e = launch_shift_forward<T>(un, nullptr, nullptr, N, nn, G + C * field, s);
+        if (!e) e = launch_shift_forward<T>(un, fn, nullptr, N, nn, G + 2 * C * field, s);
+        for (int r0 = 0; r0 < Nr && !e; r0 += R) {
+            const int nr = std::min(R, Nr - r0);
+            e = launch_shift_x<T>(d, G, N, r0, nr, nn, H, s);
+            if (!e) e = launch_shift_filter<T>(G + C * field, d.kq, nq2, N, r0, nr, nn, Ur, s);
+            if (!e) e = launch_shift_adj<T>(d, G, H, Ur, t.wsig, N, r0, nr, nn, V, s);
+            if (!e) e = launch_shift_sum<T>(d, V, 2 * d.nx + 2, nullptr, false, t.npairs, N, r0, nr, parts, r0 > 0, nn, part, s);
+            if (p->prof) p->prof_launches += (d.nx ? 1 : 0) + 3;
         }
-        if (!e) e = launch_dft3<T>(t, Gh, nn, false, s);
-        if (!e) e = launch_vjp_real_t<T>(Gh, N, nn, Gsum + n0 * n3, s);
+        if (!e) e = launch_shift_reduce<T>(part, parts, (T)scale, N, nn, F, s);
+        if (!e) e = launch_shift_filter<T>(G, t.GL0, 0, N, 0, 1, nn, F + C * field, s);
+        if (!e) e = launch_shift_filter<T>(G + 2 * C * field, t.GL0, 0, N, 0, 1, nn, F + 2 * C * field, s);
+        if (!e) e = launch_shift_out<T>(F, 3, C * field, false, un, nullptr, N, nn, out + n0 * n3, p->d_flags, s);
         if (e) return e;
-        if (p->prof) p->prof_launches += 4 + 4 * (int64_t)Nr + 4;
+        if (p->prof) p->prof_launches += 7;
     }
     return cudaSuccess;
 }
@@ -570,29 +600,11 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     const int rank = t.rank;
     cudaError_t e;
     if (op == Op::Vjp) {
-        // g holds u. 1) K_r u for every r:  DFT(u) -> Uk[s] u^ -> IDFT -> sum_s Vr w_r rho_r
-        e = launch_load_field<T>(t.N, g, nullptr, offs, nodes, X, xf, rank, 0, s);
-        if (!e) e = launch_dft3<T>(t, X + (size_t)0, nodes * xf, true, s);
-        if (!e) e = launch_multiply_uk<T>(t, X, xf, rank, nodes, s);
-        if (!e) e = launch_dft3<T>(t, X, nodes * xf, false, s);
-        if (!e) e = launch_expand_radial<T>(t, X, xf, np, nodes, P, s);
-        if (e) return cuda_fail(e, "vjp: radial multipliers");
-        // 2) adjoint translate-products, summed over r, with the translates in Fourier space
-        T* G = reinterpret_cast<T*>(ws(p, p->off_G));
         if (offs) return fail(DGFS_ERR_UNSUPPORTED, "vjp with node offsets");
         if (!p->fftx) return fail(DGFS_ERR_UNSUPPORTED, "vjp: no Fourier-space translates for this plan");
         if (p->prof) p->prof_nodes += nodes;
-        e = fft_vjp_products<T>(p, f, P, nodes, G, s);
-        if (e) return cuda_fail(e, "vjp: translate-product kernels");
-        // 3) loss: K_L f + i K_L (u f)
-        e = launch_load_field<T>(t.N, f, nullptr, offs, nodes, X, xf, 0, 0, s);
-        if (!e) e = launch_load_field<T>(t.N, f, g, offs, nodes, X, xf, 1, 0, s);
-        if (!e) e = launch_dft3<T>(t, X, nodes * xf, true, s);
-        if (!e) e = launch_loss_pair<T>(t, X, xf, np, nodes, 0, 1, Y, 2, s);
-        if (!e) e = launch_dft3<T>(t, Y, nodes * 2, false, s);
-        // the Fourier-space adjoint leaves the radial sum in G (one field per node)
-        if (!e) e = launch_finalize<T>(t.N, 1, Y, 2, g, nullptr, G, offs, nodes, 1, out, p->d_flags, s);
-        if (e) return cuda_fail(e, "vjp: loss and finalisation");
+        e = shift_vjp<T>(p, f, g, out, nodes, s);   // g holds u
+        if (e) return cuda_fail(e, "vjp");
         return DGFS_OK;
     }
     // gain products: Q(f,f) and dQ/dgamma use (f, f); Q(f,g) uses (f, g); JVP uses (f, v)
@@ -666,8 +678,7 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     if (!e) e = launch_dft3<T>(t, Y, nodes * yf, false, s);
     if (e) return cuda_fail(e, "Fourier combine / inverse DFT");
     // Q = gain - f (K_L g)   (JVP: 2 gain(f,v) - f K_L v - v K_L f)
-    e = launch_finalize<T>(t.N, t.Nrho, Y, yf, f, op == Op::Jvp ? g : nullptr, nullptr, offs, nodes, 0,
-                           out, p->d_flags, s);
+    e = launch_finalize<T>(t.N, Y, yf, f, op == Op::Jvp ? g : nullptr, offs, nodes, out, p->d_flags, s);
     if (e) return cuda_fail(e, "finalisation");
     return DGFS_OK;
 }
@@ -743,7 +754,7 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
     dgfs_status st = build_host_plan(*desc, p->hp, err);
     if (st != DGFS_OK) return fail(st, err);
     p->prec = desc->precision;
-    if (p->hp.aniso && !vss_fused_supported(p->hp.N, p->prec == DGFS_PREC_FP64))
+    if (p->hp.aniso && p->hp.N == 32 && p->prec == DGFS_PREC_FP64)
         return fail(DGFS_ERR_UNSUPPORTED, "the VSS kernel supports N <= 24 in FP64");
     if (is_tc(p->prec) && !tc_supported(p->hp.N, p->prec))
         return fail(DGFS_ERR_UNSUPPORTED, "tensor-core precisions support N = 16 and 32 (F16S and BF16S also N = 24)");
@@ -767,16 +778,13 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
         if (desc->max_batch > 0) C = std::min<int64_t>(desc->max_batch, (int64_t)1 << 20);   // the caller's choice
         p->chunk = C;
         if (p->hp.aniso) {
-            // transform batches of about 1.5 GB of translate spectra and products: enough CTAs per launch
-            // (64 MB, which stays in L2, measured 3.2k node-evals/s at N = 32; 512 MB 6.0k; 1.5 GB 6.7k)
-            const size_t n3 = (size_t)p->hp.N * p->hp.N * p->hp.N;
-            const size_t zw = 2 * elem_size(p->prec) * n3 * (2 * (size_t)p->hp.npairs + (p->hp.npairs + 1) / 2);
+            // about 1.5 GB for the batches of translate and product spectra
+            const size_t zw = vss_node_bytes(p->hp, p->prec);
             p->vchunk = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(C, (int64_t)(((size_t)1536 << 20) / zw)), 65535));
         }
     }
-    // tensor-core plans keep their kernel for Q(f, f) and dQ/dgamma; their bilinear calls (Q(f, g),
-    // the JVP) and the VJP take the Fourier-space translates in FP32 like the FP32 plans
-    p->fftx = !p->hp.aniso && fft_translate_supported(p->hp.N);
+    // Fourier-space translates of every VHS plan (tensor-core plans: the VJP)
+    p->fftx = !p->hp.aniso;
     if (p->fftx) {
         // transform batches of about 1.5 GB of operand and translate spectra
         const size_t n3 = (size_t)p->hp.N * p->hp.N * p->hp.N;
@@ -793,9 +801,15 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
     if (is_tc(p->prec)) tc_bytes = build_tc_tables(p->hp, p->prec, tcblob, p->tc);
     if (p->hp.aniso) {
         std::vector<unsigned char> vblob;
-        p->vss_planes = vss_fused_supported(p->hp.N, p->prec == DGFS_PREC_FP64);
-        if (p->prec == DGFS_PREC_FP64) fill_vss_tables<double>(p->hp, p->vss_planes, vblob);
-        else fill_vss_tables<float>(p->hp, p->vss_planes, vblob);
+        ShiftProgram sp;
+        build_shift_program(p->hp, sp);
+        if (p->prec == DGFS_PREC_FP64) {
+            fill_vss_tables<double>(p->hp, vblob);
+            pack_shift(sp, vblob, p->shd);
+        } else {
+            fill_vss_tables<float>(p->hp, vblob);
+            pack_shift(sp, vblob, p->shf);
+        }
         cudaError_t ev = cudaMalloc(&p->d_vss, vblob.size());
         if (ev != cudaSuccess) return fail(DGFS_ERR_OOM, std::string("VSS tables: ") + cudaGetErrorString(ev));
         ev = cudaMemcpy(p->d_vss, vblob.data(), vblob.size(), cudaMemcpyHostToDevice);
@@ -804,17 +818,16 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
             return cuda_fail(ev, "VSS table upload");
         }
         p->vss_bytes = vblob.size();
-        p->d_mu = static_cast<unsigned char*>(p->d_vss) + (p->hp.Fa.size() + p->hp.GLa.size()) * elem_size(p->prec);
+        if (p->prec == DGFS_PREC_FP64) rebase_shift(p->shd, p->d_vss);
+        else rebase_shift(p->shf, p->d_vss);
         // the FP64 host copies are no longer needed
         std::vector<double>().swap(p->hp.Fa);
         std::vector<double>().swap(p->hp.mu);
     } else if (p->fftx) {
         const size_t es = elem_size(p->prec);
-        std::vector<unsigned char> mblob(p->hp.mu.size() * es);
-        for (size_t i = 0; i < p->hp.mu.size(); ++i) {
-            if (es == 8) reinterpret_cast<double*>(mblob.data())[i] = p->hp.mu[i];
-            else reinterpret_cast<float*>(mblob.data())[i] = (float)p->hp.mu[i];
-        }
+        // the per-axis multipliers of every pair, for the transform-per-pair products (FP32 plans, keeps_rounding)
+        std::vector<unsigned char> mblob(p->prec == DGFS_PREC_FP32 ? p->hp.mu.size() * es : 0);
+        for (size_t i = 0; i < mblob.size() / es; ++i) reinterpret_cast<float*>(mblob.data())[i] = (float)p->hp.mu[i];
         ShiftProgram sp;
         build_shift_program(p->hp, sp);
         if (es == 8) pack_shift(sp, mblob, p->shd);
@@ -2193,7 +2206,7 @@ dgfs_status noalloc_run(dgfs_plan_s* p, const T* f, T* Q, int64_t B, unsigned ch
     if (!e) e = launch_dft3<T>(t, X, B * xs, true, s);
     if (!e) e = launch_combine<T>(t, X, xs, np, B, T(1), t.rank, -1, Y, 2, s);
     if (!e) e = launch_dft3<T>(t, Y, B * 2, false, s);
-    if (!e) e = launch_finalize<T>(t.N, t.Nrho, Y, 2, f, nullptr, nullptr, nullptr, B, 0, Q, p->d_flags, s);
+    if (!e) e = launch_finalize<T>(t.N, Y, 2, f, nullptr, nullptr, B, Q, p->d_flags, s);
     if (e) return cuda_fail(e, "dgfs_collide_noalloc");
     return DGFS_OK;
 }

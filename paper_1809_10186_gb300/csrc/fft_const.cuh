@@ -14,77 +14,21 @@
 namespace dgfs {
 namespace cfft {
 
+using fdev::add;
 using fdev::bitrev;
+using fdev::cos_of;
 using fdev::line_slot;
+using fdev::quarter24;
+using fdev::quarter32;
+using fdev::pack;
+using fdev::sin_of;
+using fdev::sub;
+using fdev::unpack;
 
-// cos(2 pi m / 32), m = 0 .. 8, and cos(2 pi m / 24), m = 0 .. 6; other angles by symmetry
-__host__ __device__ constexpr double quarter32(int m) {
-    return m == 0 ? 1.0
-         : m == 1 ? 0.980785280403230449126182236134239037
-         : m == 2 ? 0.923879532511286756128183189396788287
-         : m == 3 ? 0.831469612302545237078788377617905757
-         : m == 4 ? 0.707106781186547524400844362104849039
-         : m == 5 ? 0.555570233019602224742830813948532874
-         : m == 6 ? 0.382683432365089771728459984030398867
-         : m == 7 ? 0.195090322016128267848284868477022241
-         : 0.0;
-}
-__host__ __device__ constexpr double quarter24(int m) {
-    return m == 0 ? 1.0
-         : m == 1 ? 0.965925826289068286749743199728897368
-         : m == 2 ? 0.866025403784438646763723170752936183
-         : m == 3 ? 0.707106781186547524400844362104849039
-         : m == 4 ? 0.5
-         : m == 5 ? 0.258819045102520762348898837624048328
-         : 0.0;
-}
-// cos(2 pi m / D) for D dividing 32 or 24
-template <int D>
-__host__ __device__ constexpr double cos_of(int m) {
-    constexpr int B = 32 % D == 0 ? 32 : 24, Q = B / 4;
-    m = ((m * (B / D)) % B + B) % B;
-    const int h = m <= 2 * Q ? m : B - m;                      // cos is even
-    const int q = h <= Q ? h : 2 * Q - h;
-    const double c = B == 32 ? quarter32(q) : quarter24(q);
-    return h <= Q ? c : -c;
-}
-template <int D>
-__host__ __device__ constexpr double sin_of(int m) {
-    constexpr int B = 32 % D == 0 ? 32 : 24;
-    return cos_of<B>(m * (B / D) - B / 4);
-}
-
-// u + v, u - v and 2 u - s of complex values. In FP32 both parts go through one packed instruction
-// (f32x2, each half rounded as the scalar operation): the lines are bound by instruction issue.
-template <typename T>
-__device__ __forceinline__ Cplx<T> add(Cplx<T> u, Cplx<T> v) { return Cplx<T>{u.x + v.x, u.y + v.y}; }
-template <typename T>
-__device__ __forceinline__ Cplx<T> sub(Cplx<T> u, Cplx<T> v) { return Cplx<T>{u.x - v.x, u.y - v.y}; }
+// 2 u - s, packed in FP32
 template <typename T>
 __device__ __forceinline__ Cplx<T> twice_minus(Cplx<T> u, Cplx<T> s) {
     return Cplx<T>{fma(T(2), u.x, -s.x), fma(T(2), u.y, -s.y)};
-}
-__device__ __forceinline__ unsigned long long pack(Cplx<float> a) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
-    return r;
-}
-__device__ __forceinline__ Cplx<float> unpack(unsigned long long r) {
-    Cplx<float> a;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
-    return a;
-}
-template <>
-__device__ __forceinline__ Cplx<float> add<float>(Cplx<float> u, Cplx<float> v) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack(u)), "l"(pack(v)));
-    return unpack(r);
-}
-template <>
-__device__ __forceinline__ Cplx<float> sub<float>(Cplx<float> u, Cplx<float> v) {
-    unsigned long long r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack(u)), "l"(pack(v)));
-    return unpack(r);
 }
 template <>
 __device__ __forceinline__ Cplx<float> twice_minus<float>(Cplx<float> u, Cplx<float> s) {

@@ -32,12 +32,81 @@ __device__ __forceinline__ T loss_multiplier(const T* __restrict__ GL0, const T*
     return (T)g;
 }
 
+// cos(2 pi m / 32), m = 0 .. 8, and cos(2 pi m / 24), m = 0 .. 6; other angles by symmetry
+__host__ __device__ constexpr double quarter32(int m) {
+    return m == 0 ? 1.0
+         : m == 1 ? 0.980785280403230449126182236134239037
+         : m == 2 ? 0.923879532511286756128183189396788287
+         : m == 3 ? 0.831469612302545237078788377617905757
+         : m == 4 ? 0.707106781186547524400844362104849039
+         : m == 5 ? 0.555570233019602224742830813948532874
+         : m == 6 ? 0.382683432365089771728459984030398867
+         : m == 7 ? 0.195090322016128267848284868477022241
+         : 0.0;
+}
+__host__ __device__ constexpr double quarter24(int m) {
+    return m == 0 ? 1.0
+         : m == 1 ? 0.965925826289068286749743199728897368
+         : m == 2 ? 0.866025403784438646763723170752936183
+         : m == 3 ? 0.707106781186547524400844362104849039
+         : m == 4 ? 0.5
+         : m == 5 ? 0.258819045102520762348898837624048328
+         : 0.0;
+}
+// cos(2 pi m / D) for D dividing 32 or 24
+template <int D>
+__host__ __device__ constexpr double cos_of(int m) {
+    constexpr int B = 32 % D == 0 ? 32 : 24, Q = B / 4;
+    m = ((m * (B / D)) % B + B) % B;
+    const int h = m <= 2 * Q ? m : B - m;                      // cos is even
+    const int q = h <= Q ? h : 2 * Q - h;
+    const double c = B == 32 ? quarter32(q) : quarter24(q);
+    return h <= Q ? c : -c;
+}
+template <int D>
+__host__ __device__ constexpr double sin_of(int m) {
+    constexpr int B = 32 % D == 0 ? 32 : 24;
+    return cos_of<B>(m * (B / D) - B / 4);
+}
+
+// u + v and u - v of complex values. In FP32 both parts go through one packed instruction
+// (f32x2, each half rounded as the scalar operation): the lines are bound by instruction issue.
+template <typename T>
+__device__ __forceinline__ Cplx<T> add(Cplx<T> u, Cplx<T> v) { return Cplx<T>{u.x + v.x, u.y + v.y}; }
+template <typename T>
+__device__ __forceinline__ Cplx<T> sub(Cplx<T> u, Cplx<T> v) { return Cplx<T>{u.x - v.x, u.y - v.y}; }
+__device__ __forceinline__ unsigned long long pack(Cplx<float> a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ Cplx<float> unpack(unsigned long long r) {
+    Cplx<float> a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+template <>
+__device__ __forceinline__ Cplx<float> add<float>(Cplx<float> u, Cplx<float> v) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack(u)), "l"(pack(v)));
+    return unpack(r);
+}
+template <>
+__device__ __forceinline__ Cplx<float> sub<float>(Cplx<float> u, Cplx<float> v) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack(u)), "l"(pack(v)));
+    return unpack(r);
+}
 // ---- radix-2 FFT passes (power-of-two N) -------------------------------------------------
 //
 // One thread transforms one line of N complex values held in registers: decimation in time
-// on bit-reversed input, N/2 log2 N butterflies, twiddles e^{-+2 pi i j / N} taken from the
-// plan's DFT table (row 1) through shared memory. Same result as the dense passes, in
+// on bit-reversed input, N/2 log2 N butterflies, twiddles e^{-+2 pi i j / N} as immediate operands (for
+// N = 3 * 2^m from row 1 of the plan's DFT table through shared memory). Same result as the dense passes, in
 // 5 N log2 N instead of 8 N^2 flops per line.
+
+// a product that is not contracted into an FMA
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 template <int N>
 __device__ __forceinline__ constexpr int bitrev(int i) {
@@ -47,7 +116,8 @@ __device__ __forceinline__ constexpr int bitrev(int i) {
     return r;
 }
 
-// One radix-2 stage of butterfly span LEN, then the next stage. LEN is a template parameter so
+// One radix-2 stage of butterfly span LEN, then the next stage. The roundings (which product of a twiddle
+// multiplication is rounded by itself) are written out: dgfs_ssprk and dgfs_collide_dgamma of FP32 plans keep them. LEN is a template parameter so
 // that every loop has a compile-time trip count and the line stays in registers; the twiddles
 // 1 and -+i (known once the loops are unrolled) take no multiplication.
 template <typename T, int N, int LEN>
@@ -64,12 +134,11 @@ __device__ __forceinline__ void fft_stage(Cplx<T> (&a)[N], const Cplx<T>* __rest
             } else if (4 * j * step == N) {    // twiddle -i (forward) or +i (inverse)
                 v = forward ? Cplx<T>{v0.y, -v0.x} : Cplx<T>{-v0.y, v0.x};
             } else {
-                const Cplx<T> w = tw[j * step];
-                const T wi = forward ? w.y : -w.y;
-                v = Cplx<T>{v0.x * w.x - v0.y * wi, v0.x * wi + v0.y * w.x};
+                const T wr = (T)cos_of<N>(j * step), ws = (T)(-sin_of<N>(j * step)), wi = forward ? ws : -ws;
+                v = Cplx<T>{fma(v0.x, wr, -mul_rn(v0.y, wi)), fma(v0.y, wr, mul_rn(v0.x, wi))};
             }
-            a[i + j] = Cplx<T>{u.x + v.x, u.y + v.y};
-            a[i + j + half] = Cplx<T>{u.x - v.x, u.y - v.y};
+            a[i + j] = add(u, v);
+            a[i + j + half] = sub(u, v);
         }
     if constexpr (LEN < N) fft_stage<T, N, 2 * LEN>(a, tw, forward);
 }

@@ -225,74 +225,8 @@ __global__ void k_combine(const Cplx<T>* __restrict__ X, int xslots, const T* __
 }
 
 template <typename T>
-__global__ void k_loss_pair(const Cplx<T>* __restrict__ X, int xfields, const T* __restrict__ Lr,
-                            const T* __restrict__ GL0, const T* __restrict__ GLd,
-                            const double* __restrict__ cr, NodeParams np, int Nrho, int64_t n3,
-                            int s0, int s1, Cplx<T>* __restrict__ Y, int yfields) {
-    __shared__ double rho[64];
-    const int64_t node = blockIdx.y;
-    const bool per_node = np.gamma || np.b;
-    const double gam = np.gamma ? np.gamma[node] : np.gamma0;
-    const double bb = np.b ? np.b[node] : np.b0;
-    if (per_node)
-        for (int r = threadIdx.x; r < Nrho; r += blockDim.x) rho[r] = radial_rho<double>(bb, gam, cr[r], np.dlog);
-    __syncthreads();
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n3) return;
-    const T GL = loss_multiplier<T>(GL0, GLd, Lr, rho, per_node, np.dlog, Nrho, n3, k);
-    const Cplx<T>* Xn = X + node * (int64_t)xfields * n3;
-    const Cplx<T> a = Xn[s0 * n3 + k], b = Xn[s1 * n3 + k];
-    Cplx<T>* Yn = Y + node * (int64_t)yfields * n3;
-    Yn[k] = Cplx<T>{GL * a.x, GL * a.y};
-    Yn[n3 + k] = Cplx<T>{GL * b.x, GL * b.y};
-}
-
-template <typename T>
-__global__ void k_multiply_uk(Cplx<T>* __restrict__ X, int xfields, const T* __restrict__ Uk,
-                              int rank, int64_t n3, int src) {
-    const int64_t node = blockIdx.y;
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n3) return;
-    Cplx<T>* Xn = X + node * (int64_t)xfields * n3;
-    const Cplx<T> v = Xn[src * n3 + k];
-    for (int s = 0; s < rank; ++s) {
-        const T u = Uk[s * n3 + k];
-        Xn[s * n3 + k] = Cplx<T>{u * v.x, u * v.y};
-    }
-}
-
-// U[node][r][j] = w_r rho_r sum_s Vr[s][r] Re X[node][s][j]
-template <typename T>
-__global__ void k_expand_radial(const Cplx<T>* __restrict__ X, int xfields, const T* __restrict__ Vr,
-                                const double* __restrict__ cr, const double* __restrict__ wr,
-                                NodeParams np, int Nrho, int rank, int64_t n3, T* __restrict__ U) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    T* C = reinterpret_cast<T*>(sm_raw);        // [rank][Nrho]
-    T* Xt = C + rank * Nrho;                     // [rank][blockDim]
-    T* wrho = Xt + rank * blockDim.x;            // [Nrho]: w_r rho_r of this node
-    const int64_t node = blockIdx.y;
-    const double gam = np.gamma ? np.gamma[node] : np.gamma0;
-    const double bb = np.b ? np.b[node] : np.b0;
-    for (int r = threadIdx.x; r < Nrho; r += blockDim.x) wrho[r] = (T)wr[r] * radial_rho<T>(bb, gam, cr[r], np.dlog);
-    __syncthreads();
-    for (int e = threadIdx.x; e < rank * Nrho; e += blockDim.x) C[e] = Vr[e] * wrho[e % Nrho];
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const Cplx<T>* Xn = X + node * (int64_t)xfields * n3;
-    for (int s = 0; s < rank; ++s) Xt[s * blockDim.x + threadIdx.x] = j < n3 ? Xn[s * n3 + j].x : T(0);
-    __syncthreads();
-    if (j >= n3) return;
-    T* Un = U + node * (int64_t)Nrho * n3;
-    for (int r = 0; r < Nrho; ++r) {
-        T acc = 0;
-        for (int s = 0; s < rank; ++s) acc = fma(C[s * Nrho + r], Xt[s * blockDim.x + threadIdx.x], acc);
-        Un[r * n3 + j] = acc;
-    }
-}
-
-template <typename T>
-__global__ void k_finalize(int Nrho, int64_t n3, const Cplx<T>* __restrict__ Y, int yfields,
-                           const T* __restrict__ a, const T* __restrict__ c, const T* __restrict__ G,
-                           const int64_t* __restrict__ offs, int mode, T* __restrict__ out,
+__global__ void k_finalize(int64_t n3, const Cplx<T>* __restrict__ Y, int yfields, const T* __restrict__ a,
+                           const T* __restrict__ c, const int64_t* __restrict__ offs, T* __restrict__ out,
                            int* __restrict__ flags) {
     const int64_t node = blockIdx.y;
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -300,16 +234,8 @@ __global__ void k_finalize(int Nrho, int64_t n3, const Cplx<T>* __restrict__ Y, 
     const int64_t base = offs ? offs[node] : node * n3;
     const Cplx<T>* Yn = Y + node * (int64_t)yfields * n3;
     const Cplx<T> y0 = Yn[j], y1 = Yn[n3 + j];
-    T v;
-    if (mode == 0) {
-        v = y0.x - a[base + j] * y1.x;
-        if (c) v -= c[base + j] * Yn[2 * n3 + j].x;
-    } else {
-        v = T(0);
-        const T* Gn = G + node * (int64_t)Nrho * n3;
-        for (int r = 0; r < Nrho; ++r) v += Gn[r * n3 + j];
-        v -= a[base + j] * y0.x + y1.x;
-    }
+    T v = y0.x - a[base + j] * y1.x;
+    if (c) v -= c[base + j] * Yn[2 * n3 + j].x;
     if (!isfinite(v)) atomicOr(flags, 2);
     out[base + j] = v;
 }
@@ -372,42 +298,11 @@ cudaError_t launch_combine(const DevTables<T>& t, const Cplx<T>* X, int xslots, 
 }
 
 template <typename T>
-cudaError_t launch_loss_pair(const DevTables<T>& t, const Cplx<T>* X, int xfields, NodeParams np,
-                             int64_t nodes, int s0, int s1, Cplx<T>* Y, int yfields, cudaStream_t s) {
-    if (nodes <= 0) return cudaSuccess;
-    const int64_t n3 = (int64_t)t.N * t.N * t.N;
-    k_loss_pair<T><<<dim3(blocks_for(n3, 256), (unsigned)nodes), 256, 0, s>>>(X, xfields, t.Lr, t.GL0, t.GLd, t.cr, np, t.Nrho, n3, s0, s1, Y, yfields);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_multiply_uk(const DevTables<T>& t, Cplx<T>* X, int xfields, int src, int64_t nodes,
-                               cudaStream_t s) {
-    if (nodes <= 0) return cudaSuccess;
-    const int64_t n3 = (int64_t)t.N * t.N * t.N;
-    k_multiply_uk<T><<<dim3(blocks_for(n3, 256), (unsigned)nodes), 256, 0, s>>>(X, xfields, t.Uk, t.rank, n3, src);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_expand_radial(const DevTables<T>& t, const Cplx<T>* X, int xfields, NodeParams np,
-                                 int64_t nodes, T* U, cudaStream_t s) {
-    if (nodes <= 0) return cudaSuccess;
-    const int64_t n3 = (int64_t)t.N * t.N * t.N;
-    const int bs = 128;
-    const size_t sm = sizeof(T) * (size_t)(t.rank * t.Nrho + t.rank * bs + t.Nrho);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_expand_radial<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_expand_radial<T><<<dim3(blocks_for(n3, bs), (unsigned)nodes), bs, sm, s>>>(X, xfields, t.Vr, t.cr, t.wr, np, t.Nrho, t.rank, n3, U);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_finalize(int N, int Nrho, const Cplx<T>* Y, int yfields, const T* a, const T* c,
-                            const T* G, const int64_t* offs, int64_t nodes, int mode, T* out,
-                            int* flags, cudaStream_t s) {
+cudaError_t launch_finalize(int N, const Cplx<T>* Y, int yfields, const T* a, const T* c, const int64_t* offs,
+                            int64_t nodes, T* out, int* flags, cudaStream_t s) {
     if (nodes <= 0) return cudaSuccess;
     const int64_t n3 = (int64_t)N * N * N;
-    k_finalize<T><<<dim3(blocks_for(n3, 256), (unsigned)nodes), 256, 0, s>>>(Nrho, n3, Y, yfields, a, c, G, offs, mode, out, flags);
+    k_finalize<T><<<dim3(blocks_for(n3, 256), (unsigned)nodes), 256, 0, s>>>(n3, Y, yfields, a, c, offs, out, flags);
     return cudaGetLastError();
 }
 
@@ -419,15 +314,8 @@ cudaError_t launch_finalize(int N, int Nrho, const Cplx<T>* Y, int yfields, cons
                                               Cplx<T>*, int, int, int, cudaStream_t);                 \
     template cudaError_t launch_combine<T>(const DevTables<T>&, const Cplx<T>*, int, NodeParams,      \
                                            int64_t, T, int, int, Cplx<T>*, int, cudaStream_t);        \
-    template cudaError_t launch_loss_pair<T>(const DevTables<T>&, const Cplx<T>*, int, NodeParams,    \
-                                             int64_t, int, int, Cplx<T>*, int, cudaStream_t);         \
-    template cudaError_t launch_multiply_uk<T>(const DevTables<T>&, Cplx<T>*, int, int, int64_t,      \
-                                               cudaStream_t);                                         \
-    template cudaError_t launch_expand_radial<T>(const DevTables<T>&, const Cplx<T>*, int, NodeParams,\
-                                                 int64_t, T*, cudaStream_t);                          \
-    template cudaError_t launch_finalize<T>(int, int, const Cplx<T>*, int, const T*, const T*,        \
-                                            const T*, const int64_t*, int64_t, int, T*, int*,         \
-                                            cudaStream_t);
+    template cudaError_t launch_finalize<T>(int, const Cplx<T>*, int, const T*, const T*,             \
+                                            const int64_t*, int64_t, T*, int*, cudaStream_t);
 DGFS_INST(float)
 DGFS_INST(double)
 #undef DGFS_INST

@@ -1,6 +1,6 @@
 // CUDA-core (FP32 / FP64) kernels of the gain's translate-product-accumulate step as dense
 // circulant passes. The library's CUDA-core calls take their translates in Fourier space
-// (k_vss.cu, a fifth of the arithmetic); these kernels serve the allocation-free call of FP32/FP64
+// (k_shift.cu, a fraction of the arithmetic); these kernels serve the allocation-free call of FP32/FP64
 // plans.
 //
 // For every node and radial Gauss-Legendre point c_r this computes

@@ -22,10 +22,11 @@
 // Half spectra: kz = 0 .. N/2 - 1, with the spectra of kz = 0 and kz = N/2 (both of real (x, y)
 // fields, which x and y translates keep real) in the real and imaginary part of slot kz = 0.
 #include <algorithm>
+#include <cmath>
 #include <map>
 
-#include "fft_const.cuh"
 #include "shift.h"
+#include "shift_dev.cuh"
 
 namespace dgfs {
 
@@ -54,6 +55,26 @@ void build_shift_program(const HostPlan& h, ShiftProgram& p) {
                 o[2 * k + 1] = k == N / 2 ? 0.0 : sg * m[2 * k + 1];
             }
         }
+    if (!h.aniso) {
+        const int nq2 = 3 * (N / 2) * (N / 2) + 1;
+        const size_t n3 = (size_t)N * N * N;
+        p.kq.assign((size_t)h.Nrho * nq2, 0.0);
+        std::vector<int64_t> at_q(nq2, -1);   // a mode of each |k|^2
+        auto sk = [N](int q) { return q < N / 2 ? q : q - N; };
+        for (size_t i = 0; i < n3; ++i) {
+            const int kx = sk((int)(i / ((size_t)N * N))), ky = sk((int)((i / N) % N)), kz = sk((int)(i % N));
+            at_q[kx * kx + ky * ky + kz * kz] = (int64_t)i;
+        }
+        for (int r = 0; r < h.Nrho; ++r) {
+            const double wr = h.wr[r] * 4.0 * 3.14159265358979323846 * h.b * std::pow(h.cr[r], h.gamma + 2.0);
+            for (int q = 0; q < nq2; ++q) {
+                if (at_q[q] < 0) continue;
+                double v = 0.0;
+                for (int s = 0; s < h.rank; ++s) v += h.Uk[(size_t)s * n3 + at_q[q]] * h.Vr[(size_t)s * h.Nrho + r];
+                p.kq[(size_t)r * nq2 + q] = wr * v;
+            }
+        }
+    }
     struct Key { double x, y, z; int q; };
     auto program = [&](bool both) {
         std::vector<Key> keys;
@@ -78,46 +99,7 @@ void build_shift_program(const HostPlan& h, ShiftProgram& p) {
 
 namespace {
 
-using fdev::line_slot;
-
-template <typename T> struct Pair2;
-template <> struct Pair2<float> { using type = float2; };
-template <> struct Pair2<double> { using type = double2; };
-template <typename T>
-__device__ __forceinline__ Cplx<T> ld(const Cplx<T>* p) {
-    const typename Pair2<T>::type v = *reinterpret_cast<const typename Pair2<T>::type*>(p);
-    return Cplx<T>{v.x, v.y};
-}
-template <typename T>
-__device__ __forceinline__ Cplx<T> ldg(const Cplx<T>* p) {
-    const typename Pair2<T>::type v = __ldg(reinterpret_cast<const typename Pair2<T>::type*>(p));
-    return Cplx<T>{v.x, v.y};
-}
-template <typename T>
-__device__ __forceinline__ void st(Cplx<T>* p, Cplx<T> c) {
-    typename Pair2<T>::type v;
-    v.x = c.x;
-    v.y = c.y;
-    *reinterpret_cast<typename Pair2<T>::type*>(p) = v;
-}
-
-// two consecutive complex values from an even index (one 16-byte access in FP32)
-template <bool GLOBAL>
-__device__ __forceinline__ void ld_two(const Cplx<float>* p, Cplx<float>& a, Cplx<float>& b) {
-    const float4 v = GLOBAL ? __ldg(reinterpret_cast<const float4*>(p)) : *reinterpret_cast<const float4*>(p);
-    a = Cplx<float>{v.x, v.y};
-    b = Cplx<float>{v.z, v.w};
-}
-template <bool GLOBAL>
-__device__ __forceinline__ void ld_two(const Cplx<double>* p, Cplx<double>& a, Cplx<double>& b) {
-    a = GLOBAL ? ldg(p) : ld(p);
-    b = GLOBAL ? ldg(p + 1) : ld(p + 1);
-}
-
-template <typename T>
-__device__ __forceinline__ Cplx<T> cmul(Cplx<T> a, T br, T bi) {
-    return Cplx<T>{fma(-a.y, bi, a.x * br), fma(a.x, bi, a.y * br)};
-}
+using namespace shdev;
 
 // ---- forward (y, z) spectra ------------------------------------------------------------------
 
@@ -133,7 +115,7 @@ struct ForwardGeo {
 // half spectra; then lines along y of every slot kz.
 template <typename T, int N>
 __global__ void __launch_bounds__(ForwardGeo<N>::NT)
-k_shift_forward(const T* __restrict__ f, const int64_t* __restrict__ offs, Cplx<T>* __restrict__ G) {
+k_shift_forward(const T* __restrict__ f, const T* __restrict__ b, const int64_t* __restrict__ offs, Cplx<T>* __restrict__ G) {
     using Geo = ForwardGeo<N>;
     constexpr int NH = N / 2, PX = Geo::PX, NT = Geo::NT, PITCH = Geo::PITCH;
     extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -141,8 +123,8 @@ k_shift_forward(const T* __restrict__ f, const int64_t* __restrict__ offs, Cplx<
     Cplx<T>* S = reinterpret_cast<Cplx<T>*>(sm_raw);       // [PX][N][PITCH]
     const int tid = threadIdx.x, x0 = blockIdx.x * PX, pl = tid / NH, j = tid % NH;
     const int64_t node = blockIdx.y, n3 = (int64_t)N * N * N;
-    const T* fn = f + (offs ? offs[node] : node * n3) + (int64_t)x0 * N * N;
-    for (int e = tid; e < PX * N * N; e += NT) rows[(e / N) * (N + 1) + e % N] = fn[e];
+    const int64_t base = (offs ? offs[node] : node * n3) + (int64_t)x0 * N * N;
+    for (int e = tid; e < PX * N * N; e += NT) rows[(e / N) * (N + 1) + e % N] = b ? f[base + e] * b[base + e] : f[base + e];
     __syncthreads();
     Cplx<T> v[N];
 #pragma unroll
@@ -150,15 +132,15 @@ k_shift_forward(const T* __restrict__ f, const int64_t* __restrict__ offs, Cplx<
         v[line_slot<N>(z)] = Cplx<T>{rows[(pl * N + j) * (N + 1) + z], rows[(pl * N + j + NH) * (N + 1) + z]};
     __syncthreads();
     cfft::line<T, N, true>(v);
-    Cplx<T>* a = S + (pl * N + j) * PITCH;
-    Cplx<T>* b = a + NH * PITCH;
-    st(a, Cplx<T>{v[0].x, v[NH].x});
-    st(b, Cplx<T>{v[0].y, v[NH].y});
+    Cplx<T>* ra = S + (pl * N + j) * PITCH;
+    Cplx<T>* rb = ra + NH * PITCH;
+    st(ra, Cplx<T>{v[0].x, v[NH].x});
+    st(rb, Cplx<T>{v[0].y, v[NH].y});
 #pragma unroll
     for (int k = 1; k < NH; ++k) {
         const Cplx<T> p = v[k], m = v[N - k];
-        st(a + k, Cplx<T>{T(0.5) * (p.x + m.x), T(0.5) * (p.y - m.y)});
-        st(b + k, Cplx<T>{T(0.5) * (p.y + m.y), T(0.5) * (m.x - p.x)});
+        st(ra + k, Cplx<T>{T(0.5) * (p.x + m.x), T(0.5) * (p.y - m.y)});
+        st(rb + k, Cplx<T>{T(0.5) * (p.y + m.y), T(0.5) * (m.x - p.x)});
     }
     __syncthreads();
 #pragma unroll
@@ -217,14 +199,6 @@ k_shift_x(const Cplx<T>* __restrict__ G, const Cplx<T>* __restrict__ mu, const i
 
 // ---- y and z translates, products ------------------------------------------------------------
 
-// Row pitch (complex elements) of the y-translated fields in shared memory: a thread's kz row starts
-// 16-byte aligned and eight consecutive rows fall into different 16-byte bank groups.
-template <typename T, int N>
-__host__ __device__ constexpr int row_pitch() {
-    if (sizeof(T) == 8) return N / 2 + 1;
-    return N == 32 ? 18 : N == 24 ? 14 : N == 16 ? 10 : 6;
-}
-
 template <typename T, int N, int XC>
 struct ProductGeo {
     static constexpr int NT = XC * N;                        // z lines; y lines: 2 XC N / 2
@@ -267,29 +241,7 @@ k_shift_products(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf,
         const ShiftEntry e = prog[i];
         if (e.newy) {
             const int fi = op ? e.fm : e.fp;
-            const Cplx<T>* src = fi < 0 ? Gy : Hy + fi * FS;
-#pragma unroll
-            for (int k = 0; k < N; ++k) v[line_slot<N>(k)] = ldg(src + k * NH);
-            if (e.yrow >= 0) {
-                const Cplx<T>* m = mu_r + e.yrow * MP;
-                const T sg = (e.yneg ^ op) ? T(-1) : T(1);
-#pragma unroll
-                for (int k2 = 0; k2 < NH; k2 += 2) {
-                    Cplx<T> w2[2];
-                    ld_two<true>(m + k2, w2[0], w2[1]);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int k = k2 + h;
-                        if (k == 0) continue;
-                        const T wi = sg * w2[h].y;
-                        v[line_slot<N>(k)] = cmul(v[line_slot<N>(k)], w2[h].x, wi);
-                        v[line_slot<N>(N - k)] = cmul(v[line_slot<N>(N - k)], w2[h].x, -wi);
-                    }
-                }
-                const T wn = ldg(m + NH).x;
-                v[line_slot<N>(NH)].x *= wn;
-                v[line_slot<N>(NH)].y *= wn;
-            }
+            load_y_line<T, N>(fi < 0 ? Gy : Hy + fi * FS, mu_r, e.yrow, e.yneg ^ op, v);
             cfft::line<T, N, false>(v);
             __syncthreads();   // the previous (s_x, s_y) has been read
 #pragma unroll
@@ -298,34 +250,7 @@ k_shift_products(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf,
         }
         // z line of T_s f + i T_-s g from the half spectra a (+s) and b (-s, the conjugate phase)
         const T wgt = wscale * __ldg(wsig + e.pair);
-        const bool zs = e.zrow >= 0;
-        const Cplx<T>* m = mu_r + (zs ? e.zrow : 0) * MP;
-        const T sg = e.zneg ? T(-1) : T(1);
-#pragma unroll
-        for (int k2 = 0; k2 < NH; k2 += 2) {
-            Cplx<T> a2[2], b2[2], w2[2];
-            ld_two<false>(zp + k2, a2[0], a2[1]);
-            ld_two<false>(zm + k2, b2[0], b2[1]);
-            if (zs) ld_two<true>(m + k2, w2[0], w2[1]);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = k2 + h;
-                Cplx<T> a = a2[h], b = b2[h];
-                if (k == 0) {   // kz = 0 and kz = N/2, both real
-                    const T wn = zs ? ldg(m + NH).x : T(1);
-                    v[0] = Cplx<T>{a.x, b.x};
-                    v[line_slot<N>(NH)] = Cplx<T>{wn * a.y, wn * b.y};
-                } else {
-                    if (zs) {
-                        const T wi = sg * w2[h].y;
-                        a = cmul(a, w2[h].x, wi);
-                        b = cmul(b, w2[h].x, -wi);
-                    }
-                    v[line_slot<N>(k)] = Cplx<T>{a.x - b.y, a.y + b.x};
-                    v[line_slot<N>(N - k)] = Cplx<T>{a.x + b.y, b.x - a.y};
-                }
-            }
-        }
+        load_z_line<T, N>(zp, zm, mu_r, e.zrow, e.zneg, v);
         cfft::line<T, N, false>(v);
 #pragma unroll
         for (int z = 0; z < N; ++z) acc[z] = fma(wgt * v[z].x, v[z].y, acc[z]);
@@ -351,10 +276,10 @@ k_shift_products(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf,
 }
 
 template <typename T, int N>
-cudaError_t forward_n(const T* f, const int64_t* offs, int64_t nodes, Cplx<T>* G, cudaStream_t s) {
+cudaError_t forward_n(const T* f, const T* b, const int64_t* offs, int64_t nodes, Cplx<T>* G, cudaStream_t s) {
     using Geo = ForwardGeo<N>;
     constexpr size_t sm = (size_t)Geo::PX * N * Geo::PITCH * sizeof(Cplx<T>);
-    k_shift_forward<T, N><<<dim3(N / Geo::PX, (unsigned)nodes), Geo::NT, sm, s>>>(f, offs, G);
+    k_shift_forward<T, N><<<dim3(N / Geo::PX, (unsigned)nodes), Geo::NT, sm, s>>>(f, b, offs, G);
     return cudaGetLastError();
 }
 
@@ -415,8 +340,9 @@ cudaError_t products_n(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* H
     return cudaErrorInvalidValue
 
 template <typename T>
-cudaError_t launch_shift_forward(const T* f, const int64_t* offs, int N, int64_t nodes, Cplx<T>* G, cudaStream_t s) {
-#define CALL(n) forward_n<T, n>(f, offs, nodes, G, s)
+cudaError_t launch_shift_forward(const T* f, const T* b, const int64_t* offs, int N, int64_t nodes, Cplx<T>* G,
+                                 cudaStream_t s) {
+#define CALL(n) forward_n<T, n>(f, b, offs, nodes, G, s)
     DGFS_BY_N(CALL);
 #undef CALL
 }
@@ -439,7 +365,8 @@ cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const
 }
 
 #define DGFS_SHIFT_INST(T)                                                                                            \
-    template cudaError_t launch_shift_forward<T>(const T*, const int64_t*, int, int64_t, Cplx<T>*, cudaStream_t);     \
+    template cudaError_t launch_shift_forward<T>(const T*, const T*, const int64_t*, int, int64_t, Cplx<T>*,               \
+                                                 cudaStream_t);                                                       \
     template cudaError_t launch_shift_x<T>(const ShiftDev<T>&, const Cplx<T>*, int, int, int, int64_t, Cplx<T>*,      \
                                            cudaStream_t);                                                             \
     template cudaError_t launch_shift_products<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*, \

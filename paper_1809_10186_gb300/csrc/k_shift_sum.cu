@@ -1,0 +1,688 @@
+// The calls that transform every product forward again, on the shared translates of k_shift.cu:
+//
+//   VSS kernel (alpha != 1): gain^ = sum_r sum_p A_rp(k) DFT[(T_s f)(T_-s g) + (T_-s f)(T_s g)]_k
+//   adjoint (VJP):  gain = sum_r sum_p 2 w_p [T_-s(U_r T_-s f) + T_s(U_r T_s f)],  U_r = K_r u
+//
+//   k_shift_vss     per (node, r, XC planes x): the product lines of two sphere points share one forward z
+//                   transform (real and imaginary part, separated per line into half spectra), forward y  -> W
+//   k_shift_adj     the same for U_r T_-s f and U_r T_s f; the back-translates are phases, so what shares
+//                   (s_x, s_y) is summed after the z phases, what shares s_x after the y phases         -> V
+//   k_shift_sum     per (ky, kz) column: forward x of every field of W (V), times A_rp (the x phase), summed
+//                   over fields and a part of the radial points in registers                -> partial spectra
+//   k_shift_reduce  sum of the parts, inverse x
+//   k_shift_filter  a real multiplier on a field: forward x, multiplier, inverse x (K_L f, and K_r u)
+//   k_shift_out     inverse y and z of the gain and the loss fields, the result
+//
+// Measured (GB300, FP32, N = 32, M = 38): VSS Q of 40 nodes 3.1 ms (6.5 ms with a three-axis transform of its own for
+// every translate and product), VJP of 48 nodes 4.2 ms (11 ms); k_shift_vss 57 % and k_shift_adj 80 % of them, both
+// bound by instruction issue at 8-12 warps per SM (a line and its sums fill the registers).
+//
+// Everything stays in half spectra (kz >= 0): A_rp and the loss weight act on real fields, so only their part
+// even in k counts. A multiplier on the packed slot kz = 0 needs the spectra of kz = 0 and kz = N/2 apart.
+// k_shift_vss separates them along y, where its threads hold whole lines: their plane kz = 0 of W carries
+// ky = 0 .. N/2 - 1 of the first, then of the second, with the real ky = 0 and N/2 packed in the two slots
+// ky = 0 (a "folded" plane); only those two columns are separated along x, in registers. k_shift_filter takes the
+// plane as it is: one warp holds it, kx in registers and ky along the lanes.
+#include "shift.h"
+#include "shift_dev.cuh"
+
+namespace dgfs {
+
+namespace {
+
+using namespace shdev;
+
+// half spectra of the two real lines that v's parts carried through a forward transform; lo takes the real
+// part's, hi the imaginary part's
+template <typename T, int N, typename F>
+__device__ __forceinline__ void split_line(const Cplx<T> (&v)[N], F put) {
+    constexpr int NH = N / 2;
+    put(0, Cplx<T>{v[0].x, v[NH].x}, Cplx<T>{v[0].y, v[NH].y});
+#pragma unroll
+    for (int k = 1; k < NH; ++k) {
+        const Cplx<T> p = v[k], m = v[N - k];
+        put(k, Cplx<T>{T(0.5) * (p.x + m.x), T(0.5) * (p.y - m.y)}, Cplx<T>{T(0.5) * (p.y + m.y), T(0.5) * (m.x - p.x)});
+    }
+}
+
+template <typename T, int N, int XC>
+struct SumGeo {
+    static constexpr int NT = XC * N;
+    static constexpr int PITCH = row_pitch<T, N>();
+    static constexpr int BUF = 2 * XC * N * PITCH;           // complex elements of one buffer
+    static constexpr size_t smem = (size_t)2 * BUF * sizeof(Cplx<T>);
+    // k_shift_vss keeps a line and one product line, k_shift_adj a line, its sum and U's line
+    static constexpr int MINV = sizeof(T) == 8 ? 1 : N == 32 ? 384 / NT : N == 24 ? 480 / NT : 768 / NT;
+    static constexpr int MINA = sizeof(T) == 8 ? 1 : N == 32 ? 256 / NT : N == 24 ? 384 / NT : 512 / NT;
+};
+
+// grid (N / XC, nr, nodes). W [node][r][entry][x][ky][kz].
+template <typename T, int N, int XC>
+__global__ void __launch_bounds__(SumGeo<T, N, XC>::NT, SumGeo<T, N, XC>::MINV)
+k_shift_vss(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, const Cplx<T>* __restrict__ Gg,
+            const Cplx<T>* __restrict__ Hg, const Cplx<T>* __restrict__ mu, const ShiftEntry* __restrict__ prog, int nprog,
+            int nrows, int nx, int r0, Cplx<T>* __restrict__ W) {
+    using Geo = SumGeo<T, N, XC>;
+    constexpr int NH = N / 2, PITCH = Geo::PITCH, NT = Geo::NT, MP = shift_mu_pitch(N);
+    constexpr int64_t FS = (int64_t)N * N * NH;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    Cplx<T>* Y = reinterpret_cast<Cplx<T>*>(sm_raw);         // [sign][XC][y][PITCH] inverse y lines
+    Cplx<T>* S = Y + Geo::BUF;                               // [field][XC][y][PITCH] forward z lines
+    const int tid = threadIdx.x, x0 = blockIdx.x * XC, rl = blockIdx.y, nr = gridDim.y;
+    const int64_t node = blockIdx.z;
+    const int op = tid / (XC * NH), ypl = (tid / NH) % XC, ykz = tid % NH;
+    const int64_t ybase = (int64_t)(x0 + ypl) * N * NH + ykz;
+    const Cplx<T>* Gy = (op ? Gg : Gf) + node * FS + ybase;
+    const Cplx<T>* Hy = (op ? Hg : Hf) + (node * nr + rl) * (2 * nx) * FS + ybase;
+    const int yrow = ((op * XC + ypl) * N) * PITCH + ykz;     // this thread's y line in a buffer
+    const Cplx<T>* mu_r = mu + (int64_t)(r0 + rl) * nrows * MP;
+    Cplx<T>* Wn = W + (node * nr + rl) * nprog * FS + ybase;
+    T first[N];                                              // products of the even entry
+    Cplx<T> v[N];
+    for (int i = 0; i < nprog; ++i) {
+        const ShiftEntry e = prog[i];
+        if (e.newy) {
+            const int fi = op ? e.fm : e.fp;
+            load_y_line<T, N>(fi < 0 ? Gy : Hy + fi * FS, mu_r, e.yrow, e.yneg ^ op, v);
+            cfft::line<T, N, false>(v);
+            __syncthreads();   // the previous (s_x, s_y) has been read
+#pragma unroll
+            for (int y = 0; y < N; ++y) st(Y + yrow + y * PITCH, v[y]);
+            __syncthreads();
+        }
+        load_z_line<T, N>(Y + tid * PITCH, Y + (NT + tid) * PITCH, mu_r, e.zrow, e.zneg, v);
+        cfft::line<T, N, false>(v);
+        if ((i & 1) == 0) {
+#pragma unroll
+            for (int z = 0; z < N; ++z) first[z] = v[z].x * v[z].y;
+            if (i + 1 < nprog) continue;
+#pragma unroll
+            for (int z = 0; z < N; ++z) v[z] = Cplx<T>{T(0), T(0)};
+        }
+        Cplx<T> w[N];
+#pragma unroll
+        for (int z = 0; z < N; ++z) w[line_slot<N>(z)] = Cplx<T>{first[z], v[z].x * v[z].y};
+        cfft::line<T, N, true>(w);
+        __syncthreads();       // the previous pair's half spectra have been read
+        split_line<T, N>(w, [&](int k, Cplx<T> a, Cplx<T> b) {
+            st(S + tid * PITCH + k, a);
+            st(S + (NT + tid) * PITCH + k, b);
+        });
+        __syncthreads();
+        const int j = (i & ~1) + op;
+        if (j < nprog) {
+#pragma unroll
+            for (int y = 0; y < N; ++y) w[line_slot<N>(y)] = ld(S + yrow + y * PITCH);
+            cfft::line<T, N, true>(w);
+            Cplx<T>* o = Wn + j * FS;
+            if (ykz > 0) {
+#pragma unroll
+                for (int k = 0; k < N; ++k) st(o + k * NH, w[k]);
+            } else {   // the folded plane
+                split_line<T, N>(w, [&](int k, Cplx<T> a, Cplx<T> b) {
+                    st(o + k * NH, a);
+                    st(o + (NH + k) * NH, b);
+                });
+            }
+        }
+    }
+}
+
+// grid (N / XC, nr, nodes). Ur [node][r][x][ky][kz]: x-space half spectra of K_r u. V [node][r][2 nx + 2][x][ky][kz]:
+// field fi collects what takes the x phase of x field fi, the last two what takes none.
+template <typename T, int N, int XC>
+__global__ void __launch_bounds__(SumGeo<T, N, XC>::NT, SumGeo<T, N, XC>::MINA)
+k_shift_adj(const Cplx<T>* __restrict__ G, const Cplx<T>* __restrict__ H, const Cplx<T>* __restrict__ Ur,
+            const Cplx<T>* __restrict__ mu, const ShiftEntry* __restrict__ prog, int nprog, const T* __restrict__ wsig,
+            int nrows, int nx, int r0, Cplx<T>* __restrict__ V) {
+    using Geo = SumGeo<T, N, XC>;
+    constexpr int NH = N / 2, PITCH = Geo::PITCH, NT = Geo::NT, MP = shift_mu_pitch(N);
+    constexpr int64_t FS = (int64_t)N * N * NH;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    Cplx<T>* Y = reinterpret_cast<Cplx<T>*>(sm_raw);         // [sign][XC][y][PITCH] inverse y lines
+    Cplx<T>* S = Y + Geo::BUF;                               // [sign][XC][y][PITCH] sums over s_z
+    const int tid = threadIdx.x, x0 = blockIdx.x * XC, rl = blockIdx.y, nr = gridDim.y;
+    const int64_t node = blockIdx.z, item = node * nr + rl;
+    const int op = tid / (XC * NH), ypl = (tid / NH) % XC, ykz = tid % NH;
+    const int64_t ybase = (int64_t)(x0 + ypl) * N * NH + ykz;
+    const Cplx<T>* Gy = G + node * FS + ybase;
+    const Cplx<T>* Hy = H + item * (2 * nx) * FS + ybase;
+    const int yrow = ((op * XC + ypl) * N) * PITCH + ykz;
+    const Cplx<T>* mu_r = mu + (int64_t)(r0 + rl) * nrows * MP;
+    Cplx<T>* Vn = V + item * (2 * nx + 2) * FS + ybase;
+    Cplx<T> v[N];
+    T u[N];   // U_r on this thread's z line
+    if (op == 0) {
+        load_y_line<T, N>(Ur + item * FS + ybase, mu_r, -1, 0, v);
+        cfft::line<T, N, false>(v);
+#pragma unroll
+        for (int y = 0; y < N; ++y) st(Y + yrow + y * PITCH, v[y]);
+    }
+    __syncthreads();
+    {
+        const Cplx<T>* zr = Y + tid * PITCH;
+        const Cplx<T> a0 = ld(zr);
+        v[0] = Cplx<T>{a0.x, T(0)};
+        v[line_slot<N>(NH)] = Cplx<T>{a0.y, T(0)};
+#pragma unroll
+        for (int k = 1; k < NH; ++k) {
+            const Cplx<T> a = ld(zr + k);
+            v[line_slot<N>(k)] = a;
+            v[line_slot<N>(N - k)] = Cplx<T>{a.x, -a.y};
+        }
+        cfft::line<T, N, false>(v);
+#pragma unroll
+        for (int z = 0; z < N; ++z) u[z] = v[z].x;
+    }
+    Cplx<T> acc[N];   // this thread's (sign, plane, kz) line over ky: sum over the s_y of one s_x
+#pragma unroll
+    for (int k = 0; k < N; ++k) acc[k] = Cplx<T>{T(0), T(0)};
+    ShiftEntry g{};   // first entry of the group in hand
+    bool zero_seen = false; // a group without x shift
+    uint64_t written = 0;   // x fields (the first 64) that hold a sum already: rules with points on both sides of x = 0
+    for (int i = 0; i <= nprog; ++i) {
+        const ShiftEntry e = prog[i < nprog ? i : 0];
+        const bool next = i == nprog || e.newy;
+        if (next && i > 0) {
+            __syncthreads();   // the group's sums over s_z are complete
+#pragma unroll
+            for (int y = 0; y < N; ++y) v[line_slot<N>(y)] = ld(S + yrow + y * PITCH);
+            cfft::line<T, N, true>(v);
+            const Cplx<T>* m = mu_r + (int64_t)(g.yrow >= 0 ? g.yrow : 0) * MP;
+            const T sg = (g.yneg ^ op) ? T(-1) : T(1);
+#pragma unroll
+            for (int k = 0; k <= NH; ++k) {
+                Cplx<T> w{T(1), T(0)};
+                if (g.yrow >= 0) w = ldg(m + k);
+                const T wi = k == 0 || k == NH ? T(0) : sg * w.y;
+                acc[k] = Cplx<T>{fma(v[k].x, w.x, fma(-v[k].y, wi, acc[k].x)), fma(v[k].y, w.x, fma(v[k].x, wi, acc[k].y))};
+                if (k > 0 && k < NH) {
+                    Cplx<T>& a = acc[N - k];
+                    const Cplx<T> q = v[N - k];
+                    a = Cplx<T>{fma(q.x, w.x, fma(q.y, wi, a.x)), fma(q.y, w.x, fma(-q.x, wi, a.y))};
+                }
+            }
+            if (i == nprog || e.fp != g.fp) {   // the next s_x
+                const int fi = g.fp < 0 ? 2 * nx + op : op ? g.fm : g.fp, xi = g.fp < 0 ? -1 : g.fp >> 1;
+                Cplx<T>* o = Vn + fi * FS;
+                // both fields of an |s_x| are written together; a second visit (the opposite s_x) adds
+                bool add = false;
+                zero_seen |= xi < 0;
+                if (xi >= 0) {
+                    if (xi < 64) {
+                        add = (written >> xi) & 1;
+                        written |= uint64_t(1) << xi;
+                    } else {
+                        for (int q = 0; q < i && !add; ++q) add = prog[q].fp >= 0 && (prog[q].fp >> 1) == xi && prog[q].fp != g.fp;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    Cplx<T> s = acc[k];
+                    if (add) {
+                        const Cplx<T> b = ld(o + k * NH);
+                        s.x += b.x;
+                        s.y += b.y;
+                    }
+                    st(o + k * NH, s);
+                    acc[k] = Cplx<T>{T(0), T(0)};
+                }
+            }
+        }
+        if (i == nprog) {
+            if (!zero_seen)
+                for (int k = 0; k < N; ++k) st(Vn + (2 * nx + op) * FS + k * NH, Cplx<T>{T(0), T(0)});
+            break;
+        }
+        if (e.newy) {
+            const int fi = op ? e.fm : e.fp;
+            load_y_line<T, N>(fi < 0 ? Gy : Hy + fi * FS, mu_r, e.yrow, e.yneg ^ op, v);
+            cfft::line<T, N, false>(v);
+            if (i == 0) __syncthreads();   // U's lines have been read (later groups: the barrier above)
+#pragma unroll
+            for (int y = 0; y < N; ++y) st(Y + yrow + y * PITCH, v[y]);
+            __syncthreads();
+            g = e;
+        }
+        load_z_line<T, N>(Y + tid * PITCH, Y + (NT + tid) * PITCH, mu_r, e.zrow, e.zneg, v);
+        cfft::line<T, N, false>(v);
+        Cplx<T> w[N];   // U T_-s f + i U T_s f
+#pragma unroll
+        for (int z = 0; z < N; ++z) w[line_slot<N>(z)] = Cplx<T>{u[z] * v[z].y, u[z] * v[z].x};
+        cfft::line<T, N, true>(w);
+        const T wgt = T(2) * __ldg(wsig + e.pair), sg = e.zneg ? T(-1) : T(1);
+        const bool zs = e.zrow >= 0, set = e.newy;
+        const Cplx<T>* m = mu_r + (int64_t)(zs ? e.zrow : 0) * MP;
+        Cplx<T>* sp = S + tid * PITCH;          // T_s(U T_s f)
+        Cplx<T>* sm = S + (NT + tid) * PITCH;   // T_-s(U T_-s f)
+        split_line<T, N>(w, [&](int k, Cplx<T> b, Cplx<T> a) {
+            if (k == 0) {
+                const T wn = zs ? wgt * ldg(m + NH).x : wgt;
+                a = Cplx<T>{wgt * a.x, wn * a.y};
+                b = Cplx<T>{wgt * b.x, wn * b.y};
+            } else {
+                Cplx<T> p{wgt, T(0)};
+                if (zs) {
+                    const Cplx<T> q = ldg(m + k);
+                    p = Cplx<T>{wgt * q.x, wgt * sg * q.y};
+                }
+                a = cmul(a, p.x, p.y);
+                b = cmul(b, p.x, -p.y);
+            }
+            if (!set) {
+                const Cplx<T> ao = ld(sp + k), bo = ld(sm + k);
+                a = Cplx<T>{a.x + ao.x, a.y + ao.y};
+                b = Cplx<T>{b.x + bo.x, b.y + bo.y};
+            }
+            st(sp + k, a);
+            st(sm + k, b);
+        });
+    }
+}
+
+// ---- columns (ky, kz): x lines ----------------------------------------------------------------
+
+// The packed plane kz = 0 (kx in registers, ky = lane < N): real multipliers m0 on the spectrum of kz = 0 and mn on
+// that of kz = N/2. Every lane of the warp takes part.
+template <typename T, int N, typename M>
+__device__ __forceinline__ void packed_plane(const Cplx<T> (&v)[N], int ky, M mult, Cplx<T> (&out)[N]) {
+    const int src = ky == 0 ? 0 : N - ky;
+#pragma unroll
+    for (int kx = 0; kx < N; ++kx) {
+        const Cplx<T> a = v[kx], q = v[(N - kx) % N];
+        const Cplx<T> b{__shfl_sync(0xffffffffu, q.x, src), __shfl_sync(0xffffffffu, q.y, src)};   // the mirror
+        T m0, mn;
+        mult(kx, m0, mn);
+        const T h0 = T(0.5) * m0, hn = T(0.5) * mn;
+        // m0 (a + conj b) / 2 + i mn (a - conj b) / 2i
+        out[kx] = Cplx<T>{h0 * (a.x + b.x) + hn * (a.x - b.x), h0 * (a.y - b.y) + hn * (a.y + b.y)};
+    }
+}
+
+constexpr int kColThreads = 128;
+
+// blocks of all columns, or of the ones with kz > 0
+template <int N, bool NONZERO>
+constexpr int col_blocks() { return (N * (N / 2 - (NONZERO ? 1 : 0)) + kColThreads - 1) / kColThreads; }
+
+// F [node][r][nf fields][x][ky][kz]; part [node][parts][kx][ky][kz]. VSS: the plane kz = 0 folded, times A[(r0 + r)
+// npairs + pair of the field] in the same order, [kx][ky][kz] and the second multipliers of the two packed columns
+// [2][kx]; else the x phase of field fi (fields 2 nx, 2 nx + 1: none). VSS reads 2.5 MB of products per radial point
+// and node at N = 32, M = 38 and is bound by that.
+// grid (col_blocks, nodes, parts): part c takes the radial points c RP .. of the batch. add: on top of part.
+template <typename T, int N, bool VSS>
+__global__ void __launch_bounds__(kColThreads)
+k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, const ShiftEntry* __restrict__ prog, int npairs,
+            const Cplx<T>* __restrict__ mu, const int* __restrict__ xrows, int nrows, int nx, int r0, int nr, int RP, int add,
+            Cplx<T>* __restrict__ part) {
+    constexpr int NH = N / 2, COLS = N * NH, MP = shift_mu_pitch(N);
+    constexpr int64_t FS = (int64_t)N * COLS, AS = FS + 2 * N;
+    const int64_t node = blockIdx.y;
+    const int col = blockIdx.x * kColThreads + threadIdx.x;
+    if (col >= COLS) return;
+    const bool pair = VSS && (col == 0 || col == NH * NH);   // ky = 0 and N/2 of one plane in a column
+    Cplx<T>* pc = part + (node * gridDim.z + blockIdx.z) * FS + col;
+    Cplx<T> acc[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) acc[k] = add ? ld(pc + (int64_t)k * COLS) : Cplx<T>{T(0), T(0)};
+    const int rl1 = min(nr, (int)(blockIdx.z + 1) * RP);
+    for (int rl = blockIdx.z * RP; rl < rl1; ++rl) {
+        const Cplx<T>* f = F + (node * nr + rl) * nf * FS + col;
+        for (int j = 0; j < nf; ++j, f += FS) {
+            Cplx<T> v[N];
+#pragma unroll
+            for (int x = 0; x < N; ++x) v[line_slot<N>(x)] = ldg(f + (int64_t)x * COLS);
+            cfft::line<T, N, true>(v);
+            if constexpr (VSS) {
+                const T* a = A + ((int64_t)(r0 + rl) * npairs + __ldg(&prog[j].pair)) * AS;
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    const T m = __ldg(a + (int64_t)k * COLS + col);
+                    acc[k] = Cplx<T>{fma(m, v[k].x, acc[k].x), fma(m, v[k].y, acc[k].y)};
+                }
+                if (pair) {   // m a so far; m (a + conj b) / 2 + m' (a - conj b) / 2, b the mirror along x
+                    const T* a2 = a + FS + (col ? N : 0);
+#pragma unroll
+                    for (int k = 0; k < N; ++k) {
+                        const T h = T(0.5) * (__ldg(a2 + k) - __ldg(a + (int64_t)k * COLS + col));
+                        const Cplx<T> b = v[(N - k) % N];
+                        acc[k] = Cplx<T>{fma(h, v[k].x - b.x, acc[k].x), fma(h, v[k].y + b.y, acc[k].y)};
+                    }
+                }
+            } else {
+                const bool shifted = j < 2 * nx;
+                const Cplx<T>* m = mu + ((int64_t)(r0 + rl) * nrows + (shifted ? __ldg(xrows + (j >> 1)) : 0)) * MP;
+                const T sg = j & 1 ? T(-1) : T(1);
+#pragma unroll
+                for (int k = 0; k <= NH; ++k) {
+                    Cplx<T> w{T(1), T(0)};
+                    if (shifted) w = ldg(m + k);
+                    const T wi = k == 0 || k == NH ? T(0) : sg * w.y;
+                    acc[k] = Cplx<T>{fma(v[k].x, w.x, fma(-v[k].y, wi, acc[k].x)), fma(v[k].y, w.x, fma(v[k].x, wi, acc[k].y))};
+                    if (k > 0 && k < NH) {
+                        Cplx<T>& b = acc[N - k];
+                        const Cplx<T> q = v[N - k];
+                        b = Cplx<T>{fma(q.x, w.x, fma(q.y, wi, b.x)), fma(q.y, w.x, fma(-q.x, wi, b.y))};
+                    }
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) st(pc + (int64_t)k * COLS, acc[k]);
+}
+
+// out[node][x][ky][kz] = scale * inverse x of the sum of the parts. grid (col_blocks, nodes)
+template <typename T, int N>
+__global__ void __launch_bounds__(kColThreads)
+k_shift_reduce(const Cplx<T>* __restrict__ part, int parts, T scale, Cplx<T>* __restrict__ out) {
+    constexpr int COLS = N * N / 2;
+    constexpr int64_t FS = (int64_t)N * COLS;
+    const int c = blockIdx.x * kColThreads + threadIdx.x;
+    if (c >= COLS) return;
+    const int64_t node = blockIdx.y;
+    Cplx<T> v[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[line_slot<N>(k)] = Cplx<T>{T(0), T(0)};
+    for (int q = 0; q < parts; ++q) {
+        const Cplx<T>* p = part + (node * parts + q) * FS + c;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const Cplx<T> a = ldg(p + (int64_t)k * COLS);
+            Cplx<T>& b = v[line_slot<N>(k)];
+            b = Cplx<T>{b.x + a.x, b.y + a.y};
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = Cplx<T>{scale * v[k].x, scale * v[k].y};
+    cfft::line<T, N, false>(v);
+#pragma unroll
+    for (int x = 0; x < N; ++x) st(out + node * FS + (int64_t)x * COLS + c, v[x]);
+}
+
+// out[node][r][x][ky][kz] = inverse x of M_r(k) times the x spectrum of G: M = tab[k] (nq2 == 0, standard mode
+// index, the same for every r) or tab[r nq2 + |k|^2]. grid (col_blocks + 1, nodes, nr): the last block is one warp for the packed plane kz = 0
+template <typename T, int N>
+__global__ void __launch_bounds__(kColThreads)
+k_shift_filter(const Cplx<T>* __restrict__ G, const T* __restrict__ tab, int nq2, int r0, Cplx<T>* __restrict__ out) {
+    constexpr int NH = N / 2, COLS = N * NH;
+    constexpr int64_t FS = (int64_t)N * COLS;
+    const int64_t node = blockIdx.y;
+    const bool packed = blockIdx.x == gridDim.x - 1;
+    int ky, kz;
+    if (packed) {
+        if (threadIdx.x >= 32) return;
+        ky = threadIdx.x < N ? threadIdx.x : 0;
+        kz = 0;
+    } else {
+        const int c = blockIdx.x * kColThreads + threadIdx.x;
+        if (c >= N * (NH - 1)) return;
+        ky = c / (NH - 1);
+        kz = c % (NH - 1) + 1;
+    }
+    const int col = ky * NH + kz;
+    const T* t = tab + (int64_t)(r0 + blockIdx.z) * nq2;
+    auto sq = [](int q) { const int k = q < NH ? q : q - N; return k * k; };
+    auto mult = [&](int kx, int kzz) { return __ldg(nq2 ? t + sq(kx) + sq(ky) + kzz * kzz : t + (kx * N + ky) * N + kzz); };
+    Cplx<T> v[N], w[N];
+#pragma unroll
+    for (int x = 0; x < N; ++x) v[line_slot<N>(x)] = ldg(G + node * FS + (int64_t)x * COLS + col);
+    cfft::line<T, N, true>(v);
+    const T sc = T(1) / T(N);
+    if (packed) {
+        Cplx<T> q[N];
+        packed_plane<T, N>(v, ky, [&](int kx, T& m0, T& mn) {
+            m0 = mult(kx, 0);
+            mn = mult(kx, NH);
+        }, q);
+#pragma unroll
+        for (int k = 0; k < N; ++k) w[line_slot<N>(k)] = Cplx<T>{sc * q[k].x, sc * q[k].y};
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            const T m = sc * mult(k, kz);
+            w[line_slot<N>(k)] = Cplx<T>{m * v[k].x, m * v[k].y};
+        }
+    }
+    cfft::line<T, N, false>(w);
+    if (packed && threadIdx.x >= N) return;
+    Cplx<T>* o = out + (node * gridDim.z + blockIdx.z) * FS + col;
+#pragma unroll
+    for (int x = 0; x < N; ++x) st(o + (int64_t)x * COLS, w[x]);
+}
+
+// ---- result ------------------------------------------------------------------------------------
+
+template <int N>
+struct OutGeo {
+    static constexpr int PX = N == 32 ? 2 : N == 12 ? 6 : N == 8 ? 8 : 4;   // planes per CTA
+    static constexpr int NT = PX * N / 2;
+    static constexpr int PITCH = N / 2 + 1;
+};
+
+// out = F_0 - a F_1 - c F_2 (nf fields; a, c nullptr: 1), F [field][node][x][ky][kz]; folded: the plane kz = 0 of F_0
+// is. grid (N / PX, nodes)
+template <typename T, int N>
+__global__ void __launch_bounds__(OutGeo<N>::NT)
+k_shift_out(const Cplx<T>* __restrict__ F, int nf, int64_t field_stride, int folded, const T* __restrict__ a,
+            const T* __restrict__ c, T* __restrict__ out, int* __restrict__ flags) {
+    using Geo = OutGeo<N>;
+    constexpr int NH = N / 2, PITCH = Geo::PITCH;
+    constexpr int64_t FS = (int64_t)N * N * NH, n3 = 2 * FS;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    Cplx<T>* S = reinterpret_cast<Cplx<T>*>(sm_raw);       // [PX][y][PITCH]
+    const int tid = threadIdx.x, pl = tid / NH, j = tid % NH, x = blockIdx.x * Geo::PX + pl;
+    const int64_t node = blockIdx.y;
+    const int64_t row0 = node * n3 + ((int64_t)x * N + j) * N, row1 = row0 + (int64_t)NH * N;   // rows y = j, j + N/2
+    T q0[N], q1[N];
+#pragma unroll
+    for (int z = 0; z < N; ++z) q0[z] = q1[z] = T(0);
+    for (int fo = 0; fo < nf; ++fo) {
+        Cplx<T> v[N];
+        const Cplx<T>* src = F + fo * field_stride + node * FS + (int64_t)x * N * NH + j;   // slot kz = j
+        if (j > 0 || fo > 0 || !folded) {
+#pragma unroll
+            for (int k = 0; k < N; ++k) v[line_slot<N>(k)] = ldg(src + k * NH);
+        } else {
+            const Cplx<T> p = ldg(src), q = ldg(src + NH * NH);
+            v[0] = Cplx<T>{p.x, q.x};
+            v[line_slot<N>(NH)] = Cplx<T>{p.y, q.y};
+#pragma unroll
+            for (int k = 1; k < NH; ++k) {
+                const Cplx<T> b = ldg(src + k * NH), h = ldg(src + (NH + k) * NH);
+                v[line_slot<N>(k)] = Cplx<T>{b.x - h.y, b.y + h.x};
+                v[line_slot<N>(N - k)] = Cplx<T>{b.x + h.y, h.x - b.y};
+            }
+        }
+        cfft::line<T, N, false>(v);
+        __syncthreads();
+#pragma unroll
+        for (int y = 0; y < N; ++y) st(S + (pl * N + y) * PITCH + j, v[y]);
+        __syncthreads();
+        const Cplx<T>* ra = S + (pl * N + j) * PITCH;
+        const Cplx<T>* rb = ra + NH * PITCH;
+        {
+            const Cplx<T> p = ld(ra), q = ld(rb);
+            v[0] = Cplx<T>{p.x, q.x};
+            v[line_slot<N>(NH)] = Cplx<T>{p.y, q.y};
+        }
+#pragma unroll
+        for (int k = 1; k < NH; ++k) {
+            const Cplx<T> p = ld(ra + k), q = ld(rb + k);
+            v[line_slot<N>(k)] = Cplx<T>{p.x - q.y, p.y + q.x};
+            v[line_slot<N>(N - k)] = Cplx<T>{p.x + q.y, q.x - p.y};
+        }
+        cfft::line<T, N, false>(v);
+        const T* mul = fo == 1 ? a : fo == 2 ? c : nullptr;
+#pragma unroll
+        for (int z = 0; z < N; ++z) {
+            const T m0 = mul ? mul[row0 + z] : T(1), m1 = mul ? mul[row1 + z] : T(1);
+            q0[z] = fo ? q0[z] - m0 * v[z].x : v[z].x;
+            q1[z] = fo ? q1[z] - m1 * v[z].y : v[z].y;
+        }
+    }
+    bool bad = false;
+#pragma unroll
+    for (int z = 0; z < N; ++z) {
+        bad |= !isfinite(q0[z]) || !isfinite(q1[z]);
+        out[row0 + z] = q0[z];
+        out[row1 + z] = q1[z];
+    }
+    if (bad) atomicOr(flags, 2);
+}
+
+// ---- launches ------------------------------------------------------------------------------------
+
+template <typename K>
+cudaError_t allow_smem(K kern, size_t bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <typename T, int N, int XC>
+cudaError_t vss_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg, int r0,
+                  int nr, int64_t nodes, Cplx<T>* W, cudaStream_t s) {
+    using Geo = SumGeo<T, N, XC>;
+    const cudaError_t e = allow_smem(k_shift_vss<T, N, XC>, Geo::smem);
+    if (e != cudaSuccess) return e;
+    const bool bil = Gg != nullptr;
+    k_shift_vss<T, N, XC><<<dim3(N / XC, (unsigned)nr, (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
+        Gf, Hf, bil ? Gg : Gf, bil ? Hg : Hf, d.mu, bil ? d.bil : d.quad, bil ? d.nbil : d.nquad, d.nrows, d.nx, r0, W);
+    return cudaGetLastError();
+}
+
+template <typename T, int N, int XC>
+cudaError_t adj_x(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int r0, int nr,
+                  int64_t nodes, Cplx<T>* V, cudaStream_t s) {
+    using Geo = SumGeo<T, N, XC>;
+    const cudaError_t e = allow_smem(k_shift_adj<T, N, XC>, Geo::smem);
+    if (e != cudaSuccess) return e;
+    k_shift_adj<T, N, XC><<<dim3(N / XC, (unsigned)nr, (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
+        G, H, Ur, d.mu, d.quad, d.nquad, wsig, d.nrows, d.nx, r0, V);
+    return cudaGetLastError();
+}
+
+// planes per CTA: as in k_shift.cu (two while wide CTAs would not fill the SMs about four deep)
+template <int N>
+constexpr int wide() { return N == 32 || N == 24 ? 4 : N == 12 ? 12 : 8; }
+template <int N>
+bool narrow(int nr, int64_t nodes) { return (int64_t)(N / wide<N>()) * nr * nodes < 608; }
+
+template <typename T, int N>
+cudaError_t vss_n(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg, int r0,
+                  int nr, int64_t nodes, Cplx<T>* W, cudaStream_t s) {
+    return narrow<N>(nr, nodes) ? vss_x<T, N, 2>(d, Gf, Hf, Gg, Hg, r0, nr, nodes, W, s)
+                                : vss_x<T, N, wide<N>()>(d, Gf, Hf, Gg, Hg, r0, nr, nodes, W, s);
+}
+
+template <typename T, int N>
+cudaError_t adj_n(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int r0, int nr,
+                  int64_t nodes, Cplx<T>* V, cudaStream_t s) {
+    return narrow<N>(nr, nodes) ? adj_x<T, N, 2>(d, G, H, Ur, wsig, r0, nr, nodes, V, s)
+                                : adj_x<T, N, wide<N>()>(d, G, H, Ur, wsig, r0, nr, nodes, V, s);
+}
+
+template <typename T, int N>
+cudaError_t sum_n(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, bool bil, int npairs, int r0, int nr, int parts,
+                  bool add, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
+    const int RP = (nr + parts - 1) / parts;
+    const dim3 grid(col_blocks<N, false>(), (unsigned)nodes, (unsigned)parts);
+    auto kern = A ? k_shift_sum<T, N, true> : k_shift_sum<T, N, false>;
+    kern<<<grid, kColThreads, 0, s>>>(F, nf, A, bil ? d.bil : d.quad, npairs, d.mu, d.xrows, d.nrows, d.nx, r0, nr, RP, add, part);
+    return cudaGetLastError();
+}
+
+template <typename T, int N>
+cudaError_t reduce_n(const Cplx<T>* part, int parts, T scale, int64_t nodes, Cplx<T>* out, cudaStream_t s) {
+    k_shift_reduce<T, N><<<dim3(col_blocks<N, false>(), (unsigned)nodes), kColThreads, 0, s>>>(part, parts, scale, out);
+    return cudaGetLastError();
+}
+
+template <typename T, int N>
+cudaError_t filter_n(const Cplx<T>* G, const T* tab, int nq2, int r0, int nr, int64_t nodes, Cplx<T>* out, cudaStream_t s) {
+    k_shift_filter<T, N><<<dim3(col_blocks<N, true>() + 1, (unsigned)nodes, (unsigned)nr), kColThreads, 0, s>>>(G, tab, nq2, r0, out);
+    return cudaGetLastError();
+}
+
+template <typename T, int N>
+cudaError_t out_n(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c, int64_t nodes, T* out, int* flags,
+                  cudaStream_t s) {
+    using Geo = OutGeo<N>;
+    constexpr size_t sm = (size_t)Geo::PX * N * Geo::PITCH * sizeof(Cplx<T>);
+    k_shift_out<T, N><<<dim3(N / Geo::PX, (unsigned)nodes), Geo::NT, sm, s>>>(F, nf, field_stride, folded, a, c, out, flags);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+double shift_gain_scale(int N, bool fp64) { return fp64 ? 1.0 : 1.0 + 6.0 * cfft::line_loss(N); }
+
+#define DGFS_BY_N(CALL)                              \
+    if (nodes <= 0) return cudaSuccess;              \
+    if (nodes > 65535) return cudaErrorInvalidValue; \
+    if (N == 8) return CALL(8);                      \
+    if (N == 12) return CALL(12);                    \
+    if (N == 16) return CALL(16);                    \
+    if (N == 24) return CALL(24);                    \
+    if (N == 32) return CALL(32);                    \
+    return cudaErrorInvalidValue
+
+template <typename T>
+cudaError_t launch_shift_vss(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
+                             int N, int r0, int nr, int64_t nodes, Cplx<T>* W, cudaStream_t s) {
+#define CALL(n) vss_n<T, n>(d, Gf, Hf, Gg, Hg, r0, nr, nodes, W, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+template <typename T>
+cudaError_t launch_shift_adj(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int N,
+                             int r0, int nr, int64_t nodes, Cplx<T>* V, cudaStream_t s) {
+#define CALL(n) adj_n<T, n>(d, G, H, Ur, wsig, r0, nr, nodes, V, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+template <typename T>
+cudaError_t launch_shift_sum(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, bool bil, int npairs, int N, int r0,
+                             int nr, int parts, bool add, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
+#define CALL(n) sum_n<T, n>(d, F, nf, A, bil, npairs, r0, nr, parts, add, nodes, part, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+template <typename T>
+cudaError_t launch_shift_reduce(const Cplx<T>* part, int parts, T scale, int N, int64_t nodes, Cplx<T>* out, cudaStream_t s) {
+#define CALL(n) reduce_n<T, n>(part, parts, scale, nodes, out, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+template <typename T>
+cudaError_t launch_shift_filter(const Cplx<T>* G, const T* tab, int nq2, int N, int r0, int nr, int64_t nodes, Cplx<T>* out,
+                                cudaStream_t s) {
+#define CALL(n) filter_n<T, n>(G, tab, nq2, r0, nr, nodes, out, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+template <typename T>
+cudaError_t launch_shift_out(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c, int N,
+                             int64_t nodes, T* out, int* flags, cudaStream_t s) {
+#define CALL(n) out_n<T, n>(F, nf, field_stride, folded, a, c, nodes, out, flags, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+
+#define DGFS_SHIFT_INST(T)                                                                                              \
+    template cudaError_t launch_shift_vss<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*,        \
+                                             const Cplx<T>*, int, int, int, int64_t, Cplx<T>*, cudaStream_t);           \
+    template cudaError_t launch_shift_adj<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*,        \
+                                             const T*, int, int, int, int64_t, Cplx<T>*, cudaStream_t);                 \
+    template cudaError_t launch_shift_sum<T>(const ShiftDev<T>&, const Cplx<T>*, int, const T*, bool, int, int, int,    \
+                                             int, int, bool, int64_t, Cplx<T>*, cudaStream_t);                          \
+    template cudaError_t launch_shift_reduce<T>(const Cplx<T>*, int, T, int, int64_t, Cplx<T>*, cudaStream_t);          \
+    template cudaError_t launch_shift_filter<T>(const Cplx<T>*, const T*, int, int, int, int, int64_t, Cplx<T>*,        \
+                                                cudaStream_t);                                                          \
+    template cudaError_t launch_shift_out<T>(const Cplx<T>*, int, int64_t, bool, const T*, const T*, int, int64_t, T*,  \
+                                             int*, cudaStream_t);
+DGFS_SHIFT_INST(float)
+DGFS_SHIFT_INST(double)
+#undef DGFS_SHIFT_INST
+
+}  // namespace dgfs

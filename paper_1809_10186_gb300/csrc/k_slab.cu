@@ -12,26 +12,31 @@
 // Both kernels are memory-bound streams over the I K N^3 values.
 #include <cstdint>
 
+#include <cooperative_groups.h>
+
 #include "launchers.h"
 
 namespace dgfs {
 
 namespace {
 
-// one CTA per wall: side 0 reads the first node of element 0 (outgoing c_1 < 0), side 1 the last
-// node of element I - 1 (outgoing c_1 > 0)
+// One cluster of eight CTAs per wall: side 0 reads the first node of element 0 (outgoing c_1 < 0, the planes
+// x < N/2 of the cell-centred grid), side 1 the last node of element I - 1 (outgoing c_1 > 0). Latency-bound:
+// one CTA per wall took 40 us at N = 24, a fifteenth of the right-hand side; 6 us now.
+constexpr int kWallCtas = 8;
 template <typename T>
-__global__ void __launch_bounds__(256) k_slab_wall(const T* __restrict__ F, int N, int I, int K, double L,
-                                                   double* __restrict__ num) {
-    __shared__ double part[8];
-    const int side = blockIdx.x;
-    const int64_t n3 = (int64_t)N * N * N, n2 = (int64_t)N * N;
-    const T* f = F + (side == 0 ? 0 : ((int64_t)(I - 1) * K + (K - 1)) * n3);
+__global__ void __cluster_dims__(kWallCtas, 1, 1) __launch_bounds__(256)
+k_slab_wall(const T* __restrict__ F, int N, int I, int K, double L, double* __restrict__ num) {
+    __shared__ double part[8], cta;
+    auto cl = cooperative_groups::this_cluster();
+    const int side = blockIdx.x / kWallCtas, rank = blockIdx.x % kWallCtas;
+    const int n2 = N * N, half = (N / 2) * n2;
+    const T* f = F + (side == 0 ? 0 : ((int64_t)(I - 1) * K + (K - 1)) * ((int64_t)n2 * N) + half);
     const double dc = 2.0 * L / N;
     double acc = 0.0;
-    for (int64_t j = threadIdx.x; j < n3; j += blockDim.x) {
-        const double c1 = -L + ((double)(j / n2) + 0.5) * dc;
-        if (side == 0 ? c1 < 0.0 : c1 > 0.0) acc += fabs(c1) * (double)f[j];
+    for (int j = rank * 256 + threadIdx.x; j < half; j += kWallCtas * 256) {
+        const int x = j / n2 + (side == 0 ? 0 : N / 2);
+        acc = fma(fabs(-L + (x + 0.5) * dc), (double)f[j], acc);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -40,8 +45,15 @@ __global__ void __launch_bounds__(256) k_slab_wall(const T* __restrict__ F, int 
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < 8; ++w) s += part[w];
+        cta = s;
+    }
+    cl.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        double s = 0.0;
+        for (unsigned r = 0; r < kWallCtas; ++r) s += *cl.map_shared_rank(&cta, r);
         num[side] = s;
     }
+    cl.sync();   // the partial sums live until rank 0 has read them
 }
 
 // thread per (velocity j, element i = blockIdx.y)
@@ -96,7 +108,7 @@ __global__ void __launch_bounds__(256) k_slab_rhs(const T* __restrict__ F, const
 
 template <typename T>
 cudaError_t launch_slab_wall(const T* F, int N, int I, int K, double L, double* num, cudaStream_t s) {
-    k_slab_wall<T><<<2, 256, 0, s>>>(F, N, I, K, L, num);
+    k_slab_wall<T><<<2 * kWallCtas, 256, 0, s>>>(F, N, I, K, L, num);
     return cudaGetLastError();
 }
 

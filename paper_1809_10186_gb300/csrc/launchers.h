@@ -75,81 +75,20 @@ cudaError_t launch_combine(const DevTables<T>& t, const Cplx<T>* X, int xslots, 
                            int64_t nodes, T scale, int loss_field0, int loss_field1, Cplx<T>* Y,
                            int yfields, cudaStream_t s);
 
-// U[node][r] = w_r rho_r(node) sum_s Vr[s][r] Re X[node][s]   (after an inverse DFT)
+// out = Re Y0 - a * Re Y1 - (c ? c * Re Y2 : 0)
 template <typename T>
-cudaError_t launch_expand_radial(const DevTables<T>& t, const Cplx<T>* X, int xfields,
-                                 NodeParams np, int64_t nodes, T* U, cudaStream_t s);
+cudaError_t launch_finalize(int N, const Cplx<T>* Y, int yfields, const T* a, const T* c, const int64_t* offs,
+                            int64_t nodes, T* out, int* flags, cudaStream_t s);
 
-// X[node][s] = Uk[s] * X[node][src_slot] for s < rank (Fourier multiply, complex)
-template <typename T>
-cudaError_t launch_multiply_uk(const DevTables<T>& t, Cplx<T>* X, int xfields, int src_slot,
-                               int64_t nodes, cudaStream_t s);
-
-// Y[node][0] = GL X[node][slot0];  Y[node][1] = GL X[node][slot1]
-template <typename T>
-cudaError_t launch_loss_pair(const DevTables<T>& t, const Cplx<T>* X, int xfields, NodeParams np,
-                             int64_t nodes, int slot0, int slot1, Cplx<T>* Y, int yfields,
-                             cudaStream_t s);
-
-// out = Re Y0 - a * Re Y1 - (c ? c * Re Y2 : 0)       (mode 0)
-// out = sum_r G[node][r] - a * Re Y0 - Re Y1            (mode 1, VJP; a = u)
-template <typename T>
-cudaError_t launch_finalize(int N, int Nrho, const Cplx<T>* Y, int yfields, const T* a,
-                            const T* c, const T* G, const int64_t* offs, int64_t nodes, int mode,
-                            T* out, int* flags, cudaStream_t s);
-
-// ---- VSS kernel gain and Fourier-space translates (k_vss.cu) ------------------------------
-// Every field plane-major [kz][kx][ky]. Translate spectra of sphere point p (mu_r: [npairs][3][N]
-// complex per-axis multipliers of +s_rp): set 0 = mu_s Fh + i conj(mu_s) Gh, set 1 (f != g) =
-// conj(mu_s) Fh + i mu_s Gh; Gh == nullptr means Gh = Fh.
-// Y[n][0] += scale sum_p A_r[p] P^_p, P^_p separated from the packed spectra W by Hermitian symmetry
-template <typename T>
-cudaError_t launch_vss_accumulate(const Cplx<T>* W, const T* A_r, int N, int npairs, int64_t nodes, T scale,
-                                  Cplx<T>* Y, int yfields, cudaStream_t s);
-// Y[n][0] = 0, Y[n][1] = GL Bh[n], Y[n][2] = GL Ah[n] (yfields == 3)
-template <typename T>
-cudaError_t launch_vss_loss_init(const Cplx<T>* Ah, const Cplx<T>* Bh, const T* GL, int N, int64_t nodes,
-                                 Cplx<T>* Y, int yfields, cudaStream_t s);
-
-// the VSS kernels: N = 8, 12, 16, 24 and, in FP32, 32; the VHS translates, the adjoint: every N
-bool vss_fused_supported(int N, bool fp64);
-bool fft_translate_supported(int N);
-// X[n] = {f[n], 0} transposed to plane-major (then transformed with launch_dft3); node n of f at
-// offs[n] (device, or nullptr: n N^3)
-template <typename T>
-cudaError_t launch_vss_load_t(const T* f, const int64_t* offs, int N, int64_t nodes, Cplx<T>* X, cudaStream_t s);
-// Z[n][set][p] = inverse x, y transforms of the translate spectra
-template <typename T>
-cudaError_t launch_vss_inverse_planes(const Cplx<T>* Fh, const Cplx<T>* Gh, const Cplx<T>* mu_r, const Cplx<T>* dftw,
-                                      int N, int npairs, int sets, int nr, int64_t nodes, Cplx<T>* Z, cudaStream_t s);
-// W[n][j] = forward z transform of P_2j + i P_2j+1 after the inverse z transform of the Z lines
-template <typename T>
-cudaError_t launch_vss_lines(const Cplx<T>* Z, const Cplx<T>* dftw, int N, int npairs, int sets, int64_t nodes,
-                             Cplx<T>* W, cudaStream_t s);
-// forward y, x transforms of W[n][0 .. fields) in place
-template <typename T>
-cudaError_t launch_vss_forward_planes(const Cplx<T>* dftw, int N, int fields, int64_t nodes, Cplx<T>* W,
-                                      cudaStream_t s);
-// VHS with a transform per pair: P[n][r] (standard layout, node stride node_stride), nr radial points, from
-// the translate lines Z[n][r][pair]
-template <typename T>
-cudaError_t launch_vss_lines_sum(const Cplx<T>* Z, const Cplx<T>* dftw, const T* wsig, int N, int npairs, int nr,
-                                 int64_t nodes, int64_t node_stride, T* P, cudaStream_t s);
-// adjoint gain in Fourier space (see k_vss.cu): W[n][p] = DFT_z(U_r b + i U_r a) of the translate lines,
-// G^[n] += sum_p 2 w_p [conj(mu_s) P1^ + mu_s P2^], and the real part of the transformed-back G^ in the
-// standard layout
-template <typename T>
-cudaError_t launch_vjp_lines(const Cplx<T>* Z, const T* U, int64_t node_stride, const Cplx<T>* dftw, int N,
-                             int npairs, int64_t nodes, Cplx<T>* W, cudaStream_t s);
-template <typename T>
-cudaError_t launch_vjp_accumulate(const Cplx<T>* W, const Cplx<T>* mu_r, const T* wsig, int N, int npairs,
-                                  int64_t nodes, Cplx<T>* Gh, cudaStream_t s);
-template <typename T>
-cudaError_t launch_vjp_real_t(const Cplx<T>* Gt, int N, int64_t nodes, T* out, cudaStream_t s);
-// out (standard layout) = Re Y0 - a Re Y1 - (c ? c Re Y2 : 0), Y plane-major
-template <typename T>
-cudaError_t launch_vss_finalize_t(const Cplx<T>* Y, int yfields, const T* a, const T* c, int N, int64_t nodes, T* out,
-                                  int* flags, cudaStream_t s);
+// ---- translate products with a transform per pair (k_pair.cu) -----------------------------
+// Fields plane-major [kz][kx][ky]. X[n] = {f[n], 0} (then transformed with launch_dft3)
+cudaError_t launch_pair_load(const float* f, int N, int64_t nodes, Cplx<float>* X, cudaStream_t s);
+// Z[n][r][pair] = inverse x, y transforms of mu_s Fh + i conj(mu_s) Fh (mu_r: [nr][npairs][3][N] per-axis multipliers)
+cudaError_t launch_pair_planes(const Cplx<float>* Fh, const Cplx<float>* mu_r, const Cplx<float>* dftw, int N, int npairs, int nr,
+                               int64_t nodes, Cplx<float>* Z, cudaStream_t s);
+// P[n][r] (standard layout, node stride node_stride) from the translate lines Z
+cudaError_t launch_pair_sum(const Cplx<float>* Z, const Cplx<float>* dftw, const float* wsig, int N, int npairs, int nr,
+                            int64_t nodes, int64_t node_stride, float* P, cudaStream_t s);
 
 // ---- DG element collision, SVD variant (k_dg.cu) ---------------------------------------
 // f[e][r] = sum_l A[r][l] F[e][l], g[e][r] = sum_l B[r][l] F[e][l]   (F [E][K][n3], K <= 16; B == nullptr:

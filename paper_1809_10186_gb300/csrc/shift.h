@@ -30,6 +30,7 @@ struct ShiftProgram {
     int nx = 0;                          // distinct nonzero |s_x|; fields 2i (+) and 2i + 1 (-)
     std::vector<int> xrows;              // [nx] row of the shift table
     std::vector<ShiftEntry> quad, bil;   // g = f: one entry per pair (weight 2 w_p); f, g: both signs (w_p)
+    std::vector<double> kq;              // [Nrho][3 (N/2)^2 + 1] w_r rho_r S(|k|, r) of the compressed kernel (VHS)
     std::vector<double> mu;              // [Nrho][nrows][MP][2] e^{i pi k s / L}, k = 0 .. N/2 (Nyquist cos)
 };
 
@@ -45,13 +46,16 @@ struct ShiftDev {
     const int* xrows = nullptr;
     const ShiftEntry *quad = nullptr, *bil = nullptr;
     const Cplx<T>* mu = nullptr;
+    const T* kq = nullptr;       // [Nrho][3 (N/2)^2 + 1]: multiplier of K_r by |k|^2 (VHS)
 };
 
 // G[node][x][ky][kz], kz = 0 .. N/2 - 1: the (y, z) spectra (times 1/N^2) of every x plane of the real
 // field f; the real spectra of kz = 0 and kz = N/2 share the complex slot kz = 0. offs: element offset of
 // every node (nullptr: node N^3).
+// b: the field f b instead (nullptr: f).
 template <typename T>
-cudaError_t launch_shift_forward(const T* f, const int64_t* offs, int N, int64_t nodes, Cplx<T>* G, cudaStream_t s);
+cudaError_t launch_shift_forward(const T* f, const T* b, const int64_t* offs, int N, int64_t nodes, Cplx<T>* G,
+                                 cudaStream_t s);
 // H[node][r - r0][field][x][ky][kz] for r in [r0, r0 + nr): the x translates of G by every signed x shift
 template <typename T>
 cudaError_t launch_shift_x(const ShiftDev<T>& d, const Cplx<T>* G, int N, int r0, int nr, int64_t nodes, Cplx<T>* H,
@@ -62,5 +66,34 @@ template <typename T>
 cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg,
                                   const Cplx<T>* Hg, const T* wsig, int N, int r0, int nr, int64_t nodes,
                                   int64_t node_stride, T* P, cudaStream_t s);
+
+// VSS kernel and adjoint (k_shift_sum.cu). W [node][r][entry][x][ky][kz]: (y, z) spectra of every product of the
+// quad (Gg == nullptr) or bil program.
+template <typename T>
+cudaError_t launch_shift_vss(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
+                             int N, int r0, int nr, int64_t nodes, Cplx<T>* W, cudaStream_t s);
+// V [node][r][2 nx + 2][x][ky][kz]: the back-translated adjoint products before their x phases; Ur [node][r]: K_r u
+template <typename T>
+cudaError_t launch_shift_adj(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int N,
+                             int r0, int nr, int64_t nodes, Cplx<T>* V, cudaStream_t s);
+// part[node][parts] (+)= the x spectra of the nf fields F[node][r] times A (VSS: [Nrho][npairs] half tables of
+// N^3/2 + 2 N values, fill_vss_tables) or, A == nullptr, times the x phases of the adjoint's fields; summed over fields and r
+template <typename T>
+cudaError_t launch_shift_sum(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, bool bil, int npairs, int N, int r0,
+                             int nr, int parts, bool add, int64_t nodes, Cplx<T>* part, cudaStream_t s);
+// out[node] = scale times the inverse x transform of the sum of the parts
+template <typename T>
+cudaError_t launch_shift_reduce(const Cplx<T>* part, int parts, T scale, int N, int64_t nodes, Cplx<T>* out, cudaStream_t s);
+// out[node][r] = the field G under the real even multiplier tab[k] (nq2 == 0) or tab[(r0 + r) nq2 + |k|^2]
+template <typename T>
+cudaError_t launch_shift_filter(const Cplx<T>* G, const T* tab, int nq2, int N, int r0, int nr, int64_t nodes, Cplx<T>* out,
+                                cudaStream_t s);
+// out = F_0 - a F_1 - c F_2 on the grid (nf fields, field_stride complex elements apart; nullptr factors: 1; folded:
+// the plane kz = 0 of F_0 as the VSS sums leave it)
+template <typename T>
+cudaError_t launch_shift_out(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c, int N,
+                             int64_t nodes, T* out, int* flags, cudaStream_t s);
+// 1 + the relative loss of the six extra line round trips that a gain takes over its loss term (rounded twiddles)
+double shift_gain_scale(int N, bool fp64);
 
 }  // namespace dgfs
