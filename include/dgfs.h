@@ -65,7 +65,7 @@ typedef enum {
                              products), FP32 accumulation in tensor memory; FP32 elsewhere. N = 16, 32,
                              and 24 on the 32-point tiles (filters and data zero-padded: the exact
                              24-point result at (32/24)^3 the work of a 24-point tiling).
-                             For every tensor-core precision, Q(f,f), Q(f,g), the JVP and dQ/dgamma
+                             For F16S, BF16S and BF16X3, Q(f,f), Q(f,g), the JVP and dQ/dgamma
                              take their translates on the tensor cores (the bilinear calls by
                              polarisation: the translate-product sum is symmetric in f and g, so
                              P(f,g) = [P(f + a g) - P(f - a g)] / 4a with a = |f|/|g| per node); the
@@ -73,15 +73,18 @@ typedef enum {
                              batch against the FP64 oracle on the N = 32 two-Maxwellian workload):
                              about 8e-4 of ||Q||, 5e-5 of the loss term ||Q-||                       */
     DGFS_PREC_BF16S = 3,  /* as F16S with bf16 operands (no scaling): about 7e-3 of ||Q||           */
-    DGFS_PREC_F16X3 = 4,  /* translates on tcgen05 tensor cores with every data operand AND every
-                             filter split into an fp16 hi part and a lo part times 2^11: three
-                             products per contraction (hi hi, hi lo, lo hi), FP32 accumulation, so
-                             the translates carry about FP32 accuracy (8e-6 of ||Q||, 4e-7 of ||Q-||,
-                             as FP32); the two CTAs of a thread-block cluster share the field of one
-                             (node, radial points) item. FP32 elsewhere. N = 16, 32, and 24 on the
-                             32-point tiles as for F16S                                              */
-    DGFS_PREC_BF16X3 = 5  /* as F16X3 with bf16 hi and lo parts (lo times 2^8), 16 significand
-                             bits: about 2e-5 of ||Q||, within 1e-3 of ||Q|| at every node          */
+    DGFS_PREC_F16X3 = 4,  /* about FP32 accuracy (8e-6 of ||Q||, 4e-7 of ||Q-||). Q(f,f), Q(f,g), the JVP,
+                             ragged batches, the DG and slab calls and the VJP take the FP32 CUDA-core
+                             translates, the faster of the two engines at this accuracy; dgfs_ssprk,
+                             dgfs_collide_dgamma and dgfs_collide_noalloc run on tcgen05 tensor cores
+                             with every data operand AND every filter split into an fp16 hi part and
+                             a lo part times 2^11: three products per contraction (hi hi, hi lo, lo
+                             hi), FP32 accumulation; the two CTAs of a thread-block cluster share the
+                             field of one (node, radial points) item. N = 16, 24 (on the 32-point
+                             tiles) and 32                                                           */
+    DGFS_PREC_BF16X3 = 5  /* F16X3's tensor-core translates with bf16 hi and lo parts (lo times 2^8), 16
+                             significand bits, for every call but the VJP: about 2e-5 of ||Q||,
+                             within 1e-3 of ||Q|| at every node                                      */
 } dgfs_precision;
 
 typedef enum {

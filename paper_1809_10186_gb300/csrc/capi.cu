@@ -609,6 +609,13 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     }
     // gain products: Q(f,f) and dQ/dgamma use (f, f); Q(f,g) uses (f, g); JVP uses (f, v)
     const T* gg = quadratic(op) ? nullptr : g;
+    // F16X3 asks for about FP32 accuracy: its translates run on the CUDA cores' shared-shift kernels, which are
+    // faster than the split-data tensor-core kernel at every size (f16x3 / fp32 translates, whole Q, 600 nodes: N = 16,
+    // M = 26 2.84 / 0.99 ms; N = 24 15.7 / 5.3; N = 32, M = 38 31.2 / 21.1; JVP of 100 nodes, N = 32 10.3 / 6.6) and as
+    // accurate (2e-6 of ||Q|| at N = 32 against 3e-6). The split-data kernel keeps the calls whose rounding is kept, the
+    // allocation-free call and the failure test.
+    const bool tensor = is_tc(p->prec) && std::is_same<T, float>::value &&
+                        (p->prec != DGFS_PREC_F16X3 || keeps_rounding<T>(op) || p->fault != 0);
     // (N = 12, 24: the separate kernels where keeps_rounding holds on to their rounding)
     const bool fused = spectral_supported(t) && !(keeps_rounding<T>(op) && t.N % 3 == 0);
     NvtxRange translate_range("dgfs translate products");
@@ -619,12 +626,12 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
         p->prof_nodes += nodes;
         if (p->prof_timed < (int64_t)p->ev.size() / 2) cudaEventRecord(p->ev[2 * p->prof_timed], s);
     }
-    if (is_tc(p->prec) && std::is_same<T, float>::value && gg == nullptr) {
+    if (tensor && gg == nullptr) {
         e = launch_tc_gain_products(p->tc, p->prec, reinterpret_cast<const float*>(f),
                                     reinterpret_cast<const float*>(gg), offs, nodes,
                                     reinterpret_cast<float*>(P), p->d_flags, s, p->fault);
         p->fault = 0;
-    } else if (is_tc(p->prec) && std::is_same<T, float>::value && offs == nullptr) {
+    } else if (tensor && offs == nullptr) {
         // bilinear calls (Q(f, g), the JVP) on the tensor cores: the translate-product sum is symmetric in
         // (f, g), so P(f, g) = [P(f + a g) - P(f - a g)] / (4 a), two quadratic launches; the operands u and
         // the per-node factors live in the Fourier slots' workspace, which the Fourier stage fills only later
@@ -639,7 +646,7 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
         if (p->prof) p->prof_launches += 2;
     } else if (p->fftx) {
         if constexpr (std::is_same<T, float>::value)
-            e = keeps_rounding<T>(op) ? pair_gain_products(p, f, nodes, P, s) : shift_gain_products<T>(p, f, gg, offs, nodes, P, s);
+            e = keeps_rounding<T>(op) && !is_tc(p->prec) ? pair_gain_products(p, f, nodes, P, s) : shift_gain_products<T>(p, f, gg, offs, nodes, P, s);
         else
             e = shift_gain_products<T>(p, f, gg, offs, nodes, P, s);
     } else {
