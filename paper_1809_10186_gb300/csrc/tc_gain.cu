@@ -74,10 +74,12 @@ struct Geo {
     static constexpr int ZT = 128 / N;            // y values per pass-1/2 tile
     static constexpr int KSTEPS = N / 16;         // K = 16 steps of one contraction
     static constexpr int KG = N / 8;              // core-matrix groups along K
-    static constexpr int TW = T / 2;              // tiles per epilogue warpgroup
     static constexpr int EPI_WARPS = 8;           // epilogue warpgroups 0 and 1 (warp / 4)
     static constexpr int THREADS = 32 * EPI_WARPS + 128;   // + a warpgroup holding the MMA warp
     static constexpr int ISSUER = EPI_WARPS;      // first MMA warp (pass 1); then pass 2, pass 3 of slots 0, 1
+    // tiles in use: N = 24 on the 32-point tiles (PAD) leaves the tiles of y >= 24 (passes 1, 2) and x' >= 24
+    // (pass 3) empty, a quarter of each pass
+    static constexpr int tiles(bool pad) { return pad && N == 32 ? 24 / ZT : T; }
     // pass-1 tiles of the next step that warpgroup 0 turns into pass-2 operands while it waits for
     // the pass-3 operands of the current one (at most the two operand buffers; none when a step
     // has only two tiles)
@@ -208,7 +210,7 @@ __device__ __forceinline__ const unsigned char* item_filters(const unsigned char
     return filt + (size_t)((item % it.rblocks) * it.rpc) * npairs * Geo<N>::F_BLOCK;
 }
 
-template <int N, bool BF>
+template <int N, bool BF, int T>
 __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uint32_t sb, uint32_t tmem,
                                             const unsigned char* filt, int npairs, const Items& it, long long first,
                                             volatile long long* s_item, int* queue, volatile int* abort,
@@ -238,7 +240,7 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
             else ++waited0;
             tc::tc_fence_after();
             const uint32_t f16 = sb16 + (G::S_F + fbuf * G::F_BLOCK) / 16;   // filter block of this step
-            for (int t = 0; t < G::T; ++t) {   // pass 1 of tile t into pass-1 slot t % 2
+            for (int t = 0; t < T; ++t) {   // pass 1 of tile t into pass-1 slot t % 2
                 const int b = t & 1;
                 if (used & (1u << b)) {
                     DGFS_WAITW(&bars.free1[b], (ph_free >> b) & 1u);
@@ -299,13 +301,13 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
 }
 
 // Pass 2 of tile t reads pass-2 operand buffer t % 2 and writes pass-2/3 slot t % 2. Slot b is
-// reused within a step after the pass-2 epilogue drained it (free2, completions 0..2 of the step's
-// four); the step's first use waits for the previous step's last pass-3 drain (free3x).
-template <int N, bool BF>
+// reused within a step after the pass-2 epilogue drained it (free2, all completions of a step but the
+// last); the step's first use waits for the previous step's last pass-3 drain (free3x).
+template <int N, bool BF, int T>
 __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tmem, const Items& it,
                                             const volatile long long* s_item, volatile int* abort) {
     using G = Geo<N>;
-    uint32_t ph_a2 = 0, ph_x = 0;
+    uint32_t ph_a2 = 0, ph_x = 0, drains = 0;   // drains: pass-2 drains of a slot before this step
     constexpr uint32_t id23 = tc::idesc_f16(BF, true, false, 2 * N, 128);
     constexpr uint64_t dF = tc::sdesc_base(G::FB_LBO, G::FB_SBO);
     constexpr uint64_t dA2 = tc::sdesc_base(G::A2_LBO, G::A2_SBO);
@@ -319,7 +321,7 @@ __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tm
             DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((g >> 1) & 1));
             tc::tc_fence_after();
             const uint32_t f16 = sb16 + (G::S_F + fbuf * G::F_BLOCK) / 16;
-            for (int t = 0; t < G::T; ++t) {
+            for (int t = 0; t < T; ++t) {
                 const int b = t & 1, j = t >> 1;   // j-th use of slot b in this step
                 DGFS_WAITW(&bars.a2_full[b], (ph_a2 >> b) & 1u);
                 ph_a2 ^= 1u << b;
@@ -329,7 +331,7 @@ __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tm
                         ph_x ^= 1u << b;
                     }
                 } else {
-                    DGFS_WAITW(&bars.free2[b], (uint32_t)((j - 1) & 1));   // four completions per step
+                    DGFS_WAITW(&bars.free2[b], (drains + j - 1) & 1u);
                 }
                 tc::tc_fence_after();
                 const uint32_t d = tmem + (b ? G::C_S3 : G::C_S2);
@@ -345,6 +347,7 @@ __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tm
                 tc::mma_commit_warp(&bars.full2[b]);
                 tc::mma_commit_warp(&bars.a2_free[b]);
             }
+            drains += T / 2;
             tc::mma_commit_warp(&bars.fdone[fbuf]);
         }
     }
@@ -355,7 +358,7 @@ __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tm
 // its own completion (full3p / full3m) and release (free3p / free3m): the + MMAs of tile k + 1 wait
 // only for the + half of tile k to be read, so they run while the epilogue reads the - half and
 // forms the products. A group's second pair reads the same operands with its own y filters.
-template <int N, bool BF, int b>
+template <int N, bool BF, int T, int b>
 __device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tmem, int npairs, const Items& it,
                                             const volatile long long* s_item, volatile int* abort) {
     using G = Geo<N>;
@@ -385,7 +388,7 @@ __device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tm
                     tc::tc_fence_after();
                 }
                 const uint32_t fy16 = f16 + (i == 1 ? G::OFF_B1 : G::OFF_B3) / 16;
-                for (int k = 0; k < G::TW; ++k) {
+                for (int k = 0; k < T / 2; ++k) {
                     const int u = 2 * k + b;
                     const uint32_t d = tmem + (b ? G::C_S3 : G::C_S2);
                     const uint32_t a16 = sb16 + G::S_A3 / 16 + u * (G::A3_TS / 16);
@@ -437,6 +440,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
     // the nsrc^3 block of P_r is written)
     const int64_t n3s = PAD ? (int64_t)nsrc * nsrc * nsrc : n3;
     constexpr bool padded = PAD;
+    constexpr int T = G::tiles(PAD), TW = T / 2;   // tiles in use, per epilogue warpgroup
     const uint32_t sb = tc::smem_u32(smem);
 
     // filter copies issued and waited per buffer 0 / 1 (used by the MMA warp and the drain)
@@ -493,6 +497,11 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
             copies1 = it.nseq > 1 ? 1 : 0;
         }
         tc::tmem_alloc(&s_tmem, G::TMEM_COLS);
+    } else if (PAD && N == 32 && warp < G::EPI_WARPS) {
+        // pass-3 operand rows k = y >= 24, which no pass-2 tile writes: zero
+        for (uint32_t o = tid * 16; o < G::A3_LBO; o += 32 * G::EPI_WARPS * 16)
+            for (int gs = 0; gs < 2; ++gs) tc::st_shared_v4(sb + G::S_A3 + gs * G::A3_BYTES + 3 * G::A3_LBO + o, 0, 0, 0, 0);
+        tc::fence_proxy_async();
     }
     tc::tc_fence_before();
     __syncthreads();
@@ -503,14 +512,14 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
       tc::setmaxnreg_dec<G::REG_MMA>();   // every warp of the third warpgroup
       // ============================ MMA warps (converged) =====================================
       if (warp == G::ISSUER)
-        mma_p1_loop<N, BF>(bars, smem, sb, tmem, filt, npairs, it, first, s_item, queue, abort, copies0, copies1,
+        mma_p1_loop<N, BF, T>(bars, smem, sb, tmem, filt, npairs, it, first, s_item, queue, abort, copies0, copies1,
                            waited0, waited1, second0, second1);
       else if (warp == G::ISSUER + 1)
-        mma_p2_loop<N, BF>(bars, sb, tmem, it, s_item, abort);
+        mma_p2_loop<N, BF, T>(bars, sb, tmem, it, s_item, abort);
       else if (warp == G::ISSUER + 2)
-        mma_p3_loop<N, BF, 0>(bars, sb, tmem, npairs, it, s_item, abort);
+        mma_p3_loop<N, BF, T, 0>(bars, sb, tmem, npairs, it, s_item, abort);
       else
-        mma_p3_loop<N, BF, 1>(bars, sb, tmem, npairs, it, s_item, abort);
+        mma_p3_loop<N, BF, T, 1>(bars, sb, tmem, npairs, it, s_item, abort);
     } else {
         tc::setmaxnreg_inc<G::REG_EPI>();
         // ============================== epilogue warpgroups ===================================
@@ -527,9 +536,9 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
         const uint32_t a2_row = sb + G::S_A2 + ((uint32_t)(yl * N) >> 3) * G::A2_SBO + (lz >> 3) * G::A2_LBO + (lz & 7) * 16;
         const int mg3 = (lz * N) >> 3;
         uint32_t ph_f = 0, ph_a2free = 0, ph_a3free = 0, ph_f3p = 0, ph_f3m = 0;   // phase bits (bit b = ring slot b)
-        float2 acc[G::TW][N / 2];   // P_r of the warpgroup's pass-3 tiles: (y' = 2j, 2j + 1) per entry
+        float2 acc[TW][N / 2];   // P_r of the warpgroup's pass-3 tiles: (y' = 2j, 2j + 1) per entry
 #pragma unroll
-        for (int k = 0; k < G::TW; ++k)
+        for (int k = 0; k < TW; ++k)
 #pragma unroll
             for (int j = 0; j < N / 2; ++j) acc[k][j] = make_float2(0.f, 0.f);
         // 2^-e, the weight of the lo parts of passes 2 and 3, as a pair for the packed FMAs
@@ -586,12 +595,12 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
           if (ki > 0) DGFS_WAITE(&bars.f_free, (uint32_t)((ki - 1) & 1));
           tc::tc_fence_after();
           {
-              // tiles t = 2k + w, two at a time: both tiles' loads precede the TMEM stores (whose memory
+              // tiles t = 2k + w, two (three) at a time: their loads precede the TMEM stores (whose memory
               // clobber would otherwise keep the next tile's loads behind them)
-              constexpr int TB = G::TW >= 2 ? 2 : 1;
-              static_assert(G::TW % TB == 0, "tile batches");
+              constexpr int TB = TW % 2 == 0 ? 2 : TW;
+              static_assert(TW % TB == 0, "tile batches");
 #pragma unroll 1
-              for (int k0 = 0; k0 < G::TW; k0 += TB) {
+              for (int k0 = 0; k0 < TW; k0 += TB) {
                   uint32_t v[TB][N / 2];
 #pragma unroll
                   for (int bb = 0; bb < TB; ++bb) {
@@ -635,7 +644,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                 // LOOKAHEAD tiles (virtual tiles T, T + 1): their pass-1 MMAs and operand buffers do not
                 // depend on this step's pass 3, so warpgroup 0 fills the wait for the pass-3 operands
                 // with them (a third would wait for the next step's pass 2, i.e. for this step's back)
-                const int tend = G::T + ((pp + cnt < npairs || rr + 1 < it.rpc) ? G::LOOKAHEAD : 0);
+                const int tend = T + ((pp + cnt < npairs || rr + 1 < it.rpc) ? G::LOOKAHEAD : 0);
                 for (int t = ahead; t < tend; ++t) {   // pass-1 tile t (slot t % 2) -> pass-2 operands (buffer t % 2)
                     const int b = t & 1;
                     if (g > 0 || t >= 2) {   // pass 2 of tile t - 2 (of this or the previous step) has read buffer b
@@ -667,9 +676,9 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                     tc::fence_proxy_async();
                     tc::mbar_arrive(&bars.a2_full[b]);
                 }
-                ahead = tend - G::T;
+                ahead = tend - T;
             } else {
-                for (int t = 0; t < G::T; ++t) {   // pass-2 tile t (slot t % 2) -> rows of the pass-3 operands
+                for (int t = 0; t < T; ++t) {   // pass-2 tile t (slot t % 2) -> rows of the pass-3 operands
                     const int b = t & 1, y = t * G::ZT + yl;
                     if (t == 0 && g > 0) {   // the previous step's pass 3 has read the operands
                         DGFS_WAITE(&bars.a3_free, ph_a3free);
@@ -717,7 +726,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
 #pragma unroll 1
             for (int i = 0; i < cnt; ++i) {
 #pragma unroll
-            for (int k = 0; k < G::TW; ++k) {
+            for (int k = 0; k < TW; ++k) {
                 // + half, released before the - half is awaited
                 DGFS_WAITE(&bars.full3p[w], ph_f3p);
                 ph_f3p ^= 1u;
@@ -750,7 +759,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
                     if (c == N / 16 - 1) {
                         tc::tc_fence_before();
                         tc::mbar_arrive(&bars.free3m[w]);
-                        if (k == G::TW - 1 && i == cnt - 1) tc::mbar_arrive(&bars.free3x[w]);
+                        if (k == TW - 1 && i == cnt - 1) tc::mbar_arrive(&bars.free3x[w]);
                     }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
@@ -767,7 +776,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
               float* dst = P + ((size_t)node * Nrho + r0 + rr) * n3s;
               const float sc = out_scale * (coef ? coef[node] : 1.f);   // per-node factor (polarisation)
 #pragma unroll
-              for (int k = 0; k < G::TW; ++k) {
+              for (int k = 0; k < TW; ++k) {
                   const int m3 = (2 * k + w) * 128 + l, xp = m3 / N, zp = m3 % N;
                   if constexpr (!padded) {
                       float* o = dst + (size_t)xp * G::N2 + zp;
@@ -790,7 +799,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
               }
           }
 #pragma unroll
-          for (int k = 0; k < G::TW; ++k)
+          for (int k = 0; k < TW; ++k)
 #pragma unroll
               for (int j = 0; j < N / 2; ++j) acc[k][j] = make_float2(0.f, 0.f);
           }
