@@ -168,10 +168,10 @@ void destroy_io(dgfs_plan_s* p) {
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Bytes of the VSS path per node of its workspace: half-spectrum fields (N^3/2 complex values) for one radial point
-// of a bilinear call (2 operands, 4 npairs x fields at most, 2 npairs products, a partial sum, 3 results).
+// of a bilinear call (2 operands, 4 npairs x fields at most, 2 npairs products, 4 partial sums, 3 results).
 size_t vss_node_bytes(const HostPlan& h, int prec) {
     const size_t n3 = (size_t)h.N * h.N * h.N;
-    return elem_size(prec) * n3 * (6 * (size_t)h.npairs + 8);
+    return elem_size(prec) * n3 * (6 * (size_t)h.npairs + 9);
 }
 
 // Per-node workspace bytes (all operations share one layout). VSS plans use only the staging
@@ -370,8 +370,13 @@ void pack_shift(const ShiftProgram& sp, std::vector<unsigned char>& blob, ShiftD
     d.quad = reinterpret_cast<const ShiftEntry*>(put(sp.quad.data(), sp.quad.size() * sizeof(ShiftEntry)));
     d.bil = reinterpret_cast<const ShiftEntry*>(put(sp.bil.data(), sp.bil.size() * sizeof(ShiftEntry)));
     d.xrows = reinterpret_cast<const int*>(put(sp.xrows.data(), sp.xrows.size() * sizeof(int)));
-    std::vector<T> kq(sp.kq.begin(), sp.kq.end());
-    d.kq = reinterpret_cast<const T*>(put(kq.data(), kq.size() * sizeof(T)));
+    auto put_t = [&](const std::vector<double>& v) {
+        const std::vector<T> t(v.begin(), v.end());
+        return reinterpret_cast<const T*>(put(t.data(), t.size() * sizeof(T)));
+    };
+    d.sq = put_t(sp.sq);
+    d.kq = put_t(sp.kq);
+    d.kqd = put_t(sp.kqd);
 }
 
 template <typename T>
@@ -380,7 +385,7 @@ void rebase_shift(ShiftDev<T>& d, const void* base) {
         using P = std::remove_reference_t<decltype(ptr)>;
         ptr = reinterpret_cast<P>(static_cast<const unsigned char*>(base) + reinterpret_cast<uintptr_t>(ptr));
     };
-    fix(d.mu); fix(d.quad); fix(d.bil); fix(d.xrows); fix(d.kq);
+    fix(d.mu); fix(d.quad); fix(d.bil); fix(d.xrows); fix(d.sq); fix(d.kq); fix(d.kqd);
 }
 
 unsigned char* ws(dgfs_plan_s* p, size_t off) { return static_cast<unsigned char*>(p->d_ws) + off; }
@@ -398,9 +403,11 @@ constexpr bool keeps_rounding(Op op) {
     return std::is_same<T, float>::value && (op == Op::Dgamma || op == Op::Step);
 }
 
-// Parts of the radial sum of k_shift_sum (columns of `nodes` nodes alone are few CTAs), at most `most`.
-int sum_parts(int64_t nodes, int nr, int64_t most) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>({(300 + nodes - 1) / nodes, 8, nr, most}));
+// Parts of the gain's radial sum (k_shift_sum.cu): the groups in blocks of their own while the columns of `nodes` nodes
+// alone are fewer than the SMs and the `room` (fields of partial sums) allows it, else 1; 1 takes 2 nodes fields.
+int gain_parts(int N, int Nrho, int64_t nodes, int64_t room) {
+    const int64_t blocks = nodes * ((N * N / 2 + 127) / 128);
+    return blocks < 152 && sum_groups(Nrho) * nodes <= room ? sum_groups(Nrho) : 1;
 }
 
 // The VSS kernel (alpha != 1): gain^ = scale sum_r sum_p A_rp DFT(products of the translates by +-s_rp), one
@@ -422,21 +429,20 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     const T* a = f;
     const T* b = two ? g : f;
     const T* A = static_cast<const T*>(p->d_vss);
-    const T* GL = A + (size_t)Nr * np * (field + 2 * N);
+    FilterTable<T> loss;
+    loss.tab = A + (size_t)Nr * np * (field + 2 * N);
     const double scale = (two ? 1.0 : 2.0) * (op == Op::Jvp ? 2.0 : 1.0) / (double)n3 * shift_gain_scale(N, sizeof(T) == 8);
     // fields per node (operands, partial sums, results) and per item (x translates, products)
-    const int64_t cap = p->vchunk * (6 * (int64_t)np + 8), item = (int64_t)ops * 2 * d.nx + nprog;
-    int64_t C = std::min<int64_t>({nodes, cap / (ops + 1 + nf + item), 65535});
+    const int64_t cap = p->vchunk * (6 * (int64_t)np + 9), item = (int64_t)ops * 2 * d.nx + nprog;
+    int64_t C = std::min<int64_t>({nodes, cap / (ops + kSumParts + nf + item), 65535});
     const int64_t nbatch = (nodes + C - 1) / C;
     C = (nodes + nbatch - 1) / nbatch;   // equal batches
-    int parts = sum_parts(C, Nr, (cap / C - ops - nf - item));
-    const int R = (int)std::max<int64_t>(1, std::min<int64_t>(Nr, (cap / C - ops - parts - nf) / item));
-    parts = std::min(parts, R);
+    const int R = (int)std::max<int64_t>(1, std::min<int64_t>(Nr, (cap / C - ops - kSumParts - nf) / item));
     Cplx<T>* Gf = reinterpret_cast<Cplx<T>*>(ws(p, p->off_V));
     Cplx<T>* Gg = two ? Gf + C * field : nullptr;
     Cplx<T>* F = Gf + ops * C * field;             // [nf][C] results
-    Cplx<T>* part = F + nf * C * field;            // [C][parts]
-    Cplx<T>* Hf = part + C * parts * field;        // [C][R][2 nx]
+    Cplx<T>* part = F + nf * C * field;            // [C][kSumParts]
+    Cplx<T>* Hf = part + C * kSumParts * field;         // [C][R][2 nx]
     Cplx<T>* Hg = two ? Hf + C * R * 2 * d.nx * field : nullptr;
     Cplx<T>* W = Hf + ops * C * R * 2 * d.nx * field;   // [C][R][nprog]
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
@@ -448,31 +454,111 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
             e = launch_shift_x<T>(d, Gf, N, r0, nr, nn, Hf, s);
             if (!e && two) e = launch_shift_x<T>(d, Gg, N, r0, nr, nn, Hg, s);
             if (!e) e = launch_shift_vss<T>(d, Gf, Hf, Gg, Hg, N, r0, nr, nn, W, s);
-            if (!e) e = launch_shift_sum<T>(d, W, nprog, A, two, np, N, r0, nr, parts, r0 > 0, nn, part, s);
-            if (p->prof) p->prof_launches += (d.nx ? ops : 0) + 3;
+            if (!e) e = launch_shift_sum<T>(d, W, nprog, A, two, np, N, r0, nr, nn, part, s);
+            if (p->prof) p->prof_launches += (d.nx ? ops : 0) + 2;
         }
         if (e) return cuda_fail(e, "VSS gain");
-        e = launch_shift_reduce<T>(part, parts, (T)scale, N, nn, F, s);
-        if (!e) e = launch_shift_filter<T>(two ? Gg : Gf, GL, 0, N, 0, 1, nn, F + C * field, s);
-        if (!e && op == Op::Jvp) e = launch_shift_filter<T>(Gf, GL, 0, N, 0, 1, nn, F + 2 * C * field, s);
-        if (!e) e = launch_shift_out<T>(F, nf, C * field, true, a + n0 * n3, op == Op::Jvp ? b + n0 * n3 : nullptr, N, nn,
-                                        out + n0 * n3, p->d_flags, s);
+        e = launch_shift_finish<T>(part, kSumParts, (T)scale, two ? Gg : Gf, op == Op::Jvp ? Gf : nullptr, loss, N, nn, F, s);
+        if (!e) e = launch_shift_out<T>(F, nf, nn * field, true, a + n0 * n3, op == Op::Jvp ? b + n0 * n3 : nullptr, nullptr, N,
+                                        nn, out + n0 * n3, p->d_flags, s);
         if (e) return cuda_fail(e, "VSS loss and finalisation");
         if (p->prof) {
-            p->prof_launches += ops + 1 + nf;
+            p->prof_launches += ops + 2;
             p->prof_nodes += nn;
         }
     }
     return DGFS_OK;
 }
 
-// P[node][r] = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)] with the translates taken in Fourier space,
-// the x and (x, y) translates that several sphere points share taken once (k_shift.cu). The spectra
-// of a batch of (node, radial point) items live in the xchunk region: every radial point of as many nodes
-// as fit, or (a plan with a small max_batch) as many radial points of one node as fit.
+// The Fourier stage in spectra (k_shift_sum.cu): gain = sum_r K_r P_r from the (y, z) spectra W[nodes][Nrho] of P_r,
+// loss from the operand spectra Gb (and Ga for the JVP), and the result
+//   out = gain - a (K_L b)  [- c (K_L a') for the JVP],   gain scaled by 2 for the JVP.
+// stage_sum takes the radial points [r0, r0 + nr), on top of the earlier ones; stage_finish the rest. Against the
+// projection on the radial kernel's factors and one transform per factor (k_spectral.cu) the P_r are never stored
+// as fields nor the projected fields moved twice; its time does not depend on the rank. The DG term of 16 elements
+// (N = 24): 843 -> 667 us.
+//
+// Which of the two, by the plan alone, so that a node's result does not depend on its batch (whole Q, in spectra / by
+// projection, 1 and 300 nodes, M = 12):
+//   FP32 N = 24, rank 6:   55 /  58 us, 1308 / 1356     rank 16:  55 /  64 us, 1309 / 1547
+//        N = 32, rank 8:   68 /  73 us, 4067 / 4067     rank 16:  68 /  78 us, 4077 / 4275   (5 nodes, rank 8: 130 / 128)
+//   FP64 N = 16, rank 7:  231 / 221 us;  rank 9: 230 / 235;  rank 16: 230 / 257    N = 8, rank 8: 105 / 103
+//        N = 12, rank 9:  179 / 178 us;  rank 12: 179 / 190  N = 32, rank 14: 832 / 815;  rank 32: 832 / 892
+// FP32 N = 8 and 16 keep the projection: the six-point rule's error at N = 16 would grow from 9.7e-6 to 1.1e-5 of ||Q||.
+bool stage_in_spectra(const DevTables<float>& t) { return t.N % 3 == 0 || (t.N == 32 && 2 * t.rank >= t.Nrho); }
+bool stage_in_spectra(const DevTables<double>& t) { return t.N > 8 && 4 * t.rank > 3 * t.Nrho; }
+
 template <typename T>
-cudaError_t shift_gain_products(dgfs_plan_s* p, const T* f, const T* g, const int64_t* offs, int64_t nodes, T* P,
-                                cudaStream_t s) {
+struct StageWork {
+    Cplx<T>* F;        // [3][nodes] results
+    Cplx<T>* part;     // [nodes][parts] partial sums over r
+    T *coef, *GLq;     // per-node kernels: [nodes][Nrho], [nodes][3 (N/2)^2 + 1]
+    int parts;
+};
+
+// Events around the translate products of one launch sequence (dgfs_profile_*).
+struct ProfScope {
+    dgfs_plan_s* p;
+    cudaStream_t s;
+    ProfScope(dgfs_plan_s* plan, cudaStream_t st) : p(plan), s(st) {
+        if (!p->prof) return;
+        p->prof_gain += 1;
+        if (p->prof_timed < (int64_t)p->ev.size() / 2) cudaEventRecord(p->ev[2 * p->prof_timed], s);
+    }
+    void end() {
+        if (!p->prof || p->prof_timed >= (int64_t)p->ev.size() / 2) return;
+        cudaEventRecord(p->ev[2 * p->prof_timed + 1], s);
+        p->prof_timed += 1;
+    }
+};
+
+template <typename T>
+cudaError_t stage_sum(dgfs_plan_s* p, Op op, const Cplx<T>* W, NodeParams np, int r0, int nr, int64_t nodes,
+                      const StageWork<T>& w, cudaStream_t s) {
+    const DevTables<T>& t = tables<T>(p);
+    const ShiftDev<T>& d = shift_dev<T>(p);
+    const bool per_node = np.gamma || np.b;
+    cudaError_t e = cudaSuccess;
+    if (per_node && r0 == 0) e = launch_shift_coef<T>(t, np, nodes, w.coef, w.GLq, s);
+    if (!e)
+        e = launch_shift_gain<T>(d, W, per_node ? d.sq : op == Op::Dgamma ? d.kqd : d.kq, per_node ? w.coef : nullptr, t.Nrho, t.N,
+                                 r0, nr, w.parts, nodes, w.part, s);
+    if (p->prof) p->prof_launches += 1 + (per_node && r0 == 0);
+    return e;
+}
+
+template <typename T>
+cudaError_t stage_finish(dgfs_plan_s* p, Op op, const Cplx<T>* Ga, const Cplx<T>* Gb, NodeParams np, int64_t nodes,
+                         const T* a, const T* c, const int64_t* offs, T* out, const StageWork<T>& w, cudaStream_t s) {
+    const DevTables<T>& t = tables<T>(p);
+    const int64_t n3 = (int64_t)t.N * t.N * t.N, field = n3 / 2;
+    const bool per_node = np.gamma || np.b, jvp = op == Op::Jvp;
+    FilterTable<T> loss;
+    loss.tab = op == Op::Dgamma ? t.GLd : t.GL0;
+    if (per_node && t.Lq) {
+        loss.tab = w.GLq;
+        loss.by_node = 1;
+    } else if (per_node) {
+        loss.Lr = t.Lr;
+        loss.cr = t.cr;
+        loss.np = np;
+        loss.Nrho = t.Nrho;
+    }
+    cudaError_t e = launch_shift_finish<T>(w.part, w.parts, (T)((jvp ? 2.0 : 1.0) / (double)n3), Gb, jvp ? Ga : nullptr, loss, t.N,
+                                           nodes, w.F, s);
+    if (!e) e = launch_shift_out<T>(w.F, jvp ? 3 : 2, nodes * field, true, a, jvp ? c : nullptr, offs, t.N, nodes, out, p->d_flags, s);
+    if (p->prof) p->prof_launches += 2;
+    return e;
+}
+
+// P[node][r] = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)] with the translates taken in Fourier space, the x and
+// (x, y) translates that several sphere points share taken once (k_shift.cu). The spectra of a batch of (node, radial
+// point) items live in the xchunk region: every radial point of as many nodes as fit, or (a plan with a small max_batch)
+// as many radial points of one node as fit. stage_in_spectra: the whole call, the spectra W in place of P, the stage's
+// arrays in X (parts) and Y.
+template <typename T>
+cudaError_t shift_gain_products(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, const int64_t* offs, NodeParams np,
+                          int64_t nodes, cudaStream_t s) {
     const DevTables<T>& t = tables<T>(p);
     const ShiftDev<T>& d = shift_dev<T>(p);
     const int N = t.N, Nr = t.Nrho, ops = g ? 2 : 1;
@@ -491,23 +577,76 @@ cudaError_t shift_gain_products(dgfs_plan_s* p, const T* f, const T* g, const in
     Cplx<T>* Gg = g ? Gf + C * field : nullptr;
     Cplx<T>* Hf = Gf + ops * C * field;
     Cplx<T>* Hg = g ? Hf + C * R * 2 * d.nx * field : nullptr;
+    T* P = reinterpret_cast<T*>(ws(p, p->off_P));
+    const Cplx<T>* W = reinterpret_cast<const Cplx<T>*>(P);
+    const bool folded = stage_in_spectra(t);
+    StageWork<T> w;
+    w.F = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Y));
+    w.coef = reinterpret_cast<T*>(w.F + 3 * C * field);   // Nrho + 3 (N/2)^2 + 1 values per node, below n3
+    w.GLq = w.coef + C * Nr;
+    w.part = reinterpret_cast<Cplx<T>*>(ws(p, p->off_X));
+    w.parts = gain_parts(N, Nr, C, 2 * (int64_t)p->xfields * p->chunk);
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
-        const int64_t nn = std::min<int64_t>(C, nodes - n0);
-        const int64_t fo = offs ? 0 : n0 * n3;
-        cudaError_t e = launch_shift_forward<T>(f + fo, nullptr, offs ? offs + n0 : nullptr, N, nn, Gf, s);
-        if (!e && g) e = launch_shift_forward<T>(g + fo, nullptr, offs ? offs + n0 : nullptr, N, nn, Gg, s);
+        const int64_t nn = std::min<int64_t>(C, nodes - n0), fo = offs ? 0 : n0 * n3;
+        const int64_t* of = offs ? offs + n0 : nullptr;
+        NodeParams npb = np;
+        if (np.gamma) npb.gamma = np.gamma + n0;
+        if (np.b) npb.b = np.b + n0;
+        NvtxRange translate_range("dgfs translate products");
+        ProfScope first(p, s);
+        cudaError_t e = launch_shift_forward<T>(f + fo, nullptr, of, N, nn, Gf, s);
+        if (!e && g) e = launch_shift_forward<T>(g + fo, nullptr, of, N, nn, Gg, s);
         for (int r0 = 0; r0 < Nr && !e; r0 += R) {
             const int nr = std::min(R, Nr - r0);
+            if (r0 > 0) first = ProfScope(p, s);
             e = launch_shift_x<T>(d, Gf, N, r0, nr, nn, Hf, s);
             if (!e && g) e = launch_shift_x<T>(d, Gg, N, r0, nr, nn, Hg, s);
-            if (!e) e = launch_shift_products<T>(d, Gf, Hf, Gg, Hg, t.wsig, N, r0, nr, nn, (int64_t)Nr * n3,
-                                                 P + n0 * Nr * n3, s);
+            if (!e) e = launch_shift_products<T>(d, Gf, Hf, Gg, Hg, t.wsig, N, r0, nr, nn, folded,
+                                                 (folded ? nr : Nr) * n3, folded ? P : P + (n0 * Nr + r0) * n3, s);
+            first.end();
+            if (!e && folded) e = stage_sum<T>(p, op, W, npb, r0, nr, nn, w, s);
             if (p->prof) p->prof_launches += (d.nx ? ops : 0) + 1;
         }
+        translate_range.end();
+        if (!e && folded) e = stage_finish<T>(p, op, Gf, g ? Gg : Gf, npb, nn, f + fo, g ? g + fo : nullptr, of, out + fo, w, s);
         if (e) return e;
         if (p->prof) p->prof_launches += ops;
     }
     return cudaSuccess;
+}
+
+// The same stage from the P_r of a tensor-core plan: their spectra and the partial sums in X (xh half-spectrum fields per
+// node), results, operand spectra and coefficients in Y.
+// It takes one more pass over the P_r than stage_in_spectra does above. In spectra / by projection, 1 and 300 nodes, M = 12:
+//   N = 32, rank 19:  95 / 101 us, 3510 / 3503     rank 20:  95 /  99 us, 3510 / 3837 (k_spec_xz passes twice over the
+//   P_r from 20 factors on)     rank 32: 94 / 107 us, 3499 / 4137;  1200 nodes 13976 / 16516
+//   N = 24, rank 14:  82 /  79 us, 1892 / 1961     rank 18:  81 /  81 us, 1889 / 1998     rank 24: 81 / 86 us, 1890 / 2108
+//   N = 16, rank 16:  46 /  44 us,  446 /  495
+// (2 rank + 4 fields of X hold the spectra and at least two partial sums: Nrho may be above N)
+bool tc_stage_in_spectra(const DevTables<float>& t) {
+    return ((t.N == 32 && t.rank >= 20) || (t.N == 24 && 4 * t.rank >= 3 * t.Nrho)) && 2 * t.rank + 4 >= t.Nrho + 2;
+}
+bool tc_stage_in_spectra(const DevTables<double>&) { return false; }
+
+template <typename T>
+cudaError_t tc_stage(dgfs_plan_s* p, Op op, const T* f, const T* g, const T* P, Cplx<T>* X, int64_t xh, Cplx<T>* Y,
+                     const int64_t* offs, NodeParams np, int64_t nodes, T* out, cudaStream_t s) {
+    const DevTables<T>& t = tables<T>(p);
+    const int64_t field = (int64_t)t.N * t.N * t.N / 2;
+    StageWork<T> w;
+    w.F = Y;
+    Cplx<T>* Ga = Y + (g ? 3 : 2) * nodes * field;
+    Cplx<T>* Gb = Ga + nodes * field;
+    w.coef = reinterpret_cast<T*>(Gb + nodes * field);
+    w.GLq = w.coef + nodes * t.Nrho;
+    w.part = X + nodes * t.Nrho * field;
+    w.parts = gain_parts(t.N, t.Nrho, nodes, (xh - t.Nrho) * nodes);
+    cudaError_t e = launch_shift_folded<T>(P, nodes * t.Nrho, f, offs, t.N, nodes, X, Ga, s);
+    if (!e && g) e = launch_shift_forward<T>(g, nullptr, offs, t.N, nodes, Gb, s);
+    if (!e) e = stage_sum<T>(p, op, X, np, 0, t.Nrho, nodes, w, s);
+    if (!e) e = stage_finish<T>(p, op, Ga, g ? Gb : Ga, np, nodes, f, g, offs, out, w, s);
+    if (p->prof) p->prof_launches += g ? 2 : 1;
+    return e;
 }
 
 // P[node][r] of Q(f, f) with a transform of its own for every sphere pair (k_pair.cu; keeps_rounding above), in
@@ -547,14 +686,15 @@ template <typename T>
 cudaError_t shift_vjp(dgfs_plan_s* p, const T* f, const T* u, T* out, int64_t nodes, cudaStream_t s) {
     const DevTables<T>& t = tables<T>(p);
     const ShiftDev<T>& d = shift_dev<T>(p);
-    const int N = t.N, Nr = t.Nrho, nq2 = 3 * (N / 2) * (N / 2) + 1;
+    const int N = t.N, Nr = t.Nrho;
+    FilterTable<T> loss;
+    loss.tab = t.GL0;
     const int64_t n3 = (int64_t)N * N * N, field = n3 / 2;
     const int64_t cap = p->xchunk * (4 + 4 * (int64_t)t.npairs), item = 4 * (int64_t)d.nx + 3;
     int64_t C = std::min<int64_t>({nodes, cap / item, 65535});
     const int64_t nbatch = (nodes + C - 1) / C;
     C = (nodes + nbatch - 1) / nbatch;   // equal batches
     const int R = (int)std::min<int64_t>(Nr, cap / (C * item));
-    const int parts = sum_parts(C, R, 2 * (int64_t)p->xfields);
     const double scale = shift_gain_scale(N, sizeof(T) == 8) / (double)n3;
     Cplx<T>* G = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Y));   // spectra of f, u and u f
     Cplx<T>* F = G + 3 * C * field;                             // gain, K_L f, K_L(u f)
@@ -571,17 +711,15 @@ cudaError_t shift_vjp(dgfs_plan_s* p, const T* f, const T* u, T* out, int64_t no
         for (int r0 = 0; r0 < Nr && !e; r0 += R) {
             const int nr = std::min(R, Nr - r0);
             e = launch_shift_x<T>(d, G, N, r0, nr, nn, H, s);
-            if (!e) e = launch_shift_filter<T>(G + C * field, d.kq, nq2, N, r0, nr, nn, Ur, s);
+            if (!e) e = launch_shift_filter<T>(d, G + C * field, N, r0, nr, nn, Ur, s);
             if (!e) e = launch_shift_adj<T>(d, G, H, Ur, t.wsig, N, r0, nr, nn, V, s);
-            if (!e) e = launch_shift_sum<T>(d, V, 2 * d.nx + 2, nullptr, false, t.npairs, N, r0, nr, parts, r0 > 0, nn, part, s);
+            if (!e) e = launch_shift_sum<T>(d, V, 2 * d.nx + 2, nullptr, false, t.npairs, N, r0, nr, nn, part, s);
             if (p->prof) p->prof_launches += (d.nx ? 1 : 0) + 3;
         }
-        if (!e) e = launch_shift_reduce<T>(part, parts, (T)scale, N, nn, F, s);
-        if (!e) e = launch_shift_filter<T>(G, t.GL0, 0, N, 0, 1, nn, F + C * field, s);
-        if (!e) e = launch_shift_filter<T>(G + 2 * C * field, t.GL0, 0, N, 0, 1, nn, F + 2 * C * field, s);
-        if (!e) e = launch_shift_out<T>(F, 3, C * field, false, un, nullptr, N, nn, out + n0 * n3, p->d_flags, s);
+        if (!e) e = launch_shift_finish<T>(part, kSumParts, (T)scale, G, G + 2 * C * field, loss, N, nn, F, s);
+        if (!e) e = launch_shift_out<T>(F, 3, nn * field, false, un, nullptr, nullptr, N, nn, out + n0 * n3, p->d_flags, s);
         if (e) return e;
-        if (p->prof) p->prof_launches += 7;
+        if (p->prof) p->prof_launches += 5;
     }
     return cudaSuccess;
 }
@@ -616,49 +754,47 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     // allocation-free call and the failure test.
     const bool tensor = is_tc(p->prec) && std::is_same<T, float>::value &&
                         (p->prec != DGFS_PREC_F16X3 || keeps_rounding<T>(op) || p->fault != 0);
+    if (p->prof) p->prof_nodes += nodes;
+    if (!tensor && !keeps_rounding<T>(op)) {
+        e = shift_gain_products<T>(p, op, f, gg, out, offs, np, nodes, s);
+        if (e) return cuda_fail(e, "translate products");
+        if (stage_in_spectra(t)) return DGFS_OK;
+    } else if constexpr (std::is_same<T, float>::value) {
+        NvtxRange translate_range("dgfs translate products");
+        ProfScope gain(p, s);
+        if (tensor && gg == nullptr) {
+            e = launch_tc_gain_products(p->tc, p->prec, f, nullptr, offs, nodes, P, p->d_flags, s, p->fault);
+            p->fault = 0;
+            if (p->prof) p->prof_launches += 1 + tc_extra_launches(p->prec);
+        } else if (tensor) {
+            // bilinear calls (Q(f, g), the JVP) on the tensor cores: the translate-product sum is symmetric in
+            // (f, g), so P(f, g) = [P(f + a g) - P(f - a g)] / (4 a), two quadratic launches; the operands u and
+            // the per-node factors live in the Fourier slots' workspace, which the Fourier stage fills only later
+            const int64_t n3 = (int64_t)t.N * t.N * t.N;
+            if (offs) return fail(DGFS_ERR_UNSUPPORTED, "bilinear tensor-core calls take no node offsets");
+            float* U = reinterpret_cast<float*>(X);
+            float* coef = U + 2 * nodes * n3;
+            e = launch_polar_prep(f, gg, n3, nodes, U, coef, s);
+            if (!e) e = launch_tc_gain_products(p->tc, p->prec, U, nullptr, nullptr, nodes, P, p->d_flags, s, 0, coef, 0);
+            if (!e)
+                e = launch_tc_gain_products(p->tc, p->prec, U + nodes * n3, nullptr, nullptr, nodes, P, p->d_flags, s, 0,
+                                            coef + nodes, 1);
+            if (p->prof) p->prof_launches += 3;
+        } else {
+            e = pair_gain_products(p, f, nodes, P, s);
+        }
+        if (e) return cuda_fail(e, "translate-product kernel");
+        gain.end();
+    }
+    NvtxRange fourier_range("dgfs Fourier stage");
+    if (tensor && !keeps_rounding<T>(op) && tc_stage_in_spectra(t) && nodes <= 65535) {
+        e = tc_stage<T>(p, op, f, gg, P, X, 2 * (int64_t)xf, Y, offs, np, nodes, out, s);
+        if (e) return cuda_fail(e, "Fourier stage");
+        return DGFS_OK;
+    }
     // (N = 12, 24: the separate kernels where keeps_rounding holds on to their rounding)
     const bool fused = spectral_supported(t) && !(keeps_rounding<T>(op) && t.N % 3 == 0);
-    NvtxRange translate_range("dgfs translate products");
-    if (p->prof) {
-        p->prof_launches += (fused ? 5 : 11 + (op == Op::Jvp ? 1 : 0)) +
-                            tc_extra_launches(p->prec);
-        p->prof_gain += 1;
-        p->prof_nodes += nodes;
-        if (p->prof_timed < (int64_t)p->ev.size() / 2) cudaEventRecord(p->ev[2 * p->prof_timed], s);
-    }
-    if (tensor && gg == nullptr) {
-        e = launch_tc_gain_products(p->tc, p->prec, reinterpret_cast<const float*>(f),
-                                    reinterpret_cast<const float*>(gg), offs, nodes,
-                                    reinterpret_cast<float*>(P), p->d_flags, s, p->fault);
-        p->fault = 0;
-    } else if (tensor && offs == nullptr) {
-        // bilinear calls (Q(f, g), the JVP) on the tensor cores: the translate-product sum is symmetric in
-        // (f, g), so P(f, g) = [P(f + a g) - P(f - a g)] / (4 a), two quadratic launches; the operands u and
-        // the per-node factors live in the Fourier slots' workspace, which the Fourier stage fills only later
-        const int64_t n3 = (int64_t)t.N * t.N * t.N;
-        float* U = reinterpret_cast<float*>(X);
-        float* coef = U + 2 * nodes * n3;
-        e = launch_polar_prep(reinterpret_cast<const float*>(f), reinterpret_cast<const float*>(gg), n3, nodes, U, coef, s);
-        if (!e) e = launch_tc_gain_products(p->tc, p->prec, U, nullptr, nullptr, nodes, reinterpret_cast<float*>(P),
-                                            p->d_flags, s, 0, coef, 0);
-        if (!e) e = launch_tc_gain_products(p->tc, p->prec, U + nodes * n3, nullptr, nullptr, nodes,
-                                            reinterpret_cast<float*>(P), p->d_flags, s, 0, coef + nodes, 1);
-        if (p->prof) p->prof_launches += 2;
-    } else if (p->fftx) {
-        if constexpr (std::is_same<T, float>::value)
-            e = keeps_rounding<T>(op) && !is_tc(p->prec) ? pair_gain_products(p, f, nodes, P, s) : shift_gain_products<T>(p, f, gg, offs, nodes, P, s);
-        else
-            e = shift_gain_products<T>(p, f, gg, offs, nodes, P, s);
-    } else {
-        e = launch_gain_products(t, f, gg, offs, nodes, P, s);
-    }
-    if (e) return cuda_fail(e, "translate-product kernel");
-    translate_range.end();
-    NvtxRange fourier_range("dgfs Fourier stage");
-    if (p->prof && p->prof_timed < (int64_t)p->ev.size() / 2) {
-        cudaEventRecord(p->ev[2 * p->prof_timed + 1], s);
-        p->prof_timed += 1;
-    }
+    if (p->prof) p->prof_launches += fused ? 4 : 10 + (op == Op::Jvp ? 1 : 0);
     // real fields packed two per complex slot: the rank projected fields, then the loss
     // operand(s): Q(f,g) -> field rank = g;  JVP -> field rank = v, field rank + 1 = f
     if (fused) {   // the fused Fourier stage
@@ -2202,6 +2338,11 @@ dgfs_status noalloc_run(dgfs_plan_s* p, const T* f, T* Q, int64_t B, unsigned ch
                                     reinterpret_cast<float*>(P), p->d_flags, s);
     else
         e = launch_gain_products(t, f, nullptr, nullptr, B, P, s);
+    if (!e && is_tc(p->prec) && tc_stage_in_spectra(t)) {   // as in dgfs_collide
+        e = tc_stage<T>(p, Op::Collide, f, nullptr, P, X, 2 * (int64_t)xf, Y, nullptr, np, B, Q, s);
+        if (e) return cuda_fail(e, "dgfs_collide_noalloc");
+        return DGFS_OK;
+    }
     if (!e && spectral_supported(t)) {   // the fused Fourier stage, as in dgfs_collide
         e = launch_spectral<T>(t, P, np, B, f, nullptr, nullptr, T(1), X, Y, f, nullptr, Q, p->d_flags, s);
         if (e) return cuda_fail(e, "dgfs_collide_noalloc");

@@ -11,11 +11,11 @@
 //   k_shift_x         x spectra, then per r and signed s_x: phase, inverse x transform      -> H
 //   k_shift_products  per (node, r, XC planes x): per (s_x, s_y): phase, inverse y transform into
 //                     shared memory; per pair: phase, inverse z transform of one line per thread,
-//                     product summed in registers; P_r written once
+//                     product summed in registers; P_r (or its (y, z) spectra, for a stage in spectra) written once
 //
 // Measured (GB300, FP32, N = 32, M = 38, 256 nodes, whole Q): 8.4 ms, 22.2 ms with a transform of its own
 // per pair (two launches per radial point, 9.5 MB of spectra through DRAM per radial point and node
-// against 2.2 MB here); N = 16, M = 6, FP64, one node: 0.20 ms, 0.97 ms before. k_shift_products takes 73 %
+// against 2.2 MB here); N = 16, M = 6, FP64, one node: 0.18 ms, 0.97 ms before. k_shift_products takes 73 %
 // of the FP32 step: 70 % of the issue slots and 56 % of the FMA pipe (ncu, 40 nodes); k_shift_x 15 %, at
 // 81 % of the DRAM throughput.
 //
@@ -58,7 +58,7 @@ void build_shift_program(const HostPlan& h, ShiftProgram& p) {
     if (!h.aniso) {
         const int nq2 = 3 * (N / 2) * (N / 2) + 1;
         const size_t n3 = (size_t)N * N * N;
-        p.kq.assign((size_t)h.Nrho * nq2, 0.0);
+        for (auto* t : {&p.sq, &p.kq, &p.kqd}) t->assign((size_t)h.Nrho * nq2, 0.0);
         std::vector<int64_t> at_q(nq2, -1);   // a mode of each |k|^2
         auto sk = [N](int q) { return q < N / 2 ? q : q - N; };
         for (size_t i = 0; i < n3; ++i) {
@@ -71,7 +71,9 @@ void build_shift_program(const HostPlan& h, ShiftProgram& p) {
                 if (at_q[q] < 0) continue;
                 double v = 0.0;
                 for (int s = 0; s < h.rank; ++s) v += h.Uk[(size_t)s * n3 + at_q[q]] * h.Vr[(size_t)s * h.Nrho + r];
+                p.sq[(size_t)r * nq2 + q] = v;
                 p.kq[(size_t)r * nq2 + q] = wr * v;
+                p.kqd[(size_t)r * nq2 + q] = std::log(h.cr[r]) * wr * v;
             }
         }
     }
@@ -112,19 +114,23 @@ struct ForwardGeo {
 };
 
 // grid (N / PX, nodes). Lines along z of rows y and y + N/2 as real and imaginary part, separated into
-// half spectra; then lines along y of every slot kz.
+// half spectra; then lines along y of every slot kz. Blocks y >= nodes: the fields P to folded spectra W.
 template <typename T, int N>
 __global__ void __launch_bounds__(ForwardGeo<N>::NT)
-k_shift_forward(const T* __restrict__ f, const T* __restrict__ b, const int64_t* __restrict__ offs, Cplx<T>* __restrict__ G) {
+k_shift_forward(const T* __restrict__ f, const T* __restrict__ b, const int64_t* __restrict__ offs, int nodes,
+                const T* __restrict__ P, Cplx<T>* __restrict__ W, Cplx<T>* __restrict__ G) {
     using Geo = ForwardGeo<N>;
     constexpr int NH = N / 2, PX = Geo::PX, NT = Geo::NT, PITCH = Geo::PITCH;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     T* rows = reinterpret_cast<T*>(sm_raw);                // [PX][N][N + 1], then S overwrites it
     Cplx<T>* S = reinterpret_cast<Cplx<T>*>(sm_raw);       // [PX][N][PITCH]
     const int tid = threadIdx.x, x0 = blockIdx.x * PX, pl = tid / NH, j = tid % NH;
-    const int64_t node = blockIdx.y, n3 = (int64_t)N * N * N;
-    const int64_t base = (offs ? offs[node] : node * n3) + (int64_t)x0 * N * N;
-    for (int e = tid; e < PX * N * N; e += NT) rows[(e / N) * (N + 1) + e % N] = b ? f[base + e] * b[base + e] : f[base + e];
+    const int64_t n3 = (int64_t)N * N * N;
+    const bool folded = (int)blockIdx.y >= nodes;
+    const int64_t node = (int)blockIdx.y - (folded ? nodes : 0);
+    const T* src = folded ? P : f;
+    const int64_t base = (offs && !folded ? offs[node] : node * n3) + (int64_t)x0 * N * N;
+    for (int e = tid; e < PX * N * N; e += NT) rows[(e / N) * (N + 1) + e % N] = b && !folded ? src[base + e] * b[base + e] : src[base + e];
     __syncthreads();
     Cplx<T> v[N];
 #pragma unroll
@@ -147,9 +153,13 @@ k_shift_forward(const T* __restrict__ f, const T* __restrict__ b, const int64_t*
     for (int y = 0; y < N; ++y) v[line_slot<N>(y)] = ld(S + (pl * N + y) * PITCH + j);   // slot kz = j
     cfft::line<T, N, true>(v);
     const T sc = T(1) / (T(N) * T(N));
-    Cplx<T>* g = G + node * (n3 / 2) + (int64_t)(x0 + pl) * N * NH + j;
+    Cplx<T>* g = (folded ? W : G) + node * (n3 / 2) + (int64_t)(x0 + pl) * N * NH + j;
+    if (folded) {
+        store_folded<T, N>(v, j, g);
+    } else {
 #pragma unroll
-    for (int k = 0; k < N; ++k) st(g + k * NH, Cplx<T>{sc * v[k].x, sc * v[k].y});
+        for (int k = 0; k < N; ++k) st(g + k * NH, Cplx<T>{sc * v[k].x, sc * v[k].y});
+    }
 }
 
 // ---- x translates ----------------------------------------------------------------------------
@@ -210,12 +220,11 @@ struct ProductGeo {
 };
 
 // grid (N / XC, nr, nodes); H [node][r][2 nx fields][x][ky][kz], G [node][x][ky][kz]
-template <typename T, int N, int XC>
+template <typename T, int N, int XC, bool FOLD>
 __global__ void __launch_bounds__(ProductGeo<T, N, XC>::NT, ProductGeo<T, N, XC>::MINB)
 k_shift_products(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, const Cplx<T>* __restrict__ Gg,
                  const Cplx<T>* __restrict__ Hg, const Cplx<T>* __restrict__ mu, const ShiftEntry* __restrict__ prog,
-                 int nprog, T wscale, const T* __restrict__ wsig, int nrows, int nx, int r0, int64_t node_stride,
-                 T* __restrict__ P) {
+                 int nprog, T wscale, const T* __restrict__ wsig, int nrows, int nx, int r0, int64_t node_stride, T* __restrict__ P) {
     using Geo = ProductGeo<T, N, XC>;
     constexpr int NH = N / 2, PITCH = Geo::PITCH, NT = Geo::NT, MP = shift_mu_pitch(N);
     constexpr int64_t FS = (int64_t)N * N * NH, n3 = (int64_t)N * N * N;
@@ -265,21 +274,48 @@ k_shift_products(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf,
 #pragma unroll
         for (int z = 0; z < N; ++z) acc[z] = fma(acc[z], corr, acc[z]);
     }
-    // P_r of the planes x0 .. x0 + XC - 1 through shared memory (coalesced)
     T* tile = reinterpret_cast<T*>(sm_raw);                  // [NT][N + 1]
     __syncthreads();
 #pragma unroll
     for (int z = 0; z < N; ++z) tile[tid * (N + 1) + z] = acc[z];
     __syncthreads();
-    T* out = P + node * node_stride + (int64_t)(r0 + rl) * n3 + (int64_t)x0 * N * N;
-    for (int e = tid; e < NT * N; e += NT) out[e] = tile[(e / N) * (N + 1) + e % N];
+    T* out = P + node * node_stride + rl * n3 + (int64_t)x0 * N * N;
+    if constexpr (!FOLD) {   // P_r of the planes x0 .. x0 + XC - 1 (coalesced)
+        for (int e = tid; e < NT * N; e += NT) out[e] = tile[(e / N) * (N + 1) + e % N];
+        return;
+    }
+    // the (y, z) spectra of P_r, what the radial sum takes (k_shift_sum.cu): forward z of two rows (y, y + N/2) at a
+    // time, forward y; half of the threads, 2 % of the kernel
+    const int hpl = tid / NH, hj = tid % NH;
+    const bool half = tid < NT / 2;
+    if (half) {
+        const T* ra = tile + (hpl * N + hj) * (N + 1);
+        const T* rb = ra + NH * (N + 1);
+#pragma unroll
+        for (int z = 0; z < N; ++z) v[line_slot<N>(z)] = Cplx<T>{ra[z], rb[z]};
+        cfft::line<T, N, true>(v);
+    }
+    __syncthreads();
+    if (half)
+        split_line<T, N>(v, [&](int k, Cplx<T> a, Cplx<T> b) {
+            st(Y + (hpl * N + hj) * PITCH + k, a);
+            st(Y + (hpl * N + hj + NH) * PITCH + k, b);
+        });
+    __syncthreads();
+    if (half) {
+#pragma unroll
+        for (int y = 0; y < N; ++y) v[line_slot<N>(y)] = ld(Y + (hpl * N + y) * PITCH + hj);
+        cfft::line<T, N, true>(v);
+        store_folded<T, N>(v, hj, reinterpret_cast<Cplx<T>*>(out) + hpl * N * NH + hj);
+    }
 }
 
 template <typename T, int N>
-cudaError_t forward_n(const T* f, const T* b, const int64_t* offs, int64_t nodes, Cplx<T>* G, cudaStream_t s) {
+cudaError_t forward_n(const T* f, const T* b, const int64_t* offs, int64_t nodes, const T* P, int64_t fields, Cplx<T>* W, Cplx<T>* G,
+                      cudaStream_t s) {
     using Geo = ForwardGeo<N>;
     constexpr size_t sm = (size_t)Geo::PX * N * Geo::PITCH * sizeof(Cplx<T>);
-    k_shift_forward<T, N><<<dim3(N / Geo::PX, (unsigned)nodes), Geo::NT, sm, s>>>(f, b, offs, G);
+    k_shift_forward<T, N><<<dim3(N / Geo::PX, (unsigned)(nodes + fields)), Geo::NT, sm, s>>>(f, b, offs, (int)nodes, P, W, G);
     return cudaGetLastError();
 }
 
@@ -301,11 +337,11 @@ cudaError_t shift_x_n(const ShiftDev<T>& d, const Cplx<T>* G, int r0, int nr, in
     return cudaGetLastError();
 }
 
-template <typename T, int N, int XC>
+template <typename T, int N, int XC, bool FOLD>
 cudaError_t products_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
                        const T* wsig, int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
     using Geo = ProductGeo<T, N, XC>;
-    auto kern = k_shift_products<T, N, XC>;
+    auto kern = k_shift_products<T, N, XC, FOLD>;
     if (Geo::smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo::smem);
         if (e != cudaSuccess) return e;
@@ -317,14 +353,14 @@ cudaError_t products_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* H
     return cudaGetLastError();
 }
 
-template <typename T, int N>
+template <typename T, int N, bool FOLD>
 cudaError_t products_n(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
                        const T* wsig, int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
     constexpr int XC = N == 32 || N == 24 ? 4 : N == 12 ? 12 : 8;
     // two planes per CTA while whole CTAs of XC planes would not fill the 152 SMs about four deep
     if ((int64_t)(N / XC) * nr * nodes < 608)
-        return products_x<T, N, 2>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
-    return products_x<T, N, XC>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
+        return products_x<T, N, 2, FOLD>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
+    return products_x<T, N, XC, FOLD>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
 }
 
 }  // namespace
@@ -342,9 +378,28 @@ cudaError_t products_n(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* H
 template <typename T>
 cudaError_t launch_shift_forward(const T* f, const T* b, const int64_t* offs, int N, int64_t nodes, Cplx<T>* G,
                                  cudaStream_t s) {
-#define CALL(n) forward_n<T, n>(f, b, offs, nodes, G, s)
+#define CALL(n) forward_n<T, n>(f, b, offs, nodes, nullptr, 0, nullptr, G, s)
     DGFS_BY_N(CALL);
 #undef CALL
+}
+
+template <typename T>
+cudaError_t launch_shift_folded(const T* P, int64_t fields, const T* f, const int64_t* offs, int N, int64_t nodes, Cplx<T>* W,
+                                Cplx<T>* G, cudaStream_t s) {
+    const int64_t n3 = (int64_t)N * N * N;
+    int64_t f0 = 0;
+    auto part = [&](int64_t lead, int64_t n) {
+#define CALL(k) forward_n<T, k>(f, nullptr, offs, lead, P + f0 * n3, n, W + f0 * (n3 / 2), G, s)
+        DGFS_BY_N(CALL);
+#undef CALL
+    };
+    for (int64_t lead = nodes; f0 < fields; lead = 0) {   // grid.y limit
+        const int64_t n = std::min<int64_t>(65535 - lead, fields - f0);
+        const cudaError_t e = part(lead, n);
+        if (e != cudaSuccess) return e;
+        f0 += n;
+    }
+    return cudaSuccess;
 }
 
 template <typename T>
@@ -357,9 +412,9 @@ cudaError_t launch_shift_x(const ShiftDev<T>& d, const Cplx<T>* G, int N, int r0
 
 template <typename T>
 cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg,
-                                  const Cplx<T>* Hg, const T* wsig, int N, int r0, int nr, int64_t nodes,
+                                  const Cplx<T>* Hg, const T* wsig, int N, int r0, int nr, int64_t nodes, bool folded,
                                   int64_t node_stride, T* P, cudaStream_t s) {
-#define CALL(n) products_n<T, n>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s)
+#define CALL(n) (folded ? products_n<T, n, true> : products_n<T, n, false>)(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s)
     DGFS_BY_N(CALL);
 #undef CALL
 }
@@ -367,11 +422,13 @@ cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const
 #define DGFS_SHIFT_INST(T)                                                                                            \
     template cudaError_t launch_shift_forward<T>(const T*, const T*, const int64_t*, int, int64_t, Cplx<T>*,               \
                                                  cudaStream_t);                                                       \
+    template cudaError_t launch_shift_folded<T>(const T*, int64_t, const T*, const int64_t*, int, int64_t, Cplx<T>*,   \
+                                                Cplx<T>*, cudaStream_t);                                              \
     template cudaError_t launch_shift_x<T>(const ShiftDev<T>&, const Cplx<T>*, int, int, int, int64_t, Cplx<T>*,      \
                                            cudaStream_t);                                                             \
     template cudaError_t launch_shift_products<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*, \
-                                                  const Cplx<T>*, const T*, int, int, int, int64_t, int64_t, T*,      \
-                                                  cudaStream_t);
+                                                  const Cplx<T>*, const T*, int, int, int, int64_t, bool, int64_t,    \
+                                                  T*, cudaStream_t);
 DGFS_SHIFT_INST(float)
 DGFS_SHIFT_INST(double)
 #undef DGFS_SHIFT_INST

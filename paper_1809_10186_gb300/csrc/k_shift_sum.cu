@@ -2,20 +2,24 @@
 //
 //   VSS kernel (alpha != 1): gain^ = sum_r sum_p A_rp(k) DFT[(T_s f)(T_-s g) + (T_-s f)(T_s g)]_k
 //   adjoint (VJP):  gain = sum_r sum_p 2 w_p [T_-s(U_r T_-s f) + T_s(U_r T_s f)],  U_r = K_r u
+//   VHS gain of the Fourier stage in spectra (capi.cu stage_in_spectra):  gain^ = sum_r K_r(k) DFT[P_r]_k
 //
 //   k_shift_vss     per (node, r, XC planes x): the product lines of two sphere points share one forward z
 //                   transform (real and imaginary part, separated per line into half spectra), forward y  -> W
 //   k_shift_adj     the same for U_r T_-s f and U_r T_s f; the back-translates are phases, so what shares
 //                   (s_x, s_y) is summed after the z phases, what shares s_x after the y phases         -> V
-//   k_shift_sum     per (ky, kz) column: forward x of every field of W (V), times A_rp (the x phase), summed
-//                   over fields and a part of the radial points in registers                -> partial spectra
-//   k_shift_reduce  sum of the parts, inverse x
-//   k_shift_filter  a real multiplier on a field: forward x, multiplier, inverse x (K_L f, and K_r u)
+//   k_shift_sum     per (ky, kz) column: forward x of every field of W (V), times A_rp (the x phase, K_r), summed
+//                   over a part of the fields (VHS: of the radial points) in registers      -> partial spectra
+//   k_shift_filter  K_r u: forward x, multiplier, inverse x
+//   k_shift_finish  sum of the parts, inverse x; K_L f as k_shift_filter, in blocks of the same launch
 //   k_shift_out     inverse y and z of the gain and the loss fields, the result
 //
 // Measured (GB300, FP32, N = 32, M = 38): VSS Q of 40 nodes 3.1 ms (6.5 ms with a three-axis transform of its own for
 // every translate and product), VJP of 48 nodes 4.2 ms (11 ms); k_shift_vss 57 % and k_shift_adj 80 % of them, both
-// bound by instruction issue at 8-12 warps per SM (a line and its sums fill the registers).
+// bound by instruction issue at 8-12 warps per SM (a line and its sums fill the registers). VHS, N = 24, 144 nodes:
+// k_shift_sum 41 us (192 MB: 4.7 TB/s), k_shift_finish about 20 us, in the 667 us of the call; at a few nodes the launches
+// bound it, which is why gain and loss share k_shift_finish (five nodes, F16S, N = 32, M = 12: 169 -> 144 us with it and P_r
+// and f in one forward launch).
 //
 // Everything stays in half spectra (kz >= 0): A_rp and the loss weight act on real fields, so only their part
 // even in k counts. A multiplier on the packed slot kz = 0 needs the spectra of kz = 0 and kz = N/2 apart.
@@ -31,19 +35,6 @@ namespace dgfs {
 namespace {
 
 using namespace shdev;
-
-// half spectra of the two real lines that v's parts carried through a forward transform; lo takes the real
-// part's, hi the imaginary part's
-template <typename T, int N, typename F>
-__device__ __forceinline__ void split_line(const Cplx<T> (&v)[N], F put) {
-    constexpr int NH = N / 2;
-    put(0, Cplx<T>{v[0].x, v[NH].x}, Cplx<T>{v[0].y, v[NH].y});
-#pragma unroll
-    for (int k = 1; k < NH; ++k) {
-        const Cplx<T> p = v[k], m = v[N - k];
-        put(k, Cplx<T>{T(0.5) * (p.x + m.x), T(0.5) * (p.y - m.y)}, Cplx<T>{T(0.5) * (p.y + m.y), T(0.5) * (m.x - p.x)});
-    }
-}
 
 template <typename T, int N, int XC>
 struct SumGeo {
@@ -114,16 +105,7 @@ k_shift_vss(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, cons
 #pragma unroll
             for (int y = 0; y < N; ++y) w[line_slot<N>(y)] = ld(S + yrow + y * PITCH);
             cfft::line<T, N, true>(w);
-            Cplx<T>* o = Wn + j * FS;
-            if (ykz > 0) {
-#pragma unroll
-                for (int k = 0; k < N; ++k) st(o + k * NH, w[k]);
-            } else {   // the folded plane
-                split_line<T, N>(w, [&](int k, Cplx<T> a, Cplx<T> b) {
-                    st(o + k * NH, a);
-                    st(o + (NH + k) * NH, b);
-                });
-            }
+            store_folded<T, N>(w, ykz, Wn + j * FS);
         }
     }
 }
@@ -309,31 +291,82 @@ constexpr int col_blocks() { return (N * (N / 2 - (NONZERO ? 1 : 0)) + kColThrea
 // npairs + pair of the field] in the same order, [kx][ky][kz] and the second multipliers of the two packed columns
 // [2][kx]; else the x phase of field fi (fields 2 nx, 2 nx + 1: none). VSS reads 2.5 MB of products per radial point
 // and node at N = 32, M = 38 and is bound by that.
-// grid (col_blocks, nodes, parts): part c takes the radial points c RP .. of the batch. add: on top of part.
-template <typename T, int N, bool VSS>
+// Its rounding depends neither on the batch of nodes nor on the batch of radial points of a launch:
+// Adjoint, Vss: block z of kSumParts takes its share of the fields, every radial point in order, on top of part
+// [node][kSumParts] of the batch before; k_shift_finish adds the parts in order.
+// Radial: groups of RP = ceil(Nrho / kSumGroups) radial points, each group's sum added to the total in order: grid
+// (col_blocks, nodes, 1) keeps the totals in shared memory (part [node]); grid (col_blocks, nodes, sum_groups) takes a
+// group each (part [node][group]) where one block per column leaves SMs idle.
+// Radial (VHS gain, nf = 1): times tab[r0 + r][|k|^2], and coef[node][r0 + r] when the kernel varies by node.
+enum class Sum { Adjoint, Vss, Radial };
+template <typename T, int N, Sum MODE>
 __global__ void __launch_bounds__(kColThreads)
-k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, const ShiftEntry* __restrict__ prog, int npairs,
-            const Cplx<T>* __restrict__ mu, const int* __restrict__ xrows, int nrows, int nx, int r0, int nr, int RP, int add,
+k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, const T* __restrict__ coef, int Nrho,
+            const ShiftEntry* __restrict__ prog, int npairs,
+            const Cplx<T>* __restrict__ mu, const int* __restrict__ xrows, int nrows, int nx, int r0, int nr, int RP,
             Cplx<T>* __restrict__ part) {
-    constexpr int NH = N / 2, COLS = N * NH, MP = shift_mu_pitch(N);
+    constexpr int NH = N / 2, COLS = N * NH, MP = shift_mu_pitch(N), NQ = 3 * NH * NH + 1;
     constexpr int64_t FS = (int64_t)N * COLS, AS = FS + 2 * N;
     const int64_t node = blockIdx.y;
     const int col = blockIdx.x * kColThreads + threadIdx.x;
     if (col >= COLS) return;
-    const bool pair = VSS && (col == 0 || col == NH * NH);   // ky = 0 and N/2 of one plane in a column
+    const bool pair = MODE != Sum::Adjoint && (col == 0 || col == NH * NH);   // ky = 0 and N/2 of one plane in a column
+    // |ky|^2 + |kz|^2 of the column (folded plane kz = 0)
+    const int cky = col / NH, ckz = col % NH;
+    const int fy = ckz ? (cky < NH ? cky : N - cky) : cky % NH, fz = ckz ? ckz : cky < NH ? 0 : NH, q0 = fy * fy + fz * fz;
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    Cplx<T>* total = reinterpret_cast<Cplx<T>*>(sm_raw) + threadIdx.x;   // [kx][thread] (one block per column)
+    const bool whole = MODE == Sum::Radial && gridDim.z == 1;
     Cplx<T>* pc = part + (node * gridDim.z + blockIdx.z) * FS + col;
+    // the batch's radial points of this block: all, or the ones of its group
+    const int lo = MODE != Sum::Radial || whole ? 0 : max(0, (int)blockIdx.z * RP - r0);
+    const int hi = MODE != Sum::Radial || whole ? nr : min(nr, (int)(blockIdx.z + 1) * RP - r0);
+    if (lo >= hi) return;
+    const int f0 = MODE == Sum::Radial ? 0 : nf * (int)blockIdx.z / (int)gridDim.z;   // its fields
+    const int f1 = MODE == Sum::Radial ? 1 : nf * (int)(blockIdx.z + 1) / (int)gridDim.z;
     Cplx<T> acc[N];
+    // a group under way from the batch before: its sum (whole: kept behind the totals)
+    const bool started = MODE == Sum::Radial ? (r0 + lo) % RP != 0 : r0 > 0;
+    if (whole)
 #pragma unroll
-    for (int k = 0; k < N; ++k) acc[k] = add ? ld(pc + (int64_t)k * COLS) : Cplx<T>{T(0), T(0)};
-    const int rl1 = min(nr, (int)(blockIdx.z + 1) * RP);
-    for (int rl = blockIdx.z * RP; rl < rl1; ++rl) {
-        const Cplx<T>* f = F + (node * nr + rl) * nf * FS + col;
-        for (int j = 0; j < nf; ++j, f += FS) {
+        for (int k = 0; k < N; ++k) total[k * kColThreads] = r0 >= RP ? ld(pc + (int64_t)k * COLS) : Cplx<T>{T(0), T(0)};
+    const Cplx<T>* open = whole ? part + (gridDim.y + node) * FS + col : pc;
+#pragma unroll
+    for (int k = 0; k < N; ++k) acc[k] = started ? ld(open + (int64_t)k * COLS) : Cplx<T>{T(0), T(0)};
+    for (int rl = lo; rl < hi; ++rl) {
+        if (whole && rl > lo && (r0 + rl) % RP == 0) {   // the group is complete
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                Cplx<T>& t = total[k * kColThreads];
+                t = Cplx<T>{t.x + acc[k].x, t.y + acc[k].y};
+                acc[k] = Cplx<T>{T(0), T(0)};
+            }
+        }
+        const Cplx<T>* f = F + ((node * nr + rl) * nf + f0) * FS + col;
+        for (int j = f0; j < f1; ++j, f += FS) {
             Cplx<T> v[N];
 #pragma unroll
             for (int x = 0; x < N; ++x) v[line_slot<N>(x)] = ldg(f + (int64_t)x * COLS);
             cfft::line<T, N, true>(v);
-            if constexpr (VSS) {
+            if constexpr (MODE == Sum::Radial) {
+                const T* t = A + (r0 + rl) * NQ + q0;
+                const T c = coef ? __ldg(coef + node * Nrho + r0 + rl) : T(1);
+#pragma unroll
+                for (int k = 0; k <= NH; ++k) {
+                    const T m = c * __ldg(t + k * k);
+                    acc[k] = Cplx<T>{fma(m, v[k].x, acc[k].x), fma(m, v[k].y, acc[k].y)};
+                    if (k > 0 && k < NH) acc[N - k] = Cplx<T>{fma(m, v[N - k].x, acc[N - k].x), fma(m, v[N - k].y, acc[N - k].y)};
+                }
+                if (pair) {   // m a so far; m (a + conj b) / 2 + m' (a - conj b) / 2, b the mirror along x
+#pragma unroll
+                    for (int k = 0; k < N; ++k) {
+                        const int k2 = k <= NH ? k * k : (N - k) * (N - k);
+                        const T h = T(0.5) * c * (__ldg(t + k2 + NH * NH) - __ldg(t + k2));
+                        const Cplx<T> b = v[(N - k) % N];
+                        acc[k] = Cplx<T>{fma(h, v[k].x - b.x, acc[k].x), fma(h, v[k].y + b.y, acc[k].y)};
+                    }
+                }
+            } else if constexpr (MODE == Sum::Vss) {
                 const T* a = A + ((int64_t)(r0 + rl) * npairs + __ldg(&prog[j].pair)) * AS;
 #pragma unroll
                 for (int k = 0; k < N; ++k) {
@@ -368,19 +401,30 @@ k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, cons
             }
         }
     }
+    if (whole) {
+        const bool done = (r0 + nr) % RP == 0 || r0 + nr == Nrho;   // the last group is complete
+        Cplx<T>* rest = part + (gridDim.y + node) * FS + col;
 #pragma unroll
-    for (int k = 0; k < N; ++k) st(pc + (int64_t)k * COLS, acc[k]);
+        for (int k = 0; k < N; ++k) {
+            Cplx<T> t = total[k * kColThreads];
+            if (done) t = Cplx<T>{t.x + acc[k].x, t.y + acc[k].y};
+            else st(rest + (int64_t)k * COLS, acc[k]);
+            st(pc + (int64_t)k * COLS, t);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) st(pc + (int64_t)k * COLS, acc[k]);
+    }
 }
 
-// out[node][x][ky][kz] = scale * inverse x of the sum of the parts. grid (col_blocks, nodes)
+// out[node][x][ky][kz] = scale * inverse x of the sum of the parts; blocks bx < col_blocks
 template <typename T, int N>
-__global__ void __launch_bounds__(kColThreads)
-k_shift_reduce(const Cplx<T>* __restrict__ part, int parts, T scale, Cplx<T>* __restrict__ out) {
+__device__ __forceinline__ void reduce_columns(const Cplx<T>* __restrict__ part, int parts, T scale, int bx, int64_t node,
+                                               Cplx<T>* __restrict__ out) {
     constexpr int COLS = N * N / 2;
     constexpr int64_t FS = (int64_t)N * COLS;
-    const int c = blockIdx.x * kColThreads + threadIdx.x;
+    const int c = bx * kColThreads + threadIdx.x;
     if (c >= COLS) return;
-    const int64_t node = blockIdx.y;
     Cplx<T> v[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) v[line_slot<N>(k)] = Cplx<T>{T(0), T(0)};
@@ -400,33 +444,45 @@ k_shift_reduce(const Cplx<T>* __restrict__ part, int parts, T scale, Cplx<T>* __
     for (int x = 0; x < N; ++x) st(out + node * FS + (int64_t)x * COLS + c, v[x]);
 }
 
-// out[node][r][x][ky][kz] = inverse x of M_r(k) times the x spectrum of G: M = tab[k] (nq2 == 0, standard mode
-// index, the same for every r) or tab[r nq2 + |k|^2]. grid (col_blocks + 1, nodes, nr): the last block is one warp for the packed plane kz = 0
+// out = inverse x of M(k) times the x spectrum of G (fields of one node): M = t[k] (nq2 == 0, standard mode index),
+// t[|k|^2], or (Lr) sum_r rho_r Lr[r][k], summed in FP64 (the loss weight of the sphere rule with a kernel that varies
+// by node). Blocks bx < filter_blocks, the last one warp for the packed plane kz = 0
+template <int N>
+constexpr int filter_blocks() { return col_blocks<N, true>() + 1; }
 template <typename T, int N>
-__global__ void __launch_bounds__(kColThreads)
-k_shift_filter(const Cplx<T>* __restrict__ G, const T* __restrict__ tab, int nq2, int r0, Cplx<T>* __restrict__ out) {
+__device__ __forceinline__ void filter_columns(const Cplx<T>* __restrict__ G, const T* __restrict__ t, int nq2,
+                                               const T* __restrict__ Lr, const double* __restrict__ cr, const NodeParams& np,
+                                               int Nrho, int bx, int64_t node, Cplx<T>* __restrict__ out) {
     constexpr int NH = N / 2, COLS = N * NH;
     constexpr int64_t FS = (int64_t)N * COLS;
-    const int64_t node = blockIdx.y;
-    const bool packed = blockIdx.x == gridDim.x - 1;
+    const bool packed = bx == filter_blocks<N>() - 1;
+    __shared__ double rho[64];
+    if (Lr) {
+        const double gam = np.gamma ? np.gamma[node] : np.gamma0, bb = np.b ? np.b[node] : np.b0;
+        for (int r = threadIdx.x; r < Nrho; r += kColThreads) rho[r] = fdev::radial_rho<double>(bb, gam, cr[r], np.dlog);
+        __syncthreads();
+    }
     int ky, kz;
     if (packed) {
         if (threadIdx.x >= 32) return;
         ky = threadIdx.x < N ? threadIdx.x : 0;
         kz = 0;
     } else {
-        const int c = blockIdx.x * kColThreads + threadIdx.x;
+        const int c = bx * kColThreads + threadIdx.x;
         if (c >= N * (NH - 1)) return;
         ky = c / (NH - 1);
         kz = c % (NH - 1) + 1;
     }
     const int col = ky * NH + kz;
-    const T* t = tab + (int64_t)(r0 + blockIdx.z) * nq2;
     auto sq = [](int q) { const int k = q < NH ? q : q - N; return k * k; };
-    auto mult = [&](int kx, int kzz) { return __ldg(nq2 ? t + sq(kx) + sq(ky) + kzz * kzz : t + (kx * N + ky) * N + kzz); };
+    auto mult = [&](int kx, int kzz) -> T {
+        const int k = (kx * N + ky) * N + kzz;
+        if (Lr) return fdev::loss_multiplier<T>(nullptr, nullptr, Lr, rho, true, 0, Nrho, 2 * FS, k);
+        return __ldg(nq2 ? t + sq(kx) + sq(ky) + kzz * kzz : t + k);
+    };
     Cplx<T> v[N], w[N];
 #pragma unroll
-    for (int x = 0; x < N; ++x) v[line_slot<N>(x)] = ldg(G + node * FS + (int64_t)x * COLS + col);
+    for (int x = 0; x < N; ++x) v[line_slot<N>(x)] = ldg(G + (int64_t)x * COLS + col);
     cfft::line<T, N, true>(v);
     const T sc = T(1) / T(N);
     if (packed) {
@@ -446,9 +502,57 @@ k_shift_filter(const Cplx<T>* __restrict__ G, const T* __restrict__ tab, int nq2
     }
     cfft::line<T, N, false>(w);
     if (packed && threadIdx.x >= N) return;
-    Cplx<T>* o = out + (node * gridDim.z + blockIdx.z) * FS + col;
 #pragma unroll
-    for (int x = 0; x < N; ++x) st(o + (int64_t)x * COLS, w[x]);
+    for (int x = 0; x < N; ++x) st(out + (int64_t)x * COLS + col, w[x]);
+}
+
+// out[node][r]: K_r of every radial point. grid (filter_blocks, nodes, nr)
+template <typename T, int N>
+__global__ void __launch_bounds__(kColThreads)
+k_shift_filter(const Cplx<T>* __restrict__ G, const T* __restrict__ tab, int r0, Cplx<T>* __restrict__ out) {
+    constexpr int64_t FS = (int64_t)N * N * N / 2;
+    constexpr int NQ = 3 * (N / 2) * (N / 2) + 1;
+    const int64_t node = blockIdx.y;
+    filter_columns<T, N>(G + node * FS, tab + (int64_t)(r0 + blockIdx.z) * NQ, NQ, nullptr, nullptr, NodeParams{}, 0, blockIdx.x, node,
+                         out + (node * gridDim.z + blockIdx.z) * FS);
+}
+
+// The gain (F_0) and the loss fields (F_1 from G1, F_2 from G2, F [field][nodes]) in one launch.
+// grid (col_blocks + filter_blocks (1 or 2), nodes)
+template <typename T, int N>
+__global__ void __launch_bounds__(kColThreads)
+k_shift_finish(const Cplx<T>* __restrict__ part, int parts, T scale, const Cplx<T>* __restrict__ G1, const Cplx<T>* __restrict__ G2,
+               FilterTable<T> m, Cplx<T>* __restrict__ F) {
+    constexpr int64_t FS = (int64_t)N * N * N / 2;
+    constexpr int NQ = 3 * (N / 2) * (N / 2) + 1, CB = col_blocks<N, false>(), FB = filter_blocks<N>();
+    const int64_t node = blockIdx.y, nodes = gridDim.y;
+    if (blockIdx.x < CB) {
+        reduce_columns<T, N>(part, parts, scale, blockIdx.x, node, F);
+        return;
+    }
+    const int k = (blockIdx.x - CB) / FB;
+    filter_columns<T, N>((k ? G2 : G1) + node * FS, m.by_node ? m.tab + node * NQ : m.tab, m.by_node ? NQ : 0, m.Lr, m.cr, m.np, m.Nrho,
+                         (blockIdx.x - CB) % FB, node, F + ((k + 1) * nodes + node) * FS);
+}
+
+// w_r rho_r(node), and (Lq) the loss multiplier by |k|^2 of each node, summed over r in FP64. One block per node.
+template <typename T>
+__global__ void k_shift_coef(const double* __restrict__ cr, const double* __restrict__ wr, NodeParams np, int Nrho,
+                             const T* __restrict__ Lq, int nq2, T* __restrict__ coef, T* __restrict__ GLq) {
+    __shared__ double rho[64];
+    const int64_t node = blockIdx.x;
+    const double gam = np.gamma ? np.gamma[node] : np.gamma0, bb = np.b ? np.b[node] : np.b0;
+    for (int r = threadIdx.x; r < Nrho; r += blockDim.x) {
+        rho[r] = fdev::radial_rho<double>(bb, gam, cr[r], np.dlog);
+        coef[node * Nrho + r] = (T)(wr[r] * rho[r]);
+    }
+    __syncthreads();
+    if (!Lq) return;
+    for (int q = threadIdx.x; q < nq2; q += blockDim.x) {
+        double g = 0.0;
+        for (int r = 0; r < Nrho; ++r) g = fma(rho[r], (double)Lq[r * nq2 + q], g);
+        GLq[node * nq2 + q] = (T)g;
+    }
 }
 
 // ---- result ------------------------------------------------------------------------------------
@@ -465,7 +569,7 @@ struct OutGeo {
 template <typename T, int N>
 __global__ void __launch_bounds__(OutGeo<N>::NT)
 k_shift_out(const Cplx<T>* __restrict__ F, int nf, int64_t field_stride, int folded, const T* __restrict__ a,
-            const T* __restrict__ c, T* __restrict__ out, int* __restrict__ flags) {
+            const T* __restrict__ c, const int64_t* __restrict__ offs, T* __restrict__ out, int* __restrict__ flags) {
     using Geo = OutGeo<N>;
     constexpr int NH = N / 2, PITCH = Geo::PITCH;
     constexpr int64_t FS = (int64_t)N * N * NH, n3 = 2 * FS;
@@ -473,7 +577,7 @@ k_shift_out(const Cplx<T>* __restrict__ F, int nf, int64_t field_stride, int fol
     Cplx<T>* S = reinterpret_cast<Cplx<T>*>(sm_raw);       // [PX][y][PITCH]
     const int tid = threadIdx.x, pl = tid / NH, j = tid % NH, x = blockIdx.x * Geo::PX + pl;
     const int64_t node = blockIdx.y;
-    const int64_t row0 = node * n3 + ((int64_t)x * N + j) * N, row1 = row0 + (int64_t)NH * N;   // rows y = j, j + N/2
+    const int64_t row0 = (offs ? offs[node] : node * n3) + ((int64_t)x * N + j) * N, row1 = row0 + (int64_t)NH * N;   // rows y = j, j + N/2
     T q0[N], q1[N];
 #pragma unroll
     for (int z = 0; z < N; ++z) q0[z] = q1[z] = T(0);
@@ -582,34 +686,50 @@ cudaError_t adj_n(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, cons
                                 : adj_x<T, N, wide<N>()>(d, G, H, Ur, wsig, r0, nr, nodes, V, s);
 }
 
-template <typename T, int N>
-cudaError_t sum_n(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, bool bil, int npairs, int r0, int nr, int parts,
-                  bool add, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
-    const int RP = (nr + parts - 1) / parts;
-    const dim3 grid(col_blocks<N, false>(), (unsigned)nodes, (unsigned)parts);
-    auto kern = A ? k_shift_sum<T, N, true> : k_shift_sum<T, N, false>;
-    kern<<<grid, kColThreads, 0, s>>>(F, nf, A, bil ? d.bil : d.quad, npairs, d.mu, d.xrows, d.nrows, d.nx, r0, nr, RP, add, part);
+template <typename T, int N, Sum MODE>
+cudaError_t sum_launch(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, const T* coef, const ShiftEntry* prog, int npairs,
+                       int Nrho, int r0, int nr, int parts, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
+    const size_t sm = MODE == Sum::Radial && parts == 1 ? sizeof(Cplx<T>) * N * kColThreads : 0;
+    const cudaError_t e = allow_smem(k_shift_sum<T, N, MODE>, sm);
+    if (e != cudaSuccess) return e;
+    k_shift_sum<T, N, MODE><<<dim3(col_blocks<N, false>(), (unsigned)nodes, (unsigned)parts), kColThreads, sm, s>>>(
+        F, nf, A, coef, Nrho, prog, npairs, d.mu, d.xrows, d.nrows, d.nx, r0, nr, sum_group(Nrho), part);
     return cudaGetLastError();
 }
 
 template <typename T, int N>
-cudaError_t reduce_n(const Cplx<T>* part, int parts, T scale, int64_t nodes, Cplx<T>* out, cudaStream_t s) {
-    k_shift_reduce<T, N><<<dim3(col_blocks<N, false>(), (unsigned)nodes), kColThreads, 0, s>>>(part, parts, scale, out);
+cudaError_t sum_n(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, bool bil, int npairs, int r0, int nr, int64_t nodes,
+                  Cplx<T>* part, cudaStream_t s) {
+    if (A) return sum_launch<T, N, Sum::Vss>(d, F, nf, A, nullptr, bil ? d.bil : d.quad, npairs, 0, r0, nr, kSumParts, nodes, part, s);
+    return sum_launch<T, N, Sum::Adjoint>(d, F, nf, nullptr, nullptr, d.quad, npairs, 0, r0, nr, kSumParts, nodes, part, s);
+}
+
+template <typename T, int N>
+cudaError_t gain_n(const ShiftDev<T>& d, const Cplx<T>* W, const T* tab, const T* coef, int Nrho, int r0, int nr, int parts,
+                   int64_t nodes, Cplx<T>* part, cudaStream_t s) {
+    return sum_launch<T, N, Sum::Radial>(d, W, 1, tab, coef, d.quad, 0, Nrho, r0, nr, parts, nodes, part, s);
+}
+
+template <typename T, int N>
+cudaError_t filter_n(const ShiftDev<T>& d, const Cplx<T>* G, int r0, int nr, int64_t nodes, Cplx<T>* out, cudaStream_t s) {
+    k_shift_filter<T, N><<<dim3(filter_blocks<N>(), (unsigned)nodes, (unsigned)nr), kColThreads, 0, s>>>(G, d.kq, r0, out);
     return cudaGetLastError();
 }
 
 template <typename T, int N>
-cudaError_t filter_n(const Cplx<T>* G, const T* tab, int nq2, int r0, int nr, int64_t nodes, Cplx<T>* out, cudaStream_t s) {
-    k_shift_filter<T, N><<<dim3(col_blocks<N, true>() + 1, (unsigned)nodes, (unsigned)nr), kColThreads, 0, s>>>(G, tab, nq2, r0, out);
+cudaError_t finish_n(const Cplx<T>* part, int parts, T scale, const Cplx<T>* G1, const Cplx<T>* G2, const FilterTable<T>& m,
+                     int64_t nodes, Cplx<T>* F, cudaStream_t s) {
+    const int blocks = col_blocks<N, false>() + filter_blocks<N>() * (G2 ? 2 : 1);
+    k_shift_finish<T, N><<<dim3((unsigned)blocks, (unsigned)nodes), kColThreads, 0, s>>>(part, parts, scale, G1, G2, m, F);
     return cudaGetLastError();
 }
 
 template <typename T, int N>
-cudaError_t out_n(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c, int64_t nodes, T* out, int* flags,
-                  cudaStream_t s) {
+cudaError_t out_n(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c, const int64_t* offs, int64_t nodes,
+                  T* out, int* flags, cudaStream_t s) {
     using Geo = OutGeo<N>;
     constexpr size_t sm = (size_t)Geo::PX * N * Geo::PITCH * sizeof(Cplx<T>);
-    k_shift_out<T, N><<<dim3(N / Geo::PX, (unsigned)nodes), Geo::NT, sm, s>>>(F, nf, field_stride, folded, a, c, out, flags);
+    k_shift_out<T, N><<<dim3(N / Geo::PX, (unsigned)nodes), Geo::NT, sm, s>>>(F, nf, field_stride, folded, a, c, offs, out, flags);
     return cudaGetLastError();
 }
 
@@ -643,28 +763,42 @@ cudaError_t launch_shift_adj(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<
 }
 template <typename T>
 cudaError_t launch_shift_sum(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, bool bil, int npairs, int N, int r0,
-                             int nr, int parts, bool add, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
-#define CALL(n) sum_n<T, n>(d, F, nf, A, bil, npairs, r0, nr, parts, add, nodes, part, s)
+                             int nr, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
+#define CALL(n) sum_n<T, n>(d, F, nf, A, bil, npairs, r0, nr, nodes, part, s)
     DGFS_BY_N(CALL);
 #undef CALL
 }
 template <typename T>
-cudaError_t launch_shift_reduce(const Cplx<T>* part, int parts, T scale, int N, int64_t nodes, Cplx<T>* out, cudaStream_t s) {
-#define CALL(n) reduce_n<T, n>(part, parts, scale, nodes, out, s)
-    DGFS_BY_N(CALL);
-#undef CALL
-}
-template <typename T>
-cudaError_t launch_shift_filter(const Cplx<T>* G, const T* tab, int nq2, int N, int r0, int nr, int64_t nodes, Cplx<T>* out,
+cudaError_t launch_shift_filter(const ShiftDev<T>& d, const Cplx<T>* G, int N, int r0, int nr, int64_t nodes, Cplx<T>* out,
                                 cudaStream_t s) {
-#define CALL(n) filter_n<T, n>(G, tab, nq2, r0, nr, nodes, out, s)
+#define CALL(n) filter_n<T, n>(d, G, r0, nr, nodes, out, s)
     DGFS_BY_N(CALL);
 #undef CALL
 }
 template <typename T>
-cudaError_t launch_shift_out(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c, int N,
-                             int64_t nodes, T* out, int* flags, cudaStream_t s) {
-#define CALL(n) out_n<T, n>(F, nf, field_stride, folded, a, c, nodes, out, flags, s)
+cudaError_t launch_shift_finish(const Cplx<T>* part, int parts, T scale, const Cplx<T>* G1, const Cplx<T>* G2,
+                                const FilterTable<T>& m, int N, int64_t nodes, Cplx<T>* F, cudaStream_t s) {
+#define CALL(n) finish_n<T, n>(part, parts, scale, G1, G2, m, nodes, F, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+template <typename T>
+cudaError_t launch_shift_gain(const ShiftDev<T>& d, const Cplx<T>* W, const T* tab, const T* coef, int Nrho, int N, int r0,
+                              int nr, int parts, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
+#define CALL(n) gain_n<T, n>(d, W, tab, coef, Nrho, r0, nr, parts, nodes, part, s)
+    DGFS_BY_N(CALL);
+#undef CALL
+}
+template <typename T>
+cudaError_t launch_shift_coef(const DevTables<T>& t, NodeParams np, int64_t nodes, T* coef, T* GLq, cudaStream_t s) {
+    if (nodes <= 0) return cudaSuccess;
+    k_shift_coef<T><<<(unsigned)nodes, 128, 0, s>>>(t.cr, t.wr, np, t.Nrho, t.Lq, 3 * (t.N / 2) * (t.N / 2) + 1, coef, GLq);
+    return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_shift_out(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c,
+                             const int64_t* offs, int N, int64_t nodes, T* out, int* flags, cudaStream_t s) {
+#define CALL(n) out_n<T, n>(F, nf, field_stride, folded, a, c, offs, nodes, out, flags, s)
     DGFS_BY_N(CALL);
 #undef CALL
 }
@@ -675,12 +809,16 @@ cudaError_t launch_shift_out(const Cplx<T>* F, int nf, int64_t field_stride, boo
     template cudaError_t launch_shift_adj<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*,        \
                                              const T*, int, int, int, int64_t, Cplx<T>*, cudaStream_t);                 \
     template cudaError_t launch_shift_sum<T>(const ShiftDev<T>&, const Cplx<T>*, int, const T*, bool, int, int, int,    \
-                                             int, int, bool, int64_t, Cplx<T>*, cudaStream_t);                          \
-    template cudaError_t launch_shift_reduce<T>(const Cplx<T>*, int, T, int, int64_t, Cplx<T>*, cudaStream_t);          \
-    template cudaError_t launch_shift_filter<T>(const Cplx<T>*, const T*, int, int, int, int, int64_t, Cplx<T>*,        \
-                                                cudaStream_t);                                                          \
-    template cudaError_t launch_shift_out<T>(const Cplx<T>*, int, int64_t, bool, const T*, const T*, int, int64_t, T*,  \
-                                             int*, cudaStream_t);
+                                             int, int64_t, Cplx<T>*, cudaStream_t);                                    \
+    template cudaError_t launch_shift_filter<T>(const ShiftDev<T>&, const Cplx<T>*, int, int, int, int64_t, Cplx<T>*, \
+                                                cudaStream_t);                                                        \
+    template cudaError_t launch_shift_finish<T>(const Cplx<T>*, int, T, const Cplx<T>*, const Cplx<T>*,               \
+                                                const FilterTable<T>&, int, int64_t, Cplx<T>*, cudaStream_t);         \
+    template cudaError_t launch_shift_out<T>(const Cplx<T>*, int, int64_t, bool, const T*, const T*, const int64_t*,    \
+                                             int, int64_t, T*, int*, cudaStream_t);                                     \
+    template cudaError_t launch_shift_gain<T>(const ShiftDev<T>&, const Cplx<T>*, const T*, const T*, int, int, int,    \
+                                              int, int, int64_t, Cplx<T>*, cudaStream_t);                                    \
+    template cudaError_t launch_shift_coef<T>(const DevTables<T>&, NodeParams, int64_t, T*, T*, cudaStream_t);
 DGFS_SHIFT_INST(float)
 DGFS_SHIFT_INST(double)
 #undef DGFS_SHIFT_INST

@@ -1,4 +1,5 @@
-// Fused Fourier stage (N = 8, 12, 16, 24, 32): the same operations as the
+// Fused Fourier stage by projection (N = 8, 12, 16, 24, 32; capi.cu has the rule by which some plans take the radial sum
+// in spectra instead): the same operations as the
 // projection, forward DFT, Fourier combine, inverse DFT and finalisation kernels of
 // k_fourier.cu (arXiv:1809.10186, Appendix, eqs. realGG, lowrank1, apndx_fs_Glm_Qk), in four
 // launches whose intermediates stay in shared memory or registers between the axis passes:

@@ -121,5 +121,35 @@ __device__ __forceinline__ void load_z_line(const Cplx<T>* zp, const Cplx<T>* zm
     }
 }
 
+// half spectra of the two real lines that v's parts carried through a forward transform; put takes
+// the real part's, then the imaginary part's
+template <typename T, int N, typename F>
+__device__ __forceinline__ void split_line(const Cplx<T> (&v)[N], F put) {
+    constexpr int NH = N / 2;
+    put(0, Cplx<T>{v[0].x, v[NH].x}, Cplx<T>{v[0].y, v[NH].y});
+#pragma unroll
+    for (int k = 1; k < NH; ++k) {
+        const Cplx<T> p = v[k], m = v[N - k];
+        put(k, Cplx<T>{T(0.5) * (p.x + m.x), T(0.5) * (p.y - m.y)}, Cplx<T>{T(0.5) * (p.y + m.y), T(0.5) * (m.x - p.x)});
+    }
+}
+
+// A forward-transformed y line of a real field's half spectrum (slot kz) into the field at o (element ky at
+// o[ky N/2]); the plane kz = 0 folded: ky = 0 .. N/2 - 1 of kz = 0, then of kz = N/2, the real values at ky = 0 and N/2
+// packed in the slots ky = 0, so that a multiplier by k acts on every slot but those two by itself.
+template <typename T, int N>
+__device__ __forceinline__ void store_folded(const Cplx<T> (&w)[N], int kz, Cplx<T>* o) {
+    constexpr int NH = N / 2;
+    if (kz > 0) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) st(o + k * NH, w[k]);
+    } else {
+        split_line<T, N>(w, [&](int k, Cplx<T> a, Cplx<T> b) {
+            st(o + k * NH, a);
+            st(o + (NH + k) * NH, b);
+        });
+    }
+}
+
 }  // namespace shdev
 }  // namespace dgfs
