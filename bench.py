@@ -39,7 +39,7 @@ TOL_L = {"fp64": 1e-10, "fp32": 1e-5, "f16s": 1e-3, "bf16s": 5e-3, "f16x3": 1e-5
 MODES = ("fp32", "f16s", "bf16s", "f16x3", "bf16x3")
 DTYPES = {"fp32": "f32", "fp64": "f64", "f16s": "f16 data, f16 hi+lo filters, f32 accumulate",
           "bf16s": "bf16 data, bf16 hi+lo filters, f32 accumulate",
-          "f16x3": "f16 hi+lo data and filters (3 products), f32 accumulate",
+          "f16x3": "f32 (the FP32 translates of the CUDA cores)",
           "bf16x3": "bf16 hi+lo data and filters (3 products), f32 accumulate"}
 
 
@@ -201,6 +201,48 @@ def translate_flops_per_node(N, Nrho, npairs, prec):
     return Nrho * npairs * (mult * mma + elem)
 
 
+def on_cuda_cores(prec):
+    """F16X3 calls take the FP32 translates of the CUDA cores (all but the time stepper's and dQ/dgamma)."""
+    return prec in ("fp32", "fp64", "f16x3")
+
+
+def shared_steps(sigma):
+    """What the sphere points share: (nonzero signed s_x, distinct signed (s_x, s_y), distinct (s_x, s_z) of the
+    pairs), from one point of every antipodal pair [npairs, >= 3]."""
+    pts = [tuple(float(x) for x in p[:3]) for p in sigma]
+    both = pts + [tuple(-x for x in p) for p in pts]
+    return (len({p[0] for p in both if p[0] != 0.0}), len({(p[0] + 0.0, p[1] + 0.0) for p in both}),
+            len({(p[0] + 0.0, p[2] + 0.0) for p in pts}))
+
+
+def executed_flops_per_node(N, Nrho, sigma, prec):
+    """Flops the translate products execute per node, with what the sphere points share done once.
+
+    CUDA cores: complex lines of 5 N log2 N flops, N^2 / 2 per signed s_x (half spectra) and per signed (s_x, s_y),
+    N^2 per pair, 6 flops of phase per line point, 3 per point and pair for the product and the sum.
+    Tensor cores: passes 1 and 2 per (s_x, s_z), pass 3 and the products per pair (translate_flops_per_node)."""
+    npairs = len(sigma)
+    nx, nxy, nxz = shared_steps(sigma)
+    if on_cuda_cores(prec):
+        lines = (0.5 * nx + 0.5 * nxy + npairs) * N ** 2
+        return Nrho * (lines * (5.0 * N * math.log2(N) + 6.0 * N) + 3.0 * npairs * N ** 3)
+    mult = {"f16s": 2, "bf16s": 2, "bf16x3": 3}[prec]
+    return Nrho * (mult * 4.0 * N ** 4 * (2 * nxz + npairs) + 3.0 * N ** 3 * npairs)
+
+
+def front_share(N, prec, mma):
+    """Share of passes 1 and 2 in mma_shape_ceiling's cycles."""
+    total, _ = mma_shape_ceiling(N, prec, mma)
+    if not total:
+        return None
+    ks = N // 16
+    if prec in ("f16s", "bf16s"):
+        back = N * N // 128 * 2 * ks * mma["smem_n%d" % (2 * N)]
+    else:
+        back = N * N // 256 * 2 * ks * (mma["smem_n%d" % (2 * N)] + mma["smem_n%d" % N])
+    return 1.0 - back / total
+
+
 def shape_ceiling_fields(N, Nr, npairs, prec, measured, launch_ms, nodes, clocks):
     """The kernel's cycles per (radial point, pair) step and SM (launch time at the sampled SM clock)
     against mma_shape_ceiling: how close the kernel runs to what its MMA shapes allow."""
@@ -248,7 +290,6 @@ def fft_algorithmic_flops_per_node(N, Nrho, npairs):
 # from the ncu capture of a 512-node launch summarised in profiles/ (None for configurations
 # without a capture of the current kernel version).
 TRAFFIC_PER_NODE = {("f16s", 32, 32, 38): (180026368 + 2091159552) / 512, ("bf16s", 32, 32, 38): (185963520 + 2090830592) / 512,
-                    ("f16x3", 32, 32, 38): (109169920 + 2091046656) / 512,
                     ("fp32", 32, 32, 38): None}
 
 
@@ -803,12 +844,13 @@ def main():
     # roofline of the dominant kernel (translate-product), from the library's own events
     per_launch_ms = prof["gain_ms"] / max(1, prof["gain_timed"])
     nodes_per_launch = prof["nodes"] / max(1, prof["gain_launches"])
-    flops_node = translate_flops_per_node(N, Nr, npairs, prec)
+    sigma = binding.host_quadrature(N=N, L=cfg["L"], M=2 * npairs, N_rho=Nr)[2]
+    flops_node = executed_flops_per_node(N, Nr, sigma, prec)
     achieved = flops_node * nodes_per_launch / (per_launch_ms / 1e3) / 1e12
     peaks = _peaks()
-    if prec in ("fp32", "fp64"):
-        peak = measured["fp32_fma_tflops"] if prec == "fp32" else measured["fp64_fma_tflops"]
-        roof = {"bound": "alu", "peak_source": "measured %s FMA rate of this GPU (of measured)" % prec.upper()}
+    if on_cuda_cores(prec):
+        peak = measured["fp64_fma_tflops"] if prec == "fp64" else measured["fp32_fma_tflops"]
+        roof = {"bound": "alu", "peak_source": "measured %s FMA rate of this GPU (of measured)" % ("FP64" if prec == "fp64" else "FP32")}
     else:
         # dense fp16 and bf16 tensor rates are equal; the kernel runs for the whole step
         peak = peaks.get("bf16_tflops_sustained") or 1700.0
@@ -817,20 +859,28 @@ def main():
     # the method's own work (the translates counted as radix-2 FFTs, Appendix) over the same kernel time
     alg_node = fft_algorithmic_flops_per_node(N, Nr, npairs)
     alg_rate = alg_node * nodes_per_launch / (per_launch_ms / 1e3) / 1e12
-    alg_peak = measured["fp32_fma_tflops"] if prec in ("fp32", "fp64") else measured["fp16_dense_tflops"]
+    alg_peak = measured["fp32_fma_tflops"] if on_cuda_cores(prec) else measured["fp16_dense_tflops"]
+    shape = {}
+    if not on_cuda_cores(prec):
+        shape = shape_ceiling_fields(N, Nr, npairs, prec, measured, per_launch_ms, nodes_per_launch, clocks)
+    if shape:   # passes 1 and 2 once per (s_x, s_z)
+        front = front_share(N, prec, measured["mma_cycles"])
+        done = front * shared_steps(sigma)[2] / npairs + 1.0 - front
+        shape["mma_shape_cycles_per_step"] *= done
+        shape["frac_of_mma_shape_ceiling"] *= done
     roof.update({"achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                  "frac_basis": "flops the kernel executes (dense circulant passes, split products)"
-                 if prec not in ("fp32", "fp64") else "flops of the Fourier-space translates the kernel executes",
+                 if not on_cuda_cores(prec) else "flops of the Fourier-space translates the kernel executes",
                  "achieved_algorithmic": alg_rate, "peak_algorithmic": alg_peak,
                  "frac_algorithmic": alg_rate / alg_peak,
                  "algorithmic_basis": "N_rho (M/2) (5 N^3 log2 N^3 + 20 N^3) per node over the kernel time, against the "
-                                      "measured dense %s rate (of measured)" % ("FP32 FMA" if prec in ("fp32", "fp64")
+                                      "measured dense %s rate (of measured)" % ("FP32 FMA" if on_cuda_cores(prec)
                                                                               else "fp16 cuBLAS"),
                  "traffic": (TRAFFIC_PER_NODE.get((prec, N, Nr, 2 * npairs)) or 0) * nodes_per_launch or None,
                  "traffic_unit": "bytes per launch", "kernel": "translate-product",
                  "kernel_share": prof["gain_ms"] / ms if ms else None,
                  "flops_per_node": flops_node, "nodes_per_launch": nodes_per_launch, "launch_ms": per_launch_ms,
-                 **shape_ceiling_fields(N, Nr, npairs, prec, measured, per_launch_ms, nodes_per_launch, clocks),
+                 **shape,
                  "fft_algorithmic_tflops": fft_algorithmic_flops_per_node(N, Nr, npairs) * value / world / 1e12})
 
     line = {"metric": METRIC, "value": value, "unit": "node-evals/s", "n_gpus": world,

@@ -64,7 +64,7 @@ typedef enum {
                              power-of-two scale, every filter split into fp16 hi + lo parts (two
                              products), FP32 accumulation in tensor memory; FP32 elsewhere. N = 16, 32,
                              and 24 on the 32-point tiles (filters and data zero-padded: the exact
-                             24-point result at (32/24)^3 the work of a 24-point tiling).
+                             24-point result at 16/9 the work of a 24-point tiling).
                              For F16S, BF16S and BF16X3, Q(f,f), Q(f,g), the JVP and dQ/dgamma
                              take their translates on the tensor cores (the bilinear calls by
                              polarisation: the translate-product sum is symmetric in f and g, so
@@ -254,8 +254,9 @@ dgfs_status dgfs_collide_host(dgfs_plan_t plan, const void* f_host, void* Q_host
                               void* stream);
 
 /* Q(f,f) as dgfs_collide computes it (the same kernels, except that FP32/FP64 plans form the
-   translate products with the dense circulant kernel where dgfs_collide takes them in Fourier
-   space: equal to rounding), for callers that must not allocate device
+   translate products with the dense circulant kernel and F16X3 plans with the split-data
+   tensor-core kernel where dgfs_collide takes them in Fourier space, and the Fourier stage may
+   sum in another order: equal to rounding), for callers that must not allocate device
    memory when they run (for example code whose device memory is fully reserved up front, or
    that may not pay the device synchronisation an allocation can cause). The paper has no
    counterpart to this call. Its intermediate fields live in one fixed 64 MiB device array
@@ -277,7 +278,8 @@ dgfs_status dgfs_stream_status(dgfs_plan_t plan, void* stream);
 /* ---- space-homogeneous time stepping and moments (Secs. 3.3, 3.5) ---------------------
    dgfs_ssprk advances df/dt = scale Q(f, f) (scale: e.g. 1/Kn) by nsteps steps of dt with the
    2nd- or 3rd-order SSP Runge-Kutta scheme (eqs. SSPRK2, SSPRK3), in place: f device [B][N^3] in
-   the plan's element type. Every stage is a dgfs_collide evaluation plus one elementwise
+   the plan's element type. Every stage is an evaluation of Q(f, f) (equal to dgfs_collide
+   to rounding: some plans run other kernels here) plus one elementwise
    combination kernel; the stage fields live in the plan's workspace. Stream-ordered, no
    allocation; non-finite values raise DGFS_ERR_NUMERIC in dgfs_stream_status. */
 dgfs_status dgfs_ssprk(dgfs_plan_t plan, int order, void* f, int64_t B, double dt, double scale, int nsteps,
@@ -326,8 +328,8 @@ dgfs_status dgfs_host_dg_tensor(int K, double* nodes, double* M, double* H);
 dgfs_status dgfs_debug_inject(dgfs_plan_t plan, int mode);
 
 /* Profiling of one plan: between begin and end the library counts its kernel launches and
-   brackets every launch of the translate-product kernel (the dominant kernel) with CUDA
-   events on the call's stream. end synchronises those events and reports the totals.
+   brackets every launch (or launch sequence) of the translate-product kernels (the dominant
+   ones) with CUDA events on the call's stream. end synchronises those events and reports the totals.
    At most 65536 bracketed launches per session; later ones are counted, not timed. */
 typedef struct {
     int64_t launches;         /* kernels launched by compute calls of this plan             */
