@@ -17,7 +17,7 @@
 // Measured (GB300, FP32, N = 32, M = 38): VSS Q of 40 nodes 3.1 ms (6.5 ms with a three-axis transform of its own for
 // every translate and product), VJP of 48 nodes 4.2 ms (11 ms); k_shift_vss 57 % and k_shift_adj 80 % of them, both
 // bound by instruction issue at 8-12 warps per SM (a line and its sums fill the registers). VHS, N = 24, 144 nodes:
-// k_shift_sum 41 us (192 MB: 4.7 TB/s), k_shift_finish about 20 us, in the 667 us of the call; at a few nodes the launches
+// k_shift_sum 41 us (192 MB: 4.7 TB/s), k_shift_finish about 20 us, in the 658 us of the call; at a few nodes the launches
 // bound it, which is why gain and loss share k_shift_finish (five nodes, F16S, N = 32, M = 12: 169 -> 144 us with it and P_r
 // and f in one forward launch).
 //
