@@ -626,7 +626,8 @@ cudaError_t spectral_n(const DevTables<T>& t, const T* P, NodeParams np, int64_t
 template <typename T>
 bool spectral_supported(const DevTables<T>& t) {
     if (t.rank < 1 || t.rank > 32 || t.Nrho > 64) return false;
-    if (t.N == 8 || t.N == 12 || t.N == 16) return true;
+    if (t.N == 8 || t.N == 16) return true;
+    if (t.N == 12) return sizeof(T) == 8;   // FP32: in spectra (capi.cu), or separate kernels
     return (t.N == 24 || t.N == 32) && sizeof(T) == 4;
 }
 
@@ -677,7 +678,7 @@ cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, in
         cudaError_t e = cudaErrorNotSupported;
         switch (t.N) {
             case 8: e = spectral_n<T, 8>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
-            case 12: e = spectral_n<T, 12>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
+            case 12: if constexpr (sizeof(T) == 8) e = spectral_n<T, 12>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
             case 16: e = spectral_n<T, 16>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
             case 24: if constexpr (sizeof(T) == 4) e = spectral_n<T, 24>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
             case 32: if constexpr (sizeof(T) == 4) e = spectral_n<T, 32>(t, P0, np0, nn, la0, lb0, o, gain_scale, C0, c_stride, Q0, X0, Y0, fa0, fc0, out0, flags, s); break;
