@@ -113,6 +113,7 @@ struct dgfs_plan_s {
     const void* d_mu = nullptr;   // [Nrho][npairs][3][N] complex multipliers (inside d_vss)
     ShiftDev<float> shf;          // shared-shift program of the translate products (inside d_vss)
     ShiftDev<double> shd;
+    double project = 1.0;         // of the projection's coefficients (ShiftProgram)
     size_t off_V = 0, vss_bytes = 0;
     void* d_vss = nullptr;   // VSS: half tables A, GL [N^3], shift program; VHS: mu [Nrho][npairs][3][N], shift program
     int xfields = 0;
@@ -309,18 +310,20 @@ void fill_tables(dgfs_plan_s* p, std::vector<unsigned char>& blob, DevTables<T>&
 // (ky, 0), the others (ky - N/2, N/2)), then [2][kx] the values at ky = N/2 of its two packed columns; and the loss
 // weight [N^3], DFT index order.
 template <typename T>
-void fill_vss_tables(const HostPlan& h, std::vector<unsigned char>& blob) {
+void fill_vss_tables(const HostPlan& h, const std::vector<double>& excess, std::vector<unsigned char>& blob) {
     const int N = h.N, NH = N / 2;
     const size_t n3 = (size_t)N * N * N, half = n3 / 2 + 2 * (size_t)N, fields = h.Fa.size() / n3;
     blob.assign((fields * half + n3) * sizeof(T), 0);
     T* d = reinterpret_cast<T*>(blob.data());
+    double e = 1.0;
     auto even = [&](const double* a, int kx, int ky, int kz) {
         const size_t i = ((size_t)kx * N + ky) * N + kz;
         const size_t m = ((size_t)((N - kx) % N) * N + (N - ky) % N) * N + (N - kz) % N;
-        return (T)(0.5 * (a[i] + a[m]));
+        return (T)(e * 0.5 * (a[i] + a[m]));
     };
     for (size_t f = 0; f < fields; ++f, d += half) {
         const double* a = &h.Fa[f * n3];
+        e = excess[f % h.npairs];
         for (int kx = 0; kx < N; ++kx) {
             for (int ky = 0; ky < N; ++ky) {
                 d[((size_t)kx * N + ky) * NH] = even(a, kx, ky % NH, ky < NH ? 0 : NH);
@@ -330,6 +333,7 @@ void fill_vss_tables(const HostPlan& h, std::vector<unsigned char>& blob) {
             d[n3 / 2 + N + kx] = even(a, kx, NH, NH);
         }
     }
+    e = 1.0;
     for (size_t i = 0; i < n3; ++i) d[i] = even(h.GLa.data(), (int)(i / ((size_t)N * N)), (int)((i / N) % N), (int)(i % N));
 }
 
@@ -377,6 +381,9 @@ void pack_shift(const ShiftProgram& sp, std::vector<unsigned char>& blob, ShiftD
     d.sq = put_t(sp.sq);
     d.kq = put_t(sp.kq);
     d.kqd = put_t(sp.kqd);
+    d.st = put_t(sp.st);
+    d.kt = put_t(sp.kt);
+    d.wsig = put_t(sp.wsig);
 }
 
 template <typename T>
@@ -385,7 +392,7 @@ void rebase_shift(ShiftDev<T>& d, const void* base) {
         using P = std::remove_reference_t<decltype(ptr)>;
         ptr = reinterpret_cast<P>(static_cast<const unsigned char*>(base) + reinterpret_cast<uintptr_t>(ptr));
     };
-    fix(d.mu); fix(d.quad); fix(d.bil); fix(d.xrows); fix(d.sq); fix(d.kq); fix(d.kqd);
+    fix(d.mu); fix(d.quad); fix(d.bil); fix(d.xrows); fix(d.sq); fix(d.kq); fix(d.kqd); fix(d.st); fix(d.kt); fix(d.wsig);
 }
 
 unsigned char* ws(dgfs_plan_s* p, size_t off) { return static_cast<unsigned char*>(p->d_ws) + off; }
@@ -431,7 +438,7 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     const T* A = static_cast<const T*>(p->d_vss);
     FilterTable<T> loss;
     loss.tab = A + (size_t)Nr * np * (field + 2 * N);
-    const double scale = (two ? 1.0 : 2.0) * (op == Op::Jvp ? 2.0 : 1.0) / (double)n3 * shift_gain_scale(N, sizeof(T) == 8);
+    const double scale = (two ? 1.0 : 2.0) * (op == Op::Jvp ? 2.0 : 1.0) * shift_result_scale(N, sizeof(T) == 8);
     // fields per node (operands, partial sums, results) and per item (x translates, products)
     const int64_t cap = p->vchunk * (6 * (int64_t)np + 9), item = (int64_t)ops * 2 * d.nx + nprog;
     int64_t C = std::min<int64_t>({nodes, cap / (ops + kSumParts + nf + item), 65535});
@@ -494,6 +501,7 @@ struct StageWork {
     Cplx<T>* part;     // [nodes][parts] partial sums over r
     T *coef, *GLq;     // per-node kernels: [nodes][Nrho], [nodes][3 (N/2)^2 + 1]
     int parts;
+    bool tensor;       // the P_r are the tensor cores'
 };
 
 // Events around the translate products of one launch sequence (dgfs_profile_*).
@@ -521,7 +529,7 @@ cudaError_t stage_sum(dgfs_plan_s* p, Op op, const Cplx<T>* W, NodeParams np, in
     cudaError_t e = cudaSuccess;
     if (per_node && r0 == 0) e = launch_shift_coef<T>(t, np, nodes, w.coef, w.GLq, s);
     if (!e)
-        e = launch_shift_gain<T>(d, W, per_node ? d.sq : op == Op::Dgamma ? d.kqd : d.kq, per_node ? w.coef : nullptr, t.Nrho, t.N,
+        e = launch_shift_gain<T>(d, W, per_node ? (w.tensor ? d.st : d.sq) : op == Op::Dgamma ? d.kqd : w.tensor ? d.kt : d.kq, per_node ? w.coef : nullptr, t.Nrho, t.N,
                                  r0, nr, w.parts, nodes, w.part, s);
     if (p->prof) p->prof_launches += 1 + (per_node && r0 == 0);
     return e;
@@ -544,7 +552,7 @@ cudaError_t stage_finish(dgfs_plan_s* p, Op op, const Cplx<T>* Ga, const Cplx<T>
         loss.np = np;
         loss.Nrho = t.Nrho;
     }
-    cudaError_t e = launch_shift_finish<T>(w.part, w.parts, (T)((jvp ? 2.0 : 1.0) / (double)n3), Gb, jvp ? Ga : nullptr, loss, t.N,
+    cudaError_t e = launch_shift_finish<T>(w.part, w.parts, (T)((jvp ? 2.0 : 1.0) * shift_result_scale(t.N, sizeof(T) == 8)), Gb, jvp ? Ga : nullptr, loss, t.N,
                                            nodes, w.F, s);
     if (!e) e = launch_shift_out<T>(w.F, jvp ? 3 : 2, nodes * field, true, a, jvp ? c : nullptr, offs, t.N, nodes, out, p->d_flags, s);
     if (p->prof) p->prof_launches += 2;
@@ -586,6 +594,7 @@ cudaError_t shift_gain_products(dgfs_plan_s* p, Op op, const T* f, const T* g, T
     w.GLq = w.coef + C * Nr;
     w.part = reinterpret_cast<Cplx<T>*>(ws(p, p->off_X));
     w.parts = gain_parts(N, Nr, C, 2 * (int64_t)p->xfields * p->chunk);
+    w.tensor = false;
     for (int64_t n0 = 0; n0 < nodes; n0 += C) {
         const int64_t nn = std::min<int64_t>(C, nodes - n0), fo = offs ? 0 : n0 * n3;
         const int64_t* of = offs ? offs + n0 : nullptr;
@@ -601,7 +610,7 @@ cudaError_t shift_gain_products(dgfs_plan_s* p, Op op, const T* f, const T* g, T
             if (r0 > 0) first = ProfScope(p, s);
             e = launch_shift_x<T>(d, Gf, N, r0, nr, nn, Hf, s);
             if (!e && g) e = launch_shift_x<T>(d, Gg, N, r0, nr, nn, Hg, s);
-            if (!e) e = launch_shift_products<T>(d, Gf, Hf, Gg, Hg, t.wsig, N, r0, nr, nn, folded,
+            if (!e) e = launch_shift_products<T>(d, Gf, Hf, Gg, Hg, N, r0, nr, nn, folded,
                                                  (folded ? nr : Nr) * n3, folded ? P : P + (n0 * Nr + r0) * n3, s);
             first.end();
             if (!e && folded) e = stage_sum<T>(p, op, W, npb, r0, nr, nn, w, s);
@@ -641,6 +650,7 @@ cudaError_t tc_stage(dgfs_plan_s* p, Op op, const T* f, const T* g, const T* P, 
     w.GLq = w.coef + nodes * t.Nrho;
     w.part = X + nodes * t.Nrho * field;
     w.parts = gain_parts(t.N, t.Nrho, nodes, (xh - t.Nrho) * nodes);
+    w.tensor = true;
     cudaError_t e = launch_shift_folded<T>(P, nodes * t.Nrho, f, offs, t.N, nodes, X, Ga, s);
     if (!e && g) e = launch_shift_forward<T>(g, nullptr, offs, t.N, nodes, Gb, s);
     if (!e) e = stage_sum<T>(p, op, X, np, 0, t.Nrho, nodes, w, s);
@@ -695,7 +705,7 @@ cudaError_t shift_vjp(dgfs_plan_s* p, const T* f, const T* u, T* out, int64_t no
     const int64_t nbatch = (nodes + C - 1) / C;
     C = (nodes + nbatch - 1) / nbatch;   // equal batches
     const int R = (int)std::min<int64_t>(Nr, cap / (C * item));
-    const double scale = shift_gain_scale(N, sizeof(T) == 8) / (double)n3;
+    const double scale = shift_result_scale(N, sizeof(T) == 8);
     Cplx<T>* G = reinterpret_cast<Cplx<T>*>(ws(p, p->off_Y));   // spectra of f, u and u f
     Cplx<T>* F = G + 3 * C * field;                             // gain, K_L f, K_L(u f)
     Cplx<T>* part = reinterpret_cast<Cplx<T>*>(ws(p, p->off_X));
@@ -712,7 +722,7 @@ cudaError_t shift_vjp(dgfs_plan_s* p, const T* f, const T* u, T* out, int64_t no
             const int nr = std::min(R, Nr - r0);
             e = launch_shift_x<T>(d, G, N, r0, nr, nn, H, s);
             if (!e) e = launch_shift_filter<T>(d, G + C * field, N, r0, nr, nn, Ur, s);
-            if (!e) e = launch_shift_adj<T>(d, G, H, Ur, t.wsig, N, r0, nr, nn, V, s);
+            if (!e) e = launch_shift_adj<T>(d, G, H, Ur, N, r0, nr, nn, V, s);
             if (!e) e = launch_shift_sum<T>(d, V, 2 * d.nx + 2, nullptr, false, t.npairs, N, r0, nr, nn, part, s);
             if (p->prof) p->prof_launches += (d.nx ? 1 : 0) + 3;
         }
@@ -795,18 +805,20 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     // (N = 12, 24: the separate kernels where keeps_rounding holds on to their rounding)
     const bool fused = spectral_supported(t) && !(keeps_rounding<T>(op) && t.N % 3 == 0);
     if (p->prof) p->prof_launches += fused ? 4 : 10 + (op == Op::Jvp ? 1 : 0);
+    // the P_r of k_shift_products carry the FP32 weights of their plan
+    const double balance = std::is_same<T, float>::value && !tensor && !keeps_rounding<T>(op) ? p->project : 0.0;
     // real fields packed two per complex slot: the rank projected fields, then the loss
     // operand(s): Q(f,g) -> field rank = g;  JVP -> field rank = v, field rank + 1 = f
     if (fused) {   // the fused Fourier stage
         const T* la = quadratic(op) ? f : g;
-        e = launch_spectral<T>(t, P, np, nodes, la, op == Op::Jvp ? f : nullptr, offs,
+        e = launch_spectral<T>(t, P, np, balance, nodes, la, op == Op::Jvp ? f : nullptr, offs,
                                op == Op::Jvp ? T(2) : T(1), X, Y, f, op == Op::Jvp ? g : nullptr, out,
                                p->d_flags, s);
         if (e) return cuda_fail(e, "Fourier stage");
         return DGFS_OK;
     }
     const int nfields = rank + (op == Op::Jvp ? 2 : 1), xs = (nfields + 1) / 2;
-    e = launch_project<T>(t, P, np, nodes, X, xs, s);
+    e = launch_project<T>(t, P, np, balance, nodes, X, xs, s);
     if (e) return cuda_fail(e, "radial projection");
     const T* loss0 = quadratic(op) ? f : g;
     e = launch_load_field<T>(t.N, loss0, nullptr, offs, nodes, X, xs, rank / 2, rank % 2, s);
@@ -945,12 +957,12 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
     if (p->hp.aniso) {
         std::vector<unsigned char> vblob;
         ShiftProgram sp;
-        build_shift_program(p->hp, sp);
+        build_shift_program(p->hp, p->prec != DGFS_PREC_FP64, sp);
         if (p->prec == DGFS_PREC_FP64) {
-            fill_vss_tables<double>(p->hp, vblob);
+            fill_vss_tables<double>(p->hp, sp.excess, vblob);
             pack_shift(sp, vblob, p->shd);
         } else {
-            fill_vss_tables<float>(p->hp, vblob);
+            fill_vss_tables<float>(p->hp, sp.excess, vblob);
             pack_shift(sp, vblob, p->shf);
         }
         cudaError_t ev = cudaMalloc(&p->d_vss, vblob.size());
@@ -972,7 +984,8 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
         std::vector<unsigned char> mblob(p->prec == DGFS_PREC_FP32 ? p->hp.mu.size() * es : 0);
         for (size_t i = 0; i < mblob.size() / es; ++i) reinterpret_cast<float*>(mblob.data())[i] = (float)p->hp.mu[i];
         ShiftProgram sp;
-        build_shift_program(p->hp, sp);
+        build_shift_program(p->hp, es == 4, sp);
+        p->project = sp.project;
         if (es == 8) pack_shift(sp, mblob, p->shd);
         else pack_shift(sp, mblob, p->shf);
         cudaError_t ev = cudaMalloc(&p->d_vss, mblob.size());
@@ -2344,12 +2357,12 @@ dgfs_status noalloc_run(dgfs_plan_s* p, const T* f, T* Q, int64_t B, unsigned ch
         return DGFS_OK;
     }
     if (!e && spectral_supported(t)) {   // the fused Fourier stage, as in dgfs_collide
-        e = launch_spectral<T>(t, P, np, B, f, nullptr, nullptr, T(1), X, Y, f, nullptr, Q, p->d_flags, s);
+        e = launch_spectral<T>(t, P, np, 0.0, B, f, nullptr, nullptr, T(1), X, Y, f, nullptr, Q, p->d_flags, s);
         if (e) return cuda_fail(e, "dgfs_collide_noalloc");
         return DGFS_OK;
     }
     const int xs = (t.rank + 2) / 2;   // rank projected fields and f, packed two per slot
-    if (!e) e = launch_project<T>(t, P, np, B, X, xs, s);
+    if (!e) e = launch_project<T>(t, P, np, 0.0, B, X, xs, s);
     if (!e) e = launch_load_field<T>(t.N, f, nullptr, nullptr, B, X, xs, t.rank / 2, t.rank % 2, s);
     if (!e) e = launch_dft3<T>(t, X, B * xs, true, s);
     if (!e) e = launch_combine<T>(t, X, xs, np, B, T(1), t.rank, -1, Y, 2, s);

@@ -18,8 +18,6 @@ using fdev::add;
 using fdev::bitrev;
 using fdev::cos_of;
 using fdev::line_slot;
-using fdev::quarter24;
-using fdev::quarter32;
 using fdev::pack;
 using fdev::sin_of;
 using fdev::sub;
@@ -38,16 +36,17 @@ __device__ __forceinline__ Cplx<float> twice_minus<float>(Cplx<float> u, Cplx<fl
     return unpack(r);
 }
 
-// a + c x with the constant c in two FP32 terms (the first a multiple of 1/128, the second's rounding below
-// 4e-10): N = 12, 24 take the constants sqrt(1/2) and sqrt(3)/2 of their short stages this way, because both
-// round 1.7e-8 down and shorten every line (a round trip at N = 24 loses 1.3e-8 instead of 3.3e-8).
-constexpr double kHalfRoot = quarter32(4), kRoot34 = quarter24(2);
-template <typename T>
-__device__ __forceinline__ T plus_scaled(T a, T x, double c) {
-    if (sizeof(T) == 8) return fma((T)c, x, a);
-    const double head = (double)(int)(c * 128.0) / 128.0;
-    return fma((T)(c - head), x, fma((T)head, x, a));
+// a + sqrt(1/2) x with the constant in two FP32 terms (the first a multiple of 1/128): in one term it is 1.7e-8 short,
+// and the lines of N = 24, which meet it in every transform of length 8, lose 2.2e-8 a round trip instead of 1.4e-8.
+__device__ __forceinline__ float plus_half_root(float a, float x) {
+    constexpr double c = cos_of<8>(1), head = (double)(int)(c * 128.0) / 128.0;
+    return fma((float)(c - head), x, fma((float)head, x, a));
 }
+__device__ __forceinline__ double plus_half_root(double a, double x) { return fma(cos_of<8>(1), x, a); }
+
+// c + w x with a constant w; nothing for w = 0
+template <typename T>
+__device__ __forceinline__ T madd(T w, T x, T c) { return w == T(0) ? c : fma(w, x, c); }
 
 // radix-2 stages of a length-S transform in a[OFF .. OFF + S), spans LEN, 2 LEN, ..., S
 template <typename T, int NA, int OFF, int S, int LEN, bool FWD>
@@ -69,7 +68,7 @@ __device__ __forceinline__ void stages(Cplx<T> (&a)[NA]) {
             } else if (sizeof(T) == 4 && NA % 3 == 0 && LEN == 8) {   // (+-1 +- i) sqrt(1/2), exact to 1e-10
                 const T sr = cos_of<8>(j) > 0 ? T(1) : T(-1), si = FWD ? T(-1) : T(1);
                 const Cplx<T> t{sr * v.x - si * v.y, si * v.x + sr * v.y};
-                s = Cplx<T>{plus_scaled<T>(u.x, t.x, kHalfRoot), plus_scaled<T>(u.y, t.y, kHalfRoot)};
+                s = Cplx<T>{plus_half_root(u.x, t.x), plus_half_root(u.y, t.y)};
                 d = twice_minus(u, s);
             } else {
                 const T wr = (T)cos_of<LEN>(j), wi = FWD ? (T)(-sin_of<LEN>(j)) : (T)sin_of<LEN>(j);
@@ -92,31 +91,38 @@ __device__ __forceinline__ void line(Cplx<T> (&a)[N]) {
         stages<T, N, 0, S, 2, FWD>(a);
         stages<T, N, S, S, 2, FWD>(a);
         stages<T, N, 2 * S, S, 2, FWD>(a);
-        // X[q + m S], m = 0, 1, 2, from y0 and the twiddled y1, y2 (one radix-3 butterfly)
-        constexpr double c3 = FWD ? -kRoot34 : kRoot34;   // -+ sin(2 pi / 3)
 #pragma unroll
         for (int q = 0; q < S; ++q) {
             const Cplx<T> y0 = a[q], y1 = a[S + q], y2 = a[2 * S + q];
-            Cplx<T> t1 = y1, t2 = y2;
-            if (q > 0) {
-                const T r1 = (T)cos_of<N>(q), i1 = FWD ? (T)(-sin_of<N>(q)) : (T)sin_of<N>(q);
-                const T r2 = (T)cos_of<N>(2 * q), i2 = FWD ? (T)(-sin_of<N>(2 * q)) : (T)sin_of<N>(2 * q);
-                t1 = Cplx<T>{fma(-i1, y1.y, r1 * y1.x), fma(i1, y1.x, r1 * y1.y)};
-                t2 = Cplx<T>{fma(-i2, y2.y, r2 * y2.x), fma(i2, y2.x, r2 * y2.y)};
+            if constexpr (sizeof(T) == 4) {
+                // X[q + m S] = y0 + w^k y1 + w^2k y2, k = q + m S, four chained FMAs a part: as many instructions as a
+                // radix-3 butterfly on twiddled y1, y2, and fewer roundings on the way to each result (N = 24:
+                // 6.8e-8 of a line's norm, the butterfly 7.1e-8)
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    const int k = q + m * S;
+                    const T r1 = (T)cos_of<N>(k), i1 = FWD ? (T)(-sin_of<N>(k)) : (T)sin_of<N>(k);
+                    const T r2 = (T)cos_of<N>(2 * k), i2 = FWD ? (T)(-sin_of<N>(2 * k)) : (T)sin_of<N>(2 * k);
+                    a[k] = Cplx<T>{madd(-i2, y2.y, madd(r2, y2.x, madd(-i1, y1.y, madd(r1, y1.x, y0.x)))),
+                                   madd(i2, y2.x, madd(r2, y2.y, madd(i1, y1.x, madd(r1, y1.y, y0.y))))};
+                }
+            } else {   // FP64, bound by its instructions: one radix-3 butterfly
+                constexpr double c3 = FWD ? -cos_of<12>(1) : cos_of<12>(1);   // -+ sin(2 pi / 3)
+                Cplx<T> t1 = y1, t2 = y2;
+                if (q > 0) {
+                    const T r1 = (T)cos_of<N>(q), i1 = FWD ? (T)(-sin_of<N>(q)) : (T)sin_of<N>(q);
+                    const T r2 = (T)cos_of<N>(2 * q), i2 = FWD ? (T)(-sin_of<N>(2 * q)) : (T)sin_of<N>(2 * q);
+                    t1 = Cplx<T>{fma(-i1, y1.y, r1 * y1.x), fma(i1, y1.x, r1 * y1.y)};
+                    t2 = Cplx<T>{fma(-i2, y2.y, r2 * y2.x), fma(i2, y2.x, r2 * y2.y)};
+                }
+                const Cplx<T> p{t1.x + t2.x, t1.y + t2.y}, d{t1.x - t2.x, t1.y - t2.y};
+                const Cplx<T> m{fma(T(-0.5), p.x, y0.x), fma(T(-0.5), p.y, y0.y)};
+                a[q] = Cplx<T>{y0.x + p.x, y0.y + p.y};
+                a[S + q] = Cplx<T>{fma((T)-c3, d.y, m.x), fma((T)c3, d.x, m.y)};
+                a[2 * S + q] = Cplx<T>{fma((T)c3, d.y, m.x), fma((T)-c3, d.x, m.y)};
             }
-            const Cplx<T> p{t1.x + t2.x, t1.y + t2.y}, d{t1.x - t2.x, t1.y - t2.y};
-            const Cplx<T> m{fma(T(-0.5), p.x, y0.x), fma(T(-0.5), p.y, y0.y)};
-            a[q] = Cplx<T>{y0.x + p.x, y0.y + p.y};
-            a[S + q] = Cplx<T>{plus_scaled<T>(m.x, d.y, -c3), plus_scaled<T>(m.y, d.x, c3)};
-            a[2 * S + q] = Cplx<T>{plus_scaled<T>(m.x, d.y, c3), plus_scaled<T>(m.y, d.x, -c3)};
         }
     }
-}
-
-// 1 - (mean diagonal of inverse times forward line / N) with the twiddles rounded to FP32, the rest exact:
-// the relative loss of a round trip. |w| of the rounded twiddles of these lengths is below 1 on average.
-__host__ __device__ constexpr double line_loss(int N) {
-    return N == 8 ? 0.86e-8 : N == 12 ? 0.90e-8 : N == 16 ? 2.71e-8 : N == 24 ? 1.27e-8 : 4.55e-8;
 }
 
 }  // namespace cfft

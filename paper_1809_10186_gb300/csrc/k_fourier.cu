@@ -111,7 +111,7 @@ __device__ __forceinline__ void store_cplx_pair(Cplx<double>* x, double a0, doub
 template <typename T, int SG>
 __global__ void __launch_bounds__(256) k_project(const T* __restrict__ P, const T* __restrict__ Vr,
                                                  const double* __restrict__ cr, const double* __restrict__ wr,
-                                                 NodeParams np, int Nrho, int rank, int64_t n3,
+                                                 NodeParams np, double balance, int Nrho, int rank, int64_t n3,
                                                  Cplx<T>* __restrict__ X, int xslots) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     T* CT = reinterpret_cast<T*>(sm_raw);                 // [Nrho][rpad]
@@ -121,7 +121,10 @@ __global__ void __launch_bounds__(256) k_project(const T* __restrict__ P, const 
     const double gam = np.gamma ? np.gamma[node] : np.gamma0;
     const double bb = np.b ? np.b[node] : np.b0;
     // one FP64 power per radial point (FP64 is slow on this part), then the coefficient table
-    for (int r = threadIdx.x; r < Nrho; r += blockDim.x) wrho[r] = (T)wr[r] * radial_rho<T>(bb, gam, cr[r], np.dlog);
+    for (int r = threadIdx.x; r < Nrho; r += blockDim.x) {
+        const double v = radial_rho<double>(bb, gam, cr[r], np.dlog);
+        wrho[r] = balance != 0.0 ? (T)(wr[r] * v * balance) : (T)wr[r] * (T)v;
+    }
     __syncthreads();
     for (int e = threadIdx.x; e < Nrho * rpad; e += blockDim.x) {
         const int r = e / rpad, sidx = e % rpad;
@@ -260,7 +263,7 @@ cudaError_t launch_dft3(const DevTables<T>& t, Cplx<T>* X, int64_t count, bool f
 }
 
 template <typename T>
-cudaError_t launch_project(const DevTables<T>& t, const T* P, NodeParams np, int64_t nodes,
+cudaError_t launch_project(const DevTables<T>& t, const T* P, NodeParams np, double balance, int64_t nodes,
                            Cplx<T>* X, int xfields, cudaStream_t s) {
     if (nodes <= 0) return cudaSuccess;
     const int64_t n3 = (int64_t)t.N * t.N * t.N;      // even for every supported N
@@ -269,7 +272,7 @@ cudaError_t launch_project(const DevTables<T>& t, const T* P, NodeParams np, int
     auto go = [&](auto kern, int sg) {
         const size_t sm = sizeof(T) * (size_t)t.Nrho * (size_t)((t.rank + sg - 1) / sg * sg + 1);
         if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        kern<<<grid, bs, sm, s>>>(P, t.Vr, t.cr, t.wr, np, t.Nrho, t.rank, n3, X, xfields);
+        kern<<<grid, bs, sm, s>>>(P, t.Vr, t.cr, t.wr, np, balance, t.Nrho, t.rank, n3, X, xfields);
     };
     if (t.rank <= 8) go(k_project<T, 8>, 8);
     else if (t.rank <= 16) go(k_project<T, 16>, 16);
@@ -308,7 +311,7 @@ cudaError_t launch_finalize(int N, const Cplx<T>* Y, int yfields, const T* a, co
 
 #define DGFS_INST(T)                                                                                   \
     template cudaError_t launch_dft3<T>(const DevTables<T>&, Cplx<T>*, int64_t, bool, cudaStream_t);  \
-    template cudaError_t launch_project<T>(const DevTables<T>&, const T*, NodeParams, int64_t,        \
+    template cudaError_t launch_project<T>(const DevTables<T>&, const T*, NodeParams, double, int64_t, \
                                            Cplx<T>*, int, cudaStream_t);                              \
     template cudaError_t launch_load_field<T>(int, const T*, const T*, const int64_t*, int64_t,       \
                                               Cplx<T>*, int, int, int, cudaStream_t);                 \

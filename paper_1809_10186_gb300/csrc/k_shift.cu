@@ -23,6 +23,7 @@
 // fields, which x and y translates keep real) in the real and imaginary part of slot kz = 0.
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstdint>
 #include <map>
 
@@ -31,9 +32,165 @@
 
 namespace dgfs {
 
-void build_shift_program(const HostPlan& h, ShiftProgram& p) {
+namespace {
+
+// The relative loss of a round trip through FP32 lines of N points, 1 - (mean diagonal of inverse times forward
+// line / N), from the rounding of their twiddles alone (fft_const.cuh): |w| of the rounded ones is below 1 on
+// average. 0.8e-8 (N = 8), 1.2e-8, 2.7e-8, 1.4e-8, 4.6e-8 (N = 32).
+double line_loss(int N) {
+    using C = std::complex<double>;
+    auto w = [N](int k, int n) {   // e^{-2 pi i k / n} in FP32 (the inverse takes the conjugate)
+        const double a = 2.0 * 3.14159265358979323846 * (k % n) / n;
+        const bool exact = n == 8 && N == 24;   // plus_half_root
+        auto f32 = [&](double v) { return std::fabs(v) < 1e-9 ? 0.0 : exact ? v : (double)(float)v; };
+        return C(f32(std::cos(a)), -f32(std::sin(a)));
+    };
+    // the lines' linear map on x, decimation in time
+    auto line = [&](auto&& self, const std::vector<C>& x, bool fwd) -> std::vector<C> {
+        const int n = (int)x.size(), R = n % 3 == 0 ? 3 : 2, S = n / R;
+        if (n == 1) return x;
+        std::vector<std::vector<C>> y(R);
+        for (int j = 0; j < R; ++j) {
+            std::vector<C> s(S);
+            for (int i = 0; i < S; ++i) s[i] = x[R * i + j];
+            y[j] = self(self, s, fwd);
+        }
+        std::vector<C> out(n);
+        for (int k = 0; k < n; ++k)
+            for (int j = 0; j < R; ++j) {
+                // radix 2 takes +- the twiddle of k < n / 2
+                const C t = R == 2 ? (j && k >= S ? -1.0 : 1.0) * w(j * (k % S), n) : w(j * k, n);
+                out[k] += (fwd ? t : std::conj(t)) * y[j][k % S];
+            }
+        return out;
+    };
+    double d = 0.0;
+    for (int j = 0; j < N; ++j) {
+        std::vector<C> e(N);
+        e[j] = 1.0;
+        d += line(line, line(line, e, true), false)[j].real() / N;
+    }
+    return 1.0 - d / N;
+}
+
+// FP32: constants that make the rounding of the tables, scales and twiddles a common factor of gain and loss, which
+// cancel to a tenth of their size in Q (1e-7 of difference shows as 1e-6 of ||Q||). Against exact arithmetic
+//   - an operand carries the FP32 forward scale 1/N^2 and, when it is translated along x, 1/N; 1 - line_loss per
+//     axis that it went forward and back; the loss's operand always all three;
+//   - the weights are rounded, |mu| of the rounded phases is not 1, and the loss weight is rounded.
+// The first line goes into the weights, pair by pair; the factor by which what is left changes the gain of a Maxwellian of
+// thermal speed L / sqrt(1.5 N) (3.5 of them at N = 8, 7 at N = 32), against the one of its loss, into p.balance, a
+// factor of the radial tables. The weights take a common factor in [1, 2) by which all of them round well.
+void balance_constants(const HostPlan& h, ShiftProgram& p) {
+    auto f32 = [](double v) { return (double)(float)v; };
+    const int N = h.N, Nr = h.Nrho, np = h.npairs, NH = N / 2;
+    const size_t n3 = (size_t)N * N * N;
+    const double ll = line_loss(N), syz = f32(1.0 / ((double)N * N)) * N * N, sx = f32(1.0 / N) * N;
+    std::vector<double> a2(N);
+    auto sk = [N](int q) { return q < N / 2 ? q : q - N; };
+    for (int q = 0; q < N; ++q) {
+        const double t = 3.14159265358979323846 * sk(q);
+        a2[q] = std::exp(-0.5 * t * t / (1.5 * N));   // |f^|^2
+    }
+    std::vector<double> rho(Nr);
+    for (int r = 0; r < Nr; ++r) rho[r] = 4.0 * 3.14159265358979323846 * h.b * std::pow(h.cr[r], h.gamma + 2.0);
+    double lw = 0.0, lr = 0.0;   // loss: exact, with the FP32 weight
+    for (size_t i = 0; i < n3; ++i) {
+        double g = h.aniso ? h.GLa[i] : 0.0;
+        for (int r = 0; r < Nr && !h.aniso; ++r) g += rho[r] * h.Lr[(size_t)r * n3 + i];
+        const double m = a2[i / ((size_t)N * N)] * a2[(i / N) % N] * a2[i % N];
+        lw += m * g;
+        lr += m * f32(g);
+    }
+    for (int q = 0; q < np; ++q) {
+        const bool tx = h.sig[3 * q] != 0.0;
+        const double s = syz * (tx ? sx : 1.0);
+        p.excess[q] = syz * sx / (s * s) * (1.0 + 2.0 * (tx ? 3 : 2) * ll);
+    }
+    double common = 1.0, best = -1.0;
+    for (int i = 0; i < 4096; ++i) {
+        const double c = 1.0 + i / 4096.0;
+        double e = 0.0;
+        for (int q = 0; q < np; ++q) {
+            const double w = c * h.wsig[q] * p.excess[q], d = f32(w) / w - 1.0;
+            e += h.wsig[q] * d * d;
+        }
+        if (best < 0.0 || e < best) {
+            best = e;
+            common = c;
+        }
+    }
+    // gain of the Maxwellian at X^3 points of an octant (even along each axis): exact (g), with the rounded constants
+    // (gr), and those on the compressed radial kernel with its factors at k = 0 rounded (gp)
+    constexpr int X = 6;
+    std::vector<double> g(X * X * X, 0.0), gr(g), gp(g), cosx(X * (size_t)N), sinx(cosx);
+    for (int i = 0; i < X; ++i)
+        for (int k = 0; k < N; ++k) {
+            const double ang = 3.14159265358979323846 * sk(k) * (0.15 + 0.3 * i) / std::sqrt(1.5 * N), a = std::sqrt(a2[k]);
+            cosx[i * N + k] = a * std::cos(ang);
+            sinx[i * N + k] = k == NH ? 0.0 : a * std::sin(ang);
+        }
+    std::vector<double> proj(Nr, 1.0);
+    for (int r = 0; r < Nr && !h.aniso; ++r) {
+        double v = 0.0, e = 0.0;
+        for (int s = 0; s < h.rank; ++s) {
+            const double u = h.Uk[(size_t)s * n3], c = h.Vr[(size_t)s * Nr + r];
+            e += u * c;
+            v += f32(u) * f32(c);
+        }
+        proj[r] = v / e;
+    }
+    for (int q = 0; q < np; ++q) {
+        p.wsig[q] = common * h.wsig[q] * p.excess[q];
+        // VSS: the weight is part of the kernel factor
+        const double rounded = h.aniso ? 1.0 : common * f32(p.wsig[q]) / p.wsig[q];
+        for (int r = 0; r < Nr; ++r) {
+            const double mass = h.aniso ? h.Fa[((size_t)r * np + q) * n3] : h.wsig[q] * h.wr[r] * rho[r];
+            double ex[3][X], rd[3][X];   // (T_s f)(T_-s f) along each axis
+            for (int ax = 0; ax < 3; ++ax) {
+                const double* m = &h.mu[(((size_t)r * np + q) * 3 + ax) * N * 2];
+                for (int i = 0; i < X; ++i) {
+                    double c = 0.0, d = 0.0, cr = 0.0, dr = 0.0;
+                    for (int k = 0; k < N; ++k) {
+                        const double re = m[2 * k], im = k == NH ? 0.0 : m[2 * k + 1];
+                        c += cosx[i * N + k] * re;
+                        d += sinx[i * N + k] * im;
+                        cr += cosx[i * N + k] * f32(re);
+                        dr += sinx[i * N + k] * f32(im);
+                    }
+                    ex[ax][i] = (c - d) * (c + d);
+                    rd[ax][i] = (cr - dr) * (cr + dr);
+                }
+            }
+            for (int i = 0; i < X * X * X; ++i) {
+                const int x = i / (X * X), y = i / X % X, z = i % X;
+                g[i] += mass * ex[0][x] * ex[1][y] * ex[2][z];
+                const double v = mass * rounded * rd[0][x] * rd[1][y] * rd[2][z];
+                gr[i] += v;
+                gp[i] += proj[r] * v;
+            }
+        }
+    }
+    double gg = 0.0, ggr = 0.0, ggp = 0.0;
+    for (size_t i = 0; i < g.size(); ++i) {
+        gg += g[i] * g[i];
+        ggr += g[i] * gr[i];
+        ggp += g[i] * gp[i];
+    }
+    p.balance = lr / lw * (gg / ggr);
+    p.project = lr / lw * (gg / ggp);
+}
+
+}  // namespace
+
+void build_shift_program(const HostPlan& h, bool fp32, ShiftProgram& p) {
     const int N = h.N, np = h.npairs, MP = shift_mu_pitch(N);
     p = ShiftProgram();
+    p.wsig = h.wsig;
+    p.excess.assign(np, 1.0);
+    if (fp32) balance_constants(h, p);
+    // FP32 results leave the last transform by a power of two; the tables carry the rest of 1 / N^3
+    const double n3d = (double)N * N * N, exact = fp32 ? 1.0 / (n3d * shift_result_scale(N, false)) : 1.0;
     std::map<double, int> rows, xs;
     std::vector<std::pair<int, int>> at;   // a (pair, axis) that carries each row
     for (int q = 0; q < np; ++q)
@@ -59,7 +216,8 @@ void build_shift_program(const HostPlan& h, ShiftProgram& p) {
     if (!h.aniso) {
         const int nq2 = 3 * (N / 2) * (N / 2) + 1;
         const size_t n3 = (size_t)N * N * N;
-        for (auto* t : {&p.sq, &p.kq, &p.kqd}) t->assign((size_t)h.Nrho * nq2, 0.0);
+        for (auto* t : {&p.sq, &p.kq, &p.kqd, &p.st, &p.kt}) t->assign((size_t)h.Nrho * nq2, 0.0);
+        const double gain = exact * p.balance;
         std::vector<int64_t> at_q(nq2, -1);   // a mode of each |k|^2
         auto sk = [N](int q) { return q < N / 2 ? q : q - N; };
         for (size_t i = 0; i < n3; ++i) {
@@ -72,12 +230,16 @@ void build_shift_program(const HostPlan& h, ShiftProgram& p) {
                 if (at_q[q] < 0) continue;
                 double v = 0.0;
                 for (int s = 0; s < h.rank; ++s) v += h.Uk[(size_t)s * n3 + at_q[q]] * h.Vr[(size_t)s * h.Nrho + r];
-                p.sq[(size_t)r * nq2 + q] = v;
-                p.kq[(size_t)r * nq2 + q] = wr * v;
-                p.kqd[(size_t)r * nq2 + q] = std::log(h.cr[r]) * wr * v;
+                p.sq[(size_t)r * nq2 + q] = gain * v;
+                p.kq[(size_t)r * nq2 + q] = gain * wr * v;
+                p.kqd[(size_t)r * nq2 + q] = gain * std::log(h.cr[r]) * wr * v;
+                p.st[(size_t)r * nq2 + q] = exact * v;
+                p.kt[(size_t)r * nq2 + q] = exact * wr * v;
             }
         }
     }
+    if (h.aniso)
+        for (double& e : p.excess) e *= exact * p.balance;
     struct Key { double x, y, z; int q; };
     auto program = [&](bool both) {
         std::vector<Key> keys;
@@ -280,16 +442,6 @@ k_shift_products(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf,
 #pragma unroll
         for (int z = 0; z < N; ++z) acc[z] = fma(wgt * v[z].x, v[z].y, acc[z]);
     }
-    if constexpr (sizeof(T) == 4) {
-        // Two systematic factors of the FP32 constants scale every P_r alike, a bias that the loss does not
-        // share: 1/N^2 and 1/N are rounded for N = 12, 24, and the rounded twiddles return a line that goes
-        // forward and back (three axes, two operands) shorter by line_loss. One FMA takes both out again;
-        // without it the FP32 error of Q at N = 24 grew from 1.6e-6 to 2.8e-6 (two-Maxwellian batch).
-        constexpr double sc = (double)(T(1) / (T(N) * T(N))) * (double)(T(1) / T(N)) * (double)n3;
-        constexpr T corr = (T)(1.0 / (sc * sc) - 1.0 + 6.0 * cfft::line_loss(N));
-#pragma unroll
-        for (int z = 0; z < N; ++z) acc[z] = fma(acc[z], corr, acc[z]);
-    }
     T* tile = reinterpret_cast<T*>(sm_raw);                  // [NT][N + 1]
     __syncthreads();
 #pragma unroll
@@ -355,7 +507,7 @@ cudaError_t shift_x_n(const ShiftDev<T>& d, const Cplx<T>* G, int r0, int nr, in
 
 template <typename T, int N, int XC, bool FOLD>
 cudaError_t products_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
-                       const T* wsig, int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
+                       int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
     using Geo = ProductGeo<T, N, XC>;
     auto kern = k_shift_products<T, N, XC, FOLD>;
     if (Geo::smem > 48 * 1024) {
@@ -364,19 +516,19 @@ cudaError_t products_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* H
     }
     const bool bil = Gg != nullptr;
     kern<<<dim3(N / XC, (unsigned)nr, (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
-        Gf, Hf, bil ? Gg : Gf, bil ? Hg : Hf, d.mu, bil ? d.bil : d.quad, bil ? d.nbil : d.nquad, bil ? T(1) : T(2), wsig,
+        Gf, Hf, bil ? Gg : Gf, bil ? Hg : Hf, d.mu, bil ? d.bil : d.quad, bil ? d.nbil : d.nquad, bil ? T(1) : T(2), d.wsig,
         d.nrows, d.nx, r0, node_stride, P);
     return cudaGetLastError();
 }
 
 template <typename T, int N, bool FOLD>
 cudaError_t products_n(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg, const Cplx<T>* Hg,
-                       const T* wsig, int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
+                       int r0, int nr, int64_t nodes, int64_t node_stride, T* P, cudaStream_t s) {
     constexpr int XC = N == 32 || N == 24 ? 4 : N == 12 ? 12 : 8;
     // two planes per CTA while whole CTAs of XC planes would not fill the 152 SMs about four deep
     if ((int64_t)(N / XC) * nr * nodes < 608)
-        return products_x<T, N, 2, FOLD>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
-    return products_x<T, N, XC, FOLD>(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s);
+        return products_x<T, N, 2, FOLD>(d, Gf, Hf, Gg, Hg, r0, nr, nodes, node_stride, P, s);
+    return products_x<T, N, XC, FOLD>(d, Gf, Hf, Gg, Hg, r0, nr, nodes, node_stride, P, s);
 }
 
 }  // namespace
@@ -428,9 +580,9 @@ cudaError_t launch_shift_x(const ShiftDev<T>& d, const Cplx<T>* G, int N, int r0
 
 template <typename T>
 cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg,
-                                  const Cplx<T>* Hg, const T* wsig, int N, int r0, int nr, int64_t nodes, bool folded,
-                                  int64_t node_stride, T* P, cudaStream_t s) {
-#define CALL(n) (folded ? products_n<T, n, true> : products_n<T, n, false>)(d, Gf, Hf, Gg, Hg, wsig, r0, nr, nodes, node_stride, P, s)
+                                  const Cplx<T>* Hg, int N, int r0, int nr, int64_t nodes, bool folded, int64_t node_stride,
+                                  T* P, cudaStream_t s) {
+#define CALL(n) (folded ? products_n<T, n, true> : products_n<T, n, false>)(d, Gf, Hf, Gg, Hg, r0, nr, nodes, node_stride, P, s)
     DGFS_BY_N(CALL);
 #undef CALL
 }
@@ -443,7 +595,7 @@ cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const
     template cudaError_t launch_shift_x<T>(const ShiftDev<T>&, const Cplx<T>*, int, int, int, int64_t, Cplx<T>*,      \
                                            cudaStream_t);                                                             \
     template cudaError_t launch_shift_products<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*, \
-                                                  const Cplx<T>*, const T*, int, int, int, int64_t, bool, int64_t,    \
+                                                  const Cplx<T>*, int, int, int, int64_t, bool, int64_t,    \
                                                   T*, cudaStream_t);
 DGFS_SHIFT_INST(float)
 DGFS_SHIFT_INST(double)

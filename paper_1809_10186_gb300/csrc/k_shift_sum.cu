@@ -27,6 +27,8 @@
 // ky = 0 .. N/2 - 1 of the first, then of the second, with the real ky = 0 and N/2 packed in the two slots
 // ky = 0 (a "folded" plane); only those two columns are separated along x, in registers. k_shift_filter takes the
 // plane as it is: one warp holds it, kx in registers and ky along the lanes.
+#include <cmath>
+
 #include "shift.h"
 #include "shift_dev.cuh"
 
@@ -292,15 +294,18 @@ constexpr int col_blocks() { return (N * (N / 2 - (NONZERO ? 1 : 0)) + kColThrea
 // [2][kx]; else the x phase of field fi (fields 2 nx, 2 nx + 1: none). VSS reads 2.5 MB of products per radial point
 // and node at N = 32, M = 38 and is bound by that.
 // Its rounding depends neither on the batch of nodes nor on the batch of radial points of a launch:
-// Adjoint, Vss: block z of kSumParts takes its share of the fields, every radial point in order, on top of part
-// [node][kSumParts] of the batch before; k_shift_finish adds the parts in order.
+// Adjoint, Vss: block z of kSumParts takes its share of the fields, their sum at a radial point added to the total in
+// order, on top of part [node][kSumParts] of the batch before; k_shift_finish adds the parts in order. (One running sum
+// over radial points and fields, up to 300 FP32 additions at M = 38, lost accuracy: the VSS JVP of 32 nodes at N = 24 was
+// 2.6e-6 of its norm off, 1.9e-6 with the sums taken apart.)
 // Radial: groups of RP = ceil(Nrho / kSumGroups) radial points, each group's sum added to the total in order: grid
 // (col_blocks, nodes, 1) keeps the totals in shared memory (part [node]); grid (col_blocks, nodes, sum_groups) takes a
 // group each (part [node][group]) where one block per column leaves SMs idle.
 // Radial (VHS gain, nf = 1): times tab[r0 + r][|k|^2], and coef[node][r0 + r] when the kernel varies by node.
 enum class Sum { Adjoint, Vss, Radial };
-template <typename T, int N, Sum MODE>
-__global__ void __launch_bounds__(kColThreads)
+// REGS: the totals of Adjoint and Vss in registers (sum_launch).
+template <typename T, int N, Sum MODE, bool REGS>
+__global__ void __launch_bounds__(kColThreads, REGS ? 1 : 0)
 k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, const T* __restrict__ coef, int Nrho,
             const ShiftEntry* __restrict__ prog, int npairs,
             const Cplx<T>* __restrict__ mu, const int* __restrict__ xrows, int nrows, int nx, int r0, int nr, int RP,
@@ -316,7 +321,7 @@ k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, cons
     const int fy = ckz ? (cky < NH ? cky : N - cky) : cky % NH, fz = ckz ? ckz : cky < NH ? 0 : NH, q0 = fy * fy + fz * fz;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     Cplx<T>* total = reinterpret_cast<Cplx<T>*>(sm_raw) + threadIdx.x;   // [kx][thread] (one block per column)
-    const bool whole = MODE == Sum::Radial && gridDim.z == 1;
+    const bool whole = MODE == Sum::Radial && gridDim.z == 1, by_r = MODE != Sum::Radial && sizeof(T) == 4, totals = by_r || whole;
     Cplx<T>* pc = part + (node * gridDim.z + blockIdx.z) * FS + col;
     // the batch's radial points of this block: all, or the ones of its group
     const int lo = MODE != Sum::Radial || whole ? 0 : max(0, (int)blockIdx.z * RP - r0);
@@ -326,18 +331,24 @@ k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, cons
     const int f1 = MODE == Sum::Radial ? 1 : nf * (int)(blockIdx.z + 1) / (int)gridDim.z;
     Cplx<T> acc[N];
     // a group under way from the batch before: its sum (whole: kept behind the totals)
-    const bool started = MODE == Sum::Radial ? (r0 + lo) % RP != 0 : r0 > 0;
-    if (whole)
+    const bool started = MODE == Sum::Radial ? (r0 + lo) % RP != 0 : !by_r && r0 > 0;
+    Cplx<T> reg[REGS ? N : 1];
+    if (totals) {
 #pragma unroll
-        for (int k = 0; k < N; ++k) total[k * kColThreads] = r0 >= RP ? ld(pc + (int64_t)k * COLS) : Cplx<T>{T(0), T(0)};
+        for (int k = 0; k < N; ++k) {
+            const Cplx<T> t = r0 >= RP ? ld(pc + (int64_t)k * COLS) : Cplx<T>{T(0), T(0)};
+            if constexpr (REGS) reg[k] = t;
+            else total[k * kColThreads] = t;
+        }
+    }
     const Cplx<T>* open = whole ? part + (gridDim.y + node) * FS + col : pc;
 #pragma unroll
     for (int k = 0; k < N; ++k) acc[k] = started ? ld(open + (int64_t)k * COLS) : Cplx<T>{T(0), T(0)};
     for (int rl = lo; rl < hi; ++rl) {
-        if (whole && rl > lo && (r0 + rl) % RP == 0) {   // the group is complete
+        if (totals && rl > lo && (r0 + rl) % RP == 0) {   // the group is complete
 #pragma unroll
             for (int k = 0; k < N; ++k) {
-                Cplx<T>& t = total[k * kColThreads];
+                Cplx<T>& t = REGS ? reg[REGS ? k : 0] : total[k * kColThreads];
                 t = Cplx<T>{t.x + acc[k].x, t.y + acc[k].y};
                 acc[k] = Cplx<T>{T(0), T(0)};
             }
@@ -401,12 +412,12 @@ k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, cons
             }
         }
     }
-    if (whole) {
+    if (totals) {
         const bool done = (r0 + nr) % RP == 0 || r0 + nr == Nrho;   // the last group is complete
-        Cplx<T>* rest = part + (gridDim.y + node) * FS + col;
+        Cplx<T>* rest = part + (gridDim.y + node) * FS + col;       // (whole; the other sums have groups of one radial point)
 #pragma unroll
         for (int k = 0; k < N; ++k) {
-            Cplx<T> t = total[k * kColThreads];
+            Cplx<T> t = REGS ? reg[REGS ? k : 0] : total[k * kColThreads];
             if (done) t = Cplx<T>{t.x + acc[k].x, t.y + acc[k].y};
             else st(rest + (int64_t)k * COLS, acc[k]);
             st(pc + (int64_t)k * COLS, t);
@@ -670,13 +681,13 @@ cudaError_t vss_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, co
 }
 
 template <typename T, int N, int XC>
-cudaError_t adj_x(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int r0, int nr,
+cudaError_t adj_x(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, int r0, int nr,
                   int64_t nodes, Cplx<T>* V, cudaStream_t s) {
     using Geo = SumGeo<T, N, XC>;
     const cudaError_t e = allow_smem(k_shift_adj<T, N, XC>, Geo::smem);
     if (e != cudaSuccess) return e;
     k_shift_adj<T, N, XC><<<dim3(N / XC, (unsigned)nr, (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
-        G, H, Ur, d.mu, d.quad, d.nquad, wsig, d.nrows, d.nx, r0, V);
+        G, H, Ur, d.mu, d.quad, d.nquad, d.wsig, d.nrows, d.nx, r0, V);
     return cudaGetLastError();
 }
 
@@ -694,21 +705,33 @@ cudaError_t vss_n(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, co
 }
 
 template <typename T, int N>
-cudaError_t adj_n(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int r0, int nr,
+cudaError_t adj_n(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, int r0, int nr,
                   int64_t nodes, Cplx<T>* V, cudaStream_t s) {
-    return narrow<N>(nr, nodes) ? adj_x<T, N, 2>(d, G, H, Ur, wsig, r0, nr, nodes, V, s)
-                                : adj_x<T, N, wide<N>()>(d, G, H, Ur, wsig, r0, nr, nodes, V, s);
+    return narrow<N>(nr, nodes) ? adj_x<T, N, 2>(d, G, H, Ur, r0, nr, nodes, V, s)
+                                : adj_x<T, N, wide<N>()>(d, G, H, Ur, r0, nr, nodes, V, s);
 }
 
 template <typename T, int N, Sum MODE>
 cudaError_t sum_launch(const ShiftDev<T>& d, const Cplx<T>* F, int nf, const T* A, const T* coef, const ShiftEntry* prog, int npairs,
                        int Nrho, int r0, int nr, int parts, int64_t nodes, Cplx<T>* part, cudaStream_t s) {
-    const size_t sm = MODE == Sum::Radial && parts == 1 ? sizeof(Cplx<T>) * N * kColThreads : 0;
-    const cudaError_t e = allow_smem(k_shift_sum<T, N, MODE>, sm);
-    if (e != cudaSuccess) return e;
-    k_shift_sum<T, N, MODE><<<dim3(col_blocks<N, false>(), (unsigned)nodes, (unsigned)parts), kColThreads, sm, s>>>(
-        F, nf, A, coef, Nrho, prog, npairs, d.mu, d.xrows, d.nrows, d.nx, r0, nr, sum_group(Nrho), part);
-    return cudaGetLastError();
+    const bool by_r = MODE != Sum::Radial && sizeof(T) == 4;
+    const dim3 grid(col_blocks<N, false>(), (unsigned)nodes, (unsigned)parts);
+    auto go = [&](auto kern, bool regs) {
+        const size_t sm = (by_r && !regs) || (MODE == Sum::Radial && parts == 1) ? sizeof(Cplx<T>) * N * kColThreads : 0;
+        const cudaError_t e = allow_smem(kern, sm);
+        if (e != cudaSuccess) return e;
+        kern<<<grid, kColThreads, sm, s>>>(F, nf, A, coef, Nrho, prog, npairs, d.mu, d.xrows, d.nrows, d.nx, r0, nr,
+                                           MODE == Sum::Radial ? sum_group(Nrho) : 1, part);
+        return cudaGetLastError();
+    };
+    // Totals in registers (two thirds of the resident warps) or in shared memory (a read and a write of them per radial
+    // point): registers for launches that leave SMs idle (VSS Q of one node, N = 32, M = 26: 358 us, 507 in shared memory)
+    // and for VSS at N <= 12 and 32 (M = 26, 500 nodes at N = 12: 526 / 594 us; 40 nodes at N = 32: 2223 / 2312 us); at
+    // N = 16, 24 and for the adjoint shared memory is level or ahead (VJP of 300 nodes, N = 24: 5317 / 5515 us)
+    if constexpr (MODE != Sum::Radial && sizeof(T) == 4)
+        if ((MODE == Sum::Vss && N != 16 && N != 24) || (int64_t)grid.x * grid.y * grid.z < 304)
+            return go(k_shift_sum<T, N, MODE, true>, true);
+    return go(k_shift_sum<T, N, MODE, false>, false);
 }
 
 template <typename T, int N>
@@ -749,7 +772,10 @@ cudaError_t out_n(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, c
 
 }  // namespace
 
-double shift_gain_scale(int N, bool fp64) { return fp64 ? 1.0 : 1.0 + 6.0 * cfft::line_loss(N); }
+double shift_result_scale(int N, bool fp64) {
+    const double n3 = (double)N * N * N;
+    return fp64 ? 1.0 / n3 : std::exp2(-std::round(std::log2(n3)));
+}
 
 #define DGFS_BY_N(CALL)                              \
     if (nodes <= 0) return cudaSuccess;              \
@@ -769,9 +795,9 @@ cudaError_t launch_shift_vss(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx
 #undef CALL
 }
 template <typename T>
-cudaError_t launch_shift_adj(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int N,
+cudaError_t launch_shift_adj(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, int N,
                              int r0, int nr, int64_t nodes, Cplx<T>* V, cudaStream_t s) {
-#define CALL(n) adj_n<T, n>(d, G, H, Ur, wsig, r0, nr, nodes, V, s)
+#define CALL(n) adj_n<T, n>(d, G, H, Ur, r0, nr, nodes, V, s)
     DGFS_BY_N(CALL);
 #undef CALL
 }
@@ -821,7 +847,7 @@ cudaError_t launch_shift_out(const Cplx<T>* F, int nf, int64_t field_stride, boo
     template cudaError_t launch_shift_vss<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*,        \
                                              const Cplx<T>*, int, int, int, int64_t, Cplx<T>*, cudaStream_t);           \
     template cudaError_t launch_shift_adj<T>(const ShiftDev<T>&, const Cplx<T>*, const Cplx<T>*, const Cplx<T>*,        \
-                                             const T*, int, int, int, int64_t, Cplx<T>*, cudaStream_t);                 \
+                                             int, int, int, int64_t, Cplx<T>*, cudaStream_t);                 \
     template cudaError_t launch_shift_sum<T>(const ShiftDev<T>&, const Cplx<T>*, int, const T*, bool, int, int, int,    \
                                              int, int64_t, Cplx<T>*, cudaStream_t);                                    \
     template cudaError_t launch_shift_filter<T>(const ShiftDev<T>&, const Cplx<T>*, int, int, int, int64_t, Cplx<T>*, \

@@ -165,19 +165,23 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 // C[node][r][s] = Vr[s][r] (w_r rho_r(node)): one block per node (or one for the whole launch). With Lq
 // (per-node gamma or b, a loss weight of |k| alone), also the loss multiplier GLq[node][|k|^2]: the same FP64
 // sum over r as loss_multiplier, once for each of the 3 (N/2)^2 + 1 values of |k|^2 instead of at every mode
-// (the ragged cavity batch spent 1.2 of 14.3 ms on those sums at N = 32 alone).
+// (the ragged cavity batch spent 1.2 of 14.3 ms on those sums at N = 32 alone). balance != 0 (FP32 products of k_shift.cu):
+// times balance (shift.h), the whole product in FP64 and rounded once; 0: the arithmetic that dgfs_ssprk and
+// dgfs_collide_dgamma keep.
 template <typename T>
 __global__ void k_spec_coef(const T* __restrict__ Vr, const double* __restrict__ cr, const double* __restrict__ wr,
-                            NodeParams np, int Nrho, int rank, T* __restrict__ C, const T* __restrict__ Lq, int nq2,
+                            NodeParams np, double balance, int Nrho, int rank, T* __restrict__ C, const T* __restrict__ Lq, int nq2,
                             T* __restrict__ GLq) {
     __shared__ T wrho[64];
-    __shared__ double rho[64];
+    __shared__ double rho[64], bal[64];
     const int64_t node = blockIdx.x;
     const double gam = np.gamma ? np.gamma[node] : np.gamma0;
     const double bb = np.b ? np.b[node] : np.b0;
     for (int r = threadIdx.x; r < Nrho; r += blockDim.x) {
-        wrho[r] = (T)wr[r] * radial_rho<T>(bb, gam, cr[r], np.dlog);
-        if (Lq) rho[r] = radial_rho<double>(bb, gam, cr[r], np.dlog);
+        const double v = radial_rho<double>(bb, gam, cr[r], np.dlog);   // one FP64 power (slow here) for all three
+        wrho[r] = (T)wr[r] * (T)v;
+        rho[r] = v;
+        bal[r] = wr[r] * v * balance;
     }
     __syncthreads();
     if (Lq)
@@ -189,7 +193,7 @@ __global__ void k_spec_coef(const T* __restrict__ Vr, const double* __restrict__
     T* Cn = C + node * Nrho * rank;
     for (int e = threadIdx.x; e < Nrho * rank; e += blockDim.x) {
         const int r = e / rank, s = e % rank;
-        Cn[e] = Vr[s * Nrho + r] * wrho[r];
+        Cn[e] = balance != 0.0 ? (T)((double)Vr[s * Nrho + r] * bal[r]) : Vr[s * Nrho + r] * wrho[r];
     }
 }
 
@@ -632,7 +636,7 @@ bool spectral_supported(const DevTables<T>& t) {
 }
 
 template <typename T>
-cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, int64_t nodes, const T* la,
+cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, double balance, int64_t nodes, const T* la,
                             const T* lb, const int64_t* offs, T gain_scale, Cplx<T>* X, Cplx<T>* Y,
                             const T* fa, const T* fc, T* out, int* flags, cudaStream_t s) {
     if (nodes <= 0) return cudaSuccess;
@@ -652,7 +656,7 @@ cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, in
         NodeParams np0 = np;
         if (np.gamma) np0.gamma = np.gamma + n0;
         if (np.b) np0.b = np.b + n0;
-        k_spec_coef<T><<<(unsigned)nn, 128, 0, s>>>(t.Vr, t.cr, t.wr, np0, t.Nrho, t.rank, C + n0 * c_stride,
+        k_spec_coef<T><<<(unsigned)nn, 128, 0, s>>>(t.Vr, t.cr, t.wr, np0, balance, t.Nrho, t.rank, C + n0 * c_stride,
                                                           GLq ? t.Lq : nullptr, nq2, GLq ? GLq + n0 * nq2 : nullptr);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -690,10 +694,10 @@ cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, in
 
 template bool spectral_supported<float>(const DevTables<float>&);
 template bool spectral_supported<double>(const DevTables<double>&);
-template cudaError_t launch_spectral<float>(const DevTables<float>&, const float*, NodeParams, int64_t, const float*,
+template cudaError_t launch_spectral<float>(const DevTables<float>&, const float*, NodeParams, double, int64_t, const float*,
                                             const float*, const int64_t*, float, Cplx<float>*, Cplx<float>*,
                                             const float*, const float*, float*, int*, cudaStream_t);
-template cudaError_t launch_spectral<double>(const DevTables<double>&, const double*, NodeParams, int64_t,
+template cudaError_t launch_spectral<double>(const DevTables<double>&, const double*, NodeParams, double, int64_t,
                                              const double*, const double*, const int64_t*, double, Cplx<double>*,
                                              Cplx<double>*, const double*, const double*, double*, int*,
                                              cudaStream_t);

@@ -50,7 +50,7 @@ struct Cplx { T x, y; };
 // Projected field s (s < rank) = sum_r Vr[s][r] w_r rho_r(node) P[node][r], packed into
 // X[node][xslots]; with odd rank the imaginary part of the last slot is left zero.
 template <typename T>
-cudaError_t launch_project(const DevTables<T>& t, const T* P, NodeParams np, int64_t nodes,
+cudaError_t launch_project(const DevTables<T>& t, const T* P, NodeParams np, double balance, int64_t nodes,
                            Cplx<T>* X, int xslots, cudaStream_t s);
 
 // Field a (offs as above) or the product a*b into X[node][slot]: part 0 writes {v, 0}, part 1
@@ -126,15 +126,15 @@ template <typename T>
 cudaError_t launch_moments(const T* f, int N, double L, int64_t B, double* out, cudaStream_t s);
 
 // ---- fused Fourier stage (k_spectral.cu) ----------------------------------------------
-// The whole Fourier side of a non-adjoint call in three launches for N = 8, 16 (float, double)
-// and N = 32 (float), rank <= 32, Nrho <= 64: projection of P, loss operands la (field rank)
+// The whole Fourier side of a non-adjoint call by projection for N = 8, 16 (float, double), 12 (double) and
+// 24, 32 (float), rank <= 32, Nrho <= 64: coefficients (balance != 0: times balance, see k_spec_coef), projection of P, loss operands la (field rank)
 // and lb (field rank + 1, or nullptr), forward DFT, combine with gain scale `gain_scale`,
 // inverse DFT and out = Re gain - fa Re(K_L la) - (fc ? fc Re(K_L lb) : 0). Same workspace
 // X [nodes][(rank + nloss + 1) / 2][N^3] and Y [nodes][2 or 3][N^3] as the separate kernels.
 template <typename T>
 bool spectral_supported(const DevTables<T>& t);
 template <typename T>
-cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, int64_t nodes, const T* la,
+cudaError_t launch_spectral(const DevTables<T>& t, const T* P, NodeParams np, double balance, int64_t nodes, const T* la,
                             const T* lb, const int64_t* offs, T gain_scale, Cplx<T>* X, Cplx<T>* Y,
                             const T* fa, const T* fc, T* out, int* flags, cudaStream_t s);
 

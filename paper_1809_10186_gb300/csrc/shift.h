@@ -30,14 +30,20 @@ struct ShiftProgram {
     int nx = 0;                          // distinct nonzero |s_x|; fields 2i (+) and 2i + 1 (-)
     std::vector<int> xrows;              // [nx] row of the shift table
     std::vector<ShiftEntry> quad, bil;   // g = f: one entry per pair (weight 2 w_p); f, g: both signs (w_p)
-    std::vector<double> sq, kq, kqd;     // [Nrho][3 (N/2)^2 + 1] (VHS, see ShiftDev)
+    std::vector<double> sq, kq, kqd, st, kt;   // [Nrho][3 (N/2)^2 + 1] (VHS, see ShiftDev)
+    std::vector<double> wsig;            // [npairs] weights; FP32: times excess (balance_constants)
+    std::vector<double> excess;          // [npairs] VSS: factor of the pair's kernel factors (fill_vss_tables)
+    double balance = 1.0, project = 1.0; // FP32: factor of the gain's radial multipliers, of the projection's coefficients
     std::vector<double> mu;              // [Nrho][nrows][MP][2] e^{i pi k s / L}, k = 0 .. N/2 (Nyquist cos)
 };
 
 // Row pitch of the shift table: N/2 + 1 modes, padded to an even count (16-byte FP32 rows).
 constexpr int shift_mu_pitch(int N) { return N / 2 + 2; }
 
-void build_shift_program(const HostPlan& h, ShiftProgram& p);
+// fp32: for FP32 arithmetic
+void build_shift_program(const HostPlan& h, bool fp32, ShiftProgram& p);
+// scale of a result after its inverse transforms: 1 / N^3, FP32: the nearest power of two
+double shift_result_scale(int N, bool fp64);
 
 // Device side of the program, in the compute type.
 template <typename T>
@@ -46,9 +52,11 @@ struct ShiftDev {
     const int* xrows = nullptr;
     const ShiftEntry *quad = nullptr, *bil = nullptr;
     const Cplx<T>* mu = nullptr;
+    const T* wsig = nullptr;
     // VHS, [Nrho][3 (N/2)^2 + 1] by |k|^2: S(|k|, r) of the compressed radial kernel, w_r rho_r S (the multiplier of
-    // K_r) and its derivative by gamma
-    const T *sq = nullptr, *kq = nullptr, *kqd = nullptr;
+    // K_r) and its derivative by gamma; st, kt: S and w_r rho_r S for P_r of the tensor cores, which carry the sphere
+    // rule's own weights
+    const T *sq = nullptr, *kq = nullptr, *kqd = nullptr, *st = nullptr, *kt = nullptr;
 };
 
 // G[node][x][ky][kz], kz = 0 .. N/2 - 1: the (y, z) spectra (times 1/N^2) of every x plane of the real
@@ -67,8 +75,8 @@ cudaError_t launch_shift_x(const ShiftDev<T>& d, const Cplx<T>* G, int N, int r0
 // large as P_r.
 template <typename T>
 cudaError_t launch_shift_products(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, const Cplx<T>* Gg,
-                                  const Cplx<T>* Hg, const T* wsig, int N, int r0, int nr, int64_t nodes, bool folded,
-                                  int64_t node_stride, T* P, cudaStream_t s);
+                                  const Cplx<T>* Hg, int N, int r0, int nr, int64_t nodes, bool folded, int64_t node_stride,
+                                  T* P, cudaStream_t s);
 // W: the same (folded) spectra of real fields P[fields][N^3] (a tensor-core plan's P_r); G: launch_shift_forward of f
 template <typename T>
 cudaError_t launch_shift_folded(const T* P, int64_t fields, const T* f, const int64_t* offs, int N, int64_t nodes, Cplx<T>* W,
@@ -93,7 +101,7 @@ cudaError_t launch_shift_vss(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx
                              int N, int r0, int nr, int64_t nodes, Cplx<T>* W, cudaStream_t s);
 // V [node][r][2 nx + 2][x][ky][kz]: the back-translated adjoint products before their x phases; Ur [node][r]: K_r u
 template <typename T>
-cudaError_t launch_shift_adj(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, const T* wsig, int N,
+cudaError_t launch_shift_adj(const ShiftDev<T>& d, const Cplx<T>* G, const Cplx<T>* H, const Cplx<T>* Ur, int N,
                              int r0, int nr, int64_t nodes, Cplx<T>* V, cudaStream_t s);
 // part (+)= the x spectra of the nf fields F[node][r] times A (VSS: [Nrho][npairs] half tables of
 // N^3/2 + 2 N values, fill_vss_tables) or, A == nullptr, times the x phases of the adjoint's fields; summed over fields and r
@@ -125,7 +133,5 @@ cudaError_t launch_shift_finish(const Cplx<T>* part, int parts, T scale, const C
 template <typename T>
 cudaError_t launch_shift_out(const Cplx<T>* F, int nf, int64_t field_stride, bool folded, const T* a, const T* c,
                              const int64_t* offs, int N, int64_t nodes, T* out, int* flags, cudaStream_t s);
-// 1 + the relative loss of the six extra line round trips that a gain takes over its loss term (rounded twiddles)
-double shift_gain_scale(int N, bool fp64);
 
 }  // namespace dgfs
