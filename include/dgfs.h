@@ -73,14 +73,18 @@ typedef enum {
                              batch against the FP64 oracle on the N = 32 two-Maxwellian workload):
                              about 8e-4 of ||Q||, 5e-5 of the loss term ||Q-||                       */
     DGFS_PREC_BF16S = 3,  /* as F16S with bf16 operands (no scaling): about 7e-3 of ||Q||           */
-    DGFS_PREC_F16X3 = 4,  /* about FP32 accuracy (8e-6 of ||Q||, 4e-7 of ||Q-||). Q(f,f), Q(f,g), the JVP,
-                             ragged batches, the DG and slab calls and the VJP take the FP32 CUDA-core
-                             translates, the faster of the two engines at this accuracy; dgfs_ssprk,
-                             dgfs_collide_dgamma and dgfs_collide_noalloc run on tcgen05 tensor cores
-                             with every data operand AND every filter split into an fp16 hi part and
-                             a lo part times 2^11: three products per contraction (hi hi, hi lo, lo
-                             hi), FP32 accumulation; the two CTAs of a thread-block cluster share the
-                             field of one (node, radial points) item. N = 16, 24 (on the 32-point
+    DGFS_PREC_F16X3 = 4,  /* about FP32 accuracy (8e-6 of ||Q||, 4e-7 of ||Q-||). Two engines: the FP32
+                             CUDA-core translates (the bits of an FP32 plan's calls), and a tcgen05
+                             tensor-core kernel with every data operand AND every filter split into an
+                             fp16 hi part and a lo part times 2^11: three products per contraction (hi
+                             hi, hi lo, lo hi), FP32 accumulation; the two CTAs of a thread-block cluster
+                             share the field of one (node, radial points) item. dgfs_ssprk,
+                             dgfs_collide_dgamma and dgfs_collide_noalloc take the tensor cores, the VJP
+                             the CUDA cores. Q(f,f), Q(f,g), the JVP, ragged batches, the DG and slab
+                             calls take the CUDA cores, which are faster where sphere points share
+                             components; the tensor cores when more than half of the rule's weight lies on
+                             the coordinate axes (M = 6; N = 16, 32: more exact there) and, at N = 32, when
+                             nearly every pair has an x component of its own. N = 16, 24 (on the 32-point
                              tiles) and 32                                                           */
     DGFS_PREC_BF16X3 = 5  /* F16X3's tensor-core translates with bf16 hi and lo parts (lo times 2^8), 16
                              significand bits, for every call but the VJP: about 2e-5 of ||Q||,
@@ -255,7 +259,7 @@ dgfs_status dgfs_collide_host(dgfs_plan_t plan, const void* f_host, void* Q_host
 
 /* Q(f,f) as dgfs_collide computes it (the same kernels, except that FP32/FP64 plans form the
    translate products with the dense circulant kernel and F16X3 plans with the split-data
-   tensor-core kernel where dgfs_collide takes them in Fourier space, and the Fourier stage may
+   tensor-core kernel where dgfs_collide takes them in Fourier space (see DGFS_PREC_F16X3), and the Fourier stage may
    sum in another order: equal to rounding), for callers that must not allocate device
    memory when they run (for example code whose device memory is fully reserved up front, or
    that may not pay the device synchronisation an allocation can cause). The paper has no

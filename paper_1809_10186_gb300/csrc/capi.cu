@@ -113,6 +113,7 @@ struct dgfs_plan_s {
     const void* d_mu = nullptr;   // [Nrho][npairs][3][N] complex multipliers (inside d_vss)
     ShiftDev<float> shf;          // shared-shift program of the translate products (inside d_vss)
     ShiftDev<double> shd;
+    bool split_data = false;      // F16X3: every call but the VJP on the split-data kernel (split_data_ahead)
     double project = 1.0;         // of the projection's coefficients (ShiftProgram)
     size_t off_V = 0, vss_bytes = 0;
     void* d_vss = nullptr;   // VSS: half tables A, GL [N^3], shift program; VHS: mu [Nrho][npairs][3][N], shift program
@@ -408,6 +409,33 @@ constexpr bool quadratic(Op op) { return op == Op::Collide || op == Op::Dgamma |
 template <typename T>
 constexpr bool keeps_rounding(Op op) {
     return std::is_same<T, float>::value && (op == Op::Dgamma || op == Op::Step);
+}
+
+// F16X3 asks for about FP32 accuracy: its translates run on the CUDA cores' shared-shift kernels, which are
+// faster than the split-data tensor-core kernel for the rules whose points share shifts (f16x3 / fp32 translates, whole
+// Q, 600 nodes: N = 16, M = 26 2.84 / 0.99 ms; N = 24 15.7 / 5.3; N = 32, M = 38 31.2 / 21.1; JVP of 100 nodes, N = 32
+// 10.3 / 6.6) and as accurate (2e-6 of ||Q|| at N = 32 against 3e-6). The split-data kernel keeps the calls whose
+// rounding is kept, the allocation-free call, the failure test, and every call of the plans where it is ahead:
+//   - N = 32 and nearly a shift along x of its own for every pair: the x translates pass through DRAM, 1.25 us a node and
+//     |s_x| (17 generic pairs, 160 nodes: 8.5 / 10.2 ms; N = 24, where its tiles are padded, 300 nodes: 12.2 / 6.0 ms);
+//   - more than half of the weight on the axes (M = 6): most translates then leave two axes alone, and f takes the same
+//     rounding through these axes' transforms in every term. Error of Q at N = 16: 1.1e-6 / 1.6e-6, N = 32: 2.1e-6 /
+//     3.3e-6; at N = 24 1.9e-6 / 1.7e-6.
+bool split_data_ahead(const HostPlan& h, int nx) {
+    double axes = 0.0, all = 0.0;
+    for (int q = 0; q < h.npairs; ++q) {
+        const double* s = &h.sig[3 * q];
+        all += h.wsig[q];
+        if ((s[0] != 0.0) + (s[1] != 0.0) + (s[2] != 0.0) == 1) axes += h.wsig[q];
+    }
+    return (h.N == 32 && 5 * nx > 3 * h.npairs + 5) || (h.N != 24 && 2.0 * axes > all);
+}
+
+// The engine of a call's translates: true for a tensor-core kernel (a pending injected failure aside).
+template <typename T>
+bool on_tensor_cores(const dgfs_plan_s* p, Op op) {
+    return is_tc(p->prec) && std::is_same<T, float>::value && op != Op::Vjp &&
+           (p->prec != DGFS_PREC_F16X3 || p->split_data || keeps_rounding<T>(op));
 }
 
 // Parts of the gain's radial sum (k_shift_sum.cu): the groups in blocks of their own while the columns of `nodes` nodes
@@ -757,13 +785,7 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     }
     // gain products: Q(f,f) and dQ/dgamma use (f, f); Q(f,g) uses (f, g); JVP uses (f, v)
     const T* gg = quadratic(op) ? nullptr : g;
-    // F16X3 asks for about FP32 accuracy: its translates run on the CUDA cores' shared-shift kernels, which are
-    // faster than the split-data tensor-core kernel at every size (f16x3 / fp32 translates, whole Q, 600 nodes: N = 16,
-    // M = 26 2.84 / 0.99 ms; N = 24 15.7 / 5.3; N = 32, M = 38 31.2 / 21.1; JVP of 100 nodes, N = 32 10.3 / 6.6) and as
-    // accurate (2e-6 of ||Q|| at N = 32 against 3e-6). The split-data kernel keeps the calls whose rounding is kept, the
-    // allocation-free call and the failure test.
-    const bool tensor = is_tc(p->prec) && std::is_same<T, float>::value &&
-                        (p->prec != DGFS_PREC_F16X3 || keeps_rounding<T>(op) || p->fault != 0);
+    const bool tensor = on_tensor_cores<T>(p, op) || (p->prec == DGFS_PREC_F16X3 && p->fault != 0);
     if (p->prof) p->prof_nodes += nodes;
     if (!tensor && !keeps_rounding<T>(op)) {
         e = shift_gain_products<T>(p, op, f, gg, out, offs, np, nodes, s);
@@ -986,6 +1008,7 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
         ShiftProgram sp;
         build_shift_program(p->hp, es == 4, sp);
         p->project = sp.project;
+        p->split_data = p->prec == DGFS_PREC_F16X3 && split_data_ahead(p->hp, sp.nx);
         if (es == 8) pack_shift(sp, mblob, p->shd);
         else pack_shift(sp, mblob, p->shf);
         cudaError_t ev = cudaMalloc(&p->d_vss, mblob.size());
