@@ -358,7 +358,8 @@ dgfs_status dgfs_profile_end(dgfs_plan_t plan, dgfs_profile_t* out);
    arithmetic is the same in every configuration). Synchronous; not for use inside a stream
    capture. The output goes to the plan's own staging buffer. VSS plans: DGFS_ERR_UNSUPPORTED. */
 typedef struct {
-    int rpc;                        /* radial points per item chosen (0 for plans without tensor cores) */
+    int rpc;                        /* radial points per item chosen (0 for plans without tensor cores; not timed, the
+                                       batch-size rule's value, for F16X3 plans whose Q(f, f) runs on the CUDA cores) */
     int64_t chunk_nodes;            /* nodes per chunk chosen                                          */
     double ms_per_node_default;     /* time per node with the batch-size rule and the plan's chunk     */
     double ms_per_node_tuned;       /* time per node with the choice                                   */

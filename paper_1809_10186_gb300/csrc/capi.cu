@@ -2079,13 +2079,14 @@ dgfs_status dgfs_profile_end(dgfs_plan_t plan, dgfs_profile_t* out) {
 namespace {
 
 struct TuneKey {
-    int N, npairs, Nrho, rank, prec, bucket;
+    int N, npairs, Nrho, rank, prec, bucket, tensor;
     bool operator<(const TuneKey& o) const {
-        return std::tie(N, npairs, Nrho, rank, prec, bucket) < std::tie(o.N, o.npairs, o.Nrho, o.rank, o.prec, o.bucket);
+        return std::tie(N, npairs, Nrho, rank, prec, bucket, tensor) <
+               std::tie(o.N, o.npairs, o.Nrho, o.rank, o.prec, o.bucket, o.tensor);
     }
 };
 struct TuneVal {
-    int rpc;
+    int rpc;   // of the plan; 0 (the batch-size rule) where the timed call does not read it
     int64_t chunk;
     double ms_default, ms_tuned;
 };
@@ -2111,31 +2112,37 @@ dgfs_status dgfs_plan_autotune(dgfs_plan_t plan, const void* f, int64_t B, void*
     NvtxRange range("dgfs autotune");
     dgfs_plan_s* p = plan;
     const int64_t nodes = std::min<int64_t>(B, p->chunk);
-    const TuneKey key{p->hp.N, p->hp.npairs, p->hp.Nrho, p->hp.rank, p->prec, floor_log2(nodes)};
+    // Radial points per work item are a candidate only where the timed call runs the kernel that reads them: the
+    // split-data kernel of an F16X3 plan whose Q(f, f) is on the CUDA cores serves other calls, which keep the rule
+    const bool tensor = on_tensor_cores<float>(p, Op::Collide);
+    const TuneKey key{p->hp.N, p->hp.npairs, p->hp.Nrho, p->hp.rank, p->prec, floor_log2(nodes), tensor};
     std::memset(report, 0, sizeof *report);
+    DGFS_ON_DEVICE(p->device);
+    int sms = 0;
+    DGFS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device), "cudaDeviceGetAttribute");
+    auto take = [&](const TuneVal& v) {
+        p->tc.rpc = v.rpc;
+        p->run_chunk = v.chunk;
+        report->rpc = is_tc(p->prec) ? tc_resolve_rpc(p->tc, p->prec, v.chunk, sms) : v.rpc;
+        report->chunk_nodes = v.chunk;
+        report->ms_per_node_default = v.ms_default;
+        report->ms_per_node_tuned = v.ms_tuned;
+    };
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune.find(key);
         if (it != g_tune.end()) {   // the same shape was tuned before in this process
-            p->tc.rpc = it->second.rpc;
-            p->run_chunk = it->second.chunk;
-            report->rpc = it->second.rpc;
-            report->chunk_nodes = it->second.chunk;
-            report->ms_per_node_default = it->second.ms_default;
-            report->ms_per_node_tuned = it->second.ms_tuned;
+            take(it->second);
             report->cached = 1;
             return DGFS_OK;
         }
     }
-    DGFS_ON_DEVICE(p->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int sms = 0;
-    DGFS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device), "cudaDeviceGetAttribute");
     const size_t n3 = (size_t)p->hp.N * p->hp.N * p->hp.N, es = elem_size(p->prec);
     void* Q = ws(p, p->off_io) + (size_t)p->chunk * n3 * es;   // the output half of the host staging area
     // candidates: radial points per work item (tensor-core plans; 0 = the batch-size rule) x nodes per chunk
     std::vector<int> rpcs{0};
-    if (is_tc(p->prec))
+    if (tensor)
         for (int c : {1, 2, 4, 8})
             if (p->hp.Nrho % c == 0) rpcs.push_back(c);
     std::vector<int64_t> chunks{nodes};
@@ -2190,20 +2197,16 @@ dgfs_status dgfs_plan_autotune(dgfs_plan_t plan, const void* f, int64_t B, void*
     }
     // record the resolved value of the batch-size rule, so that a cached choice means the same (the
     // rule reads the plan's rpc, which still holds the last candidate: clear it first)
-    if (best_rpc == 0 && is_tc(p->prec)) {
+    if (best_rpc == 0 && tensor) {
         p->tc.rpc = 0;
         best_rpc = tc_resolve_rpc(p->tc, p->prec, best_chunk, sms);
     }
-    p->tc.rpc = best_rpc;
-    p->run_chunk = best_chunk;
+    const TuneVal val{best_rpc, best_chunk, ms_default, best};
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
-        g_tune[key] = TuneVal{best_rpc, best_chunk, ms_default, best};
+        g_tune[key] = val;
     }
-    report->rpc = best_rpc;
-    report->chunk_nodes = best_chunk;
-    report->ms_per_node_default = ms_default;
-    report->ms_per_node_tuned = best;
+    take(val);
     report->candidates = count;
     report->cached = 0;
     return DGFS_OK;

@@ -46,3 +46,21 @@ def test_six_point_error(N):
     ref = binding.Plan(precision="fp64", **kw).collide(f.double())
     err = lambda q: (q.double() - ref).norm().item()
     assert err(plan.collide(f)) <= 1.1 * err(plan.collide_noalloc(f))
+
+
+@pytest.mark.parametrize("rule,candidates", [(12, 3), (6, 15)])
+def test_autotune_times_radial_points_only_where_they_count(rule, candidates):
+    """Three chunk sizes; five choices of radial points per item where Q(f, f) runs the kernel that reads them, else the
+    batch-size rule stays in force (per calls of this batch: two CTAs an item, 16 items per SM)."""
+    N, B = 32, 40
+    plan = binding.Plan(N=N, L=7.0, gamma=0.4, N_rho=N, M=rule, precision="f16x3", max_batch=B)
+    f = torch.from_numpy(W.two_maxwellian(B, N, 7.0, 5)[0]).cuda().float()
+    plan.set_tuning(8, 0)
+    rep = plan.autotune(f)
+    assert rep["cached"] == 0 and rep["candidates"] == candidates
+    if rule == 12:
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        want = next((c for c in (4, 2) if 2 * (N // c) * rep["chunk_nodes"] >= 16 * sms), 1)
+        assert rep["rpc"] == want
+    again = binding.Plan(N=N, L=7.0, gamma=0.4, N_rho=N, M=rule, precision="f16x3", max_batch=B).autotune(f)
+    assert again["cached"] == 1 and again["rpc"] == rep["rpc"]
