@@ -49,6 +49,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -210,7 +211,7 @@ __device__ __forceinline__ const unsigned char* item_filters(const unsigned char
     return filt + (size_t)((item % it.rblocks) * it.rpc) * npairs * Geo<N>::F_BLOCK;
 }
 
-template <int N, bool BF, int T>
+template <int N, bool BF, bool GR, int T>
 __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uint32_t sb, uint32_t tmem,
                                             const unsigned char* filt, int npairs, const Items& it, long long first,
                                             volatile long long* s_item, int* queue, volatile int* abort,
@@ -233,7 +234,7 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
         int pair = 0, off = 0;   // first pair of the step's group, its filter block within the item
         for (int s = 0; s < it.nseq; ++s, ++g) {
             const int fbuf = (int)(g & 1);
-            const int cnt = it.groups.count(pair);
+            const int cnt = it.groups.count<GR>(pair);
             const unsigned char* fstep = fcur + (size_t)off * G::F_BLOCK;
             DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((g >> 1) & 1));
             if (fbuf) ++waited1;
@@ -303,7 +304,7 @@ __device__ __forceinline__ void mma_p1_loop(Bars& bars, unsigned char* smem, uin
 // Pass 2 of tile t reads pass-2 operand buffer t % 2 and writes pass-2/3 slot t % 2. Slot b is
 // reused within a step after the pass-2 epilogue drained it (free2, all completions of a step but the
 // last); the step's first use waits for the previous step's last pass-3 drain (free3x).
-template <int N, bool BF, int T>
+template <int N, bool BF, bool GR, int T>
 __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tmem, const Items& it,
                                             const volatile long long* s_item, volatile int* abort) {
     using G = Geo<N>;
@@ -358,7 +359,7 @@ __device__ __forceinline__ void mma_p2_loop(Bars& bars, uint32_t sb, uint32_t tm
 // its own completion (full3p / full3m) and release (free3p / free3m): the + MMAs of tile k + 1 wait
 // only for the + half of tile k to be read, so they run while the epilogue reads the - half and
 // forms the products. A group's second pair reads the same operands with its own y filters.
-template <int N, bool BF, int T, int b>
+template <int N, bool BF, bool GR, int T, int b>
 __device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tmem, int npairs, const Items& it,
                                             const volatile long long* s_item, volatile int* abort) {
     using G = Geo<N>;
@@ -374,7 +375,7 @@ __device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tm
         int pair = 0;
         for (int s = 0; s < it.nseq; ++s, ++g) {
             const int fbuf = (int)(g & 1);
-            const int cnt = it.groups.count(pair);
+            const int cnt = it.groups.count<GR>(pair);
             pair = pair + cnt < npairs ? pair + cnt : 0;
             DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((g >> 1) & 1));
             const uint32_t f16 = sb16 + (G::S_F + fbuf * G::F_BLOCK) / 16;
@@ -418,7 +419,7 @@ __device__ __forceinline__ void mma_p3_loop(Bars& bars, uint32_t sb, uint32_t tm
 // Persistent: one CTA per SM pulls work items (node, block of rpc radial points) from the queue
 // counter queue[0] (zero at launch) until the items run out. PAD: f and P_r on an nsrc^3 grid,
 // nsrc < N (N = 24 on the 32-point tiles).
-template <int N, bool BF, bool PAD>
+template <int N, bool BF, bool PAD, bool GR>
 __global__ void __launch_bounds__(Geo<N>::THREADS, 1)
 k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const unsigned char* __restrict__ filt,
           int npairs, int Nrho, Items it, int nsrc, int* __restrict__ queue, float* __restrict__ P,
@@ -488,7 +489,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
             for (int p = 0; p < 2 && p < it.nseq; ++p) {   // the first two groups
                 tc::mbar_expect_tx(&bars.filt[p], G::F_BLOCK);
                 tc::bulk_g2s(smem + G::S_F + p * G::F_BLOCK, f0, G::F_BLOCK, &bars.filt[p]);
-                f0 += (size_t)it.groups.count(0) * G::F_BLOCK;
+                f0 += (size_t)it.groups.count<GR>(0) * G::F_BLOCK;
             }
         }
         __syncwarp();
@@ -512,14 +513,14 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
       tc::setmaxnreg_dec<G::REG_MMA>();   // every warp of the third warpgroup
       // ============================ MMA warps (converged) =====================================
       if (warp == G::ISSUER)
-        mma_p1_loop<N, BF, T>(bars, smem, sb, tmem, filt, npairs, it, first, s_item, queue, abort, copies0, copies1,
+        mma_p1_loop<N, BF, GR, T>(bars, smem, sb, tmem, filt, npairs, it, first, s_item, queue, abort, copies0, copies1,
                            waited0, waited1, second0, second1);
       else if (warp == G::ISSUER + 1)
-        mma_p2_loop<N, BF, T>(bars, sb, tmem, it, s_item, abort);
+        mma_p2_loop<N, BF, GR, T>(bars, sb, tmem, it, s_item, abort);
       else if (warp == G::ISSUER + 2)
-        mma_p3_loop<N, BF, T, 0>(bars, sb, tmem, npairs, it, s_item, abort);
+        mma_p3_loop<N, BF, GR, T, 0>(bars, sb, tmem, npairs, it, s_item, abort);
       else
-        mma_p3_loop<N, BF, T, 1>(bars, sb, tmem, npairs, it, s_item, abort);
+        mma_p3_loop<N, BF, GR, T, 1>(bars, sb, tmem, npairs, it, s_item, abort);
     } else {
         tc::setmaxnreg_inc<G::REG_EPI>();
         // ============================== epilogue warpgroups ===================================
@@ -638,7 +639,7 @@ k_tc_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const u
           for (int rr = 0; rr < it.rpc; ++rr) {
           int cnt = 1;   // pairs of the step's group
           for (int pp = 0; pp < npairs; pp += cnt, ++g) {
-            cnt = it.groups.count(pp);
+            cnt = it.groups.count<GR>(pp);
             if (w == 0) {
                 // the step's remaining tiles, then, when the next step belongs to this item, its first
                 // LOOKAHEAD tiles (virtual tiles T, T + 1): their pass-1 MMAs and operand buffers do not
@@ -840,7 +841,13 @@ cudaError_t launch_n(const TcTables& t, const float* f, const int64_t* offs, int
                      int* flags, cudaStream_t s, int fault, const float* coef, int accum) {
     using G = Geo<N>;
     const int nsrc = t.nsrc > 0 ? t.nsrc : N;
-    auto kern = nsrc == N ? k_tc_gain<N, BF, false> : k_tc_gain<N, BF, true>;
+    auto pick = [&](auto gr) {
+        constexpr bool GR = decltype(gr)::value;
+        if constexpr (N == 32)
+            if (nsrc != N) return k_tc_gain<N, BF, true, GR>;
+        return k_tc_gain<N, BF, false, GR>;
+    };
+    auto kern = t.ngroups < t.npairs ? pick(std::true_type{}) : pick(std::false_type{});
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::S_TOTAL);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;

@@ -42,6 +42,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -146,7 +147,7 @@ struct Bars3 {
     } while (0)
 
 // Pass 1 of the CTA's front tiles i (both signs) into the pass-1 slot; refills the filter buffers.
-template <int N, bool BF>
+template <int N, bool BF, bool GR>
 __device__ __forceinline__ void mma3_p1_loop(Bars3& bars, unsigned char* smem, uint32_t sb, uint32_t tmem,
                                              const unsigned char* fglob, int npairs, const TcGroups& groups, int nseq,
                                              volatile int* abort, int& copies0, int& copies1, int& waited0, int& waited1,
@@ -163,7 +164,7 @@ __device__ __forceinline__ void mma3_p1_loop(Bars3& bars, unsigned char* smem, u
     const uint32_t sb16 = sb >> 4;
     for (int p = 0; p < nseq; ++p) {
         const int fbuf = p & 1;
-        const int cnt = groups.count(pair);
+        const int cnt = groups.count<GR>(pair);
         DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((p >> 1) & 1));
         if (fbuf) ++waited1;
         else ++waited0;
@@ -278,7 +279,7 @@ __device__ __forceinline__ void mma3_p2_loop(Bars3& bars, uint32_t sb, uint32_t 
 // Pass 3 of back tiles k = b, b + 2, ... (both signs) into slot 2 + b once the pass-3 operands of
 // both CTAs' epilogues are complete (warpgroup b drains the slot); the release of the operands is
 // signalled to both CTAs (multicast commit).
-template <int N, bool BF, int b>
+template <int N, bool BF, bool GR, int b>
 __device__ __forceinline__ void mma3_p3_loop(Bars3& bars, uint32_t sb, uint32_t tmem, int npairs, const TcGroups& groups, int nseq,
                                              volatile int* abort) {
     using G = Geo3<N>;
@@ -290,7 +291,7 @@ __device__ __forceinline__ void mma3_p3_loop(Bars3& bars, uint32_t sb, uint32_t 
     constexpr uint64_t dA3 = tc::sdesc_base(G::A3_LBO, G::A3_SBO);
     const uint32_t sb16 = sb >> 4;
     for (int p = 0; p < nseq; ++p) {
-        const int fbuf = p & 1, cnt = groups.count(pair);
+        const int fbuf = p & 1, cnt = groups.count<GR>(pair);
         pair = pair + cnt < npairs ? pair + cnt : 0;
         DGFS_WAITW(&bars.filt[fbuf], (uint32_t)((p >> 1) & 1));
         const uint32_t f16 = sb16 + (G::S_F + fbuf * G::F_BLOCK) / 16;
@@ -336,7 +337,7 @@ __device__ __forceinline__ void mma3_p3_loop(Bars3& bars, uint32_t sb, uint32_t 
 // PAD: f and P_r on an nsrc^3 grid, nsrc < N (N = 24 on the 32-point tiles: the filters are zero
 // outside the nsrc x nsrc block, f is read with zeros outside it and only the nsrc^3 block of P_r is
 // written).
-template <int N, bool BF, bool PAD>
+template <int N, bool BF, bool PAD, bool GR>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Geo3<N>::THREADS, 1)
 k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const unsigned char* __restrict__ filt,
            int npairs, int Nrho, int rpc, TcGroups groups, int ngroups, int nsrc, float* __restrict__ P,
@@ -393,7 +394,7 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
             s_abort = 0;
             for (int p = 0; p < 2 && p < nseq; ++p) {
                 tc::mbar_expect_tx(&bars.filt[p], G::F_BLOCK);
-                tc::bulk_g2s(smem + G::S_F + p * G::F_BLOCK, fglob + (size_t)(p ? groups.count(0) : 0) * G::F_BLOCK,
+                tc::bulk_g2s(smem + G::S_F + p * G::F_BLOCK, fglob + (size_t)(p ? groups.count<GR>(0) : 0) * G::F_BLOCK,
                              G::F_BLOCK, &bars.filt[p]);   // the first two groups
             }
         }
@@ -479,14 +480,14 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
     if (warp >= G::EPI_WARPS) {
         tc::setmaxnreg_dec<G::REG_MMA>();
         if (warp == G::ISSUER)
-            mma3_p1_loop<N, BF>(bars, smem, sb, tmem, fglob, npairs, groups, nseq, abort, copies0, copies1, waited0, waited1,
+            mma3_p1_loop<N, BF, GR>(bars, smem, sb, tmem, fglob, npairs, groups, nseq, abort, copies0, copies1, waited0, waited1,
                                 second0, second1);
         else if (warp == G::ISSUER + 1)
             mma3_p2_loop<N, BF>(bars, sb, tmem, nseq, abort);
         else if (warp == G::ISSUER + 2)
-            mma3_p3_loop<N, BF, 0>(bars, sb, tmem, npairs, groups, nseq, abort);
+            mma3_p3_loop<N, BF, GR, 0>(bars, sb, tmem, npairs, groups, nseq, abort);
         else
-            mma3_p3_loop<N, BF, 1>(bars, sb, tmem, npairs, groups, nseq, abort);
+            mma3_p3_loop<N, BF, GR, 1>(bars, sb, tmem, npairs, groups, nseq, abort);
     } else {
         tc::setmaxnreg_inc<G::REG_EPI>();
         // warpgroup w: the epilogues of sign w (w = 0: +s, 1: -s) and the back tiles k = w, w + 2, ...
@@ -524,7 +525,7 @@ k_tc3_gain(const float* __restrict__ f, const int64_t* __restrict__ offs, const 
         int p = 0;   // (radial point, group) step
         for (int rr = 0; rr < rpc; ++rr) {
           for (int pp = 0, cnt; pp < npairs; pp += cnt, ++p) {
-            cnt = groups.count(pp);
+            cnt = groups.count<GR>(pp);
             // front, software-pipelined over the front tiles: pass-1 epilogue of tile s, then the pass-2
             // epilogue of tile s - 1 (whose pass-2 MMAs ran meanwhile)
             for (int st = 0; st <= G::TH; ++st) {
@@ -742,7 +743,13 @@ cudaError_t launch3_n(const TcTables& t, const float* f, const int64_t* offs, in
                       cudaStream_t s, int fault, const float* coef, int accum) {
     using G = Geo3<N>;
     const int nsrc = t.nsrc > 0 ? t.nsrc : N;
-    auto kern = nsrc == N ? k_tc3_gain<N, BF, false> : k_tc3_gain<N, BF, true>;
+    auto pick = [&](auto gr) {
+        constexpr bool GR = decltype(gr)::value;
+        if constexpr (N == 32)
+            if (nsrc != N) return k_tc3_gain<N, BF, true, GR>;
+        return k_tc3_gain<N, BF, false, GR>;
+    };
+    auto kern = t.ngroups < t.npairs ? pick(std::true_type{}) : pick(std::false_type{});
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::S_TOTAL);
     if (e != cudaSuccess) return e;
     const int64_t n3 = (int64_t)nsrc * nsrc * nsrc;   // f and P_r grid
