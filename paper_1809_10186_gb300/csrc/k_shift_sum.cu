@@ -27,6 +27,7 @@
 // ky = 0 .. N/2 - 1 of the first, then of the second, with the real ky = 0 and N/2 packed in the two slots
 // ky = 0 (a "folded" plane); only those two columns are separated along x, in registers. k_shift_filter takes the
 // plane as it is: one warp holds it, kx in registers and ky along the lanes.
+#include <algorithm>
 #include <cmath>
 
 #include "shift.h"
@@ -49,19 +50,21 @@ struct SumGeo {
     static constexpr int MINA = sizeof(T) == 8 ? 1 : N == 32 ? 256 / NT : N == 24 ? 384 / NT : 512 / NT;
 };
 
-// grid (N / XC, nr, nodes). W [node][r][entry][x][ky][kz].
+// grid (N / XC, nr parts, nodes): part q of a radial point takes its share of the program, whole pairs of entries, so that
+// the bits do not depend on it. W [node][r][entry][x][ky][kz].
 template <typename T, int N, int XC>
 __global__ void __launch_bounds__(SumGeo<T, N, XC>::NT, SumGeo<T, N, XC>::MINV)
 k_shift_vss(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, const Cplx<T>* __restrict__ Gg,
             const Cplx<T>* __restrict__ Hg, const Cplx<T>* __restrict__ mu, const ShiftEntry* __restrict__ prog, int nprog,
-            int nrows, int nx, int r0, Cplx<T>* __restrict__ W) {
+            int nrows, int nx, int r0, int parts, Cplx<T>* __restrict__ W) {
     using Geo = SumGeo<T, N, XC>;
     constexpr int NH = N / 2, PITCH = Geo::PITCH, NT = Geo::NT, MP = shift_mu_pitch(N);
     constexpr int64_t FS = (int64_t)N * N * NH;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     Cplx<T>* Y = reinterpret_cast<Cplx<T>*>(sm_raw);         // [sign][XC][y][PITCH] inverse y lines
     Cplx<T>* S = Y + Geo::BUF;                               // [field][XC][y][PITCH] forward z lines
-    const int tid = threadIdx.x, x0 = blockIdx.x * XC, rl = blockIdx.y, nr = gridDim.y;
+    const int tid = threadIdx.x, x0 = blockIdx.x * XC, rl = blockIdx.y / parts, nr = gridDim.y / parts;
+    const int pq = blockIdx.y % parts, pairs = (nprog + 1) / 2, i0 = 2 * (pairs * pq / parts), i1 = min(nprog, 2 * (pairs * (pq + 1) / parts));
     const int64_t node = blockIdx.z;
     const int op = tid / (XC * NH), ypl = (tid / NH) % XC, ykz = tid % NH;
     const int64_t ybase = (int64_t)(x0 + ypl) * N * NH + ykz;
@@ -72,9 +75,9 @@ k_shift_vss(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, cons
     Cplx<T>* Wn = W + (node * nr + rl) * nprog * FS + ybase;
     T first[N];                                              // products of the even entry
     Cplx<T> v[N];
-    for (int i = 0; i < nprog; ++i) {
+    for (int i = i0; i < i1; ++i) {
         const ShiftEntry e = prog[i];
-        if (e.newy) {
+        if (e.newy || i == i0) {
             const int fi = op ? e.fm : e.fp;
             load_y_line<T, N>(fi < 0 ? Gy : Hy + fi * FS, mu_r, e.yrow, e.yneg ^ op, v);
             cfft::line<T, N, false>(v);
@@ -675,8 +678,13 @@ cudaError_t vss_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, co
     const cudaError_t e = allow_smem(k_shift_vss<T, N, XC>, Geo::smem);
     if (e != cudaSuccess) return e;
     const bool bil = Gg != nullptr;
-    k_shift_vss<T, N, XC><<<dim3(N / XC, (unsigned)nr, (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
-        Gf, Hf, bil ? Gg : Gf, bil ? Hg : Hf, d.mu, bil ? d.bil : d.quad, bil ? d.nbil : d.nquad, d.nrows, d.nx, r0, W);
+    const int nprog = bil ? d.nbil : d.nquad;
+    // shares of the program while the (x, r, node) blocks have fewer than eight warps for each of the 152 SMs: the JVP of
+    // one node in FP64, N = 8, M = 26 took 514 us with one share, 336 with 13
+    const int64_t threads = (int64_t)(N / XC) * nr * nodes * Geo::NT;
+    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((nprog + 1) / 2, 152 * 256 / threads));
+    k_shift_vss<T, N, XC><<<dim3(N / XC, (unsigned)(nr * parts), (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
+        Gf, Hf, bil ? Gg : Gf, bil ? Hg : Hf, d.mu, bil ? d.bil : d.quad, nprog, d.nrows, d.nx, r0, parts, W);
     return cudaGetLastError();
 }
 
