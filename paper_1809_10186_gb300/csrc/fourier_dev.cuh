@@ -181,7 +181,7 @@ __device__ __forceinline__ void fft_stage_sub(Cplx<T> (&a)[NA], const Cplx<T>* _
             } else {
                 const Cplx<T> w = tw[j * step * tstride];
                 const T wi = forward ? w.y : -w.y;
-                v = Cplx<T>{v0.x * w.x - v0.y * wi, v0.x * wi + v0.y * w.x};
+                v = Cplx<T>{fma(v0.x, w.x, -mul_rn(v0.y, wi)), fma(v0.y, w.x, mul_rn(v0.x, wi))};
             }
             a[OFF + i + j] = Cplx<T>{u.x + v.x, u.y + v.y};
             a[OFF + i + j + half] = Cplx<T>{u.x - v.x, u.y - v.y};
@@ -206,8 +206,8 @@ __device__ __forceinline__ void line_fft(Cplx<T> (&a)[N], const Cplx<T>* __restr
             const Cplx<T> y0 = a[q], y1 = a[S + q], y2 = a[2 * S + q];
             const Cplx<T> w1 = tw[k], w2 = tw[(2 * k) % N];
             const T s1 = forward ? w1.y : -w1.y, s2 = forward ? w2.y : -w2.y;
-            b[k] = Cplx<T>{y0.x + (y1.x * w1.x - y1.y * s1) + (y2.x * w2.x - y2.y * s2),
-                           y0.y + (y1.x * s1 + y1.y * w1.x) + (y2.x * s2 + y2.y * w2.x)};
+            b[k] = Cplx<T>{y0.x + fma(y1.x, w1.x, -mul_rn(y1.y, s1)) + fma(y2.x, w2.x, -mul_rn(y2.y, s2)),
+                           y0.y + fma(y1.y, w1.x, mul_rn(y1.x, s1)) + fma(y2.y, w2.x, mul_rn(y2.x, s2))};
         }
 #pragma unroll
         for (int k = 0; k < N; ++k) a[k] = b[k];

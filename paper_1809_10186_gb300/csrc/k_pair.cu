@@ -19,6 +19,7 @@ namespace {
 
 using fdev::line_fft;
 using fdev::line_slot;
+using fdev::mul_rn;
 
 // X[n][z][x][y] = {f[n][x][y][z], 0}: a real field into a plane-major complex field
 template <typename T>
@@ -54,8 +55,8 @@ struct PlaneGeo {
 // ky: coalesced), the y lines go through shared memory.
 template <typename T, int N>
 __global__ void __launch_bounds__(PlaneGeo<T, N>::NT)
-    k_pair_planes(const Cplx<T>* __restrict__ Fh, const Cplx<T>* __restrict__ Gh, const Cplx<T>* __restrict__ mu_r,
-                  const Cplx<T>* __restrict__ dftw, int npairs, int nr, Cplx<T>* __restrict__ X) {
+    k_pair_planes(const Cplx<T>* __restrict__ Fh, const Cplx<T>* __restrict__ mu_r, const Cplx<T>* __restrict__ dftw, int nr,
+                  Cplx<T>* __restrict__ X) {
     using G = PlaneGeo<T, N>;
     constexpr int KZ = G::KZ, NT = G::NT, P = G::P;
     constexpr int64_t n2 = (int64_t)N * N, n3 = n2 * N;
@@ -63,31 +64,26 @@ __global__ void __launch_bounds__(PlaneGeo<T, N>::NT)
     Cplx<T>* S = reinterpret_cast<Cplx<T>*>(sm_raw);   // [KZ][N][P]
     __shared__ Cplx<T> tw[N];
     __shared__ Cplx<T> m[3 * N];
-    const int tid = threadIdx.x, kz0 = blockIdx.x * KZ, f = blockIdx.y, nf = gridDim.y;
+    const int tid = threadIdx.x, kz0 = blockIdx.x * KZ, p = blockIdx.y, npairs = gridDim.y;
     const unsigned node = nr > 1 ? blockIdx.z / (unsigned)nr : blockIdx.z;
     const int rl = (int)(blockIdx.z - node * (unsigned)nr);   // radial point of the item
-    const int64_t n = node, item = blockIdx.z;
+    const int64_t item = blockIdx.z;
     const int pl = tid / N, ln = tid % N;
     if (tid < N) tw[tid] = dftw[N + tid];
-    Cplx<T>* Xf = X + (item * nf + f) * n3 + (int64_t)kz0 * n2;
+    Cplx<T>* Xf = X + (item * npairs + p) * n3 + (int64_t)kz0 * n2;
     Cplx<T> v[N];
-    const int p = f % npairs;
-    const T sgn = f < npairs ? T(1) : T(-1);
     for (int i = tid; i < 3 * N; i += NT) m[i] = mu_r[((int64_t)rl * npairs + p) * 3 * N + i];
     __syncthreads();
-    const Cplx<T>* Fp = Fh + n * n3 + (int64_t)(kz0 + pl) * n2 + ln;
-    const Cplx<T>* Gp = (Gh ? Gh : Fh) + n * n3 + (int64_t)(kz0 + pl) * n2 + ln;
+    const Cplx<T>* Fp = Fh + (int64_t)node * n3 + (int64_t)(kz0 + pl) * n2 + ln;
+    // which product of a sum is rounded by itself is written out: it is part of the rounding that is kept
     const Cplx<T> my = m[N + ln], mz = m[2 * N + kz0 + pl];
-    const Cplx<T> myz{my.x * mz.x - my.y * mz.y, my.x * mz.y + my.y * mz.x};
+    const Cplx<T> myz{fma(my.x, mz.x, -mul_rn(my.y, mz.y)), fma(my.y, mz.x, mul_rn(my.x, mz.y))};
 #pragma unroll
     for (int kx = 0; kx < N; ++kx) {
-        const Cplx<T> mx = m[kx];
-        const T a = mx.x * myz.x - mx.y * myz.y, b = sgn * (mx.x * myz.y + mx.y * myz.x);
-        const Cplx<T> fv = Fp[kx * N];
-        // Gh is nullptr in every launch and field f < npairs: the general form of f and g is kept as it is written,
-        // because which of its products the compiler contracts into FMAs is part of the rounding that is kept
-        const Cplx<T> gv = Gh ? Gp[kx * N] : fv;
-        v[line_slot<N>(kx)] = Cplx<T>{a * fv.x - b * fv.y - a * gv.y + b * gv.x, a * fv.y + b * fv.x + a * gv.x + b * gv.y};
+        const Cplx<T> mx = m[kx], fv = Fp[kx * N];
+        const T a = fma(mx.x, myz.x, -mul_rn(mx.y, myz.y)), b = fma(mx.x, myz.y, mul_rn(mx.y, myz.x));
+        v[line_slot<N>(kx)] = Cplx<T>{fma(b, fv.x, fma(-a, fv.y, fma(a, fv.x, -mul_rn(b, fv.y)))),
+                                      fma(b, fv.y, fma(a, fv.x, fma(a, fv.y, mul_rn(b, fv.x))))};
     }
     // x lines (fixed ky = ln)
     line_fft<T, N>(v, tw, false);
@@ -154,8 +150,7 @@ cudaError_t planes_n(const Cplx<float>* Fh, const Cplx<float>* mu_r, const Cplx<
                      Cplx<float>* Z, cudaStream_t s) {
     using G = PlaneGeo<float, N>;
     static_assert(G::smem <= 48 * 1024, "static shared memory limit");
-    k_pair_planes<float, N><<<dim3(N / G::KZ, (unsigned)npairs, (unsigned)(nodes * nr)), G::NT, G::smem, s>>>(Fh, nullptr, mu_r, dftw,
-                                                                                                          npairs, nr, Z);
+    k_pair_planes<float, N><<<dim3(N / G::KZ, (unsigned)npairs, (unsigned)(nodes * nr)), G::NT, G::smem, s>>>(Fh, mu_r, dftw, nr, Z);
     return cudaGetLastError();
 }
 
