@@ -58,13 +58,13 @@ k_shift_vss(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, cons
             const Cplx<T>* __restrict__ Hg, const Cplx<T>* __restrict__ mu, const ShiftEntry* __restrict__ prog, int nprog,
             int nrows, int nx, int r0, int parts, Cplx<T>* __restrict__ W) {
     using Geo = SumGeo<T, N, XC>;
+    const int shares = XC == 2 ? parts : 1;   // the wide blocks take it all (and spare the registers of a share)
     constexpr int NH = N / 2, PITCH = Geo::PITCH, NT = Geo::NT, MP = shift_mu_pitch(N);
     constexpr int64_t FS = (int64_t)N * N * NH;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     Cplx<T>* Y = reinterpret_cast<Cplx<T>*>(sm_raw);         // [sign][XC][y][PITCH] inverse y lines
     Cplx<T>* S = Y + Geo::BUF;                               // [field][XC][y][PITCH] forward z lines
-    const int tid = threadIdx.x, x0 = blockIdx.x * XC, rl = blockIdx.y / parts, nr = gridDim.y / parts;
-    const int pq = blockIdx.y % parts, pairs = (nprog + 1) / 2, i0 = 2 * (pairs * pq / parts), i1 = min(nprog, 2 * (pairs * (pq + 1) / parts));
+    const int tid = threadIdx.x, x0 = blockIdx.x * XC, rl = blockIdx.y / shares, nr = gridDim.y / shares;
     const int64_t node = blockIdx.z;
     const int op = tid / (XC * NH), ypl = (tid / NH) % XC, ykz = tid % NH;
     const int64_t ybase = (int64_t)(x0 + ypl) * N * NH + ykz;
@@ -73,11 +73,17 @@ k_shift_vss(const Cplx<T>* __restrict__ Gf, const Cplx<T>* __restrict__ Hf, cons
     const int yrow = ((op * XC + ypl) * N) * PITCH + ykz;     // this thread's y line in a buffer
     const Cplx<T>* mu_r = mu + (int64_t)(r0 + rl) * nrows * MP;
     Cplx<T>* Wn = W + (node * nr + rl) * nprog * FS + ybase;
+    if constexpr (XC == 2) {   // this block's share
+        const int pq = blockIdx.y % parts, pairs = (nprog + 1) / 2, i0 = 2 * (pairs * pq / parts);
+        nprog = min(nprog, 2 * (pairs * (pq + 1) / parts)) - i0;
+        prog += i0;
+        Wn += i0 * FS;
+    }
     T first[N];                                              // products of the even entry
     Cplx<T> v[N];
-    for (int i = i0; i < i1; ++i) {
+    for (int i = 0; i < nprog; ++i) {
         const ShiftEntry e = prog[i];
-        if (e.newy || i == i0) {
+        if (e.newy || i == 0) {
             const int fi = op ? e.fm : e.fp;
             load_y_line<T, N>(fi < 0 ? Gy : Hy + fi * FS, mu_r, e.yrow, e.yneg ^ op, v);
             cfft::line<T, N, false>(v);
@@ -352,7 +358,7 @@ k_shift_sum(const Cplx<T>* __restrict__ F, int nf, const T* __restrict__ A, cons
 #pragma unroll
             for (int k = 0; k < N; ++k) {
                 Cplx<T>& t = REGS ? reg[REGS ? k : 0] : total[k * kColThreads];
-                t = Cplx<T>{t.x + acc[k].x, t.y + acc[k].y};
+                t = fdev::add(t, acc[k]);
                 acc[k] = Cplx<T>{T(0), T(0)};
             }
         }
@@ -679,10 +685,10 @@ cudaError_t vss_x(const ShiftDev<T>& d, const Cplx<T>* Gf, const Cplx<T>* Hf, co
     if (e != cudaSuccess) return e;
     const bool bil = Gg != nullptr;
     const int nprog = bil ? d.nbil : d.nquad;
-    // shares of the program while the (x, r, node) blocks have fewer than eight warps for each of the 152 SMs: the JVP of
-    // one node in FP64, N = 8, M = 26 took 514 us with one share, 336 with 13
+    // shares of the program while the (x, r, node) blocks have fewer than eight warps for each of the 152 SMs (narrow blocks
+    // only, see narrow()): the JVP of one node in FP64, N = 8, M = 26 took 514 us with one share, 336 with 13
     const int64_t threads = (int64_t)(N / XC) * nr * nodes * Geo::NT;
-    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((nprog + 1) / 2, 152 * 256 / threads));
+    const int parts = XC == 2 ? (int)std::max<int64_t>(1, std::min<int64_t>((nprog + 1) / 2, 152 * 256 / threads)) : 1;
     k_shift_vss<T, N, XC><<<dim3(N / XC, (unsigned)(nr * parts), (unsigned)nodes), Geo::NT, Geo::smem, s>>>(
         Gf, Hf, bil ? Gg : Gf, bil ? Hg : Hf, d.mu, bil ? d.bil : d.quad, nprog, d.nrows, d.nx, r0, parts, W);
     return cudaGetLastError();
