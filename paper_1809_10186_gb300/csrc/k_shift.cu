@@ -13,11 +13,11 @@
 //                     shared memory; per pair: phase, inverse z transform of one line per thread,
 //                     product summed in registers; P_r (or its (y, z) spectra, for a stage in spectra) written once
 //
-// Measured (GB300, FP32, N = 32, M = 38, 256 nodes, whole Q): 8.4 ms, 22.2 ms with a transform of its own
+// Measured (GB300, FP32, N = 32, M = 38, 256 nodes, whole Q): 8.35 ms, 22.2 ms with a transform of its own
 // per pair (two launches per radial point, 9.5 MB of spectra through DRAM per radial point and node
-// against 2.2 MB here); N = 16, M = 6, FP64, one node: 0.18 ms, 0.97 ms before. k_shift_products takes 73 %
-// of the FP32 step: 70 % of the issue slots and 56 % of the FMA pipe (ncu, 40 nodes); k_shift_x 15 %, at
-// 81 % of the DRAM throughput.
+// against 2.2 MB here); N = 16, M = 6, FP64, one node: 0.17 ms, 0.97 ms before. k_shift_products takes 77 %
+// of the FP32 step: 2.45 instructions a cycle (61 % of the issue slots), 49 % of the FMA pipe (ncu, 40 nodes); k_shift_x
+// 15 %, at 82 % of the DRAM throughput.
 //
 // Half spectra: kz = 0 .. N/2 - 1, with the spectra of kz = 0 and kz = N/2 (both of real (x, y)
 // fields, which x and y translates keep real) in the real and imaginary part of slot kz = 0.

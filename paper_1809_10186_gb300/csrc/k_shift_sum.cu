@@ -15,9 +15,10 @@
 //   k_shift_out     inverse y and z of the gain and the loss fields, the result
 //
 // Measured (GB300, FP32, N = 32, M = 38): VSS Q of 40 nodes 3.1 ms (6.5 ms with a three-axis transform of its own for
-// every translate and product), VJP of 48 nodes 4.2 ms (11 ms); k_shift_vss 57 % and k_shift_adj 80 % of them, both
-// bound by instruction issue at 8-12 warps per SM (a line and its sums fill the registers). VHS, N = 24, 144 nodes:
-// k_shift_sum 41 us (192 MB: 4.7 TB/s), k_shift_finish about 20 us, in the 658 us of the call; at a few nodes the launches
+// every translate and product), VJP of 48 nodes 3.9 ms (11 ms). k_shift_vss is 65 % of the first (1.75 instructions a cycle
+// at 11 warps per SM, waiting on its loads), k_shift_sum 27 % (its products from DRAM); k_shift_adj 79 % of the second (2.1
+// instructions a cycle at 8 warps per SM: a line and its sums fill the registers). VHS, N = 24, 144 nodes: k_shift_sum 41 us
+// (192 MB: 4.7 TB/s), k_shift_finish about 20 us, in the 655 us of the call; at a few nodes the launches
 // bound it, which is why gain and loss share k_shift_finish (five nodes, F16S, N = 32, M = 12: 169 -> 144 us with it and P_r
 // and f in one forward launch).
 //
