@@ -108,7 +108,7 @@ void balance_constants(const HostPlan& h, ShiftProgram& p) {
         p.excess[q] = syz * sx / (s * s) * (1.0 + 2.0 * (tx ? 3 : 2) * ll);
     }
     double common = 1.0, best = -1.0;
-    for (int i = 0; i < 4096; ++i) {
+    for (int i = 0; i < 4096 && !h.aniso; ++i) {   // (VSS: the weight is part of the kernel factor)
         const double c = 1.0 + i / 4096.0;
         double e = 0.0;
         for (int q = 0; q < np; ++q) {
@@ -130,19 +130,18 @@ void balance_constants(const HostPlan& h, ShiftProgram& p) {
             cosx[i * N + k] = a * std::cos(ang);
             sinx[i * N + k] = k == NH ? 0.0 : a * std::sin(ang);
         }
-    std::vector<double> proj(Nr, 1.0);
+    // the compressed radial kernel at k = 0, and with its factors rounded (either may pass zero at a low rank)
+    std::vector<double> rad(Nr, 1.0), proj(Nr, 1.0);
     for (int r = 0; r < Nr && !h.aniso; ++r) {
-        double v = 0.0, e = 0.0;
+        rad[r] = proj[r] = 0.0;
         for (int s = 0; s < h.rank; ++s) {
             const double u = h.Uk[(size_t)s * n3], c = h.Vr[(size_t)s * Nr + r];
-            e += u * c;
-            v += f32(u) * f32(c);
+            rad[r] += u * c;
+            proj[r] += f32(u) * f32(c);
         }
-        proj[r] = v / e;
     }
     for (int q = 0; q < np; ++q) {
         p.wsig[q] = common * h.wsig[q] * p.excess[q];
-        // VSS: the weight is part of the kernel factor
         const double rounded = h.aniso ? 1.0 : common * f32(p.wsig[q]) / p.wsig[q];
         for (int r = 0; r < Nr; ++r) {
             const double mass = h.aniso ? h.Fa[((size_t)r * np + q) * n3] : h.wsig[q] * h.wr[r] * rho[r];
@@ -164,9 +163,9 @@ void balance_constants(const HostPlan& h, ShiftProgram& p) {
             }
             for (int i = 0; i < X * X * X; ++i) {
                 const int x = i / (X * X), y = i / X % X, z = i % X;
-                g[i] += mass * ex[0][x] * ex[1][y] * ex[2][z];
+                g[i] += rad[r] * mass * ex[0][x] * ex[1][y] * ex[2][z];
                 const double v = mass * rounded * rd[0][x] * rd[1][y] * rd[2][z];
-                gr[i] += v;
+                gr[i] += rad[r] * v;
                 gp[i] += proj[r] * v;
             }
         }
@@ -177,8 +176,13 @@ void balance_constants(const HostPlan& h, ShiftProgram& p) {
         ggr += g[i] * gr[i];
         ggp += g[i] * gp[i];
     }
-    p.balance = lr / lw * (gg / ggr);
-    p.project = lr / lw * (gg / ggp);
+    // rounded constants move it by 1e-7; anything else (a kernel without a gain or a loss) is left alone
+    auto factor = [&](double gain) {
+        const double x = lr / lw * (gg / gain) * common;
+        return (std::fabs(x - 1.0) < 1e-4 ? x : 1.0) / common;
+    };
+    p.balance = factor(ggr);
+    p.project = factor(ggp);
 }
 
 }  // namespace

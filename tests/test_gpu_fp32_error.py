@@ -91,3 +91,15 @@ def test_more_radial_points_than_the_fused_stage_takes(prec, N, N_rho):
     packed = binding.collide_ragged([plan], [0, 0, 0], [i * N ** 3 for i in range(3)], f.reshape(-1), node_gamma=[0.38] * 3,
                                     node_b=[p64.info["b"]] * 3)
     assert (packed.reshape(f.shape).double() - p64.collide(f.double())).norm() < bound
+
+
+@pytest.mark.parametrize("rank", [1, 2, 3, 5])
+@pytest.mark.parametrize("N", [8, 16, 32])
+def test_low_ranks(N, rank):
+    """A radial kernel of a few factors, which passes zero at some radial points: 1e-5 of the loss term."""
+    kw = dict(N=N, L=L_OF[N], gamma=0.38, M=12, N_rho=N, svd_rank=rank)
+    f, g = (torch.from_numpy(W.two_maxwellian(3, N, L_OF[N], seed)[0]).cuda().float() for seed in (11, 12))
+    p32, p64 = binding.Plan(precision="fp32", **kw), binding.Plan(precision="fp64", **kw)
+    bound = 1e-5 * (f.double() * f.double().sum((1, 2, 3), keepdim=True) * (2 * L_OF[N] / N) ** 3).norm()   # b n f bounds the loss
+    assert (p32.collide(f).double() - p64.collide(f.double())).norm() < bound
+    assert (p32.collide2(f, g).double() - p64.collide2(f.double(), g.double())).norm() < 1.5 * bound   # norms of f and g differ
